@@ -51,11 +51,14 @@ struct SplitIn {
   // several matrices side by side whose widths are not whole tiles (0 = not the case): the columns
   // at which the second and third matrix start, and the tiles before them
   unsigned sk_m0, sk_m1, sk_t0, sk_t1;
-  __device__ __forceinline__ int count(int c) const {
+  // several token tiles of sk_tt rows dealt in the same launch: tile = weight tile * sk_zt + row / sk_tt
+  unsigned sk_zt, sk_tt;
+  __device__ __forceinline__ int count(int r, int c) const {
     if (sk_ctas == 0) return n;
     const unsigned sh = 7u + sk_wide, uc = (unsigned)c;
     unsigned tile = uc >> sh;
     if (sk_m0 != 0 && uc >= sk_m0) tile = uc < sk_m1 ? sk_t0 + ((uc - sk_m0) >> sh) : sk_t1 + ((uc - sk_m1) >> sh);
+    if (sk_zt > 1) tile = tile * sk_zt + (unsigned)r / sk_tt;
     const unsigned u0 = tile * sk_kb;
     const unsigned first = ((u0 + 1u) * sk_ctas - 1u) / sk_units;
     const unsigned last = ((u0 + sk_kb) * sk_ctas - 1u) / sk_units;
@@ -63,7 +66,7 @@ struct SplitIn {
   }
   __device__ __forceinline__ float at(int r, int c) const {
     const float *q = p + (size_t)r * ld + c;
-    const int k = count(c);
+    const int k = count(r, c);
     float v = q[0];
     for (int s = 1; s < k; ++s) v += q[(size_t)s * stride];
     return v;

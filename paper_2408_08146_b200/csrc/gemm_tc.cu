@@ -446,7 +446,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
   const unsigned u_hi = (unsigned)(((unsigned long long)(cid + 1) * P.sk_units) / (unsigned)P.sk_ctas);
   const int n_units = (int)(u_hi - u_lo);
   const int n_epi = (int)(blockDim.x >> 5) - 2;
-  const int tt = P.tt;                                   // 128 or 256 tokens per tile
+  const int tt = P.tt;                                   // tokens per tile: a multiple of 32, at most 256
   const int x_part = (tt >> 1) * BK * 2;                  // this CTA's tokens, value or residual rows
   const int stage_bytes = 2 * PAIR_PART_BYTES + 2 * x_part;
   const int n_stages = P.stages;
@@ -495,27 +495,37 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       uint32_t full_even[PAIR_MAX_STAGES];
       for (int s = 0; s < PAIR_MAX_STAGES; ++s) full_even[s] = cluster_addr_of(smem_u32(&full_bar[s]), 0);
       int tile = (int)(u_lo / KB), kb = (int)(u_lo % KB), row0;
-      const CUtensorMap *tmW = tile_map(tile, row0);
+      int tok0 = (tile % P.ztiles) * tt;
+      const CUtensorMap *tmW = tile_map(tile / P.ztiles, row0);
+      auto next_unit = [&]() {
+        if (++kb == KB) {
+          kb = 0;
+          ++tile;
+          tok0 = (tile % P.ztiles) * tt;
+          tmW = tile_map(tile / P.ztiles, row0);
+        }
+      };
       auto load_w = [&](int s) {
         unsigned char *dst = tiles + (size_t)s * stage_bytes;
         if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * (uint32_t)stage_bytes);
         tma_load_2d_pair(tmW, full_even[s], dst, kb * BK, row0 + (int)rank * BM);
         tma_load_2d_pair(tmW, full_even[s], dst + PAIR_PART_BYTES, kb * BK, row0 + 2 * BM + (int)rank * BM);
       };
-      auto load_x = [&](int s, int kbx) {
+      auto load_x = [&](int s, int kbx, int tokx) {
         unsigned char *dst = tiles + (size_t)s * stage_bytes + 2 * PAIR_PART_BYTES;
-        tma_load_2d_pair(&tmX, full_even[s], dst, kbx * BK, (int)rank * (tt >> 1));
-        tma_load_2d_pair(&tmXlo, full_even[s], dst + x_part, kbx * BK, (int)rank * (tt >> 1));
+        tma_load_2d_pair(&tmX, full_even[s], dst, kbx * BK, tokx + (int)rank * (tt >> 1));
+        tma_load_2d_pair(&tmXlo, full_even[s], dst + x_part, kbx * BK, tokx + (int)rank * (tt >> 1));
       };
       // the first stages' weights do not depend on the kernel before this one
-      int kb_first[PAIR_MAX_STAGES];
+      int kb_first[PAIR_MAX_STAGES], tok_first[PAIR_MAX_STAGES];
       for (int it = 0; it < pre; ++it) {
         kb_first[it] = kb;
+        tok_first[it] = tok0;
         load_w(it);
-        if (++kb == KB) { kb = 0; ++tile; tmW = tile_map(tile, row0); }
+        next_unit();
       }
       pdl_wait();
-      for (int it = 0; it < pre; ++it) load_x(it, kb_first[it]);
+      for (int it = 0; it < pre; ++it) load_x(it, kb_first[it], tok_first[it]);
       bool ok = true;
       int s = pre % n_stages;
       uint32_t ph = (uint32_t)(pre / n_stages) & 1u;
@@ -523,8 +533,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
         ok = mbar_wait(&empty_bar[s], ph ^ 1u);
         if (!ok) break;
         load_w(s);
-        load_x(s, kb);
-        if (++kb == KB) { kb = 0; ++tile; tmW = tile_map(tile, row0); }
+        load_x(s, kb, tok0);
+        next_unit();
         if (++s == n_stages) { s = 0; ph ^= 1u; }
       }
       if (!ok) atomicExch(&s_error, 1);
@@ -600,9 +610,10 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       int row0, col_off = 0, n_rows = P.n0;
-      if (tile >= P.tiles1) { row0 = (tile - P.tiles1) * PAIR_ROWS; col_off = P.n0 + P.n1; n_rows = P.n2; }
-      else if (tile >= P.tiles0) { row0 = (tile - P.tiles0) * PAIR_ROWS; col_off = P.n0; n_rows = P.n1; }
-      else row0 = tile * PAIR_ROWS;
+      const int wt = tile / P.ztiles, tok0 = (tile % P.ztiles) * tt;
+      if (wt >= P.tiles1) { row0 = (wt - P.tiles1) * PAIR_ROWS; col_off = P.n0 + P.n1; n_rows = P.n2; }
+      else if (wt >= P.tiles0) { row0 = (wt - P.tiles0) * PAIR_ROWS; col_off = P.n0; n_rows = P.n1; }
+      else row0 = wt * PAIR_ROWS;
       if (dry) n_rows = 0;
       // partial-sum slot = rank of this cluster among the tile's contributors
       const int slot = (int)cid - (int)sk_owner((unsigned)tile * KB, (unsigned)P.sk_ctas, P.sk_units);
@@ -615,7 +626,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
           if (feat < n_rows) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              const int t = c0 + j;
+              const int t = tok0 + c0 + j;
               if (t < P.R) Yp[(size_t)t * P.ldy] = __uint_as_float(v[j]);
             }
           }
@@ -773,9 +784,9 @@ int tc_init_driver(char *err, size_t errlen) {
   }
   // the CTA-pair kernel: shared-memory opt-in, and how many pairs fit on this device at once
   {
-    const size_t smem = (size_t)3 * (2 * PAIR_PART_BYTES + 256 * BK * 2) + 1024;   // = four stages of the 128-token form
+    const size_t smem = (size_t)d.smem_optin - 1024;       // as many stages as fit, see gemm_tc()
     d.pair_clusters = 0;
-    if ((size_t)d.smem_optin >= smem + 1024 &&
+    if ((size_t)d.smem_optin >= (size_t)3 * (2 * PAIR_PART_BYTES + 256 * BK * 2) + 2048 &&
         cudaFuncSetAttribute(gemm_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(2 * (d.num_sms / 2));
@@ -942,7 +953,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   // two CTAs per SM measured 6-7 % faster than 256 rows with one: 7B verify 5.7 against 6.1 ms.)
   bool wide = !g_tune_no_wide && accp && bn == 256 && g_smem_optin - 2048 >= 2 * (2 * W_STAGE_BYTES + x_bytes);
   for (int i = 0; i < m.n && wide; ++i) wide = (m.n_out[i] % (2 * BM)) == 0;
-  // CTA pairs (512 weight rows per cluster, each CTA loading half of the tokens): 113 to 256 tokens
+  // CTA pairs (512 weight rows per cluster, each CTA loading half of the tokens): 113 tokens and more
   // as a pair, stream-K over the clusters that fit on the device at once.  The last tile of a
   // matrix may be ragged (rows beyond the matrix are zero-filled by the loads and not stored).
   // Measured per verification, 7B shapes: 128 rows 5.67-5.85 against 5.78-5.90 ms, 2 x 64 rows
@@ -951,11 +962,17 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   // with 32- and 64-token tiles the pair form measured 13-15 % slower at 16 to 64 rows, where two
   // independent CTAs per SM overlap each other's start and end).
   const int pair_min_rows = g_tune_pair_min > 0 ? g_tune_pair_min : 113;
-  if (pair && R >= pair_min_rows && R <= 256 && !(g_tune_no_pair2 & 1) && g_pair_clusters > 0 && split == 0 &&
+  if (pair && R >= pair_min_rows && !(g_tune_no_pair2 & 1) && g_pair_clusters > 0 && split == 0 &&
       out != nullptr && max_slots >= 2 && m.n <= 3 && (R > 128 || !(g_tune_no_pair2 & 2))) {
     const int q0 = (m.n_out[0] + PAIR_ROWS - 1) / PAIR_ROWS, q1 = m.n > 1 ? (m.n_out[1] + PAIR_ROWS - 1) / PAIR_ROWS : 0,
               q2 = m.n > 2 ? (m.n_out[2] + PAIR_ROWS - 1) / PAIR_ROWS : 0;
-    const int n_tiles = q0 + q1 + q2, KB = K_in / BK;
+    // Token tiles: equal up to 32 rows (the MMA's N follows the tile, so 300 rows cost 320 and not 512),
+    // all in one launch, the token tiles of a weight tile next to one another in the deal of units:
+    // the clusters that share a weight tile then read it at about the same time.
+    const int zt = (R + 255) / 256;
+    int ptt = ((R + zt - 1) / zt + 31) / 32 * 32;
+    if (ptt < 128) ptt = 128;
+    const int n_tiles = (q0 + q1 + q2) * zt, KB = K_in / BK;
     const long long units = (long long)n_tiles * KB;
     long long g = g_pair_clusters;
     if (g > units / 8) g = units / 8;
@@ -966,31 +983,30 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
     };
     while (g > 1 && slots_of(g) > max_slots) --g;
     if (slots_of(g) <= max_slots) {
-      const int ptt = R > 128 ? 256 : 128;
-      P.tt = ptt;
-      P.bn = ptt;
-      P.nbuf = ptt == 128 ? 2 : 1;
-      P.stages = ptt == 128 ? 4 : 3;
       P.tiles0 = q0;
       P.tiles1 = q0 + q1;
       P.n0 = m.n_out[0];
       P.n1 = m.n > 1 ? m.n_out[1] : 0;
       P.n2 = m.n > 2 ? m.n_out[2] : 0;
       P.kblocks = KB;
+      P.tt = ptt;
+      P.bn = ptt;
+      P.nbuf = ptt <= 128 ? 2 : 1;
+      P.ztiles = zt;
       P.sk_ctas = (int)g;
       P.sk_units = (unsigned)units;
       P.split = 1;
       P.split_stride = split_stride;
       P.status = status;
       P.epi_dry = g_tune_epi_dry;
-      CUtensorMap mw[3], mx, mxlo;
+      CUtensorMap mw[3];
       for (int i = 0; i < 3; ++i) {
         const int j = i < m.n ? i : 0;
         if (!get_map(m.W[j], m.n_out[j], K_in, BM, &mw[i])) return cudaErrorInvalidValue;
       }
-      if (!get_map(X.hi, x_rows_alloc, K_in, ptt / 2, &mx)) return cudaErrorInvalidValue;
-      if (!get_map(X.lo, x_rows_alloc, K_in, ptt / 2, &mxlo)) return cudaErrorInvalidValue;
       SplitIn si{Y, slots_of(g), split_stride, ldy, (unsigned)g, (unsigned)units, (unsigned)KB, 2u};
+      si.sk_zt = (unsigned)zt;
+      si.sk_tt = (unsigned)ptt;
       bool ragged = false;
       for (int i = 0; i + 1 < m.n; ++i) ragged = ragged || (m.n_out[i] % PAIR_ROWS) != 0;
       if (ragged) {
@@ -1000,10 +1016,15 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
         si.sk_t1 = (unsigned)(q0 + q1);
       }
       *out = si;
+      const int stage = 2 * PAIR_PART_BYTES + ptt * BK * 2;
+      P.stages = (g_smem_optin - 2048) / stage < PAIR_MAX_STAGES ? (g_smem_optin - 2048) / stage : PAIR_MAX_STAGES;
+      CUtensorMap mx, mxlo;
+      if (!get_map(X.hi, x_rows_alloc, K_in, ptt / 2, &mx)) return cudaErrorInvalidValue;
+      if (!get_map(X.lo, x_rows_alloc, K_in, ptt / 2, &mxlo)) return cudaErrorInvalidValue;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)(2 * g));
       cfg.blockDim = dim3(PAIR_THREADS);
-      cfg.dynamicSmemBytes = (size_t)P.stages * (2 * PAIR_PART_BYTES + ptt * BK * 2) + 1024;
+      cfg.dynamicSmemBytes = (size_t)P.stages * stage + 1024;
       cfg.stream = L.st;
       cudaLaunchAttribute attr[2];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

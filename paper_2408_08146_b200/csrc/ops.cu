@@ -97,7 +97,7 @@ __global__ void row_epilogue_kernel(int mode, float *__restrict__ x, SplitIn P,
 template <int AHEAD = 8>
 __device__ __forceinline__ float4 split_sum4(const SplitIn &P, int r, int c) {
   const float *q = P.p + (size_t)r * P.ld + c;
-  const int k = P.count(c);
+  const int k = P.count(r, c);
   float4 u[AHEAD];
 #pragma unroll
   for (int s = 0; s < AHEAD; ++s)
@@ -376,7 +376,7 @@ __global__ void rope_kv_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__
 // one head with 8-byte loads.
 __device__ __forceinline__ float2 split_sum2(const SplitIn &P, int r, int c) {
   const float *q = P.p + (size_t)r * P.ld + c;
-  const int k = P.count(c);
+  const int k = P.count(r, c);
   float2 u[4];
 #pragma unroll
   for (int s = 0; s < 4; ++s)

@@ -97,3 +97,39 @@ def test_cta_pair_form_and_one_cta_form_agree(shape):
     finally:
         lib.koala_set_tuning(17, 0)
     assert np.abs(outs[0] - outs[1]).max() <= 4e-5 * np.sqrt(K) + 1e-6
+
+
+@pytest.mark.parametrize("shape", [(140, 1024, 512), (257, 1536, 512), (300, 700 * 16, 256), (512, 1024, 4096),
+                                   (1000, 640, 1024), (600, 512, 11008)])
+def test_cta_pairs_with_token_tiles_of_any_width(shape):
+    """More than 128 rows: token tiles of a multiple of 32 rows (ragged last tile), several of them sharing
+    the deal of K blocks; the consumer's count of partial sums follows the row and the column."""
+    M, N, K = shape
+    xf = normal_tensor(13, f"xf{M}.{N}.{K}", (M, K), 1.0, 0.0, torch.float32, "cuda:0")
+    w = normal_tensor(14, f"w{M}.{N}.{K}", (N, K), 0.02, 0.0, torch.bfloat16, "cuda:0")
+    hi = xf.to(torch.bfloat16)
+    lo = (xf - hi.float()).to(torch.bfloat16)
+    ref = (hi.double() + lo.double()).cpu().numpy() @ w.double().cpu().numpy().T
+    status = torch.zeros(1, dtype=torch.int32, device="cuda:0")
+    y = koala_gemm_bf16(hi, w, True, 0, status, x_lo=lo)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert np.abs(y.cpu().numpy() - ref).max() <= 2e-5 * np.sqrt(K) + 1e-6      # fp32 accumulation of K products
+
+
+@pytest.mark.parametrize("shape", [(1, 9, 4), (2, 8, 128), (3, 250, 68), (4, 17, 772), (9, 64, 1028), (17, 33, 2052),
+                                   (31, 2500, 256), (5, 20, 66)])
+@pytest.mark.parametrize("pair", [False, True])
+def test_cuda_core_gemm_of_few_rows(shape, pair):
+    """Rows per warp 2 to 16, K with and without a tail past the pre-read weights, K not a multiple of four
+    (the staged kernel), features that leave the last block partly empty."""
+    M, N, K = shape
+    xf = normal_tensor(15, f"xf{M}.{N}.{K}", (M, K), 1.0, 0.0, torch.float32, "cuda:0")
+    w = normal_tensor(16, f"w{M}.{N}.{K}", (N, K), 0.02, 0.0, torch.bfloat16, "cuda:0")
+    hi = xf.to(torch.bfloat16)
+    lo = (xf - hi.float()).to(torch.bfloat16) if pair else None
+    full = hi.double() + lo.double() if pair else hi.double()
+    y = koala_gemm_bf16(hi, w, False, 0, None, x_lo=lo)
+    torch.cuda.synchronize()
+    ref = full.cpu().numpy() @ w.double().cpu().numpy().T
+    assert np.abs(y.cpu().numpy() - ref).max() <= 2e-5 * np.sqrt(K) + 1e-6

@@ -120,3 +120,17 @@ def test_sampling_needs_chain_drafts():
         eng.koala_set_sampling(torch.zeros(1, 4, device=DEV))
     assert e.value.code == 1
     eng.close()
+
+
+@pytest.mark.parametrize("V", [1000, 1500, 3100])
+def test_draws_over_vocabularies_that_do_not_fill_the_segments(V):
+    """1024 threads draw from V ids in segments of ceil(V / 1024): threads without ids, a short last segment."""
+    cfg = TINY_EAGLE.with_(topk=1, D=3, N=4, S_max=128, B=2, prompt_len=24, prompt_len_min=20, seed=11, V=V)
+    eng, orc, _ = make_pair(cfg)
+    pr = prompts(cfg)
+    eng.prefill(pr, cfg.N)
+    orc.prefill(pr, cfg.N)
+    for it in range(3):
+        _iteration(cfg, eng, orc, 300 + it, True)
+    assert eng.device_status() == 0
+    eng.close()
