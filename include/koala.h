@@ -180,6 +180,15 @@ int koala_expand_tree(koala_ctx *ctx, int pass);
  * tree built by koala_expand_tree. */
 int koala_verify(koala_ctx *ctx, const koala_tree *tree);
 
+/* Prompt ingestion in forwards wider than a tree.  Every prompt is cut into n_parts equal parts (the
+ * first len % n_parts of them one token longer); all parts but the last are taken into the caches as if
+ * each had been verified as a chain and accepted in full, followed, for an EAGLE-style head, by
+ * koala_draft(0) with the next prompt token as root: target and head caches, seq_len and the acceptance
+ * counters are as after those calls.  Up to 1024 tokens go through one forward and no logits are formed.
+ * The caller continues with koala_verify(chain of the last part) and koala_accept.
+ * tok: DEVICE [B][stride] prompts; len: HOST [B], copied. */
+int koala_ingest(koala_ctx *ctx, const int32_t *tok, int32_t stride, const int32_t *len, int32_t n_parts);
+
 /* Greedy acceptance (Section 4.1: a draft token is kept only if it equals the target's greedy
  * token) of the longest matching root path, then KV compaction: the accepted nodes' K/V move to
  * slots S..S+l-1 of every target layer and seq_len += l.  out_tokens[b][0..l-1] = the path's

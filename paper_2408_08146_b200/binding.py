@@ -122,6 +122,8 @@ def load_library(rebuild: bool = False) -> C.CDLL:
     lib.koala_poll.argtypes = [C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_int)]
     lib.koala_last_error.restype = C.c_char_p
     lib.koala_last_error.argtypes = [C.c_void_p]
+    lib.koala_ingest.restype = C.c_int
+    lib.koala_ingest.argtypes = [C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_int32]
     lib.koala_destroy.restype = None
     lib.koala_destroy.argtypes = [C.c_void_p]
     lib.koala_gemm_x_rows.restype = C.c_int
@@ -380,20 +382,22 @@ class Koala:
 
     def prefill(self, prompts: Sequence[Sequence[int]], chunk: int):
         """Ingests the prompts as chain trees with full forced acceptance (EAGLE-style heads also
-        run draft pass 0 over every chunk but the last, with the next prompt token as root)."""
+        run draft pass 0 over every chunk but the last, with the next prompt token as root); the
+        chunks before the last go through koala_ingest, many at a time."""
         c = self.cfg
         chunk = min(chunk, c.N)
         n_chunks = max(-(-len(p) // chunk) for p in prompts)
-        parts = [np.array_split(np.asarray(p, dtype=np.int64), n_chunks) for p in prompts]
-        bufs = self.buffers()
-        for ci in range(n_chunks):
-            tree = self.chain_tree([parts[b][ci] for b in range(c.B)])
-            self.koala_verify(tree)
-            self.koala_accept(tree[2])
-            if c.head_kind == KOALA_EAGLE and ci + 1 < n_chunks:
-                nxt = torch.tensor([int(parts[b][ci + 1][0]) for b in range(c.B)], dtype=torch.int32)
-                bufs["root_tok"].copy_(nxt.to(self.dev))
-                self.koala_draft(0)
+        lens = [len(p) for p in prompts]
+        last = [n // n_chunks for n in lens]             # the last of n_chunks equal parts
+        if n_chunks > 1:
+            host = np.zeros((c.B, max(lens)), np.int32)
+            for b, p in enumerate(prompts):
+                host[b, :lens[b]] = np.asarray(p)
+            toks = torch.from_numpy(host).to(self.dev)
+            self._check(self.lib.koala_ingest(self._ctx, toks.data_ptr(), toks.shape[1], _i32_array(lens), n_chunks))
+        tree = self.chain_tree([np.asarray(p)[lens[b] - last[b]:] for b, p in enumerate(prompts)])
+        self.koala_verify(tree)
+        self.koala_accept(tree[2])
 
     def step(self, forced_len: Optional[torch.Tensor] = None):
         """One whole iteration: D x (draft, expand_tree), verify, accept."""

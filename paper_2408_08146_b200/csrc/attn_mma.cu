@@ -93,8 +93,9 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
   const int n_tiles = (kv_len + TILE - 1) / TILE;
   const int tile_lo = (int)(((long long)n_tiles * c) / chunks);
   const int tile_hi = (int)(((long long)n_tiles * (c + 1)) / chunks);
-  const bf16 *kb = kc + ((size_t)b * n_heads + h) * S_max * DH;
-  const bf16 *vb = vc + ((size_t)b * n_heads + h) * S_max * DH;
+  const int cb = plan.cache_of(b);
+  const bf16 *kb = kc + ((size_t)cb * n_heads + h) * S_max * DH;
+  const bf16 *vb = vc + ((size_t)cb * n_heads + h) * S_max * DH;
   const uint32_t sbase = smem_addr(smem);
 
   auto load_tile = [&](int tile, int buf) {

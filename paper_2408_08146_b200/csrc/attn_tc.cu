@@ -252,7 +252,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   if (warp == 4) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      const int y0 = (b * P.n_heads + h) * P.S_max;
+      const int y0 = (P.plan.cache_of(b) * P.n_heads + h) * P.S_max;
       bool ok = true;
       int issued = 0;
       auto request_l2 = [&](int t) {
@@ -677,7 +677,7 @@ bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max) {
 }
 
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
-                              RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks,
+                              RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
                               int *status) {
   static SmemOptIn optin_dup, optin_full;
   const size_t smem = (size_t)SMEM_BYTES + 1024;
@@ -686,7 +686,7 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
   if (e != cudaSuccess) return e;
   if (chunks != 1 && chunks != 2 && chunks != 4 && chunks != 8) return cudaErrorInvalidValue;
   if (q_pair.hi == nullptr || q_pair.lo == nullptr) return cudaErrorInvalidValue;
-  const long long rows = (long long)B * n_heads * S_max;
+  const long long rows = (long long)cache_seqs * n_heads * S_max;
   if (rows > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int H = n_heads * DH;
   CUtensorMap tmQh, tmQl, tmK, tmV;

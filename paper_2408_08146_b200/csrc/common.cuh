@@ -88,6 +88,13 @@ struct RowScale {
   }
 };
 
+// Where row r of a forward goes in a per-node buffer: a forward runs `rows` rows per sequence, the
+// buffer holds `n` per sequence (rows == 0: the two are the same).
+struct RowMap {
+  int rows, n;
+  __device__ __forceinline__ int operator()(int r) const { return rows == 0 ? r : (r / rows) * n + r % rows; }
+};
+
 // Per-row plan of one forward over R rows (rows_per_seq consecutive rows per sequence).
 struct RowPlan {
   const int32_t *pos;     // [R] RoPE position
@@ -96,6 +103,8 @@ struct RowPlan {
   const int32_t *ctx_len; // [B] slots 0..ctx_len-1 are visible to every row of the sequence
   const int32_t *kv_len;  // [B] slots in use after this forward's writes
   const float2 *rope;     // [R][head_dim/2] (cos, sin)
+  const int32_t *seq;     // cache sequence of each group of rows_per_seq rows; null = the group's own index
+  __device__ __forceinline__ int cache_of(int group) const { return seq == nullptr ? group : seq[group]; }
 };
 
 extern unsigned long long g_launches;   // kernels launched by the library (defined in koala_api.cu)
@@ -161,9 +170,9 @@ struct GemmMats {         // up to three weight matrices sharing K_in, outputs c
 cudaError_t embed_norm(Launch L, int dtype, const int32_t *tok, const void *E, const void *g,
                        float *x, Operand xn, int R, int H, int V, float eps);
 // mode 0: v = x + sum(P); 1: v = sum(P) + bias; 2: v = x + SiLU(sum(P) + bias).  x <- v;
-// n = g ? rmsnorm(v) * g : v;  xn <- T(n) if xn;  out_f32 <- n if out_f32.
+// n = g ? rmsnorm(v) * g : v;  xn <- T(n) if xn;  out_f32[out_map(row)] <- n if out_f32.
 cudaError_t row_epilogue(Launch L, int dtype, int mode, float *x, SplitIn P, const void *bias,
-                         const void *g, Operand xn, float *out_f32, int R, int H, float eps);
+                         const void *g, Operand xn, float *out_f32, RowMap out_map, int R, int H, float eps);
 cudaError_t eagle_concat(Launch L, int dtype, const float *feat_src, const int32_t *row_src,
                          const int32_t *row_tok, const void *E, Operand cat, int R, int H, int V);
 // x <- x + sum(P); xg <- T(x * g) (not normalised); sumsq[r][chunk] <- partial sums of x^2 over
@@ -191,7 +200,8 @@ cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, in
 cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_cache,
                            const void *v_cache, RowPlan plan, Operand out, int R, int rows_per_seq,
                            int B, int n_heads, int head_dim, int S_max);
-cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, int R, int V);
+// row r of the forward: logits row and output index map(r)
+cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, RowMap map, int R, int V);
 cudaError_t topk_logp(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k);
 // dst[r] = T(src[row_src ? row_src[r] : r]); optionally dst32[r * dst32_stride] = the same row in fp32
 cudaError_t cast_rows(Launch L, int dtype, const float *src, const int32_t *row_src, Operand dst,
@@ -210,21 +220,22 @@ cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, co
 int attn_tc_chunks(int B, int n_heads, int S_max, int num_sms);
 bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max);
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
-                              RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks,
+                              RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
                               int *status);
 
 // gemm_simt.cu : Y[R][sum n_out] (fp32, ld ldy) = X[R][K_in] * W^T, X and W of `dtype`
 cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int R, float *Y,
-                      int ldy);
+                      int ldy, RowMap ymap);
 
 // gemm_tc.cu : bf16 tensor-core path; writes `split` partial matrices `split_stride` apart.
 int tc_init_driver(char *err, size_t errlen);   // 0 on success
 bool tc_supported(const GemmMats &m, int K_in);
 int tc_default_split(int n_tiles, int kblocks, int tokens);
+// Row r of the product is row ymap(r) of Y (not the identity only with split == 1).
 // split >= 1: classic split-K; split == 0: automatic (stream-K where it applies).  `max_slots`
 // bounds the partial matrices written; *out describes them for the consumer.
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
-                    float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
+                    float *Y, int ldy, RowMap ymap, int split, size_t split_stride, int *status, int max_slots,
                     SplitIn *out);
 
 // layer_tc.cu : several GEMMs of a decoder layer and the row-wise steps between them in one
@@ -282,7 +293,21 @@ struct TreeBufs {
   unsigned long long *alpha_hits, *alpha_trials;   // [128] position-wise acceptance counters
   float *pend_hid;
 };
+constexpr int INGEST_MAX_BLOCKS = 64;
+// Prompt tokens of one forward, cut into blocks of `q` consecutive tokens of one sequence: block v holds
+// tokens start[v] .. start[v] + count[v] - 1 of sequence seq[v]; its rows are v * q ...
+struct IngestBlocks {
+  int n, q;
+  int32_t start[INGEST_MAX_BLOCKS];
+  int16_t seq[INGEST_MAX_BLOCKS], count[INGEST_MAX_BLOCKS];
+};
+// Prompt of each sequence: len tokens in n_parts equal parts, all but the last of which are ingested.
+struct IngestLens {
+  int n_parts;
+  int32_t len[64], count[64];
+};
 struct PlanBufs {
+  int32_t *seq;           // [INGEST_MAX_BLOCKS]
   int32_t *pos, *slot, *ctx_len, *kv_len, *row_src, *row_tok, *last_row;
   uint64_t *mask;
   float2 *rope;
@@ -290,8 +315,21 @@ struct PlanBufs {
 cudaError_t tree_from_caller(Launch L, TreeBufs t, const int32_t *tok, const int32_t *parent,
                              const int32_t *n_nodes, int stride, int B, int N, int *status);
 cudaError_t tree_ancestors(Launch L, TreeBufs t, int B, int N);
-cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
+// rows <= N: plan rows per sequence (row b * rows + u is node u of sequence b)
+cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows,
                         int head_dim, float rope_base, int S_max, int *status);
+// Plan of a forward over prompt blocks (chains on top of their own earlier tokens); row_tok = the token
+// `shift` places further on (0: the row's own; 1: the one the draft head pairs with it).
+cudaError_t plan_ingest(Launch L, PlanBufs p, IngestBlocks k, const int32_t *tok, int stride, int shift,
+                        const int32_t *seq_len, int head_dim, float rope_base, int S_max, int *status);
+// Rows of a forward whose hidden state stays in the pending buffer: pend_hid row dst[i] <- hid row src[i].
+struct IngestKeep {
+  int n;
+  int32_t src[64], dst[64];
+};
+cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, int H);
+// seq_len += count; acceptance counters as if every ingested part had been accepted as a chain
+cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, int32_t *seq_len, int B);
 cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
                         int rows, int head_dim, float rope_base, int S_max, int *status);
 cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k,

@@ -20,7 +20,7 @@ unsigned long long g_launches = 0;
 
 namespace {
 
-enum Phase { PH_READY = 0, PH_DRAFTED, PH_EXPANDED, PH_TREE, PH_VERIFIED };
+enum Phase { PH_READY = 0, PH_DRAFTED, PH_EXPANDED, PH_TREE, PH_VERIFIED, PH_INGESTED };
 
 struct LayerW {
   const void *attn_norm, *wq, *wk, *wv, *wo, *ffn_norm, *wg, *wu, *wd;
@@ -48,6 +48,11 @@ struct Carver {
 };
 
 constexpr int MAX_SPLIT = 12;     // partial-sum matrices the workspace holds per GEMM
+// Prompt tokens per forward of koala_ingest: enough for the multiplies to be bound by the tensor cores
+// (256-token tiles, four of them), few enough for the workspace to stay small (four partial-sum
+// matrices of that many rows; 7B shape: 0.36 GB).
+constexpr int INGEST_ROWS = 1024;
+constexpr int INGEST_SPLIT = 4;
 
 }  // namespace
 
@@ -61,7 +66,8 @@ struct koala_ctx {
   void *tk, *tv, *dk, *dv;
   int32_t *seq_len;
   // derived sizes
-  int M, Mp, pool, draft_rows_max, esz;
+  int M, Mp, ingest_rows, pool, draft_rows_max, esz;    // Mp: rows of the forward's operands (whole token tiles)
+  size_t p_floats;        // capacity of P
   size_t pcols;           // widest GEMM output
   // workspace
   float *attn_part;
@@ -87,6 +93,7 @@ struct koala_ctx {
   Phase phase;
   int last_pass, pend_cap, draft_rows, expand_mode;
   bool last_tree_from_caller;
+  int ingest_blocks;      // > 0 while koala_ingest enqueues a forward: its groups of rows (else one group per sequence)
   int *host_status;       // pinned
   cudaEvent_t poll_ev;
   bool poll_pending;
@@ -162,17 +169,22 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   if (cfg.head_kind == KOALA_MEDUSA && cfg.n_medusa_heads * B > draft_rows) draft_rows = cfg.n_medusa_heads * B;
   int rows = M > draft_rows ? M : draft_rows;
   // padded row count: the tensor-core GEMM reads whole token tiles (up to 256 rows) of its input
-  const int Mp = (int)align_up((size_t)rows + 16, rows > 128 ? 256 : 16);
+  const int Mt = (int)align_up((size_t)rows + 16, rows > 128 ? 256 : 16);      // a tree's rows
+  const size_t held = (size_t)B * (cfg.S_max > 0 ? cfg.S_max : 1);
+  const int wide = (int)align_up(held < (size_t)INGEST_ROWS ? held : (size_t)INGEST_ROWS, held > 128 ? 256 : 16);
+  const int Mp = Mt > wide ? Mt : wide;
+  c->ingest_rows = wide;
   const int pool = cfg.head_kind == KOALA_EAGLE ? k + (cfg.D - 1) * k * k : k;
   const size_t pcols = (size_t)(3 * H > 2 * F ? 3 * H : 2 * F);
   const size_t esz = cfg.dtype == KOALA_FP32 ? 4 : 2;
   c->M = M; c->Mp = Mp; c->pool = pool; c->draft_rows_max = draft_rows; c->esz = (int)esz; c->pcols = pcols;
   c->x = w.take<float>((size_t)Mp * H);
   c->qbuf = w.take<float>((size_t)Mp * H);
-  c->P = w.take<float>((size_t)MAX_SPLIT * Mp * pcols);
-  c->verify_logits = w.take<float>((size_t)Mp * V);
+  c->p_floats = (size_t)(MAX_SPLIT * Mt > INGEST_SPLIT * wide ? MAX_SPLIT * Mt : INGEST_SPLIT * wide) * pcols;
+  c->P = w.take<float>(c->p_floats);
+  c->verify_logits = w.take<float>((size_t)Mt * V);
   c->draft_logits = w.take<float>((size_t)(draft_rows + 16) * V);
-  c->verify_hid = w.take<float>((size_t)Mp * H);
+  c->verify_hid = w.take<float>((size_t)Mt * H);
   c->feat[0] = w.take<float>((size_t)(B * k + 16) * H);
   c->feat[1] = w.take<float>((size_t)(B * k + 16) * H);
   c->mx = w.take<float>((size_t)Mp * H);
@@ -197,12 +209,12 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   c->lmin = operand(H);
   c->attn_chunks = 16;     // largest chunk count any launch may choose
   c->attn_part = (cfg.dtype == KOALA_BF16 && cfg.head_dim == 128)
-                     ? w.take<float>(attn_mma_scratch_floats(Mp, cfg.n_heads, c->attn_chunks))
+                     ? w.take<float>(attn_mma_scratch_floats(Mt, cfg.n_heads, c->attn_chunks))
                      : nullptr;
   c->sumsq[0] = w.take<float>((size_t)Mp * 32);
   c->sumsq[1] = w.take<float>((size_t)Mp * 32);
   c->layer_sync = w.take<unsigned>(LAYER_SYNC_WORDS);
-  c->verify_tgt = w.take<int32_t>(Mp);
+  c->verify_tgt = w.take<int32_t>(Mt);
   c->s_parent = w.take<int32_t>(N);
   c->s_level = w.take<int32_t>(N);
   c->s_rank = w.take<int32_t>(N);
@@ -235,10 +247,11 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   t.alpha_trials = w.take<unsigned long long>(128);
   t.pend_hid = w.take<float>((size_t)M * H);
   PlanBufs &p = c->p;
+  p.seq = w.take<int32_t>(INGEST_MAX_BLOCKS);
   p.pos = w.take<int32_t>(Mp);
   p.slot = w.take<int32_t>(Mp);
-  p.ctx_len = w.take<int32_t>(B);
-  p.kv_len = w.take<int32_t>(B);
+  p.ctx_len = w.take<int32_t>(B > INGEST_MAX_BLOCKS ? B : INGEST_MAX_BLOCKS);
+  p.kv_len = w.take<int32_t>(B > INGEST_MAX_BLOCKS ? B : INGEST_MAX_BLOCKS);
   p.row_src = w.take<int32_t>(Mp);
   p.row_tok = w.take<int32_t>(Mp);
   p.last_row = w.take<int32_t>(B);
@@ -277,29 +290,31 @@ void time_end(koala_ctx *c, int i) {
 }
 
 RowPlan row_plan(koala_ctx *c) {
-  return RowPlan{c->p.pos, c->p.slot, c->p.mask, c->p.ctx_len, c->p.kv_len, c->p.rope};
+  return RowPlan{c->p.pos, c->p.slot, c->p.mask, c->p.ctx_len, c->p.kv_len, c->p.rope,
+                 c->ingest_blocks > 0 ? c->p.seq : nullptr};
 }
 
 // Y = X * [W...]^T as a (possibly split) fp32 result in the partial buffer, or directly into
 // `direct` (ld = ld_direct) when given.
 int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct, int ld_direct,
-            SplitIn *out) {
+            SplitIn *out, RowMap ymap = RowMap{0, 0}) {
   int ncols = 0;
   for (int i = 0; i < m.n; ++i) ncols += m.n_out[i];
   float *Y = direct ? direct : c->P + c->p_off;
   const int ld = direct ? ld_direct : ncols;
   const uint64_t wbytes = (uint64_t)ncols * K_in * c->esz;
   if (c->use_tc && c->cfg.dtype == KOALA_BF16 && tc_supported(m, K_in)) {
-    const size_t stride = (size_t)c->Mp * ld;
+    const size_t stride = align_up((size_t)R, 16) * ld;
+    const size_t fit = (c->p_slots > 0 ? (size_t)c->p_slots : c->p_floats / stride);
+    const int slots = fit < (size_t)MAX_SPLIT ? (int)fit : MAX_SPLIT;
     const int tb = time_begin(c, KOALA_CLS_GEMM_TC, wbytes);
     SplitIn res;
-    CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, direct ? 1 : 0, stride, c->status,
-                   c->p_slots > 0 ? c->p_slots : MAX_SPLIT, &res));
+    CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, ymap, direct ? 1 : 0, stride, c->status, slots, &res));
     time_end(c, tb);
     if (out) *out = res;
   } else {
     const int tb = time_begin(c, KOALA_CLS_GEMM_SIMT, wbytes);
-    CU_TRY(gemm_simt(LN(c), c->cfg.dtype, X, m, K_in, R, Y, ld));
+    CU_TRY(gemm_simt(LN(c), c->cfg.dtype, X, m, K_in, R, Y, ld, ymap));
     time_end(c, tb);
     if (out) *out = SplitIn{Y, 1, 0, ld, 0u, 0u, 0u};
   }
@@ -316,17 +331,18 @@ int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct,
 // cache, writes the O projection's operand pair.
 int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq) {
   const koala_config &g = c->cfg;
+  const int groups = c->ingest_blocks > 0 ? c->ingest_blocks : g.B;
   const int ta = time_begin(c, KOALA_CLS_ATTENTION, 0);
   if (c->use_tc && g.dtype == KOALA_BF16 && c->qpair.lo != nullptr &&
       attn_tc_supported(rows_per_seq, g.head_dim, g.S_max)) {
-    CU_TRY(tree_attention_tc(LN(c), c->qpair, c->Mp, kc, vc, row_plan(c), c->attn_out, rows_per_seq, g.B, g.n_heads,
-                             g.S_max, attn_tc_chunks(g.B, g.n_heads, g.S_max, 148), c->status));
+    CU_TRY(tree_attention_tc(LN(c), c->qpair, c->Mp, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups,
+                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, 148), c->status));
   } else if (c->use_tc && g.head_dim == 128 && c->attn_part != nullptr && rows_per_seq <= 128) {
     CU_TRY(tree_attention_mma(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, c->attn_part, rows_per_seq,
-                              g.B, g.n_heads, g.S_max,
-                              attn_mma_chunks(g.B, g.n_heads, rows_per_seq, g.S_max, 148)));
+                              groups, g.n_heads, g.S_max,
+                              c->ingest_blocks > 0 ? 1 : attn_mma_chunks(g.B, g.n_heads, rows_per_seq, g.S_max, 148)));
   } else {
-    CU_TRY(tree_attention(LN(c), g.dtype, c->qbuf, kc, vc, row_plan(c), c->attn_out, R, rows_per_seq, g.B,
+    CU_TRY(tree_attention(LN(c), g.dtype, c->qbuf, kc, vc, row_plan(c), c->attn_out, R, rows_per_seq, groups,
                           g.n_heads, g.head_dim, g.S_max));
   }
   time_end(c, ta);
@@ -340,19 +356,22 @@ int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq) {
 // of the attention block: normalised, or x * gain with the scale still pending in c->pending.
 // On exit x is updated; if `defer` the next layer's input is left in c->xn as x * next_g with its
 // scale pending, otherwise `next_xn` holds T(rmsnorm(x) * next_g) (or T(x) if next_g is null) and
-// `out_f32` optionally the same in fp32.
+// `out_f32` optionally the same in fp32.  kv_only: the layer's keys and values are all that is wanted.
 int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows_per_seq,
-              const void *next_g, Operand next_xn, float *out_f32, bool defer) {
+              const void *next_g, Operand next_xn, float *out_f32, RowMap out_map, bool defer,
+              bool kv_only = false) {
   const koala_config &g = c->cfg;
   const int H = g.H, F = g.F;
   const bool can_defer = (H % 4) == 0 && H <= 8192;
   const RowScale none{nullptr, 0, 0.f, 0.f};
+  const RowMap same{0, 0};
   SplitIn s;
   GemmMats qkv{{w.wq, w.wk, w.wv}, {H, H, H}, 3};
   K_TRY(do_gemm(c, c->xn, H, qkv, R, nullptr, 0, &s));
   CU_TRY(rope_kv_write(LN(c), g.dtype, s, c->pending, row_plan(c), c->qbuf, c->qpair, kc, vc, R, rows_per_seq, g.n_heads,
                        g.head_dim, g.S_max));
   c->pending = none;
+  if (kv_only) return KOALA_OK;
   K_TRY(run_attention(c, kc, vc, R, rows_per_seq));
   GemmMats o{{w.wo, nullptr, nullptr}, {H, 0, 0}, 1};
   K_TRY(do_gemm(c, c->attn_out, H, o, R, nullptr, 0, &s));
@@ -361,7 +380,7 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
     CU_TRY(row_update(LN(c), g.dtype, c->x, s, w.ffn_norm, c->xn, c->sumsq[0], R, H));
     ffn = RowScale{c->sumsq[0], (H + 1023) / 1024, 1.f / (float)H, g.rms_eps};
   } else {
-    CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, w.ffn_norm, c->xn, nullptr, R, H, g.rms_eps));
+    CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, w.ffn_norm, c->xn, nullptr, same, R, H, g.rms_eps));
   }
   GemmMats gu{{w.wg, w.wu, nullptr}, {F, F, 0}, 2};
   K_TRY(do_gemm(c, c->xn, H, gu, R, nullptr, 0, &s));
@@ -372,31 +391,32 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
     CU_TRY(row_update(LN(c), g.dtype, c->x, s, next_g, c->xn, c->sumsq[1], R, H));
     c->pending = RowScale{c->sumsq[1], (H + 1023) / 1024, 1.f / (float)H, g.rms_eps};
   } else {
-    CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, next_g, next_xn, out_f32, R, H, g.rms_eps));
+    CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, next_g, next_xn, out_f32, out_map, R, H, g.rms_eps));
   }
   return KOALA_OK;
 }
 
 
 // n_layers pre-norm decoder layers over R rows.  On entry x holds the residual stream and c->xn the
-// first layer's input (normalised, or x * gain with its scale pending in c->pending).  After the
+// first layer's input (normalised, or x * gain with its scale pending in c->pending).  last_kv_only: the
+// last layer only writes its keys and values (prompt positions whose hidden state nobody reads).  After the
 // last layer the output is rmsnorm(x) * final_g (or x if final_g is null) as an operand in
 // `final_xn` and, optionally, in fp32 in `out_f32`.
 // Where the persistent layer kernel applies (bf16 pairs, at most 128 rows, head_dim 128, matrices
 // of whole 128-row tiles) a layer is two launches: attention, and one launch that runs
 // O -> residual -> gate/up -> SwiGLU -> down -> residual -> the next layer's Q/K/V -> rotary/cache.
 int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, void *kbase, void *vbase, int R,
-               int rows_per_seq, const void *final_g, Operand final_xn, float *out_f32) {
+               int rows_per_seq, const void *final_g, Operand final_xn, float *out_f32, RowMap out_map,
+               bool last_kv_only = false) {
   const koala_config &g = c->cfg;
   const int H = g.H, F = g.F;
   const size_t le = kv_layer_elems(g) * c->esz;
   auto kc_of = [&](int l) { return (void *)((unsigned char *)kbase + (size_t)l * le); };
   auto vc_of = [&](int l) { return (void *)((unsigned char *)vbase + (size_t)l * le); };
   bool streamed = c->stream_layers && g.dtype == KOALA_BF16 && c->pair && g.head_dim == 128 && R <= 128 &&
-                  c->qpair.lo != nullptr && n_layers > 0;
+                  c->qpair.lo != nullptr && n_layers > 0 && c->ingest_blocks == 0;
   LayerJob job;
-  const size_t stride = (size_t)c->Mp * c->pcols;     // one partial-sum matrix of the widest GEMM
-  auto base_job = [&]() {
+    auto base_job = [&]() {
     memset(&job, 0, sizeof(job));
     job.R = R;
     job.x_rows_alloc = c->Mp;
@@ -412,10 +432,9 @@ int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, vo
     LayerPhaseJob &j = job.ph[i];
     int ncols = 0;
     for (int q = 0; q < m.n; ++q) ncols += m.n_out[q];
-    j.X = X; j.K_in = K_in; j.m = m; j.Y = c->P; j.ldy = ncols; j.split_stride = (size_t)c->Mp * ncols;
+    j.X = X; j.K_in = K_in; j.m = m; j.Y = c->P; j.ldy = ncols; j.split_stride = align_up((size_t)R, 16) * ncols;
     j.max_slots = MAX_SPLIT; j.post = post;
     j.sc = RowScale{nullptr, 0, 0.f, 0.f};
-    (void)stride;
     return j;
   };
   const int chunks = (H + 511) / 512;
@@ -451,7 +470,7 @@ int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, vo
     for (int l = 0; l < n_layers; ++l) {
       const bool last = l == n_layers - 1;
       K_TRY(run_layer(c, layers[l], kc_of(l), vc_of(l), R, rows_per_seq, last ? final_g : layers[l + 1].attn_norm,
-                      last ? final_xn : c->xn, last ? out_f32 : nullptr, !last));
+                      last ? final_xn : c->xn, last ? out_f32 : nullptr, out_map, !last, last && last_kv_only));
     }
     return KOALA_OK;
   }
@@ -492,9 +511,49 @@ int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, vo
     CU_TRY(layer_stream(LN(c), job, c->layer_sync, c->layer_use, c->status, outs));
     time_end(c, tb);
     if (last)
-      CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, outs[2], nullptr, final_g, final_xn, out_f32, R, H, g.rms_eps));
+      CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, outs[2], nullptr, final_g, final_xn, out_f32, out_map, R, H, g.rms_eps));
   }
   return KOALA_OK;
+}
+
+// x and the first target layer's input from the plan's tokens
+int embed_rows(koala_ctx *c, int R) {
+  const koala_config &g = c->cfg;
+  if ((g.H % 4) == 0 && g.H <= 8192) {
+    // the embedding rows in the deferred form: their RMSNorm scale is applied by the first layer's consumer
+    CU_TRY(embed_update(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, c->sumsq[1],
+                        R, g.H, g.V));
+    c->pending = RowScale{c->sumsq[1], (g.H + 1023) / 1024, 1.f / (float)g.H, g.rms_eps};
+  } else {
+    CU_TRY(embed_norm(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, R, g.H, g.V,
+                      g.rms_eps));
+  }
+  return KOALA_OK;
+}
+
+// One forward of the target over prompt blocks, then of an EAGLE-style head over the same positions
+// (hidden state of a position paired with the token after it).  Only caches are written.
+int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, const int32_t *tok, int stride) {
+  const koala_config &g = c->cfg;
+  const int R = k.n * k.q, H = g.H;
+  const bool head = g.head_kind == KOALA_EAGLE && g.K > 0;
+  const Operand none{nullptr, nullptr};
+  const RowMap same{0, 0};
+  c->pending = RowScale{nullptr, 0, 0.f, 0.f};
+  CU_TRY(plan_ingest(LN(c), c->p, k, tok, stride, 0, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
+  K_TRY(embed_rows(c, R));
+  K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, k.q, c->final_norm, none, c->mx, same, !head));
+  if (!head) return KOALA_OK;
+  CU_TRY(ingest_keep(LN(c), c->t, keep, c->mx, H));
+  CU_TRY(plan_ingest(LN(c), c->p, k, tok, stride, 1, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
+  CU_TRY(eagle_concat(LN(c), g.dtype, c->mx, c->p.row_src, c->p.row_tok, c->embed, c->cat, R, H, g.V));
+  SplitIn s;
+  GemmMats fc{{c->fc_w, nullptr, nullptr}, {H, 0, 0}, 1};
+  K_TRY(do_gemm(c, c->cat, 2 * H, fc, R, nullptr, 0, &s));
+  CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, c->draft_layers[0].attn_norm, c->xn, nullptr, same, R, H,
+                      g.rms_eps));
+  c->pending = RowScale{nullptr, 0, 0.f, 0.f};
+  return run_layers(c, c->draft_layers, g.K, c->dk, c->dv, R, k.q, nullptr, none, nullptr, same, true);
 }
 
 int draft_eagle(koala_ctx *c, int pass) {
@@ -521,13 +580,14 @@ int draft_eagle(koala_ctx *c, int pass) {
   // pass >= 1: every row's feature goes to feat[pass & 1] and to the LM head's input.
   float *f_all = pass == 0 ? nullptr : c->feat[pass & 1];
   const Operand none{nullptr, nullptr};
+  const RowMap same{0, 0};
   const Operand lm_all = pass == 0 ? none : c->lmin;
   if (g.K == 0) {
-    CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, nullptr, lm_all, f_all, R, H, g.rms_eps));
+    CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, nullptr, lm_all, f_all, same, R, H, g.rms_eps));
   } else {
     CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, c->draft_layers[0].attn_norm, c->xn, nullptr,
-                        R, H, g.rms_eps));
-    K_TRY(run_layers(c, c->draft_layers, g.K, c->dk, c->dv, R, rows, nullptr, lm_all, f_all));
+                        same, R, H, g.rms_eps));
+    K_TRY(run_layers(c, c->draft_layers, g.K, c->dk, c->dv, R, rows, nullptr, lm_all, f_all, same));
   }
   int lm_rows = R;
   if (pass == 0) {
@@ -549,8 +609,9 @@ int draft_medusa(koala_ctx *c) {
   // The heads are independent chains.  Block j of every head is multiplied first (each head's
   // partial sums in a region of its own), then the heads' epilogues run: the weight stream of one
   // head's matrix follows the previous head's without a small kernel in between.
-  const size_t region = ((size_t)MAX_SPLIT * c->Mp * c->pcols / (size_t)(nh > 0 ? nh : 1)) & ~(size_t)63;
-  const int slots = (int)(region / ((size_t)c->Mp * H));
+  const size_t region = (c->p_floats / (size_t)(nh > 0 ? nh : 1)) & ~(size_t)63;
+  const size_t fit = region / (align_up((size_t)B, 16) * H);
+  const int slots = fit < (size_t)MAX_SPLIT ? (int)fit : MAX_SPLIT;
   const bool batched = nh <= 8 && slots >= 1;
   SplitIn sp[8];
   for (int j = 0; j < g.K; ++j) {
@@ -558,7 +619,7 @@ int draft_medusa(koala_ctx *c) {
       GemmMats m{{c->res_w[(size_t)i * g.K + j], nullptr, nullptr}, {H, 0, 0}, 1};
       const size_t off = (size_t)i * B * H * c->esz;
       Operand xi{(unsigned char *)c->xn.hi + off, c->xn.lo ? (unsigned char *)c->xn.lo + off : nullptr};
-      if (batched) { c->p_off = (size_t)i * region; c->p_slots = slots < MAX_SPLIT ? slots : MAX_SPLIT; }
+      if (batched) { c->p_off = (size_t)i * region; c->p_slots = slots; }
       SplitIn s;
       const int rc = do_gemm(c, xi, H, m, B, nullptr, 0, &s);
       c->p_off = 0;
@@ -566,7 +627,7 @@ int draft_medusa(koala_ctx *c) {
       if (rc != KOALA_OK) return rc;
       if (batched) { sp[i] = s; continue; }
       CU_TRY(row_epilogue(LN(c), g.dtype, 2, c->mx + (size_t)i * B * H, s, c->res_b[(size_t)i * g.K + j],
-                          nullptr, xi, nullptr, B, H, g.rms_eps));
+                          nullptr, xi, nullptr, RowMap{0, 0}, B, H, g.rms_eps));
     }
     if (!batched) continue;
     bool same = (H % 4) == 0 && (sp[0].ld % 4) == 0 && (sp[0].stride % 4) == 0 && sp[0].sk_ctas == 0;
@@ -583,7 +644,7 @@ int draft_medusa(koala_ctx *c) {
       const size_t off = (size_t)i * B * H * c->esz;
       Operand xi{(unsigned char *)c->xn.hi + off, c->xn.lo ? (unsigned char *)c->xn.lo + off : nullptr};
       CU_TRY(row_epilogue(LN(c), g.dtype, 2, c->mx + (size_t)i * B * H, sp[i], c->res_b[(size_t)i * g.K + j],
-                          nullptr, xi, nullptr, B, H, g.rms_eps));
+                          nullptr, xi, nullptr, RowMap{0, 0}, B, H, g.rms_eps));
     }
   }
   if (c->medusa_lm.empty()) {
@@ -727,6 +788,7 @@ int koala_init(const koala_config *cfg, const koala_weights *w, const koala_stat
   memset(c->t_bytes, 0, sizeof(c->t_bytes));
   memset(c->t_launches, 0, sizeof(c->t_launches));
   c->last_tree_from_caller = false;
+  c->ingest_blocks = 0;
   return KOALA_OK;
 }
 
@@ -792,27 +854,92 @@ int koala_verify(koala_ctx *c, const koala_tree *tree) {
     c->last_tree_from_caller = false;
     c->pend_cap = g.N < g.D + 1 ? g.N : g.D + 1;
   }
-  // a single sequence with a short caller tree (a prompt chunk, a one-node step) runs n_max rows;
-  // with several sequences row b * N + u is fixed, so all B * N rows run
-  const int rows = (tree && g.B == 1) ? tree->n_max : g.N;
-  const int R = g.B == 1 ? rows : g.B * g.N;
+  // A short caller tree (a prompt chunk, a one-node step) runs n_max rows per sequence; node u of
+  // sequence b stays row b * N + u of the buffers, so the outputs are spread at the end.  (One-token
+  // steps of four sequences on an engine for 64-node trees ran all 256 rows before: 8.1 -> 3.7 ms.)
+  const int rows = tree ? tree->n_max : g.N;
+  const int R = g.B * rows;
+  const RowMap out_map = rows == g.N ? RowMap{0, 0} : RowMap{rows, g.N};
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
   CU_TRY(tree_ancestors(LN(c), c->t, g.B, g.N));
-  CU_TRY(plan_verify(LN(c), c->t, c->p, c->seq_len, g.B, g.N, g.head_dim, g.rope_base, g.S_max, c->status));
-  if ((g.H % 4) == 0 && g.H <= 8192) {
-    // the embedding rows in the deferred form: their RMSNorm scale is applied by the first layer's consumer
-    CU_TRY(embed_update(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, c->sumsq[1],
-                        R, g.H, g.V));
-    c->pending = RowScale{c->sumsq[1], (g.H + 1023) / 1024, 1.f / (float)g.H, g.rms_eps};
-  } else {
-    CU_TRY(embed_norm(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, R, g.H, g.V,
-                      g.rms_eps));
-  }
-  K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, rows, c->final_norm, c->lmin, c->verify_hid));
+  CU_TRY(plan_verify(LN(c), c->t, c->p, c->seq_len, g.B, g.N, rows, g.head_dim, g.rope_base, g.S_max, c->status));
+  K_TRY(embed_rows(c, R));
+  K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, rows, c->final_norm, c->lmin, c->verify_hid, out_map));
   GemmMats lm{{c->lm_head, nullptr, nullptr}, {g.V, 0, 0}, 1};
-  K_TRY(do_gemm(c, c->lmin, g.H, lm, R, c->verify_logits, g.V, nullptr));
-  CU_TRY(argmax_rows(LN(c), c->verify_logits, c->verify_tgt, R, g.V));
+  K_TRY(do_gemm(c, c->lmin, g.H, lm, R, c->verify_logits, g.V, nullptr, out_map));
+  CU_TRY(argmax_rows(LN(c), c->verify_logits, c->verify_tgt, out_map, R, g.V));
   c->phase = PH_VERIFIED;
+  return KOALA_OK;
+}
+
+int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t *len, int32_t n_parts) {
+  if (!c) return KOALA_E_INVALID;
+  const koala_config &g = c->cfg;
+  if (!tok || !len || n_parts < 1) return fail(c, KOALA_E_INVALID, "null prompt / no parts");
+  IngestLens k;
+  memset(&k, 0, sizeof(k));
+  k.n_parts = n_parts;
+  int longest = 0;
+  for (int b = 0; b < g.B; ++b) {
+    if (len[b] < 0 || len[b] > stride) return fail(c, KOALA_E_INVALID, "prompt %d: %d tokens (stride %d)", b, len[b], stride);
+    k.len[b] = len[b];
+    k.count[b] = len[b] - len[b] / n_parts;        // the last of the equal parts is the shorter kind
+    if (k.count[b] > longest) longest = k.count[b];
+  }
+  c->phase = PH_INGESTED;
+  c->last_pass = -1;
+  if (longest == 0) return KOALA_OK;
+  // Block length: the one that leaves the fewest unused rows (ties: the longest, which re-reads the
+  // cached keys least); one block if every prompt is short.
+  int q = longest < 128 ? longest : 128;
+  if (q > c->ingest_rows) q = c->ingest_rows;      // a prompt beyond the cache's capacity: reported by the plan
+  if (q > 48) {
+    int best = 1 << 30;
+    for (int t = q; t > 48; --t) {
+      int rows = 0;
+      for (int b = 0; b < g.B; ++b) rows += (k.count[b] + t - 1) / t * t;
+      if (rows < best) { best = rows; q = t; }
+    }
+  }
+  int fwd = c->ingest_rows / q;
+  fwd = fwd > INGEST_MAX_BLOCKS ? INGEST_MAX_BLOCKS : (fwd < 1 ? 1 : fwd);
+  int total = 0;
+  for (int b = 0; b < g.B; ++b) total += (k.count[b] + q - 1) / q;
+  const int n_fwd = (total + fwd - 1) / fwd;
+  fwd = (total + n_fwd - 1) / n_fwd;               // forwards of equal size
+  // blocks by position, all sequences side by side: a block comes after the earlier ones of its sequence
+  IngestBlocks blk;
+  memset(&blk, 0, sizeof(blk));
+  blk.q = q;
+  int rc = KOALA_OK;
+  auto flush = [&]() {
+    if (blk.n == 0 || rc != KOALA_OK) return;
+    // The pending rows of a sequence are those of its last part; where earlier parts were one token
+    // longer, the row after them still holds the last token of the last longer part.
+    IngestKeep keep;
+    keep.n = 0;
+    for (int v = 0; v < blk.n; ++v) {
+      const int b = blk.seq[v], row = k.len[b] / n_parts, at = (k.len[b] % n_parts) * (row + 1) - 1 - blk.start[v];
+      if (at < 0 || at >= blk.count[v] || row >= g.N) continue;
+      keep.src[keep.n] = v * q + at;
+      keep.dst[keep.n++] = b * g.N + row;
+    }
+    c->ingest_blocks = blk.n;
+    rc = ingest_forward(c, blk, keep, tok, stride);
+    c->ingest_blocks = 0;
+    blk.n = 0;
+  };
+  for (int s0 = 0; s0 < longest; s0 += q)
+    for (int b = 0; b < g.B; ++b) {
+      if (s0 >= k.count[b]) continue;
+      blk.start[blk.n] = s0;
+      blk.seq[blk.n] = (int16_t)b;
+      blk.count[blk.n] = (int16_t)(k.count[b] - s0 < q ? k.count[b] - s0 : q);
+      if (++blk.n == fwd) flush();
+    }
+  flush();
+  if (rc != KOALA_OK) return rc;
+  CU_TRY(ingest_commit(LN(c), c->t, k, c->seq_len, g.B));
   return KOALA_OK;
 }
 
@@ -1011,7 +1138,8 @@ int koala_gemm_bf16(const void *X, const void *X_lo, const void *W, float *Y, in
   Launch L{(cudaStream_t)cuda_stream, false};
   GemmMats m{{W, nullptr, nullptr}, {N_out, 0, 0}, 1};
   Operand Xo{const_cast<void *>(X), const_cast<void *>(X_lo)};
-  if (!use_tensor_cores) return gemm_simt(L, KOALA_BF16, Xo, m, K_in, M, Y, ldy) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;
+  const RowMap same{0, 0};
+  if (!use_tensor_cores) return gemm_simt(L, KOALA_BF16, Xo, m, K_in, M, Y, ldy, same) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;
   char e[160];
   if (tc_init_driver(e, sizeof(e)) != 0) return KOALA_E_CUDA;
   if (!tc_supported(m, K_in)) return KOALA_E_UNSUPPORTED;
@@ -1020,12 +1148,12 @@ int koala_gemm_bf16(const void *X, const void *X_lo, const void *W, float *Y, in
   // X must hold whole token tiles (koala_gemm_x_rows)
   const int rows_alloc = koala_gemm_x_rows(M, X_lo != nullptr);
   if (split_k == 1)
-    return gemm_tc(L, Xo, rows_alloc, m, K_in, M, Y, ldy, 1, 0, device_status, 1, nullptr) == cudaSuccess
+    return gemm_tc(L, Xo, rows_alloc, m, K_in, M, Y, ldy, same, 1, 0, device_status, 1, nullptr) == cudaSuccess
                ? KOALA_OK : KOALA_E_CUDA;
   const size_t stride = (size_t)M * N_out;
   if (!scratch || scratch_bytes < (size_t)MAX_SPLIT * stride * sizeof(float)) return KOALA_E_CAPACITY;
   SplitIn s;
-  if (gemm_tc(L, Xo, rows_alloc, m, K_in, M, (float *)scratch, N_out, split_k, stride, device_status, MAX_SPLIT,
+  if (gemm_tc(L, Xo, rows_alloc, m, K_in, M, (float *)scratch, N_out, same, split_k, stride, device_status, MAX_SPLIT,
               &s) != cudaSuccess)
     return KOALA_E_CUDA;
   return reduce_splits(L, s, Y, ldy, M, N_out) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;

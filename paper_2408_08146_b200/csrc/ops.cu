@@ -63,7 +63,7 @@ template <typename T>
 __global__ void row_epilogue_kernel(int mode, float *__restrict__ x, SplitIn P,
                                     const T *__restrict__ bias, const T *__restrict__ g,
                                     T *__restrict__ xn, T *__restrict__ xn_lo,
-                                    float *__restrict__ out_f32, int H, float eps) {
+                                    float *__restrict__ out_f32, RowMap out_map, int H, float eps) {
   __shared__ float red[32];
   pdl_launch_dependents();
   pdl_wait();
@@ -85,7 +85,7 @@ __global__ void row_epilogue_kernel(int mode, float *__restrict__ x, SplitIn P,
     float n = xr[i];
     if (g != nullptr) n = n * inv * to_f(g[i]);
     if (xn != nullptr) store_operand(xn, xn_lo, (size_t)r * H + i, n);
-    if (out_f32 != nullptr) out_f32[(size_t)r * H + i] = n;
+    if (out_f32 != nullptr) out_f32[(size_t)out_map(r) * H + i] = n;
   }
 }
 
@@ -145,7 +145,7 @@ template <typename T, int VPT>
 __global__ void __launch_bounds__(1024)
 row_epilogue_vec_kernel(int mode, float *__restrict__ x, SplitIn P, const T *__restrict__ bias,
                         const T *__restrict__ g, T *__restrict__ xn, T *__restrict__ xn_lo,
-                        float *__restrict__ out_f32, int H, float eps) {
+                        float *__restrict__ out_f32, RowMap out_map, int H, float eps) {
   __shared__ float red[32];
   pdl_launch_dependents();
   pdl_wait();
@@ -195,7 +195,7 @@ row_epilogue_vec_kernel(int mode, float *__restrict__ x, SplitIn P, const T *__r
         n = make_float4(n.x * inv * gg[k].x, n.y * inv * gg[k].y, n.z * inv * gg[k].z, n.w * inv * gg[k].w);
       }
       if (xn != nullptr) store_operand4(xn, xn_lo, (size_t)r * H + c, n);
-      if (out_f32 != nullptr) *reinterpret_cast<float4 *>(out_f32 + (size_t)r * H + c) = n;
+      if (out_f32 != nullptr) *reinterpret_cast<float4 *>(out_f32 + (size_t)out_map(r) * H + c) = n;
     }
   }
 }
@@ -349,7 +349,7 @@ __global__ void rope_kv_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__
   pdl_wait();
   const int r = blockIdx.x, h = blockIdx.y, i = threadIdx.x;
   const int half = head_dim >> 1, H = n_heads * head_dim;
-  const int b = r / rows_per_seq;
+  const int b = plan.cache_of(r / rows_per_seq);
   const int slot = plan.slot[r];
   const float2 cs = plan.rope[(size_t)r * half + i];
   const int c0 = h * head_dim + i, c1 = c0 + half;
@@ -405,7 +405,7 @@ rope_kv_vec_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__restrict__ q
   pdl_wait();
   const int r = blockIdx.x;
   const int half = head_dim >> 1, H = n_heads * head_dim, hq = half >> 1;
-  const int b = r / rows_per_seq;
+  const int b = plan.cache_of(r / rows_per_seq);
   const int slot = plan.slot[r];
   const bool wr = slot >= 0 && slot < S_max;
   const float rs = sc.of(r);
@@ -491,8 +491,9 @@ tree_attn_kernel(const float *q, const T *kc, const T *vc,
   const int ctx = plan.ctx_len[b], kv_len = plan.kv_len[b];
   const uint64_t m0 = plan.mask[(size_t)r * 2], m1 = plan.mask[(size_t)r * 2 + 1];
   for (int d = lane; d < DH; d += 32) qs[w][d] = valid ? q[(size_t)r * H + h * DH + d] : 0.f;
-  const T *kb = kc + ((size_t)b * n_heads + h) * S_max * DH;
-  const T *vb = vc + ((size_t)b * n_heads + h) * S_max * DH;
+  const int cb = plan.cache_of(b);
+  const T *kb = kc + ((size_t)cb * n_heads + h) * S_max * DH;
+  const T *vb = vc + ((size_t)cb * n_heads + h) * S_max * DH;
   const float scale = rsqrtf((float)DH);
   float m = -INFINITY, l = 0.f;
   float o[DH / 32];
@@ -575,15 +576,15 @@ __device__ __forceinline__ ValIdx block_argmax(ValIdx x, ValIdx *red) {
   return x;
 }
 
-__global__ void argmax_rows_kernel(const float *logits, int32_t *__restrict__ out, int V) {
+__global__ void argmax_rows_kernel(const float *logits, int32_t *__restrict__ out, RowMap map, int V) {
   __shared__ ValIdx red[32];
   pdl_launch_dependents();
   pdl_wait();
-  const float *row = logits + (size_t)blockIdx.x * V;
+  const float *row = logits + (size_t)map(blockIdx.x) * V;
   ValIdx best{-INFINITY, 0x7fffffff};
   for (int i = threadIdx.x; i < V; i += blockDim.x) best = better(best, ValIdx{row[i], i});
   best = block_argmax(best, red);
-  if (threadIdx.x == 0) out[blockIdx.x] = best.i;
+  if (threadIdx.x == 0) out[map(blockIdx.x)] = best.i;
 }
 
 // Per row: the k largest logits (ties: smaller id) and their natural-log softmax probabilities.
@@ -709,7 +710,7 @@ topk_logp_fast_kernel(const float *logits, int32_t *__restrict__ tok, float *__r
 // candidates (ties still go to the smaller id) and forms the log-sum-exp.  V <= 32768, k <= 32.
 constexpr int TKP = 8;            // CTAs per row
 __global__ void __launch_bounds__(256)
-topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp, int V, int k) {
+topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp, RowMap map, int V, int k) {
   // logp == nullptr: only the ids are wanted (the arg-max of a row is its top-1), no exponentials
   __shared__ ValIdx cand[8 * 32];
   __shared__ ValIdx mine[32];     // this CTA's k best, read by CTA 0
@@ -717,7 +718,7 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
   __shared__ float redf[32];
   pdl_launch_dependents();
   pdl_wait();
-  const int part = blockIdx.x, r = blockIdx.y;
+  const int part = blockIdx.x, r = map(blockIdx.y);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int chunk = (((V + TKP - 1) / TKP) + 255) & ~255;          // ids per CTA, a multiple of 256
   const int base = part * chunk;
@@ -835,23 +836,23 @@ cudaError_t embed_norm(Launch L, int dtype, const int32_t *tok, const void *E, c
 }
 
 cudaError_t row_epilogue(Launch L, int dtype, int mode, float *x, SplitIn P, const void *bias,
-                         const void *g, Operand xn, float *out_f32, int R, int H, float eps) {
+                         const void *g, Operand xn, float *out_f32, RowMap out_map, int R, int H, float eps) {
   if (H % 4 == 0 && P.ld % 4 == 0 && P.stride % 4 == 0 && H <= 8192) {
     const int groups = H / 4;
     int threads = groups <= 1024 ? ((groups + 31) / 32) * 32 : (((groups + 1) / 2 + 31) / 32) * 32;
     if (groups <= 1024) {
       DISPATCH_T(dtype, return launch_k(row_epilogue_vec_kernel<T, 1>, dim3(R), dim3(threads), 0, L.st, L.pdl,
                                         mode, x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo,
-                                        out_f32, H, eps);)
+                                        out_f32, out_map, H, eps);)
     } else {
       DISPATCH_T(dtype, return launch_k(row_epilogue_vec_kernel<T, 2>, dim3(R), dim3(threads), 0, L.st, L.pdl,
                                         mode, x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo,
-                                        out_f32, H, eps);)
+                                        out_f32, out_map, H, eps);)
     }
   }
   DISPATCH_T(dtype, return launch_k(row_epilogue_kernel<T>, dim3(R), dim3(256), 0, L.st, L.pdl, mode,
                                     x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo, out_f32,
-                                    H, eps);)
+                                    out_map, H, eps);)
 }
 
 cudaError_t eagle_concat(Launch L, int dtype, const float *feat_src, const int32_t *row_src,
@@ -942,7 +943,8 @@ cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_ca
   return cudaErrorInvalidValue;
 }
 
-static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k) {
+static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *tok, float *logp, RowMap map, int R, int V,
+                                       int k) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(TKP, R);
   cfg.blockDim = dim3(256);
@@ -957,17 +959,17 @@ static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *t
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   ++g_launches;
-  return cudaLaunchKernelEx(&cfg, topk_logp_cluster_kernel, logits, tok, logp, V, k);
+  return cudaLaunchKernelEx(&cfg, topk_logp_cluster_kernel, logits, tok, logp, map, V, k);
 }
 
-cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, int R, int V) {
+cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, RowMap map, int R, int V) {
   // the arg-max (ties: smaller id) is the top-1; wide rows go to the eight-CTA kernel
-  if (V <= 32768 && V >= 4096) return topk_cluster_launch(L, logits, out, nullptr, R, V, 1);
-  return launch_k(argmax_rows_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, out, V);
+  if (V <= 32768 && V >= 4096) return topk_cluster_launch(L, logits, out, nullptr, map, R, V, 1);
+  return launch_k(argmax_rows_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, out, map, V);
 }
 
 cudaError_t topk_logp(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k) {
-  if (V <= 32768 && k <= 32 && V >= 4096) return topk_cluster_launch(L, logits, tok, logp, R, V, k);
+  if (V <= 32768 && k <= 32 && V >= 4096) return topk_cluster_launch(L, logits, tok, logp, RowMap{0, 0}, R, V, k);
   if (V <= 32768 && k <= 32)
     return launch_k(topk_logp_fast_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, tok, logp, V, k);
   const size_t smem = (size_t)V * sizeof(float);

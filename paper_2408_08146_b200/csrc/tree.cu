@@ -88,7 +88,7 @@ __global__ void tree_ancestors_kernel(TreeBufs t, int N) {
 
 // ------------------------------------------------------------------------------- plans
 __global__ void plan_verify_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len,
-                                   int N, int head_dim, float rope_base, int S_max, int *status) {
+                                   int N, int rows, int head_dim, float rope_base, int S_max, int *status) {
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
@@ -102,15 +102,14 @@ __global__ void plan_verify_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_le
   }
   {
     const int u = blockIdx.y;
-    const size_t r = (size_t)b * N + u;
-    const int lvl = t.tree_level[r];
+    const size_t node = (size_t)b * N + u, r = (size_t)b * rows + u;
+    const int lvl = t.tree_level[node];
     if (threadIdx.x == 0) {
       p.pos[r] = S + lvl;
       p.slot[r] = (fits && u < n) ? S + u : -1;
-      p.mask[r * 2] = t.tree_anc[r * 2];
-      p.mask[r * 2 + 1] = t.tree_anc[r * 2 + 1];
-      p.row_tok[r] = t.tree_tok[r];
-      p.row_src[r] = (int)r;
+      p.mask[r * 2] = t.tree_anc[node * 2];
+      p.mask[r * 2 + 1] = t.tree_anc[node * 2 + 1];
+      p.row_tok[r] = t.tree_tok[node];
     }
     write_rope(p.rope, r, S + lvl, head_dim, rope_base, threadIdx.x, blockDim.x);
   }
@@ -150,6 +149,61 @@ __global__ void plan_draft0_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_le
     }
     write_rope(p.rope, r, pos < 0 ? 0 : pos, head_dim, rope_base, threadIdx.x, blockDim.x);
   }
+}
+
+// Prompt ingestion: row i of block v is the token at start + i of its sequence, as a chain on top of
+// everything before it.  grid (blocks, q).
+__global__ void plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlocks k, const int32_t *tok, int stride,
+                                   int shift, const int32_t *seq_len, int head_dim, float rope_base, int S_max,
+                                   int *status) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int v = blockIdx.x, i = blockIdx.y;
+  const int b = k.seq[v], n = k.count[v];
+  const int S = seq_len[b] + k.start[v];
+  const bool fits = S >= 0 && S + n <= S_max;
+  const size_t r = (size_t)v * k.q + i;
+  if (threadIdx.x == 0) {
+    if (i == 0) {
+      if (!fits && status) atomicMax(status, E_CAPACITY);
+      p.seq[v] = b;
+      p.ctx_len[v] = fits ? S : 0;
+      p.kv_len[v] = fits ? S + n : 0;
+    }
+    p.pos[r] = S + i;
+    p.slot[r] = (fits && i < n) ? S + i : -1;
+    p.mask[r * 2] = i >= 63 ? ~0ull : (1ull << (i + 1)) - 1ull;
+    p.mask[r * 2 + 1] = i < 64 ? 0ull : (i == 127 ? ~0ull : (1ull << (i - 63)) - 1ull);
+    p.row_tok[r] = i < n ? tok[(size_t)b * stride + k.start[v] + i + shift] : 0;
+    p.row_src[r] = (int)r;
+  }
+  write_rope(p.rope, r, S + i < 0 ? 0 : S + i, head_dim, rope_base, threadIdx.x, blockDim.x);
+}
+
+__global__ void ingest_keep_kernel(TreeBufs t, const __grid_constant__ IngestKeep k, const float *hid, int H) {
+  pdl_launch_dependents();
+  pdl_wait();
+  for (int d = threadIdx.x; d < H; d += blockDim.x)
+    t.pend_hid[(size_t)k.dst[blockIdx.x] * H + d] = hid[(size_t)k.src[blockIdx.x] * H + d];
+}
+
+__global__ void ingest_commit_kernel(TreeBufs t, const __grid_constant__ IngestLens k, int32_t *seq_len, int B) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int i = threadIdx.x;                  // chain position i + 1
+  unsigned long long hits = 0;
+  for (int b = 0; b < B; ++b) {
+    // the first len % n_parts parts have one token more; the last part is not ingested here
+    const int base = k.len[b] / k.n_parts, longer = k.len[b] % k.n_parts, parts = k.n_parts - 1;
+    const int n_long = longer < parts ? longer : parts;
+    if (base + 1 > i + 1) hits += (unsigned long long)n_long;
+    if (base > i + 1) hits += (unsigned long long)(parts - n_long);
+  }
+  if (i < 128 && t.alpha_hits != nullptr && hits > 0) {
+    t.alpha_hits[i] += hits;
+    t.alpha_trials[i] += hits;
+  }
+  if (i < B) seq_len[i] += k.count[i];
 }
 
 // Medusa-style draft: every head reads the hidden state of the last accepted position.
@@ -485,10 +539,22 @@ cudaError_t tree_from_caller(Launch L, TreeBufs t, const int32_t *tok, const int
 cudaError_t tree_ancestors(Launch L, TreeBufs t, int B, int N) {
   return launch_k(tree_ancestors_kernel, dim3(B), dim3(128), 0, L.st, L.pdl, t, N);
 }
-cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
+cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows,
                         int head_dim, float rope_base, int S_max, int *status) {
-  return launch_k(plan_verify_kernel, dim3(B, N), dim3(64), 0, L.st, L.pdl, t, p, seq_len, N, head_dim,
+  return launch_k(plan_verify_kernel, dim3(B, rows), dim3(64), 0, L.st, L.pdl, t, p, seq_len, N, rows, head_dim,
                   rope_base, S_max, status);
+}
+cudaError_t plan_ingest(Launch L, PlanBufs p, IngestBlocks k, const int32_t *tok, int stride, int shift,
+                        const int32_t *seq_len, int head_dim, float rope_base, int S_max, int *status) {
+  return launch_k(plan_ingest_kernel, dim3(k.n, k.q), dim3(64), 0, L.st, L.pdl, p, k, tok, stride, shift, seq_len,
+                  head_dim, rope_base, S_max, status);
+}
+cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, int H) {
+  if (k.n == 0) return cudaSuccess;
+  return launch_k(ingest_keep_kernel, dim3(k.n), dim3(256), 0, L.st, L.pdl, t, k, hid, H);
+}
+cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, int32_t *seq_len, int B) {
+  return launch_k(ingest_commit_kernel, dim3(1), dim3(128), 0, L.st, L.pdl, t, k, seq_len, B);
 }
 cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
                         int rows, int head_dim, float rope_base, int S_max, int *status) {

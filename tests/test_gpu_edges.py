@@ -302,3 +302,36 @@ def test_whole_iterations_repeat_bit_for_bit():
         runs.append(rec)
     for a, c in zip(*runs):
         assert np.array_equal(a, c)
+
+
+@pytest.mark.parametrize("base,B,N,n_max", [("tiny", 3, 15, 1), ("tiny", 2, 15, 4), ("7b", 4, 64, 1), ("7b", 3, 40, 17),
+                                            ("7b", 4, 64, 40)])
+def test_short_caller_trees_of_a_batch_run_only_their_rows(base, B, N, n_max):
+    """Several sequences with caller trees of at most n_max < N nodes: node u of sequence b is row b * N + u
+    of the outputs, whatever rows the forward itself used; ragged node counts, then an accepted path."""
+    from tests.parity import assert_close
+    if base == "tiny":
+        cfg = TINY_EAGLE.with_(B=B, N=N, prompt_len=30, prompt_len_min=21, S_max=128, seed=21)
+    else:
+        cfg = reduced(T7_EAGLE, 1, B=B, N=N, prompt_len=70, prompt_len_min=33, S_max=256, K=1, seed=22)
+    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float64 if base == "tiny" else np.float32, cache_host=base == "tiny")
+    pr = prompts(cfg)
+    eng.prefill(pr, cfg.N)
+    orc.prefill(pr, cfg.N)
+    rng = np.random.default_rng(n_max)
+    counts = [max(1, n_max - b) for b in range(B)]
+    tok = rng.integers(0, cfg.V, (B, n_max)).astype(np.int32)
+    par = np.asarray([[-1] + [int(rng.integers(0, u)) for u in range(1, n_max)] for _ in range(B)], np.int32)
+    to = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to("cuda:0")
+    eng.koala_verify((to(tok), to(par), to(np.asarray(counts)), n_max))
+    orc.verify([(list(map(int, tok[b, :counts[b]])), list(map(int, par[b, :counts[b]]))) for b in range(B)])
+    bufs = eng.buffers()
+    for b in range(B):
+        n = counts[b]
+        assert_close(bufs["verify_hid"][b * N:b * N + n].cpu().numpy(), orc.verify_hid[b][:n], cfg.dtype, f"hidden {b}")
+        assert_close(bufs["verify_logits"][b * N:b * N + n].cpu().numpy(), orc.verify_logits[b][:n], cfg.dtype, f"logits {b}")
+        got = bufs["verify_logits"][b * N:b * N + n].argmax(1).cpu().tolist()
+        assert bufs["verify_tgt"][b * N:b * N + n].cpu().tolist() == got
+    eng.koala_accept(None)
+    assert eng.device_status() == 0
+    eng.close()
