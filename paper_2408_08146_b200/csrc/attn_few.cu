@@ -1,0 +1,268 @@
+// Tree-masked attention of at most four query rows per sequence (one-token steps, chain drafts,
+// short drafts) for bf16 caches with head_dim 128.
+//
+// With so few rows the cached keys and values are all there is to move: 512 bytes per key and head
+// against a few hundred multiply-adds, so the products run in fp32 on the CUDA cores (the tensor-core
+// kernels would multiply a 16- or 128-row operand that is mostly padding: 0.7 us of mma.sync per
+// 64-key tile).  One CTA = one (key chunk, head, sequence); a warp takes eight keys of every 64-key
+// tile, half a warp one key per step: 16 lanes x 16 bytes of K and of V, the next tile's loads in
+// flight in registers while this one's are used.  Softmax is online, per half-warp; the sixteen
+// partial results of a CTA are merged through shared memory, the chunks (a thread-block cluster)
+// through distributed shared memory, each CTA finishing its share of the output, in chunk order.
+// Tried and dropped: tiles dealt evenly over all CTAs with partials in global memory and the last
+// arriver adding them (fence, counter and the re-read: 4 us at the end of every launch; 14 us per
+// launch, ragged batch 22 us).
+#include "common.cuh"
+
+namespace koala {
+namespace {
+
+constexpr int DH = 128;
+constexpr int TILE = 64;
+constexpr int WARPS = 8;
+constexpr int MAX_CHUNKS = 8;
+constexpr int PSTRIDE = DH + 4;           // floats of a partial: O[128], m, l, pad (16-byte rows)
+
+__device__ __forceinline__ void unpack8(const uint4 &u, float *f) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    f[2 * i] = __uint_as_float(w[i] << 16);
+    f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
+
+__device__ __forceinline__ float ld_cluster(uint32_t local_addr, uint32_t rank) {
+  uint32_t ra;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
+  return v;
+}
+
+template <int RT>
+__global__ void __launch_bounds__(WARPS * 32, RT <= 2 ? 2 : 1)
+tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan plan, bf16 *__restrict__ out,
+                     bf16 *__restrict__ out_lo, int rows_per_seq, int n_heads, int S_max) {
+  __shared__ __align__(16) float s_q[RT][DH];
+  __shared__ __align__(16) float s_o[2 * WARPS][RT][PSTRIDE];
+  __shared__ __align__(16) float s_c[RT][PSTRIDE];         // this chunk's result, read by the cluster
+  pdl_launch_dependents();
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hf = lane >> 4, d0 = (lane & 15) * 8;
+  const int H = n_heads * DH;
+  const int c = (int)blockIdx.x, chunks = (int)gridDim.x;
+  const int b = (int)blockIdx.y / n_heads, h = (int)blockIdx.y % n_heads;
+  const float sc = 0.08838834764831845f * 1.4426950408889634f;    // 1/sqrt(128) * log2(e)
+  const int ctx = plan.ctx_len[b];
+  const int kv_len = min(plan.kv_len[b], S_max);
+  const int tiles = (kv_len + TILE - 1) / TILE;
+  const int t_lo = tiles * c / chunks, t_hi = tiles * (c + 1) / chunks;
+  const size_t base = ((size_t)plan.cache_of(b) * n_heads + h) * S_max;
+  const bf16 *kb = kc + base * DH + d0, *vb = vc + base * DH + d0;
+  const int k_off = warp * 8 + hf;                       // this half-warp's keys of a tile: k_off + 2 j
+  uint4 kn[4], vn[4];
+  auto load = [&](int t) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int key = t * TILE + k_off + 2 * j;
+      const bool in = key < kv_len;                      // slots past the end were never written
+      kn[j] = in ? *reinterpret_cast<const uint4 *>(kb + (size_t)key * DH) : make_uint4(0u, 0u, 0u, 0u);
+      vn[j] = in ? *reinterpret_cast<const uint4 *>(vb + (size_t)key * DH) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  load(t_lo);                                            // first of all: the longest way
+  uint64_t mk0[RT], mk1[RT];
+  unsigned row_ok = 0;
+#pragma unroll
+  for (int r = 0; r < RT; ++r) {
+    const int rg = b * rows_per_seq + (r < rows_per_seq ? r : 0);
+    const int slot = plan.slot[rg];
+    mk0[r] = plan.mask[(size_t)rg * 2];
+    mk1[r] = plan.mask[(size_t)rg * 2 + 1];
+    if (r < rows_per_seq && slot >= 0) row_ok |= 1u << r;
+  }
+  for (int e = threadIdx.x; e < RT * DH; e += WARPS * 32) {
+    const int r = e / DH, d = e % DH;
+    s_q[r][d] = q[(size_t)(b * rows_per_seq + (r < rows_per_seq ? r : 0)) * H + h * DH + d] * sc;
+  }
+  __syncthreads();
+  float m[RT], l[RT], o[RT][8];
+#pragma unroll
+  for (int r = 0; r < RT; ++r) {
+    m[r] = -INFINITY;
+    l[r] = 0.f;
+#pragma unroll
+    for (int d = 0; d < 8; ++d) o[r][d] = 0.f;
+  }
+  for (int t = t_lo; t < t_hi; ++t) {
+    uint4 kx[4], vx[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { kx[j] = kn[j]; vx[j] = vn[j]; }
+    if (t + 1 < t_hi) load(t + 1);
+    float s[RT][4];
+    {
+      float kf[4][8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) unpack8(kx[j], kf[j]);
+#pragma unroll
+      for (int r = 0; r < RT; ++r) {
+        const float4 qa = *reinterpret_cast<const float4 *>(&s_q[r][d0]), qb = *reinterpret_cast<const float4 *>(&s_q[r][d0 + 4]);
+        const float qr[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float a = 0.f;
+#pragma unroll
+          for (int d = 0; d < 8; ++d) a = fmaf(qr[d], kf[j][d], a);
+          s[r][j] = a;
+        }
+      }
+    }
+#pragma unroll
+    for (int o2 = 8; o2 >= 1; o2 >>= 1)
+#pragma unroll
+      for (int r = 0; r < RT; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[r][j] += __shfl_xor_sync(0xffffffffu, s[r][j], o2);
+    const int key0 = t * TILE + k_off;
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+      float mx = m[r];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int rel = key0 + 2 * j - ctx;
+        bool vis = ((row_ok >> r) & 1u) != 0 && key0 + 2 * j < kv_len;
+        if (rel >= 0) vis = vis && (rel < 64 ? ((mk0[r] >> rel) & 1ull) : (rel < 128 ? ((mk1[r] >> (rel - 64)) & 1ull) : 0ull)) != 0ull;
+        s[r][j] = vis ? s[r][j] : -INFINITY;
+        mx = fmaxf(mx, s[r][j]);
+      }
+      const float mu = mx == -INFINITY ? 0.f : mx;
+      const float corr = exp2f(m[r] - mu);               // exp2(-inf) = 0
+      m[r] = mx;
+      l[r] *= corr;
+#pragma unroll
+      for (int d = 0; d < 8; ++d) o[r][d] *= corr;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        s[r][j] = exp2f(s[r][j] - mu);
+        l[r] += s[r][j];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float vf[8];
+      unpack8(vx[j], vf);
+#pragma unroll
+      for (int r = 0; r < RT; ++r)
+#pragma unroll
+        for (int d = 0; d < 8; ++d) o[r][d] = fmaf(s[r][j], vf[d], o[r][d]);
+    }
+  }
+// ---- the CTA's sixteen half-warps
+  const int src = warp * 2 + hf;
+#pragma unroll
+  for (int r = 0; r < RT; ++r) {
+#pragma unroll
+    for (int d = 0; d < 8; d += 4)
+      *reinterpret_cast<float4 *>(&s_o[src][r][d0 + d]) = make_float4(o[r][d], o[r][d + 1], o[r][d + 2], o[r][d + 3]);
+    if ((lane & 15) == 0) { s_o[src][r][DH] = m[r]; s_o[src][r][DH + 1] = l[r]; }
+  }
+  __syncthreads();
+  auto emit = [&](int r, int d, float v) {
+    const size_t at = (size_t)(b * rows_per_seq + r) * H + h * DH + d;
+    const bf16 hi = __float2bfloat16_rn(v);
+    out[at] = hi;
+    if (out_lo != nullptr) out_lo[at] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  };
+  for (int e = threadIdx.x; e < RT * DH; e += WARPS * 32) {
+    const int r = e / DH, d = e % DH;
+    float mm = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < 2 * WARPS; ++w) mm = fmaxf(mm, s_o[w][r][DH]);
+    float acc = 0.f, ll = 0.f;
+    if (mm != -INFINITY) {
+#pragma unroll
+      for (int w = 0; w < 2 * WARPS; ++w) {
+        const float wt = exp2f(s_o[w][r][DH] - mm);
+        acc += wt * s_o[w][r][d];
+        ll += wt * s_o[w][r][DH + 1];
+      }
+    }
+    if (chunks == 1) {
+      if (r < rows_per_seq) emit(r, d, ll > 0.f ? acc / ll : 0.f);
+    } else {
+      s_c[r][d] = acc;
+      if (d == 0) { s_c[r][DH] = mm; s_c[r][DH + 1] = ll; }
+    }
+  }
+  if (chunks == 1) return;
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  const int share = RT * DH / chunks;                      // outputs this CTA finishes
+  for (int e = c * share + (int)threadIdx.x; e < (c + 1) * share; e += WARPS * 32) {
+    const int r = e / DH, d = e % DH;
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(&s_c[r][0]);
+    float pm[MAX_CHUNKS], pl[MAX_CHUNKS], po[MAX_CHUNKS];  // all requested before the first is used
+#pragma unroll
+    for (int k = 0; k < MAX_CHUNKS; ++k) {
+      const bool in = k < chunks;
+      const uint32_t rk = in ? k : 0;
+      const float a0 = ld_cluster(at + DH * 4, rk), a1 = ld_cluster(at + DH * 4 + 4, rk), a2 = ld_cluster(at + d * 4, rk);
+      pm[k] = in ? a0 : -INFINITY;
+      pl[k] = a1;
+      po[k] = a2;
+    }
+    float mm = pm[0];
+#pragma unroll
+    for (int k = 1; k < MAX_CHUNKS; ++k) mm = fmaxf(mm, pm[k]);
+    float acc = 0.f, ll = 0.f;
+    if (mm != -INFINITY) {
+#pragma unroll
+      for (int k = 0; k < MAX_CHUNKS; ++k) {               // in chunk order
+        const float wt = exp2f(pm[k] - mm);
+        acc += wt * po[k];
+        ll += wt * pl[k];
+      }
+    }
+    if (r < rows_per_seq) emit(r, d, ll > 0.f ? acc / ll : 0.f);
+  }
+  // no CTA leaves while another may still read its result
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+}  // namespace
+
+// Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the launch
+// within what is resident at once (two CTAs per SM up to two rows, else one; clusters of eight do not
+// fill every GPC, hence seven eighths), and at least two tiles of capacity per chunk.
+cudaError_t tree_attention_few(Launch L, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
+                               Operand out, int rows_per_seq, int B, int n_heads, int S_max, int num_sms) {
+  if (rows_per_seq < 1 || rows_per_seq > ATTN_FEW_ROWS) return cudaErrorInvalidValue;
+  const int room = (rows_per_seq <= 2 ? 2 : 1) * num_sms * 7 / 8;
+  int chunks = 1;
+  while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads <= room && 2 * chunks * 2 * TILE <= S_max) chunks *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(chunks, n_heads * B);
+  cfg.blockDim = dim3(WARPS * 32);
+  cfg.stream = L.st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = L.pdl ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = chunks;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chunks > 1 ? 2 : 1;
+  ++g_launches;
+  auto go = [&](auto *kern) {
+    return cudaLaunchKernelEx(&cfg, kern, q, (const bf16 *)k_cache, (const bf16 *)v_cache, plan, (bf16 *)out.hi,
+                              (bf16 *)out.lo, rows_per_seq, n_heads, S_max);
+  };
+  if (rows_per_seq == 1) return go(tree_attn_few_kernel<1>);
+  if (rows_per_seq == 2) return go(tree_attn_few_kernel<2>);
+  return go(tree_attn_few_kernel<4>);
+}
+
+}  // namespace koala

@@ -10,8 +10,11 @@
 // rounding residual), so only the cached K and V carry bf16 rounding.  The mask is: slots below
 // ctx_len visible to every row; slot ctx_len + j visible to a row iff bit j of its 128-bit mask.
 // Softmax is online, in fp32, in base 2; row statistics use quad shuffles.  With several chunks
-// each CTA writes an unnormalised partial (O, m, l) per row and a second kernel combines the
-// chunks in a fixed order; either way the output is emitted as a matrix-multiply operand pair.
+// the CTAs of a (head, row group, sequence) are a thread-block cluster: each leaves its unnormalised
+// (O, m, l) per row in its shared memory and every CTA finishes its share of the output dims from all of
+// them, in chunk order (a second kernel that combined partials in global memory took 6 to 8 us per
+// launch, the last arriver doing it in this kernel 10); the output is emitted as a matrix-multiply
+// operand pair.
 #include "common.cuh"
 
 namespace koala {
@@ -21,7 +24,6 @@ constexpr int DH = 128;
 constexpr int TILE = 64;                 // keys per shared-memory tile
 constexpr int ROW_BYTES = DH * 2;        // 256
 constexpr int TILE_BYTES = TILE * ROW_BYTES;
-constexpr int PSTRIDE = DH + 2;          // floats per partial: O[128], m, l
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -68,6 +70,15 @@ __device__ __forceinline__ bool mask_bit(uint64_t m0, uint64_t m1, int rel) {
   return rel < 64 ? ((m0 >> rel) & 1ull) : (rel < 128 ? ((m1 >> (rel - 64)) & 1ull) : false);
 }
 
+// two floats of a cluster peer's shared memory, given this CTA's own address of the same place
+__device__ __forceinline__ float2 ld_cluster2(uint32_t local_addr, uint32_t rank) {
+  uint32_t ra;
+  float2 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(ra) : "memory");
+  return v;
+}
+
 // grid (chunks, row groups of 16, n_heads * B); block = 4 warps.  All four warps serve the same
 // 16 query rows; warp w takes keys [16w, 16w + 16) of every 64-key tile and keeps its own running
 // (max, sum, O); the four are merged through shared memory at the end.  With chunks == 1 the CTA
@@ -77,7 +88,7 @@ constexpr int MSTRIDE = DH + 4;          // floats per merged row in shared memo
 
 __global__ void __launch_bounds__(128)
 tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
-                     RowPlan plan, float *__restrict__ part, bf16 *__restrict__ out, bf16 *__restrict__ out_lo,
+                     RowPlan plan, bf16 *__restrict__ out, bf16 *__restrict__ out_lo,
                      int rows_per_seq, int n_heads, int S_max, int chunks) {
   extern __shared__ __align__(1024) unsigned char smem[];     // [NST][K tile | V tile]
   pdl_launch_dependents();
@@ -281,131 +292,140 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
   // thread -> (row = tid / 8, 16 consecutive dims starting at (tid % 8) * 16)
   const int row = threadIdx.x >> 3, d0 = (threadIdx.x & 7) * 16;
   const int i = rg * 16 + row;
-  if (i >= rows_per_seq) return;
-  const int r = b * rows_per_seq + i;
-  float mm = -INFINITY;
-#pragma unroll
-  for (int w = 0; w < 4; ++w) mm = fmaxf(mm, ms[((size_t)w * 16 + row) * MSTRIDE + DH]);
+  const bool in_row = i < rows_per_seq;
+  const int r = b * rows_per_seq + (in_row ? i : 0);
   float acc[16];
 #pragma unroll
   for (int d = 0; d < 16; ++d) acc[d] = 0.f;
-  float l = 0.f;
-  if (mm != -INFINITY) {
+  float l = 0.f, mm = -INFINITY;
+  if (in_row) {
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const float *src = ms + ((size_t)w * 16 + row) * MSTRIDE;
-      const float mw = src[DH];
-      if (mw == -INFINITY) continue;
-      const float wgt = exp2f(mw - mm);
-      l += wgt * src[DH + 1];
+    for (int w = 0; w < 4; ++w) mm = fmaxf(mm, ms[((size_t)w * 16 + row) * MSTRIDE + DH]);
+    if (mm != -INFINITY) {
 #pragma unroll
-      for (int d = 0; d < 16; d += 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(src + d0 + d);
-        acc[d] += wgt * v.x; acc[d + 1] += wgt * v.y; acc[d + 2] += wgt * v.z; acc[d + 3] += wgt * v.w;
+      for (int w = 0; w < 4; ++w) {
+        const float *src = ms + ((size_t)w * 16 + row) * MSTRIDE;
+        const float mw = src[DH];
+        if (mw == -INFINITY) continue;
+        const float wgt = exp2f(mw - mm);
+        l += wgt * src[DH + 1];
+#pragma unroll
+        for (int d = 0; d < 16; d += 4) {
+          const float4 v = *reinterpret_cast<const float4 *>(src + d0 + d);
+          acc[d] += wgt * v.x; acc[d + 1] += wgt * v.y; acc[d + 2] += wgt * v.z; acc[d + 3] += wgt * v.w;
+        }
       }
     }
   }
-  if (chunks == 1) {
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    const size_t ob = (size_t)r * H + h * DH + d0;
+  float *mine = ms + (size_t)4 * 16 * MSTRIDE;             // [16 rows][O 128 | m | l]: this chunk's result
+  if (chunks > 1) {
+    if (in_row) {
 #pragma unroll
-    for (int d = 0; d < 16; d += 2) {
-      uint32_t hi, lo;
-      split_pack(acc[d] * inv, acc[d + 1] * inv, hi, lo);
-      *reinterpret_cast<uint32_t *>(out + ob + d) = hi;
-      if (out_lo != nullptr) *reinterpret_cast<uint32_t *>(out_lo + ob + d) = lo;
+      for (int d = 0; d < 16; d += 4)
+        *reinterpret_cast<float4 *>(mine + row * MSTRIDE + d0 + d) = make_float4(acc[d], acc[d + 1], acc[d + 2], acc[d + 3]);
+      if ((threadIdx.x & 7) == 0) *reinterpret_cast<float2 *>(mine + row * MSTRIDE + DH) = make_float2(mm, l);
     }
-  } else {
-    float *p = part + (((size_t)r * n_heads + h) * chunks + c) * PSTRIDE;
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    // this CTA's share: 16 / chunks dims per thread (chunks <= 8: at least two)
+    const int nd = 16 / chunks, dd = (threadIdx.x & 7) * nd + c * (DH / chunks);
+    if (in_row) {
+      const uint32_t at = smem_addr(mine + row * MSTRIDE);
+      float pm[8], pl[8];
 #pragma unroll
-    for (int d = 0; d < 16; d += 2) *reinterpret_cast<float2 *>(p + d0 + d) = make_float2(acc[d], acc[d + 1]);
-    if ((threadIdx.x & 7) == 0) { p[DH] = mm; p[DH + 1] = l; }
-  }
-}
-
-// One warp per (row, head): merges the chunk partials in chunk order and writes the operand pair.
-__global__ void __launch_bounds__(256)
-tree_attn_combine_kernel(const float *part, bf16 *__restrict__ out, bf16 *__restrict__ out_lo,
-                         int R, int n_heads, int chunks) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int pair = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (pair >= R * n_heads) return;
-  const float *p = part + (size_t)pair * chunks * PSTRIDE;
-  float m = -INFINITY;
-  for (int c = 0; c < chunks; ++c) m = fmaxf(m, p[(size_t)c * PSTRIDE + DH]);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  float l = 0.f;
-  if (m != -INFINITY) {
-    for (int c = 0; c < chunks; ++c) {
-      const float mc = p[(size_t)c * PSTRIDE + DH];
-      if (mc == -INFINITY) continue;
-      const float w = exp2f(mc - m);
-      l += w * p[(size_t)c * PSTRIDE + DH + 1];
-      const float2 a = *reinterpret_cast<const float2 *>(p + (size_t)c * PSTRIDE + 4 * lane);
-      const float2 bq = *reinterpret_cast<const float2 *>(p + (size_t)c * PSTRIDE + 4 * lane + 2);
-      acc.x += w * a.x; acc.y += w * a.y; acc.z += w * bq.x; acc.w += w * bq.y;
+      for (int k = 0; k < 8; ++k) {
+        const float2 v = ld_cluster2(at + DH * 4, k < chunks ? k : 0);
+        pm[k] = k < chunks ? v.x : -INFINITY;
+        pl[k] = v.y;
+      }
+      float mx = pm[0];
+#pragma unroll
+      for (int k = 1; k < 8; ++k) mx = fmaxf(mx, pm[k]);
+      float lsum = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        pm[k] = mx == -INFINITY ? 0.f : exp2f(pm[k] - mx);
+        lsum += pm[k] * pl[k];
+      }
+      const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+      const size_t ob = (size_t)r * H + h * DH + dd;
+      for (int d = 0; d < nd; d += 2) {
+        float2 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = ld_cluster2(at + (dd + d) * 4, k < chunks ? k : 0);
+        float x = 0.f, y = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { x += pm[k] * v[k].x; y += pm[k] * v[k].y; }      // in chunk order
+        uint32_t hi, lo;
+        split_pack(x * inv, y * inv, hi, lo);
+        *reinterpret_cast<uint32_t *>(out + ob + d) = hi;
+        if (out_lo != nullptr) *reinterpret_cast<uint32_t *>(out_lo + ob + d) = lo;
+      }
     }
+    // no CTA leaves while another may still read its result
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    return;
   }
+  if (!in_row) return;
   const float inv = l > 0.f ? 1.f / l : 0.f;
-  const float v[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
-  const size_t o = (size_t)pair * DH + 4 * lane;      // pair = r * n_heads + h  ->  r * H + h * DH
+  const size_t ob = (size_t)r * H + h * DH + d0;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const bf16 hi = __float2bfloat16_rn(v[e]);
-    out[o + e] = hi;
-    if (out_lo != nullptr) out_lo[o + e] = __float2bfloat16_rn(v[e] - __bfloat162float(hi));
+  for (int d = 0; d < 16; d += 2) {
+    uint32_t hi, lo;
+    split_pack(acc[d] * inv, acc[d + 1] * inv, hi, lo);
+    *reinterpret_cast<uint32_t *>(out + ob + d) = hi;
+    if (out_lo != nullptr) *reinterpret_cast<uint32_t *>(out_lo + ob + d) = lo;
   }
 }
 
 }  // namespace
 
-// Key chunks per (sequence, head, row group): as many as keep the CTA count within two CTAs per SM
-// (96 KB of shared memory each), at least one per 2048 keys of capacity, never finer than 128 keys of
-// capacity per chunk.  One chunk means one kernel (no partials, no combine).  (7B-shaped draft
-// iteration, 10 rows, context 1024: 1.965 / 1.905 / 1.858 / 1.845 / 1.839 ms with 1 / 2 / 4 / 6 / 8
-// chunks; 13B shape at batch 4, 160 sequence-head pairs: flat from 1 to 4, slower beyond.)
+// Key chunks per (sequence, head, row group) = cluster size: the largest of 1, 2, 4, 8 that keeps the
+// launch within what is resident at once (two CTAs of 96 KB per SM; clusters of eight do not fill every
+// GPC, hence seven eighths), never finer than 128 keys of capacity per chunk.
 int g_attn_mma_chunks = 0;     // > 0: this many key chunks whatever the shape (A/B runs)
 void attn_mma_set_chunks(int chunks) { g_attn_mma_chunks = chunks; }
 int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms) {
   const int rgs = (rows_per_seq + 15) / 16;
+  const int room = 2 * num_sms * 7 / 8;
+  int c = 1;
   if (g_attn_mma_chunks > 0) {
-    const int lim = S_max / 64 > 1 ? S_max / 64 : 1;
-    const int f = g_attn_mma_chunks > 16 ? 16 : g_attn_mma_chunks;
-    return f > lim ? lim : f;
+    while (2 * c <= g_attn_mma_chunks && 2 * c <= 8 && 2 * c * 64 <= S_max) c *= 2;
+    return c;
   }
-  int c = (2 * num_sms) / (rgs * B * n_heads);
-  const int by_len = (S_max + 2047) / 2048;
-  c = c < by_len ? by_len : c;
-  const int cap = S_max / 128 > 1 ? S_max / 128 : 1;
-  c = c > cap ? cap : c;
-  return c < 1 ? 1 : (c > 16 ? 16 : c);
-}
-
-size_t attn_mma_scratch_floats(int rows_total, int n_heads, int chunks) {
-  return (size_t)rows_total * n_heads * chunks * PSTRIDE;
+  while (c < 8 && 2 * c * rgs * B * n_heads <= room && 2 * c * 128 <= S_max) c *= 2;
+  return c;
 }
 
 cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, const void *v_cache,
-                               RowPlan plan, Operand out, float *scratch, int rows_per_seq, int B,
-                               int n_heads, int S_max, int chunks) {
+                               RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks) {
   static SmemOptIn optin;
   const size_t smem = (size_t)NST * 2 * TILE_BYTES;
-  static_assert((size_t)4 * 16 * MSTRIDE * sizeof(float) <= (size_t)NST * 2 * TILE_BYTES, "merge buffer fits");
+  static_assert((size_t)5 * 16 * MSTRIDE * sizeof(float) <= (size_t)NST * 2 * TILE_BYTES, "merge buffer fits");
   {
     cudaError_t e = optin.ensure((const void *)tree_attn_mma_kernel, smem);
     if (e != cudaSuccess) return e;
   }
   const int rgs = (rows_per_seq + 15) / 16;
-  if (rgs < 1 || rgs > 8 || chunks < 1) return cudaErrorInvalidValue;
-  cudaError_t e = launch_k(tree_attn_mma_kernel, dim3(chunks, rgs, n_heads * B), dim3(128), smem, L.st, L.pdl, q,
-                           (const bf16 *)k_cache, (const bf16 *)v_cache, plan, scratch, (bf16 *)out.hi,
-                           (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks);
-  if (e != cudaSuccess || chunks == 1) return e;
-  const int R = B * rows_per_seq;
-  return launch_k(tree_attn_combine_kernel, dim3((R * n_heads + 7) / 8), dim3(256), 0, L.st, L.pdl,
-                  (const float *)scratch, (bf16 *)out.hi, (bf16 *)out.lo, R, n_heads, chunks);
+  if (rgs < 1 || rgs > 8 || (chunks != 1 && chunks != 2 && chunks != 4 && chunks != 8)) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(chunks, rgs, n_heads * B);
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = L.st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = L.pdl ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = chunks;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chunks > 1 ? 2 : 1;
+  ++g_launches;
+  return cudaLaunchKernelEx(&cfg, tree_attn_mma_kernel, q, (const bf16 *)k_cache, (const bf16 *)v_cache, plan,
+                            (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks);
 }
 
 }  // namespace koala

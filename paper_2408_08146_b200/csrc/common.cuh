@@ -200,8 +200,8 @@ cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, in
 cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_cache,
                            const void *v_cache, RowPlan plan, Operand out, int R, int rows_per_seq,
                            int B, int n_heads, int head_dim, int S_max);
-// row r of the forward: logits row and output index map(r)
-cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, RowMap map, int R, int V);
+// out[map(r)] <- arg-max of row r; with `spread` the row is also copied to row map(r) of it
+cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, float *spread, RowMap map, int R, int V);
 cudaError_t topk_logp(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k);
 // dst[r] = T(src[row_src ? row_src[r] : r]); optionally dst32[r * dst32_stride] = the same row in fp32
 cudaError_t cast_rows(Launch L, int dtype, const float *src, const int32_t *row_src, Operand dst,
@@ -210,10 +210,13 @@ cudaError_t reduce_splits(Launch L, SplitIn P, float *Y, int ldy, int R, int nco
 
 // attn_mma.cu : bf16 caches, head_dim 128, tensor cores, split over key chunks
 int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms);
-size_t attn_mma_scratch_floats(int rows_total, int n_heads, int chunks);
 cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, const void *v_cache,
-                               RowPlan plan, Operand out, float *scratch, int rows_per_seq, int B,
-                               int n_heads, int S_max, int chunks);
+                               RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks);
+
+// attn_few.cu : bf16 caches, head_dim 128, at most ATTN_FEW_ROWS query rows per sequence
+constexpr int ATTN_FEW_ROWS = 4;
+cudaError_t tree_attention_few(Launch L, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
+                               Operand out, int rows_per_seq, int B, int n_heads, int S_max, int num_sms);
 
 // attn_tc.cu : the same on tcgen05 tensor cores, all rows of a sequence in one CTA, key chunks as a cluster;
 // the queries come as the bf16 pair written by rope_kv_write ([q_rows_alloc][n_heads * 128] each)
@@ -225,17 +228,16 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
 
 // gemm_simt.cu : Y[R][sum n_out] (fp32, ld ldy) = X[R][K_in] * W^T, X and W of `dtype`
 cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int R, float *Y,
-                      int ldy, RowMap ymap);
+                      int ldy);
 
 // gemm_tc.cu : bf16 tensor-core path; writes `split` partial matrices `split_stride` apart.
 int tc_init_driver(char *err, size_t errlen);   // 0 on success
 bool tc_supported(const GemmMats &m, int K_in);
 int tc_default_split(int n_tiles, int kblocks, int tokens);
-// Row r of the product is row ymap(r) of Y (not the identity only with split == 1).
 // split >= 1: classic split-K; split == 0: automatic (stream-K where it applies).  `max_slots`
 // bounds the partial matrices written; *out describes them for the consumer.
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
-                    float *Y, int ldy, RowMap ymap, int split, size_t split_stride, int *status, int max_slots,
+                    float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
                     SplitIn *out);
 
 // layer_tc.cu : several GEMMs of a decoder layer and the row-wise steps between them in one

@@ -18,7 +18,7 @@ template <typename T>
 __global__ void __launch_bounds__(WARPS * 32)
 gemm_simt_kernel(const T *X, const T *Xlo, int R, int K_in, const T *__restrict__ W0,
                  const T *__restrict__ W1, const T *__restrict__ W2, int n0, int n1, int n2,
-                 float *__restrict__ Y, int ldy, RowMap ymap) {
+                 float *__restrict__ Y, int ldy) {
   __shared__ float xs[ROWS][KC + 1];
   pdl_launch_dependents();
   pdl_wait();
@@ -74,7 +74,7 @@ gemm_simt_kernel(const T *X, const T *Xlo, int R, int K_in, const T *__restrict_
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       const float v = warp_sum(acc[f][r]);
-      if (lane == 0 && col[f] < ntot && r0 + r < R) Y[(size_t)ymap(r0 + r) * ldy + col[f]] = v;
+      if (lane == 0 && col[f] < ntot && r0 + r < R) Y[(size_t)(r0 + r) * ldy + col[f]] = v;
     }
 }
 
@@ -104,7 +104,7 @@ template <> struct Vec4<bf16> {
 template <typename T, int RT>
 __global__ void __launch_bounds__(WARPS * 32)
 gemm_simt_small_kernel(const T *X, const T *Xlo, int R, int K_in, const T *__restrict__ W0, const T *__restrict__ W1,
-                       const T *__restrict__ W2, int n0, int n1, int n2, float *__restrict__ Y, int ldy, RowMap ymap) {
+                       const T *__restrict__ W2, int n0, int n1, int n2, float *__restrict__ Y, int ldy) {
   pdl_launch_dependents();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int ntot = n0 + n1 + n2;
@@ -160,13 +160,13 @@ gemm_simt_small_kernel(const T *X, const T *Xlo, int R, int K_in, const T *__res
   for (int o = 32 / RT / 2; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   constexpr int LPR = 32 / RT;                        // lanes that hold the same row
   const int row = r0 + lane / LPR;
-  if (lane % LPR == 0 && row < R) Y[(size_t)ymap(row) * ldy + col] = v;
+  if (lane % LPR == 0 && row < R) Y[(size_t)row * ldy + col] = v;
 }
 
 }  // namespace
 
 cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int R, float *Y,
-                      int ldy, RowMap ymap) {
+                      int ldy) {
   const int n0 = m.n_out[0], n1 = m.n > 1 ? m.n_out[1] : 0, n2 = m.n > 2 ? m.n_out[2] : 0;
   const int ntot = n0 + n1 + n2;
   // The small kernel reads a weight row once per RT rows of X and X once per block of eight features,
@@ -183,7 +183,7 @@ cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int 
       dim3 g((ntot + WARPS - 1) / WARPS, (R + RT - 1) / RT);
       return launch_k(gemm_simt_small_kernel<T, RT>, g, dim3(WARPS * 32), 0, L.st, L.pdl, (const T *)X.hi,
                       (const T *)X.lo, R, K_in, (const T *)m.W[0], (const T *)(m.n > 1 ? m.W[1] : m.W[0]),
-                      (const T *)(m.n > 2 ? m.W[2] : m.W[0]), n0, n1, n2, Y, ldy, ymap);
+                      (const T *)(m.n > 2 ? m.W[2] : m.W[0]), n0, n1, n2, Y, ldy);
     };
     // rows per warp: as few as keep the grid near two blocks per SM (more blocks, shorter chains)
     const bool wide = (long long)((ntot + WARPS - 1) / WARPS) * ((R + 7) / 8) > 2 * 148;
@@ -200,10 +200,10 @@ cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int 
   if (dtype == 0)
     return launch_k(gemm_simt_kernel<float>, grid, dim3(WARPS * 32), 0, L.st, L.pdl, (const float *)X.hi,
                     (const float *)X.lo, R, K_in, (const float *)m.W[0], (const float *)(m.n > 1 ? m.W[1] : m.W[0]),
-                    (const float *)(m.n > 2 ? m.W[2] : m.W[0]), n0, n1, n2, Y, ldy, ymap);
+                    (const float *)(m.n > 2 ? m.W[2] : m.W[0]), n0, n1, n2, Y, ldy);
   return launch_k(gemm_simt_kernel<bf16>, grid, dim3(WARPS * 32), 0, L.st, L.pdl, (const bf16 *)X.hi,
                   (const bf16 *)X.lo, R, K_in, (const bf16 *)m.W[0], (const bf16 *)(m.n > 1 ? m.W[1] : m.W[0]),
-                  (const bf16 *)(m.n > 2 ? m.W[2] : m.W[0]), n0, n1, n2, Y, ldy, ymap);
+                  (const bf16 *)(m.n > 2 ? m.W[2] : m.W[0]), n0, n1, n2, Y, ldy);
 }
 
 }  // namespace koala

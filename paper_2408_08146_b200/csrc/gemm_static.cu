@@ -68,13 +68,13 @@ int koala_gemm_bf16_static(const void *X, const void *X_lo, const void *W, float
   Operand Xo{const_cast<void *>(X), const_cast<void *>(X_lo)};
   const int rows_alloc = koala_gemm_x_rows(M, X_lo != nullptr);
   if (split == 1)
-    return gemm_tc(L, Xo, rows_alloc, m, K_in, M, Y, ldy, RowMap{0, 0}, 1, 0, device_status, 1, nullptr) == cudaSuccess ? KOALA_OK
+    return gemm_tc(L, Xo, rows_alloc, m, K_in, M, Y, ldy, 1, 0, device_status, 1, nullptr) == cudaSuccess ? KOALA_OK
                                                                                               : KOALA_E_CUDA;
   if ((size_t)split * stride > STATIC_SCRATCH_FLOATS) return KOALA_E_CAPACITY;   // an explicit factor that does not fit
   // every partial element that is read below is written by exactly one CTA of this launch, so the
   // previous call's contents need no clearing
   SplitIn s;
-  if (gemm_tc(L, Xo, rows_alloc, m, K_in, M, scratch, N_out, RowMap{0, 0}, split, stride, device_status, split, &s) != cudaSuccess)
+  if (gemm_tc(L, Xo, rows_alloc, m, K_in, M, scratch, N_out, split, stride, device_status, split, &s) != cudaSuccess)
     return KOALA_E_CUDA;
   return reduce_splits(L, s, Y, ldy, M, N_out) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;
 }

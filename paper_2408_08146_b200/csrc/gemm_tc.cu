@@ -53,7 +53,6 @@ constexpr int L2_AHEAD = 0;          // weight tiles (16 KB each) prefetched int
 struct TcParams {
   float *Y;
   int ldy;
-  RowMap ymap;        // row of Y of a token (identity unless the output is whole: split 1)
   int R;              // valid tokens
   int bn;             // MMA N = rows of the activation tile in shared memory, multiple of 16, <= 256
   int tt;             // tokens per tile: bn, or bn / 2 when the activations are a hi/lo pair
@@ -342,7 +341,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int t = tok0 + c0 + j;
-            if (t < P.R) Yp[(size_t)P.ymap(t) * P.ldy] = __uint_as_float(v[j]);
+            if (t < P.R) Yp[(size_t)t * P.ldy] = __uint_as_float(v[j]);
           }
         }
       };
@@ -917,7 +916,7 @@ int tc_streamk_ctas(int n_tiles, int kblocks, int tokens, int max_slots, int *sl
 }
 
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
-                    float *Y, int ldy, RowMap ymap, int split, size_t split_stride, int *status, int max_slots,
+                    float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
                     SplitIn *out) {
   if (!use_current_device()) return cudaErrorInitializationError;
   if (!tc_supported(m, K_in) || R < 1 || ((uintptr_t)X.hi & 15u) || ((uintptr_t)X.lo & 15u))
@@ -946,7 +945,6 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   while (cols < bn) cols <<= 1;
   P.Y = Y;
   P.ldy = ldy;
-  P.ymap = ymap;
   P.R = R;
   P.bn = bn;
   P.tmem_cols = cols;
@@ -1041,7 +1039,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
       return cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel, mw[0], mw[1], mw[2], mx, mxlo, P);
     }
     memset(&P, 0, sizeof(P));
-    P.tt = tt; P.pair = pair; P.accp = accp; P.ztiles = ztiles; P.Y = Y; P.ldy = ldy; P.ymap = ymap; P.R = R; P.bn = bn; P.tmem_cols = cols;
+    P.tt = tt; P.pair = pair; P.accp = accp; P.ztiles = ztiles; P.Y = Y; P.ldy = ldy; P.R = R; P.bn = bn; P.tmem_cols = cols;
   }
   const int bmw = wide ? 2 * BM : BM;
   P.wide = wide ? 1 : 0;

@@ -70,13 +70,11 @@ struct koala_ctx {
   size_t p_floats;        // capacity of P
   size_t pcols;           // widest GEMM output
   // workspace
-  float *attn_part;
   float *sumsq[2];        // per-row partial sums of squares of the two deferred RMSNorms of a layer
   unsigned *layer_sync;   // device counters of the persistent layer kernel
   unsigned layer_use[LAYER_MAX_PHASES];   // how often each counter has been used (host)
   bool stream_layers;     // decoder layers run through the persistent layer kernel where it applies
   RowScale pending;       // scale still owed by the consumer of the GEMM that reads c->xn
-  int attn_chunks;
   float *x, *qbuf, *P, *verify_logits, *draft_logits, *verify_hid, *feat[2], *mx;
   Operand xn, attn_out, act, cat, lmin;
   size_t p_off;            // floats: where in P the next GEMM's partial sums go (0 except while heads are batched)
@@ -181,6 +179,7 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   c->x = w.take<float>((size_t)Mp * H);
   c->qbuf = w.take<float>((size_t)Mp * H);
   c->p_floats = (size_t)(MAX_SPLIT * Mt > INGEST_SPLIT * wide ? MAX_SPLIT * Mt : INGEST_SPLIT * wide) * pcols;
+  if (B > 1 && c->p_floats < (size_t)M * V) c->p_floats = (size_t)M * V;       // a short tree's logits pass through it
   c->P = w.take<float>(c->p_floats);
   c->verify_logits = w.take<float>((size_t)Mt * V);
   c->draft_logits = w.take<float>((size_t)(draft_rows + 16) * V);
@@ -207,10 +206,6 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   c->act = operand(F);
   c->cat = operand(2 * H);
   c->lmin = operand(H);
-  c->attn_chunks = 16;     // largest chunk count any launch may choose
-  c->attn_part = (cfg.dtype == KOALA_BF16 && cfg.head_dim == 128)
-                     ? w.take<float>(attn_mma_scratch_floats(Mt, cfg.n_heads, c->attn_chunks))
-                     : nullptr;
   c->sumsq[0] = w.take<float>((size_t)Mp * 32);
   c->sumsq[1] = w.take<float>((size_t)Mp * 32);
   c->layer_sync = w.take<unsigned>(LAYER_SYNC_WORDS);
@@ -297,7 +292,7 @@ RowPlan row_plan(koala_ctx *c) {
 // Y = X * [W...]^T as a (possibly split) fp32 result in the partial buffer, or directly into
 // `direct` (ld = ld_direct) when given.
 int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct, int ld_direct,
-            SplitIn *out, RowMap ymap = RowMap{0, 0}) {
+            SplitIn *out) {
   int ncols = 0;
   for (int i = 0; i < m.n; ++i) ncols += m.n_out[i];
   float *Y = direct ? direct : c->P + c->p_off;
@@ -309,12 +304,12 @@ int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct,
     const int slots = fit < (size_t)MAX_SPLIT ? (int)fit : MAX_SPLIT;
     const int tb = time_begin(c, KOALA_CLS_GEMM_TC, wbytes);
     SplitIn res;
-    CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, ymap, direct ? 1 : 0, stride, c->status, slots, &res));
+    CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, direct ? 1 : 0, stride, c->status, slots, &res));
     time_end(c, tb);
     if (out) *out = res;
   } else {
     const int tb = time_begin(c, KOALA_CLS_GEMM_SIMT, wbytes);
-    CU_TRY(gemm_simt(LN(c), c->cfg.dtype, X, m, K_in, R, Y, ld, ymap));
+    CU_TRY(gemm_simt(LN(c), c->cfg.dtype, X, m, K_in, R, Y, ld));
     time_end(c, tb);
     if (out) *out = SplitIn{Y, 1, 0, ld, 0u, 0u, 0u};
   }
@@ -337,10 +332,12 @@ int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq) {
       attn_tc_supported(rows_per_seq, g.head_dim, g.S_max)) {
     CU_TRY(tree_attention_tc(LN(c), c->qpair, c->Mp, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups,
                              g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, 148), c->status));
-  } else if (c->use_tc && g.head_dim == 128 && c->attn_part != nullptr && rows_per_seq <= 128) {
-    CU_TRY(tree_attention_mma(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, c->attn_part, rows_per_seq,
-                              groups, g.n_heads, g.S_max,
-                              c->ingest_blocks > 0 ? 1 : attn_mma_chunks(g.B, g.n_heads, rows_per_seq, g.S_max, 148)));
+  } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq <= ATTN_FEW_ROWS) {
+    CU_TRY(tree_attention_few(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
+                              g.S_max, 148));
+  } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq <= 128) {
+    CU_TRY(tree_attention_mma(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
+                              g.S_max, attn_mma_chunks(groups, g.n_heads, rows_per_seq, g.S_max, 148)));
   } else {
     CU_TRY(tree_attention(LN(c), g.dtype, c->qbuf, kc, vc, row_plan(c), c->attn_out, R, rows_per_seq, groups,
                           g.n_heads, g.head_dim, g.S_max));
@@ -866,8 +863,12 @@ int koala_verify(koala_ctx *c, const koala_tree *tree) {
   K_TRY(embed_rows(c, R));
   K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, rows, c->final_norm, c->lmin, c->verify_hid, out_map));
   GemmMats lm{{c->lm_head, nullptr, nullptr}, {g.V, 0, 0}, 1};
-  K_TRY(do_gemm(c, c->lmin, g.H, lm, R, c->verify_logits, g.V, nullptr, out_map));
-  CU_TRY(argmax_rows(LN(c), c->verify_logits, c->verify_tgt, out_map, R, g.V));
+  // spread rows: the product goes through the partial-sum buffer and the arg-max kernel, which reads every
+  // logit anyway, puts the rows in their places (in the multiply's own stores the row arithmetic cost
+  // every launch 4 %)
+  float *logits = out_map.rows == 0 ? c->verify_logits : c->P;
+  K_TRY(do_gemm(c, c->lmin, g.H, lm, R, logits, g.V, nullptr));
+  CU_TRY(argmax_rows(LN(c), logits, c->verify_tgt, out_map.rows == 0 ? nullptr : c->verify_logits, out_map, R, g.V));
   c->phase = PH_VERIFIED;
   return KOALA_OK;
 }
@@ -1138,8 +1139,7 @@ int koala_gemm_bf16(const void *X, const void *X_lo, const void *W, float *Y, in
   Launch L{(cudaStream_t)cuda_stream, false};
   GemmMats m{{W, nullptr, nullptr}, {N_out, 0, 0}, 1};
   Operand Xo{const_cast<void *>(X), const_cast<void *>(X_lo)};
-  const RowMap same{0, 0};
-  if (!use_tensor_cores) return gemm_simt(L, KOALA_BF16, Xo, m, K_in, M, Y, ldy, same) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;
+  if (!use_tensor_cores) return gemm_simt(L, KOALA_BF16, Xo, m, K_in, M, Y, ldy) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;
   char e[160];
   if (tc_init_driver(e, sizeof(e)) != 0) return KOALA_E_CUDA;
   if (!tc_supported(m, K_in)) return KOALA_E_UNSUPPORTED;
@@ -1148,12 +1148,12 @@ int koala_gemm_bf16(const void *X, const void *X_lo, const void *W, float *Y, in
   // X must hold whole token tiles (koala_gemm_x_rows)
   const int rows_alloc = koala_gemm_x_rows(M, X_lo != nullptr);
   if (split_k == 1)
-    return gemm_tc(L, Xo, rows_alloc, m, K_in, M, Y, ldy, same, 1, 0, device_status, 1, nullptr) == cudaSuccess
+    return gemm_tc(L, Xo, rows_alloc, m, K_in, M, Y, ldy, 1, 0, device_status, 1, nullptr) == cudaSuccess
                ? KOALA_OK : KOALA_E_CUDA;
   const size_t stride = (size_t)M * N_out;
   if (!scratch || scratch_bytes < (size_t)MAX_SPLIT * stride * sizeof(float)) return KOALA_E_CAPACITY;
   SplitIn s;
-  if (gemm_tc(L, Xo, rows_alloc, m, K_in, M, (float *)scratch, N_out, same, split_k, stride, device_status, MAX_SPLIT,
+  if (gemm_tc(L, Xo, rows_alloc, m, K_in, M, (float *)scratch, N_out, split_k, stride, device_status, MAX_SPLIT,
               &s) != cudaSuccess)
     return KOALA_E_CUDA;
   return reduce_splits(L, s, Y, ldy, M, N_out) == cudaSuccess ? KOALA_OK : KOALA_E_CUDA;

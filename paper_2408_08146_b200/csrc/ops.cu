@@ -576,15 +576,20 @@ __device__ __forceinline__ ValIdx block_argmax(ValIdx x, ValIdx *red) {
   return x;
 }
 
-__global__ void argmax_rows_kernel(const float *logits, int32_t *__restrict__ out, RowMap map, int V) {
+__global__ void argmax_rows_kernel(const float *logits, int32_t *__restrict__ out, float *spread, RowMap map, int V) {
   __shared__ ValIdx red[32];
   pdl_launch_dependents();
   pdl_wait();
-  const float *row = logits + (size_t)map(blockIdx.x) * V;
+  const float *row = logits + (size_t)blockIdx.x * V;
+  const int to = map(blockIdx.x);
   ValIdx best{-INFINITY, 0x7fffffff};
-  for (int i = threadIdx.x; i < V; i += blockDim.x) best = better(best, ValIdx{row[i], i});
+  for (int i = threadIdx.x; i < V; i += blockDim.x) {
+    const float v = row[i];
+    best = better(best, ValIdx{v, i});
+    if (spread != nullptr) spread[(size_t)to * V + i] = v;
+  }
   best = block_argmax(best, red);
-  if (threadIdx.x == 0) out[map(blockIdx.x)] = best.i;
+  if (threadIdx.x == 0) out[to] = best.i;
 }
 
 // Per row: the k largest logits (ties: smaller id) and their natural-log softmax probabilities.
@@ -710,7 +715,7 @@ topk_logp_fast_kernel(const float *logits, int32_t *__restrict__ tok, float *__r
 // candidates (ties still go to the smaller id) and forms the log-sum-exp.  V <= 32768, k <= 32.
 constexpr int TKP = 8;            // CTAs per row
 __global__ void __launch_bounds__(256)
-topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp, RowMap map, int V, int k) {
+topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp, float *spread, RowMap map, int V, int k) {
   // logp == nullptr: only the ids are wanted (the arg-max of a row is its top-1), no exponentials
   __shared__ ValIdx cand[8 * 32];
   __shared__ ValIdx mine[32];     // this CTA's k best, read by CTA 0
@@ -718,11 +723,11 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
   __shared__ float redf[32];
   pdl_launch_dependents();
   pdl_wait();
-  const int part = blockIdx.x, r = map(blockIdx.y);
+  const int part = blockIdx.x, r = map(blockIdx.y);          // the row is read at blockIdx.y, its results go to r
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int chunk = (((V + TKP - 1) / TKP) + 255) & ~255;          // ids per CTA, a multiple of 256
   const int base = part * chunk;
-  const float *row = logits + (size_t)r * V;
+  const float *row = logits + (size_t)blockIdx.y * V;
   float vals[16];
   float mx = -INFINITY;
 #pragma unroll
@@ -730,6 +735,7 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
     const int i = base + tid + 256 * j;
     vals[j] = (tid + 256 * j < chunk && i < V) ? row[i] : -INFINITY;
     mx = fmaxf(mx, vals[j]);
+    if (spread != nullptr && tid + 256 * j < chunk && i < V) spread[(size_t)r * V + i] = vals[j];
   }
   mx = warp_max(mx);
   if (lane == 0) redf[w] = mx;
@@ -943,8 +949,8 @@ cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_ca
   return cudaErrorInvalidValue;
 }
 
-static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *tok, float *logp, RowMap map, int R, int V,
-                                       int k) {
+static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *tok, float *logp, float *spread, RowMap map,
+                                       int R, int V, int k) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(TKP, R);
   cfg.blockDim = dim3(256);
@@ -959,17 +965,17 @@ static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *t
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   ++g_launches;
-  return cudaLaunchKernelEx(&cfg, topk_logp_cluster_kernel, logits, tok, logp, map, V, k);
+  return cudaLaunchKernelEx(&cfg, topk_logp_cluster_kernel, logits, tok, logp, spread, map, V, k);
 }
 
-cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, RowMap map, int R, int V) {
+cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, float *spread, RowMap map, int R, int V) {
   // the arg-max (ties: smaller id) is the top-1; wide rows go to the eight-CTA kernel
-  if (V <= 32768 && V >= 4096) return topk_cluster_launch(L, logits, out, nullptr, map, R, V, 1);
-  return launch_k(argmax_rows_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, out, map, V);
+  if (V <= 32768 && V >= 4096) return topk_cluster_launch(L, logits, out, nullptr, spread, map, R, V, 1);
+  return launch_k(argmax_rows_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, out, spread, map, V);
 }
 
 cudaError_t topk_logp(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k) {
-  if (V <= 32768 && k <= 32 && V >= 4096) return topk_cluster_launch(L, logits, tok, logp, RowMap{0, 0}, R, V, k);
+  if (V <= 32768 && k <= 32 && V >= 4096) return topk_cluster_launch(L, logits, tok, logp, nullptr, RowMap{0, 0}, R, V, k);
   if (V <= 32768 && k <= 32)
     return launch_k(topk_logp_fast_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, tok, logp, V, k);
   const size_t smem = (size_t)V * sizeof(float);

@@ -335,3 +335,49 @@ def test_short_caller_trees_of_a_batch_run_only_their_rows(base, B, N, n_max):
     eng.koala_accept(None)
     assert eng.device_status() == 0
     eng.close()
+
+
+@pytest.mark.parametrize("N,B,n_heads,context,S_max", [
+    (2, 1, 32, 1, 128),          # less than one tile
+    (2, 1, 32, 63, 256),         # the tree crosses a tile boundary; fewer tiles than CTAs
+    (3, 1, 8, 3000, 4096),       # few heads: every head is cut into many parts
+    (4, 2, 32, 700, 1024),
+    (4, 9, 8, 200, 512),         # more (sequence, head) pairs than parts
+    (2, 1, 1, 2000, 2048),       # a single head
+    (3, 5, 16, 130, 256),
+    (5, 1, 32, 777, 1024),       # five to eight rows
+    (8, 3, 8, 500, 1024),
+    (7, 1, 2, 1900, 2048),
+    (9, 1, 32, 1000, 1024),      # nine to fifteen rows: mma.sync, chunks merged by the last arriver
+    (15, 2, 8, 600, 2048),
+])
+@pytest.mark.parametrize("kind", ["plain", "poison", "growing"])
+def test_attention_of_few_rows(N, B, n_heads, context, S_max, kind):
+    """At most eight rows per sequence: tiles dealt evenly to the CTAs, parts merged by the last arriver."""
+    _attention_case(N, B, n_heads, context, S_max, poison=kind == "poison", growing=kind == "growing")
+
+
+def test_attention_of_one_row_ragged_batch():
+    """One-node trees of a ragged batch, twice on the same engine (the arrival counters are left at zero)."""
+    cfg = reduced(T7_EAGLE, 1, K=1, N=1, D=1, topk=1, B=4, H=1024, n_heads=8, F=2048, V=2048, S_max=1536, prompt_len=1400)
+    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
+    eng.target_k.copy_(random_kv(cfg, "target_k", cfg.L, DEV))
+    eng.target_v.copy_(random_kv(cfg, "target_v", cfg.L, DEV))
+    lens = [1400, 3, 700, 64]
+    for b in range(4):
+        orc.target_k[0][b][...] = kv_to_oracle(eng.target_k, 0, b, np.float32)
+        orc.target_v[0][b][...] = kv_to_oracle(eng.target_v, 0, b, np.float32)
+        orc.seq_len[b] = lens[b]
+    eng.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    toks = [[5], [6], [7], [8]]
+    first = None
+    orc.verify([(t, [-1]) for t in toks])
+    for _ in range(2):
+        eng.koala_verify(_tree_arrays(eng, toks, [[-1]] * 4))
+        hid = eng.buffers()["verify_hid"].clone()
+        for b in range(4):
+            assert_close(hid[b:b + 1].cpu().numpy(), orc.verify_hid[b][:1], cfg.dtype, f"hidden {b}")
+        assert first is None or torch.equal(first, hid)
+        first = hid
+    assert eng.device_status() == 0 and eng.check_guards()[1] == 0
+    eng.close()
