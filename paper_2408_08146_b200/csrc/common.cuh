@@ -37,6 +37,16 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// CTAs (= partial sums) that share stream-K tile `tile` of sk_kb K-blocks.  Not inlined: the kernels that
+// add partial sums run each instruction once or twice per launch, so what they cost is mostly the fetch
+// of their instructions, and two integer divisions per column group are a large part of them.
+static __device__ __noinline__ int sk_count(unsigned tile, unsigned ctas, unsigned units, unsigned kb) {
+  const unsigned u0 = tile * kb;
+  const unsigned first = ((u0 + 1u) * ctas - 1u) / units;
+  const unsigned last = ((u0 + kb) * ctas - 1u) / units;
+  return (int)(last - first) + 1;
+}
+
 // A matrix given as the sum of partial matrices `stride` floats apart (split-K results).
 // Classic split-K: every column has `n` partials.  Stream-K (sk_ctas > 0): column c belongs to
 // weight tile c / 128 (c / 256 with sk_wide), whose K-blocks were dealt to the CTAs owning units
@@ -53,21 +63,22 @@ struct SplitIn {
   unsigned sk_m0, sk_m1, sk_t0, sk_t1;
   // several token tiles of sk_tt rows dealt in the same launch: tile = weight tile * sk_zt + row / sk_tt
   unsigned sk_zt, sk_tt;
-  __device__ __forceinline__ int count(int r, int c) const {
-    if (sk_ctas == 0) return n;
+  // Stream-K tile that column c (of row r) belongs to.
+  __device__ __forceinline__ unsigned tile_of(int r, int c) const {
     const unsigned sh = 7u + sk_wide, uc = (unsigned)c;
     unsigned tile = uc >> sh;
     if (sk_m0 != 0 && uc >= sk_m0) tile = uc < sk_m1 ? sk_t0 + ((uc - sk_m0) >> sh) : sk_t1 + ((uc - sk_m1) >> sh);
     if (sk_zt > 1) tile = tile * sk_zt + (unsigned)r / sk_tt;
-    const unsigned u0 = tile * sk_kb;
-    const unsigned first = ((u0 + 1u) * sk_ctas - 1u) / sk_units;
-    const unsigned last = ((u0 + sk_kb) * sk_ctas - 1u) / sk_units;
-    return (int)(last - first) + 1;
+    return tile;
+  }
+  __device__ __forceinline__ int count(int r, int c) const {
+    return sk_ctas == 0 ? n : sk_count(tile_of(r, c), sk_ctas, sk_units, sk_kb);
   }
   __device__ __forceinline__ float at(int r, int c) const {
     const float *q = p + (size_t)r * ld + c;
     const int k = count(r, c);
     float v = q[0];
+#pragma unroll 1
     for (int s = 1; s < k; ++s) v += q[(size_t)s * stride];
     return v;
   }
@@ -77,16 +88,26 @@ struct SplitIn {
 // row, `n` partial sums of squares; the consumer of the GEMM's output multiplies by
 // rsqrt(sum / H + eps).  n == 0: nothing pending (the input was already normalised).
 struct RowScale {
-  const float *sumsq;   // [rows][n]
+  const float *sumsq;   // [rows][stride], the first n of each row in use
   int n;
   float inv_h, eps;
+  int stride;           // ROW_SUMS wherever n <= ROW_SUMS (two vector loads), else n (layer kernel)
   __device__ __forceinline__ float of(int r) const {
     if (n == 0) return 1.f;
-    float s = 0.f;
-    for (int i = 0; i < n; ++i) s += sumsq[(size_t)r * n + i];
+    const float4 a = *reinterpret_cast<const float4 *>(sumsq + (size_t)r * 8);
+    const float4 b = *reinterpret_cast<const float4 *>(sumsq + (size_t)r * 8 + 4);
+    float s = a.x;
+    if (n > 1) s += a.y;
+    if (n > 2) s += a.z;
+    if (n > 3) s += a.w;
+    if (n > 4) s += b.x;
+    if (n > 5) s += b.y;
+    if (n > 6) s += b.z;
+    if (n > 7) s += b.w;
     return rsqrtf(s * inv_h + eps);
   }
 };
+constexpr int ROW_SUMS = 8;   // H <= 8192 in chunks of 1024 columns
 
 // Where row r of a forward goes in a per-node buffer: a forward runs `rows` rows per sequence, the
 // buffer holds `n` per sequence (rows == 0: the two are the same).

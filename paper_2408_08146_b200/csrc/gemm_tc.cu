@@ -7,8 +7,8 @@
 // K = 16, both operands K-major in shared memory with the 128-byte swizzle that TMA writes.
 // The fp32 accumulator [128 x tokens] lives in tensor memory.  Warp 0 streams weight and
 // activation tiles with TMA through a ring of shared-memory stages (mbarrier full/empty pairs),
-// warp 1 issues the MMAs, four to sixteen epilogue warps read the accumulator back (tcgen05.ld,
-// one step ahead of the stores) and store it.
+// warp 1 issues the MMAs, eight or sixteen epilogue warps read the accumulator back (tcgen05.ld)
+// and store it.
 // The weight stream does not depend on the previous kernel, so under programmatic dependent
 // launch the first stages are requested before waiting for the producer of X.
 // Activations may come as a pair hi + lo of bf16 matrices (lo = rounding residual of hi): the
@@ -47,8 +47,6 @@ constexpr int THREADS_WIDE = 576;   // most threads a launch uses: producer warp
 constexpr int W_STAGE_BYTES = BM * BK * 2;
 constexpr int E_TIMEOUT = 6;
 constexpr int MAX_STAGES = 12;
-constexpr int L2_AHEAD = 0;          // weight tiles (16 KB each) prefetched into L2 beyond the ring (measured: any
-                                     // depth slows the small kernels that run meanwhile more than it helps)
 
 struct TcParams {
   float *Y;
@@ -56,7 +54,6 @@ struct TcParams {
   int R;              // valid tokens
   int bn;             // MMA N = rows of the activation tile in shared memory, multiple of 16, <= 256
   int tt;             // tokens per tile: bn, or bn / 2 when the activations are a hi/lo pair
-  int pair;           // 1: hi/lo pair
   int ztiles;         // token tiles (classic mode; fastest-varying part of blockIdx.x)
   int tmem_cols;      // power of two >= max(32, bn), per accumulator buffer
   int nbuf;           // accumulator buffers in tensor memory (2 when they fit in 256 columns)
@@ -68,12 +65,7 @@ struct TcParams {
   unsigned sk_units;  // tiles * kblocks
   size_t split_stride;
   int stages;
-  int wide;           // 1: 256 weight rows per CTA (two accumulators), N = 256, one CTA per SM
-  int accp;           // 1: the pair's residual rows are a second, accumulating MMA into the same columns
-                      //    (bn = tt: up to 256 tokens per tile) instead of extra columns (bn = 2 tt)
-  int pf_ahead;       // weight tiles requested into L2 this many units ahead of the ring (0 = none)
   int early_w;        // how many of the first stages' weight tiles are requested before the dependency wait
-  int l2_ahead;       // weight tiles prefetched into L2 beyond the ring before the dependency wait
   int epi_dry;        // 1: the epilogue warps make a dry pass over their loop body (nothing stored) at kernel start
   int *status;
 };
@@ -83,6 +75,18 @@ __device__ __forceinline__ unsigned sk_owner(unsigned u, unsigned ctas, unsigned
   return ((u + 1u) * ctas - 1u) / units;
 }
 
+// The form of the activations is a template argument: a launch fetches its instructions anew (the
+// kernels of a layer together overflow the instruction caches), so a body holds one form's code only.
+//   FORM_PLAIN  one matrix
+//   FORM_COLS   pair, the residual rows as extra accumulator columns (up to 128 tokens per tile)
+//   FORM_ACC    pair, the residual rows as a second MMA into the same columns (up to 256 tokens)
+// WIDE: 256 weight rows per CTA (FORM_ACC only).  One form for all and unrolled double-buffered stores
+// were 49 KB of instructions, FORM_COLS is 21 KB now: with the same
+// treatment of the row-wise kernels (rotary 42 -> 6 KB, SwiGLU 16 -> 7, residual 9 -> 4) a 7B one-token step
+// went from 3.33 to 3.02 ms, a 60-node EAGLE iteration from 5.76 to 5.24 ms.
+enum { FORM_PLAIN = 0, FORM_COLS = 1, FORM_ACC = 2 };
+
+template <int FORM, bool WIDE>
 __global__ void __launch_bounds__(THREADS_WIDE, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
                const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmX,
@@ -99,23 +103,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char *tiles = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-  const int x_stage_bytes = (P.accp ? 2 : 1) * P.bn * BK * 2;
-  const int w_stage_bytes = P.wide ? 2 * W_STAGE_BYTES : W_STAGE_BYTES;
+  const int x_stage_bytes = (FORM == FORM_ACC ? 2 : 1) * P.bn * BK * 2;
+  const int w_stage_bytes = WIDE ? 2 * W_STAGE_BYTES : W_STAGE_BYTES;
   const int stage_bytes = w_stage_bytes + x_stage_bytes;   // both multiples of 1024
-  const int bm = P.wide ? 2 * BM : BM;                     // weight rows per tile
+  const int bm = WIDE ? 2 * BM : BM;                     // weight rows per tile
   const int KB = P.kblocks;
 
   // this CTA's run of (tile, K-block) units, tile-major; a run may cross tile boundaries (stream-K)
   unsigned u_lo, u_hi;
   int tok0 = 0;
   if (P.sk_ctas > 0) {
-    u_lo = (unsigned)(((unsigned long long)blockIdx.x * P.sk_units) / (unsigned)P.sk_ctas);
-    u_hi = (unsigned)(((unsigned long long)(blockIdx.x + 1) * P.sk_units) / (unsigned)P.sk_ctas);
+    u_lo = blockIdx.x * P.sk_units / (unsigned)P.sk_ctas;           // units x CTAs fits in 32 bits (host)
+    u_hi = (blockIdx.x + 1u) * P.sk_units / (unsigned)P.sk_ctas;
   } else {
     const int tile = blockIdx.x / P.ztiles;
     tok0 = (blockIdx.x % P.ztiles) * P.tt;
-    u_lo = (unsigned)(tile * KB + (int)(((long long)KB * blockIdx.y) / P.split));
-    u_hi = (unsigned)(tile * KB + (int)(((long long)KB * (blockIdx.y + 1)) / P.split));
+    u_lo = (unsigned)(tile * KB) + (unsigned)KB * blockIdx.y / (unsigned)P.split;
+    u_hi = (unsigned)(tile * KB) + (unsigned)KB * (blockIdx.y + 1u) / (unsigned)P.split;
   }
   const int n_units = (int)(u_hi - u_lo);
 
@@ -129,7 +133,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
   // one weight tile of a stage: 128 rows per copy
   auto load_w = [&](const CUtensorMap *tmW, uint64_t *bar, unsigned char *dst, int kb, int row0) {
     tma_load_2d(tmW, bar, dst, kb * BK, row0);
-    if (P.wide) tma_load_2d(tmW, bar, dst + W_STAGE_BYTES, kb * BK, row0 + BM);
+    if (WIDE) tma_load_2d(tmW, bar, dst + W_STAGE_BYTES, kb * BK, row0 + BM);
   };
   const int pre = n_units < P.stages ? n_units : P.stages;
 
@@ -148,32 +152,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // The weight stream starts right here, before the block-wide set-up barrier and before the
-    // dependency wait: weights do not depend on the kernel before this one.  A few more of this
-    // CTA's weight tiles are requested into L2 (bounded, so that all CTAs together stay well
-    // inside the L2).
+    // dependency wait: weights do not depend on the kernel before this one.
     int tile = (int)(u_lo / KB), kb = (int)(u_lo % KB), row0;
     const CUtensorMap *tmW = tile_map(tile, row0);
     const int early = pre < P.early_w ? pre : P.early_w;
-    const int ahead = early == pre ? (n_units < pre + P.l2_ahead ? n_units : pre + P.l2_ahead) : early;
-    for (int it = 0; it < ahead; ++it) {
-      if (it < early) {
-        mbar_expect_tx(&full_bar[it], (uint32_t)stage_bytes);
-        load_w(tmW, &full_bar[it], tiles + (size_t)it * stage_bytes, kb, row0);
-      } else {
-        asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                     ::"l"(tmW), "r"(kb * BK), "r"(row0) : "memory");
-        if (P.wide)
-          asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                       ::"l"(tmW), "r"(kb * BK), "r"(row0 + BM) : "memory");
-      }
+#pragma unroll 1
+    for (int it = 0; it < early; ++it) {
+      mbar_expect_tx(&full_bar[it], (uint32_t)stage_bytes);
+      load_w(tmW, &full_bar[it], tiles + (size_t)it * stage_bytes, kb, row0);
       if (++kb == KB) { kb = 0; ++tile; tmW = tile_map(tile, row0); }
     }
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
-    if (P.pair) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmXlo) : "memory");
+    if (FORM != FORM_PLAIN) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmXlo) : "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(smem_u32(&tmem_base_slot)), "r"((uint32_t)(P.tmem_cols * P.nbuf * (P.wide ? 2 : 1)))
+                 ::"r"(smem_u32(&tmem_base_slot)), "r"((uint32_t)(P.tmem_cols * P.nbuf * (WIDE ? 2 : 1)))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -192,6 +186,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       tile = (int)(u_lo / KB);
       kb = (int)(u_lo % KB);
       tmW = tile_map(tile, row0);
+#pragma unroll 1
       for (int it = 0; it < pre; ++it) {
         unsigned char *xd = tiles + (size_t)it * stage_bytes + w_stage_bytes;
         if (it >= P.early_w) {
@@ -199,40 +194,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
           load_w(tmW, &full_bar[it], tiles + (size_t)it * stage_bytes, kb, row0);
         }
         tma_load_2d(&tmX, &full_bar[it], xd, kb * BK, tok0);
-        if (P.pair) tma_load_2d(&tmXlo, &full_bar[it], xd + lo_off, kb * BK, tok0);
+        if (FORM != FORM_PLAIN) tma_load_2d(&tmXlo, &full_bar[it], xd + lo_off, kb * BK, tok0);
         if (++kb == KB) { kb = 0; ++tile; tmW = tile_map(tile, row0); }
       }
       bool ok = true;
       int s = pre % P.stages;
       uint32_t ph = (uint32_t)(pre / P.stages) & 1u;
-      // Optional (tuning key 14): the weight tiles of the units `pf_ahead` beyond the one being loaded are
-      // requested into L2.  With the two 96 KB stages of the 256-token mode this was measured slower
-      // than no lookahead (13B shapes: 18.2 against 17.7 ms per verification), so it is off.
-      int pf_tile = tile, pf_kb = kb, pf_row0 = row0, pf_it = pre;
-      const CUtensorMap *pf_map = tmW;
-      auto pf_step = [&]() {
-        if (++pf_kb == KB) { pf_kb = 0; ++pf_tile; pf_map = tile_map(pf_tile, pf_row0); }
-        ++pf_it;
-      };
-      auto pf_request = [&]() {
-        asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                     ::"l"(pf_map), "r"(pf_kb * BK), "r"(pf_row0) : "memory");
-        if (P.wide)
-          asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                       ::"l"(pf_map), "r"(pf_kb * BK), "r"(pf_row0 + BM) : "memory");
-      };
-      if (P.pf_ahead > 0) {
-        for (int q = 0; q < P.pf_ahead && pf_it < n_units; ++q) { pf_request(); pf_step(); }
-      }
+#pragma unroll 1
       for (int it = pre; it < n_units; ++it) {
-        if (P.pf_ahead > 0 && pf_it < n_units) { pf_request(); pf_step(); }
         ok = mbar_wait(&empty_bar[s], ph ^ 1u);
         if (!ok) break;
         mbar_expect_tx(&full_bar[s], (uint32_t)stage_bytes);
         unsigned char *dst = tiles + (size_t)s * stage_bytes;
         load_w(tmW, &full_bar[s], dst, kb, row0);
         tma_load_2d(&tmX, &full_bar[s], dst + w_stage_bytes, kb * BK, tok0);
-        if (P.pair) tma_load_2d(&tmXlo, &full_bar[s], dst + w_stage_bytes + lo_off, kb * BK, tok0);
+        if (FORM != FORM_PLAIN) tma_load_2d(&tmXlo, &full_bar[s], dst + w_stage_bytes + lo_off, kb * BK, tok0);
         if (++kb == KB) { kb = 0; ++tile; tmW = tile_map(tile, row0); }
         if (++s == P.stages) { s = 0; ph ^= 1u; }
       }
@@ -274,10 +250,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
           // advance 32 bytes (16 bf16) inside the swizzled row: +2 in the 16-byte address field
           const uint32_t acc = (!seg_start || k > 0) ? 1u : 0u;
           umma_bf16(dacc, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc);
-          if (P.accp) umma_bf16(dacc, da + (uint64_t)(2 * k), db2 + (uint64_t)(2 * k), idesc, 1u);
-          if (P.wide) {
+          if (FORM == FORM_ACC) umma_bf16(dacc, da + (uint64_t)(2 * k), db2 + (uint64_t)(2 * k), idesc, 1u);
+          if (WIDE) {
             umma_bf16(dacc + (uint32_t)P.tmem_cols, da2 + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, acc);
-            if (P.accp) umma_bf16(dacc + (uint32_t)P.tmem_cols, da2 + (uint64_t)(2 * k), db2 + (uint64_t)(2 * k), idesc, 1u);
+            if (FORM == FORM_ACC) umma_bf16(dacc + (uint32_t)P.tmem_cols, da2 + (uint64_t)(2 * k), db2 + (uint64_t)(2 * k), idesc, 1u);
           }
         }
         umma_commit(&empty_bar[s]);      // stage reusable once these MMAs have read it
@@ -328,45 +304,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       int slot = blockIdx.y;
       if (P.sk_ctas > 0)
         slot = (int)blockIdx.x - (int)sk_owner((unsigned)tile * KB, (unsigned)P.sk_ctas, P.sk_units);
-      for (int hw = 0; hw < (P.wide ? 2 : 1); ++hw) {      // wide: one accumulator per 128 weight rows
+#pragma unroll 1
+      for (int hw = 0; hw < (WIDE ? 2 : 1); ++hw) {      // wide: one accumulator per 128 weight rows
       const int feat = row0 + hw * BM + quarter * 32 + lane;
       float *Yp = P.Y + (size_t)slot * P.split_stride + col_off + feat;
       const uint32_t lane_base = tmem_acc + (uint32_t)((buf + hw) * P.tmem_cols) + ((uint32_t)(quarter * 32) << 16);
-      // 16 token columns per step; the next step's accumulator read is in flight while this
-      // step's values are stored
-      // (registers of a read in flight are not touched before its wait)
-      uint32_t va[16], vb[16];
-      auto store16 = [&](const uint32_t (&v)[16], int c0) {
-        if (feat < n_rows) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int t = tok0 + c0 + j;
-            if (t < P.R) Yp[(size_t)t * P.ldy] = __uint_as_float(v[j]);
-          }
-        }
-      };
-      if (P.pair && !P.accp) {
-        // value and residual rows in separate accumulator columns: added here
-        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-          tmem_ld16(lane_base + (uint32_t)c0, va);
+      // 16 token columns per step, in a rolled loop: with eight or sixteen warps the accumulator reads
+      // of one hide behind the stores of the others, and the loop's instructions are fetched once.
+#pragma unroll 1
+      for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+        uint32_t va[16];
+        tmem_ld16(lane_base + (uint32_t)c0, va);
+        if constexpr (FORM == FORM_COLS) {
+          // value and residual rows in separate accumulator columns: added here
+          uint32_t vb[16];
           tmem_ld16(lane_base + (uint32_t)(P.tt + c0), vb);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
           for (int j = 0; j < 16; ++j) va[j] = __float_as_uint(__uint_as_float(va[j]) + __uint_as_float(vb[j]));
-          store16(va, c0);
-        }
-      } else {
-        if (c_lo < c_hi) tmem_ld16(lane_base + (uint32_t)c_lo, va);
-        for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+        } else {
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          const bool has_b = c0 + 16 < c_hi;
-          if (has_b) tmem_ld16(lane_base + (uint32_t)(c0 + 16), vb);
-          store16(va, c0);
-          if (has_b) {
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (c0 + 32 < c_hi) tmem_ld16(lane_base + (uint32_t)(c0 + 32), va);
-            store16(vb, c0 + 16);
-          }
+        }
+        const int left = feat < n_rows ? P.R - (tok0 + c0) : 0;      // tokens of this step that exist
+        float *yp = Yp + (size_t)(tok0 + c0) * P.ldy;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          if (j < left) *yp = __uint_as_float(va[j]);
+          yp += P.ldy;
         }
       }
       }
@@ -397,7 +361,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       __syncwarp();
     }
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                 ::"r"(tmem_acc), "r"((uint32_t)(P.tmem_cols * P.nbuf * (P.wide ? 2 : 1)))
+                 ::"r"(tmem_acc), "r"((uint32_t)(P.tmem_cols * P.nbuf * (WIDE ? 2 : 1)))
                  : "memory");
   }
   if (threadIdx.x == 0 && s_error && P.status) atomicMax(P.status, E_TIMEOUT);
@@ -442,8 +406,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char *tiles = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   const int KB = P.kblocks;
-  const unsigned u_lo = (unsigned)(((unsigned long long)cid * P.sk_units) / (unsigned)P.sk_ctas);
-  const unsigned u_hi = (unsigned)(((unsigned long long)(cid + 1) * P.sk_units) / (unsigned)P.sk_ctas);
+  const unsigned u_lo = cid * P.sk_units / (unsigned)P.sk_ctas;              // fits in 32 bits (host)
+  const unsigned u_hi = (cid + 1u) * P.sk_units / (unsigned)P.sk_ctas;
   const int n_units = (int)(u_hi - u_lo);
   const int n_epi = (int)(blockDim.x >> 5) - 2;
   const int tt = P.tt;                                   // tokens per tile: a multiple of 32, at most 256
@@ -617,30 +581,22 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       if (dry) n_rows = 0;
       // partial-sum slot = rank of this cluster among the tile's contributors
       const int slot = (int)cid - (int)sk_owner((unsigned)tile * KB, (unsigned)P.sk_ctas, P.sk_units);
+#pragma unroll 1
       for (int a = 0; a < 2; ++a) {
         const int feat = row0 + a * 2 * BM + (int)rank * BM + quarter * 32 + lane;
         float *Yp = P.Y + (size_t)slot * P.split_stride + col_off + feat;
         const uint32_t lane_base = tmem_acc + (uint32_t)((buf * 2 + a) * tt) + ((uint32_t)(quarter * 32) << 16);
-        uint32_t va[16], vb[16];
-        auto store16 = [&](const uint32_t (&v)[16], int c0) {
-          if (feat < n_rows) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int t = tok0 + c0 + j;
-              if (t < P.R) Yp[(size_t)t * P.ldy] = __uint_as_float(v[j]);
-            }
-          }
-        };
-        if (c_lo < c_hi) tmem_ld16(lane_base + (uint32_t)c_lo, va);
-        for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {       // rolled, as in the one-CTA kernel
+          uint32_t va[16];
+          tmem_ld16(lane_base + (uint32_t)c0, va);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          const bool has_b = c0 + 16 < c_hi;
-          if (has_b) tmem_ld16(lane_base + (uint32_t)(c0 + 16), vb);
-          store16(va, c0);
-          if (has_b) {
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (c0 + 32 < c_hi) tmem_ld16(lane_base + (uint32_t)(c0 + 32), va);
-            store16(vb, c0 + 16);
+          const int left = feat < n_rows ? P.R - (tok0 + c0) : 0;
+          float *yp = Yp + (size_t)(tok0 + c0) * P.ldy;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            if (j < left) *yp = __uint_as_float(va[j]);
+            yp += P.ldy;
           }
         }
       }
@@ -707,7 +663,6 @@ bool use_current_device() {
 int g_tune_stages = 0;      // 0 = as many as fit (at most 8)
 int g_tune_max_split = 0;   // 0 = default rule
 int g_tune_no_streamk = 0;  // 1 = always the per-tile decomposition
-int g_tune_l2_ahead = -1;   // < 0 = default
 int g_tune_late_w = 0;      // 1 = weights wait for the dependency too
 int g_tune_early_stages = -1; // < 0 = all stages
 int g_tune_no_wave_split = 0; // 1 = several token tiles keep the one-wave rule's split factor
@@ -717,7 +672,6 @@ int g_tune_epi_narrow = 0;  // 1, 2, 4: epilogue warps per lane quarter for 128-
 int g_tune_no_pair2 = 0;    // 1 = no CTA-pair kernel; 2 = not for 65 to 128 tokens
 int g_tune_pair_min = 0;    // > 0: fewest rows for the CTA-pair kernel
 int g_tune_epi_dry = 1;
-int g_tune_pf = 0;           // > 0: weight tiles requested into L2 ahead of the ring in that mode
 int g_tune_no_wide = 0;      // 1 = 128 weight rows per CTA also for wide token tiles
 int g_tune_traffic_div = 8; // split <= K_in / (div * tokens)
 
@@ -777,7 +731,10 @@ int tc_init_driver(char *err, size_t errlen) {
   DevInfo d{};
   cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem_optin - 1024);
+  const void *forms[4] = {(const void *)gemm_tc_kernel<FORM_PLAIN, false>, (const void *)gemm_tc_kernel<FORM_COLS, false>,
+                          (const void *)gemm_tc_kernel<FORM_ACC, false>, (const void *)gemm_tc_kernel<FORM_ACC, true>};
+  for (const void *f : forms)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem_optin - 1024);
   if (e != cudaSuccess) {
     snprintf(err, errlen, "cannot raise the GEMM kernel's shared memory: %s", cudaGetErrorString(e));
     return 1;
@@ -824,7 +781,6 @@ void tc_set_tuning(int key, int value) {
   if (key == 10) g_tune_no_wave_split = value;
   if (key == 11) g_tune_no_wide = value;
   if (key == 13) g_tune_no_accp = value;
-  if (key == 14) g_tune_pf = value;
   if (key == 15) g_tune_epi = value;
   if (key == 16) g_tune_epi_narrow = value;
   if (key == 17) g_tune_no_pair2 = value;
@@ -833,7 +789,6 @@ void tc_set_tuning(int key, int value) {
   if (key == 22) attn_mma_set_chunks(value);
   if (key == 2) g_tune_max_split = value;
   if (key == 3) g_tune_no_streamk = value;
-  if (key == 5) g_tune_l2_ahead = value;
   if (key == 6) g_tune_late_w = value;
   if (key == 8) g_tune_early_stages = value;
   if (key == 7 && value > 0) g_tune_traffic_div = value;
@@ -938,8 +893,6 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   // the last token tile may reach past R: those rows must exist (they are read, results dropped)
   if (ztiles * tt > x_rows_alloc) return cudaErrorInvalidValue;
   P.tt = tt;
-  P.pair = pair;
-  P.accp = accp;
   P.ztiles = ztiles;
   int cols = 32;
   while (cols < bn) cols <<= 1;
@@ -982,7 +935,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
       return (int)((KB + per - 1) / per) + ((units % gg) || (KB % per) ? 1 : 0);
     };
     while (g > 1 && slots_of(g) > max_slots) --g;
-    if (slots_of(g) <= max_slots) {
+    if (slots_of(g) <= max_slots && (g + 1) * units < (1LL << 32)) {
       P.tiles0 = q0;
       P.tiles1 = q0 + q1;
       P.n0 = m.n_out[0];
@@ -1039,10 +992,9 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
       return cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel, mw[0], mw[1], mw[2], mx, mxlo, P);
     }
     memset(&P, 0, sizeof(P));
-    P.tt = tt; P.pair = pair; P.accp = accp; P.ztiles = ztiles; P.Y = Y; P.ldy = ldy; P.R = R; P.bn = bn; P.tmem_cols = cols;
+    P.tt = tt; P.ztiles = ztiles; P.Y = Y; P.ldy = ldy; P.R = R; P.bn = bn; P.tmem_cols = cols;
   }
   const int bmw = wide ? 2 * BM : BM;
-  P.wide = wide ? 1 : 0;
   const int t0 = (m.n_out[0] + bmw - 1) / bmw;
   const int t1 = m.n > 1 ? (m.n_out[1] + bmw - 1) / bmw : 0;
   const int t2 = m.n > 2 ? (m.n_out[2] + bmw - 1) / bmw : 0;
@@ -1055,7 +1007,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   P.kblocks = K_in / BK;
   // stream-K (split == 0): needs a single token tile and 128-row-aligned matrices, so that a
   // column's tile (and with it the number of partial sums to add) follows from the column index
-  bool sk = split == 0 && ztiles == 1 && max_slots >= 2 && out != nullptr && !g_tune_no_streamk;
+  bool sk = split == 0 && ztiles == 1 && 2LL * (g_num_sms + 1) * n_tiles * P.kblocks < (1LL << 32) && max_slots >= 2 && out != nullptr && !g_tune_no_streamk;
   for (int i = 0; i < m.n && sk; ++i) sk = (m.n_out[i] % bmw) == 0;
   // stream-K pays off where the per-tile decomposition cannot be split further and leaves the SMs
   // unevenly loaded (more tiles than SMs, not a whole number of two-per-SM waves); elsewhere
@@ -1120,8 +1072,6 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   if (g_tune_stages > 0 && g_tune_stages < stages) stages = g_tune_stages;
   if (stages < 2) return cudaErrorInvalidValue;
   P.stages = stages;
-  P.l2_ahead = g_tune_l2_ahead >= 0 ? g_tune_l2_ahead : L2_AHEAD;
-  P.pf_ahead = (accp && stages < 4 && g_tune_pf > 0) ? g_tune_pf : 0;   // measured: no lookahead is fastest (13B, 256 rows)
   P.early_w = g_tune_late_w ? 0 : (g_tune_early_stages >= 0 && g_tune_early_stages < stages ? g_tune_early_stages : stages);
   CUtensorMap mw[3], mx, mxlo;
   for (int i = 0; i < 3; ++i) {
@@ -1144,7 +1094,12 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   int groups = wide ? 4 : 2;
   const int forced = wide ? g_tune_epi : g_tune_epi_narrow;
   if (forced == 1 || forced == 2 || forced == 4) groups = forced;
-  return launch_k(gemm_tc_kernel, grid, dim3(64 + 128 * groups), smem, L.st, L.pdl, mw[0], mw[1], mw[2], mx, mxlo, P);
+  auto go = [&](auto *kern) {
+    return launch_k(kern, grid, dim3(64 + 128 * groups), smem, L.st, L.pdl, mw[0], mw[1], mw[2], mx, mxlo, P);
+  };
+  if (!pair) return go(gemm_tc_kernel<FORM_PLAIN, false>);
+  if (!accp) return go(gemm_tc_kernel<FORM_COLS, false>);
+  return wide ? go(gemm_tc_kernel<FORM_ACC, true>) : go(gemm_tc_kernel<FORM_ACC, false>);
 }
 
 }  // namespace koala

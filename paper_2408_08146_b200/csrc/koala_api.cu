@@ -375,7 +375,7 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
   RowScale ffn = none;
   if (can_defer && (s.ld % 4) == 0 && (s.stride % 4) == 0) {
     CU_TRY(row_update(LN(c), g.dtype, c->x, s, w.ffn_norm, c->xn, c->sumsq[0], R, H));
-    ffn = RowScale{c->sumsq[0], (H + 1023) / 1024, 1.f / (float)H, g.rms_eps};
+    ffn = RowScale{c->sumsq[0], (H + 1023) / 1024, 1.f / (float)H, g.rms_eps, ROW_SUMS};
   } else {
     CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, w.ffn_norm, c->xn, nullptr, same, R, H, g.rms_eps));
   }
@@ -386,7 +386,7 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
   K_TRY(do_gemm(c, c->act, F, dn, R, nullptr, 0, &s));
   if (defer && can_defer && next_g != nullptr && (s.ld % 4) == 0 && (s.stride % 4) == 0) {
     CU_TRY(row_update(LN(c), g.dtype, c->x, s, next_g, c->xn, c->sumsq[1], R, H));
-    c->pending = RowScale{c->sumsq[1], (H + 1023) / 1024, 1.f / (float)H, g.rms_eps};
+    c->pending = RowScale{c->sumsq[1], (H + 1023) / 1024, 1.f / (float)H, g.rms_eps, ROW_SUMS};
   } else {
     CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, next_g, next_xn, out_f32, out_map, R, H, g.rms_eps));
   }
@@ -472,8 +472,8 @@ int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, vo
     return KOALA_OK;
   }
   const RowScale none{nullptr, 0, 0.f, 0.f};
-  const RowScale ffn_scale{c->sumsq[0], chunks, 1.f / (float)H, g.rms_eps};
-  const RowScale attn_scale{c->sumsq[1], chunks, 1.f / (float)H, g.rms_eps};
+  const RowScale ffn_scale{c->sumsq[0], chunks, 1.f / (float)H, g.rms_eps, chunks};
+  const RowScale attn_scale{c->sumsq[1], chunks, 1.f / (float)H, g.rms_eps, chunks};
   // the first layer's Q/K/V with the rotary step
   base_job();
   qkv_phase(0, layers[0], c->pending);
@@ -520,7 +520,7 @@ int embed_rows(koala_ctx *c, int R) {
     // the embedding rows in the deferred form: their RMSNorm scale is applied by the first layer's consumer
     CU_TRY(embed_update(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, c->sumsq[1],
                         R, g.H, g.V));
-    c->pending = RowScale{c->sumsq[1], (g.H + 1023) / 1024, 1.f / (float)g.H, g.rms_eps};
+    c->pending = RowScale{c->sumsq[1], (g.H + 1023) / 1024, 1.f / (float)g.H, g.rms_eps, ROW_SUMS};
   } else {
     CU_TRY(embed_norm(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, R, g.H, g.V,
                       g.rms_eps));

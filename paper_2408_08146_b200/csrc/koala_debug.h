@@ -16,8 +16,7 @@ extern "C" {
 /* Process-wide tuning of the tensor-core matrix multiply (the defaults are chosen for B200):
  * key 1 = shared-memory pipeline stages per CTA (0 = as many as fit, at most 8); key 2 = upper
  * bound on the automatic split-K factor (0 = default); key 3 = 1 switches stream-K off (every CTA
- * stays inside one weight tile); key 5 = weight tiles prefetched into L2 ahead of the pipeline
- * (< 0 = default 0); key 6 = 1 delays the weight stream until the previous kernel has finished;
+ * stays inside one weight tile); key 6 = 1 delays the weight stream until the previous kernel has finished;
  * key 7 = divisor of the split-K partial-sum traffic bound (default 8); key 8 = how many pipeline
  * stages request their weight tile before that wait (< 0 = all, the default); key 9 = fewest query
  * rows per sequence for which the tcgen05 attention kernel is used (default 16); key 10 = 1 keeps
@@ -26,8 +25,7 @@ extern "C" {
  * key 12 = key chunks per (sequence, head) of the tcgen05 attention kernel (0 = chosen from the shape);
  * key 13 = 1 runs pairs of more than 128 tokens as 128-token tiles with the residual rows as extra
  * accumulator columns (the form used up to 128 tokens) instead of 256-token tiles with two accumulating
- * MMAs; key 14 = weight tiles requested into L2 ahead of the ring in the 256-token form (default 0);
- * keys 15 (256-row weight tiles) and 16 (128-row tiles) = 1, 2 or 4: that many epilogue warps per
+ * MMAs; keys 15 (256-row weight tiles) and 16 (128-row tiles) = 1, 2 or 4: that many epilogue warps per
  * 32 accumulator lanes instead of the default; key 17 = 1: no CTA-pair GEMM kernel, 2: not up to 128
  * rows; key 18 = fewest rows for it (default 113); key 19 = K/V tiles the
  * tcgen05 attention requests into L2 ahead of its ring (default 0); key 20 = 0: no dry pass over its

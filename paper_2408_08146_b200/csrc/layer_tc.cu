@@ -153,7 +153,7 @@ __device__ __forceinline__ float silu_f(float v) { return __fdividef(v, 1.f + __
 __device__ __forceinline__ float row_scale(const RowScale &sc, int r) {
   if (sc.n == 0) return 1.f;
   float s = 0.f;
-  for (int i = 0; i < sc.n; ++i) s += __ldcg(sc.sumsq + (size_t)r * sc.n + i);
+  for (int i = 0; i < sc.n; ++i) s += __ldcg(sc.sumsq + (size_t)r * sc.stride + i);
   return rsqrtf(s * sc.inv_h + sc.eps);
 }
 

@@ -23,7 +23,8 @@ __device__ __forceinline__ float block_sum(float v, float *red) {
   return t;
 }
 
-__device__ __forceinline__ float silu_f(float v) { return v / (1.f + expf(-v)); }
+// (not inlined: an exponential and a division, used a dozen times by kernels that run their instructions once)
+__device__ __noinline__ float silu_f(float v) { return v / (1.f + expf(-v)); }
 
 // Stores v as a matrix-multiply operand.  bf16 operands are kept as a pair hi + lo (lo = the
 // rounding residual of hi, itself rounded to bf16), which carries 16 significant bits into the
@@ -92,25 +93,28 @@ __global__ void row_epilogue_kernel(int mode, float *__restrict__ x, SplitIn P,
 // Vectorised variant for H % 4 == 0: one CTA per row, every thread owns up to VPT groups of four
 // consecutive columns, keeps them in registers between the two passes and issues all split-K
 // partial loads of a group back to back.
-// (The first eight partial loads are issued before any is used - one trip to L2 instead of one
-// per partial; the additions keep the slot order.)
-template <int AHEAD = 8>
-__device__ __forceinline__ float4 split_sum4(const SplitIn &P, int r, int c) {
+// NS bounds the partial sums of a column: all of them are requested before the first is added - one
+// trip to L2 instead of one per partial; the additions keep the slot order.  SK: the number varies
+// with the tile (stream-K).  NS is a template argument so that the code is as short as the launch
+// allows: with one body for every factor the rotary kernel was 42 KB of instructions run once each,
+// and fetching them was most of its time (see the dispatch, FOR_SPLIT).
+template <int NS, bool SK>
+__device__ __forceinline__ int slots_at(const SplitIn &P, int r, int c) {
+  if (!SK) return P.n;
+  return sk_count(P.tile_of(r, c), P.sk_ctas, P.sk_units, P.sk_kb);
+}
+template <int NS>
+__device__ __forceinline__ float4 split_sum4(const SplitIn &P, int r, int c, int k) {
   const float *q = P.p + (size_t)r * P.ld + c;
-  const int k = P.count(r, c);
-  float4 u[AHEAD];
+  float4 u[NS];
 #pragma unroll
-  for (int s = 0; s < AHEAD; ++s)
-    u[s] = s < k ? *reinterpret_cast<const float4 *>(q + (size_t)s * P.stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s = 0; s < NS; ++s) {
+    u[s] = (s == 0 || s < k) ? *reinterpret_cast<const float4 *>(q) : make_float4(0.f, 0.f, 0.f, 0.f);
+    q += P.stride;
+  }
   float4 v = u[0];
 #pragma unroll
-  for (int s = 1; s < AHEAD; ++s) {
-    if (s < k) { v.x += u[s].x; v.y += u[s].y; v.z += u[s].z; v.w += u[s].w; }
-  }
-  for (int s = AHEAD; s < k; ++s) {
-    const float4 w = *reinterpret_cast<const float4 *>(q + (size_t)s * P.stride);
-    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-  }
+  for (int s = 1; s < NS; ++s) { v.x += u[s].x; v.y += u[s].y; v.z += u[s].z; v.w += u[s].w; }
   return v;
 }
 template <typename T> __device__ __forceinline__ float4 load4(const T *p);
@@ -141,7 +145,7 @@ __device__ __forceinline__ void store_operand4(bf16 *hi, bf16 *lo, size_t i, flo
   }
 }
 
-template <typename T, int VPT>
+template <typename T, int VPT, int NS, bool SK>
 __global__ void __launch_bounds__(1024)
 row_epilogue_vec_kernel(int mode, float *__restrict__ x, SplitIn P, const T *__restrict__ bias,
                         const T *__restrict__ g, T *__restrict__ xn, T *__restrict__ xn_lo,
@@ -157,7 +161,7 @@ row_epilogue_vec_kernel(int mode, float *__restrict__ x, SplitIn P, const T *__r
   for (int k = 0; k < VPT; ++k) {
     const int c = (threadIdx.x + k * blockDim.x) * 4;
     if (c < H) {
-      const float4 p = split_sum4(P, r, c);
+      const float4 p = split_sum4<NS>(P, r, c, slots_at<NS, SK>(P, r, c));
       float4 o;
       if (mode == 0) {
         const float4 xv = *reinterpret_cast<const float4 *>(xr + c);
@@ -203,7 +207,7 @@ row_epilogue_vec_kernel(int mode, float *__restrict__ x, SplitIn P, const T *__r
 // Residual update with the RMSNorm deferred: grid (chunks of 1024 columns, rows).  Many CTAs per
 // row pull the split-K partial sums; the row statistic is left as per-chunk partial sums of
 // squares for the consumer of the next GEMM's output (RowScale).
-template <typename T>
+template <typename T, int NS, bool SK>
 __global__ void __launch_bounds__(256)
 row_update_kernel(float *__restrict__ x, SplitIn P, const T *__restrict__ g, T *__restrict__ xg,
                   T *__restrict__ xg_lo, float *__restrict__ sumsq, int H) {
@@ -215,7 +219,7 @@ row_update_kernel(float *__restrict__ x, SplitIn P, const T *__restrict__ g, T *
   float ss = 0.f;
   if (c < H) {
     const float4 gg = load4<T>(g + c);
-    const float4 p = split_sum4(P, r, c);
+    const float4 p = split_sum4<NS>(P, r, c, slots_at<NS, SK>(P, r, c));
     float *xr = x + (size_t)r * H + c;
     const float4 xv = *reinterpret_cast<const float4 *>(xr);
     const float4 o = make_float4(xv.x + p.x, xv.y + p.y, xv.z + p.z, xv.w + p.w);
@@ -224,10 +228,10 @@ row_update_kernel(float *__restrict__ x, SplitIn P, const T *__restrict__ g, T *
     store_operand4(xg, xg_lo, (size_t)r * H + c, make_float4(o.x * gg.x, o.y * gg.y, o.z * gg.z, o.w * gg.w));
   }
   const float tot = block_sum(ss, red);
-  if (threadIdx.x == 0) sumsq[(size_t)r * gridDim.x + blockIdx.x] = tot;
+  if (threadIdx.x == 0) sumsq[(size_t)r * ROW_SUMS + blockIdx.x] = tot;
 }
 
-template <typename T>
+template <typename T, int NS>
 __global__ void __launch_bounds__(256)
 resblock_update_kernel(float *__restrict__ x, SplitIn P, HeadTab tab, T *__restrict__ xn, T *__restrict__ xn_lo, int H) {
   pdl_launch_dependents();
@@ -237,7 +241,7 @@ resblock_update_kernel(float *__restrict__ x, SplitIn P, HeadTab tab, T *__restr
   if (c >= H) return;
   const int head = r / tab.rows_per_head;
   P.p = tab.p[head];
-  const float4 p = split_sum4(P, r - head * tab.rows_per_head, c);
+  const float4 p = split_sum4<NS>(P, r - head * tab.rows_per_head, c, P.n);
   const float4 b = load4<T>(reinterpret_cast<const T *>(tab.bias[head]) + c);
   float *xr = x + (size_t)r * H + c;
   const float4 xv = *reinterpret_cast<const float4 *>(xr);
@@ -269,7 +273,7 @@ embed_update_kernel(const int32_t *tok, const T *__restrict__ E, const T *__rest
     store_operand4(xg, xg_lo, (size_t)r * H + c, make_float4(o.x * gg.x, o.y * gg.y, o.z * gg.z, o.w * gg.w));
   }
   const float tot = block_sum(ss, red);
-  if (threadIdx.x == 0) sumsq[(size_t)r * gridDim.x + blockIdx.x] = tot;
+  if (threadIdx.x == 0) sumsq[(size_t)r * ROW_SUMS + blockIdx.x] = tot;
 }
 
 // ------------------------------------------------------------------------------- EAGLE fc input
@@ -374,30 +378,26 @@ __global__ void rope_kv_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__
 
 // One CTA per row; a thread rotates two adjacent pairs (i, i+1) and (i + half, i + half + 1) of
 // one head with 8-byte loads.
-__device__ __forceinline__ float2 split_sum2(const SplitIn &P, int r, int c) {
+template <int NS>
+__device__ __forceinline__ float2 split_sum2(const SplitIn &P, int r, int c, int k) {
   const float *q = P.p + (size_t)r * P.ld + c;
-  const int k = P.count(r, c);
-  float2 u[4];
+  float2 u[NS];
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
-    u[s] = s < k ? *reinterpret_cast<const float2 *>(q + (size_t)s * P.stride) : make_float2(0.f, 0.f);
+  for (int s = 0; s < NS; ++s) {
+    u[s] = (s == 0 || s < k) ? *reinterpret_cast<const float2 *>(q) : make_float2(0.f, 0.f);
+    q += P.stride;
+  }
   float2 v = u[0];
 #pragma unroll
-  for (int s = 1; s < 4; ++s) {
-    if (s < k) { v.x += u[s].x; v.y += u[s].y; }
-  }
-  for (int s = 4; s < k; ++s) {
-    const float2 w = *reinterpret_cast<const float2 *>(q + (size_t)s * P.stride);
-    v.x += w.x; v.y += w.y;
-  }
+  for (int s = 1; s < NS; ++s) { v.x += u[s].x; v.y += u[s].y; }
   return v;
 }
 __device__ __forceinline__ void store2(float *p, float a, float b) { *reinterpret_cast<float2 *>(p) = make_float2(a, b); }
 __device__ __forceinline__ void store2(bf16 *p, float a, float b) {
   *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
-template <typename T>
-__global__ void __launch_bounds__(1024)
+template <typename T, int NS, bool SK>
+__global__ void __launch_bounds__(128)
 rope_kv_vec_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__restrict__ q_out, bf16 *__restrict__ qp_hi,
                    bf16 *__restrict__ qp_lo, T *__restrict__ k_cache, T *__restrict__ v_cache, int rows_per_seq,
                    int n_heads, int head_dim, int S_max) {
@@ -410,14 +410,17 @@ rope_kv_vec_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__restrict__ q
   const bool wr = slot >= 0 && slot < S_max;
   const float rs = sc.of(r);
   // grid.y slices the row's work so that many SMs pull the partial sums
-  for (int p = blockIdx.y * blockDim.x + threadIdx.x; p < n_heads * hq; p += gridDim.y * blockDim.x) {
+  const int p = blockIdx.y * blockDim.x + threadIdx.x;
+  if (p < n_heads * hq) {
     const int h = p / hq, i = (p - h * hq) * 2;
     const float4 cs = *reinterpret_cast<const float4 *>(&plan.rope[(size_t)r * half + i]);   // c0 s0 c1 s1
     const int c0 = h * head_dim + i, c1 = c0 + half;
-    // all partial sums of this thread are requested before the first store
-    float2 qa = split_sum2(qkv, r, c0), qb = split_sum2(qkv, r, c1);
-    float2 ka = split_sum2(qkv, r, H + c0), kb = split_sum2(qkv, r, H + c1);
-    float2 va = split_sum2(qkv, r, 2 * H + c0), vb = split_sum2(qkv, r, 2 * H + c1);
+    // all partial sums of this thread are requested before the first store (a head lies in one weight
+    // tile where tiles are dealt unevenly: there head_dim is 128 and a tile is a multiple of it)
+    const int kq = slots_at<NS, SK>(qkv, r, c0), kk = slots_at<NS, SK>(qkv, r, H + c0), kv = slots_at<NS, SK>(qkv, r, 2 * H + c0);
+    float2 qa = split_sum2<NS>(qkv, r, c0, kq), qb = split_sum2<NS>(qkv, r, c1, kq);
+    float2 ka = split_sum2<NS>(qkv, r, H + c0, kk), kb = split_sum2<NS>(qkv, r, H + c1, kk);
+    float2 va = split_sum2<NS>(qkv, r, 2 * H + c0, kv), vb = split_sum2<NS>(qkv, r, 2 * H + c1, kv);
     qa.x *= rs; qa.y *= rs; qb.x *= rs; qb.y *= rs;
     const float2 ra = make_float2(qa.x * cs.x - qb.x * cs.y, qa.y * cs.z - qb.y * cs.w);
     const float2 rb = make_float2(qb.x * cs.x + qa.x * cs.y, qb.y * cs.z + qa.y * cs.w);
@@ -431,7 +434,7 @@ rope_kv_vec_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__restrict__ q
       *reinterpret_cast<__nv_bfloat162 *>(qp_lo + (size_t)r * H + c0) = __floats2bfloat162_rn(ra.x - fa.x, ra.y - fa.y);
       *reinterpret_cast<__nv_bfloat162 *>(qp_lo + (size_t)r * H + c1) = __floats2bfloat162_rn(rb.x - fb.x, rb.y - fb.y);
     }
-    if (!wr) continue;
+    if (!wr) return;
     ka.x *= rs; ka.y *= rs; kb.x *= rs; kb.y *= rs;
     va.x *= rs; va.y *= rs; vb.x *= rs; vb.y *= rs;
     const size_t base = (((size_t)b * n_heads + h) * S_max + slot) * head_dim + i;
@@ -454,15 +457,15 @@ __global__ void swiglu_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *_
   store_operand(act, act_lo, (size_t)r * F + f, silu_f(rs * gu.at(r, f)) * (rs * gu.at(r, F + f)));
 }
 
-template <typename T>
-__global__ void swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int F) {
+template <typename T, int NS, bool SK>
+__global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int F) {
   pdl_launch_dependents();
   pdl_wait();
   const int r = blockIdx.y;
   const int f = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (f >= F) return;
   const float rs = sc.of(r);
-  const float4 a = split_sum4<3>(gu, r, f), b = split_sum4<3>(gu, r, F + f);
+  const float4 a = split_sum4<NS>(gu, r, f, slots_at<NS, SK>(gu, r, f)), b = split_sum4<NS>(gu, r, F + f, slots_at<NS, SK>(gu, r, F + f));
   store_operand4(act, act_lo, (size_t)r * F + f,
                  make_float4(silu_f(rs * a.x) * (rs * b.x), silu_f(rs * a.y) * (rs * b.y),
                              silu_f(rs * a.z) * (rs * b.z), silu_f(rs * a.w) * (rs * b.w)));
@@ -835,6 +838,36 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
     __VA_ARGS__                               \
   }
 
+// Runs BODY with NS (a bound of the partial sums per column) and SK (whether their number varies) as
+// constants.  fp32 operands come from the CUDA-core multiply, which leaves one whole result.
+#define SPLIT_CASE(n_, sk_, ...)              \
+  {                                           \
+    constexpr int NS = n_;                    \
+    constexpr bool SK = sk_;                  \
+    __VA_ARGS__                               \
+  }
+#define FOR_SPLIT(dtype, P, ...)                                                  \
+  if ((dtype) == 0) {                                                             \
+    typedef float T;                                                              \
+    if ((P).n != 1 || (P).sk_ctas != 0) return cudaErrorInvalidValue;             \
+    SPLIT_CASE(1, false, __VA_ARGS__)                                             \
+  } else {                                                                        \
+    typedef bf16 T;                                                               \
+    if ((P).n > 12) return cudaErrorInvalidValue;                                 \
+    if ((P).sk_ctas == 0) {                                                       \
+      if ((P).n <= 1) SPLIT_CASE(1, false, __VA_ARGS__)                           \
+      if ((P).n == 2) SPLIT_CASE(2, false, __VA_ARGS__)                           \
+      if ((P).n == 3) SPLIT_CASE(3, false, __VA_ARGS__)                           \
+      if ((P).n <= 5) SPLIT_CASE(5, false, __VA_ARGS__)                           \
+      if ((P).n <= 8) SPLIT_CASE(8, false, __VA_ARGS__)                           \
+      SPLIT_CASE(12, false, __VA_ARGS__)                                          \
+    }                                                                             \
+    if ((P).n <= 3) SPLIT_CASE(3, true, __VA_ARGS__)                              \
+    if ((P).n <= 5) SPLIT_CASE(5, true, __VA_ARGS__)                              \
+    if ((P).n <= 8) SPLIT_CASE(8, true, __VA_ARGS__)                              \
+    SPLIT_CASE(12, true, __VA_ARGS__)                                             \
+  }
+
 cudaError_t embed_norm(Launch L, int dtype, const int32_t *tok, const void *E, const void *g,
                        float *x, Operand xn, int R, int H, int V, float eps) {
   DISPATCH_T(dtype, return launch_k(embed_norm_kernel<T>, dim3(R), dim3(256), 0, L.st, L.pdl, tok,
@@ -847,14 +880,13 @@ cudaError_t row_epilogue(Launch L, int dtype, int mode, float *x, SplitIn P, con
     const int groups = H / 4;
     int threads = groups <= 1024 ? ((groups + 31) / 32) * 32 : (((groups + 1) / 2 + 31) / 32) * 32;
     if (groups <= 1024) {
-      DISPATCH_T(dtype, return launch_k(row_epilogue_vec_kernel<T, 1>, dim3(R), dim3(threads), 0, L.st, L.pdl,
-                                        mode, x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo,
-                                        out_f32, out_map, H, eps);)
-    } else {
-      DISPATCH_T(dtype, return launch_k(row_epilogue_vec_kernel<T, 2>, dim3(R), dim3(threads), 0, L.st, L.pdl,
-                                        mode, x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo,
-                                        out_f32, out_map, H, eps);)
+      FOR_SPLIT(dtype, P, return launch_k(row_epilogue_vec_kernel<T, 1, NS, SK>, dim3(R), dim3(threads), 0, L.st, L.pdl,
+                                          mode, x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo,
+                                          out_f32, out_map, H, eps);)
     }
+    FOR_SPLIT(dtype, P, return launch_k(row_epilogue_vec_kernel<T, 2, NS, SK>, dim3(R), dim3(threads), 0, L.st, L.pdl,
+                                        mode, x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo,
+                                        out_f32, out_map, H, eps);)
   }
   DISPATCH_T(dtype, return launch_k(row_epilogue_kernel<T>, dim3(R), dim3(256), 0, L.st, L.pdl, mode,
                                     x, P, (const T *)bias, (const T *)g, (T *)xn.hi, (T *)xn.lo, out_f32,
@@ -887,8 +919,9 @@ cudaError_t reduce_splits(Launch L, SplitIn P, float *Y, int ldy, int R, int nco
 
 cudaError_t resblock_update(Launch L, int dtype, float *x, SplitIn P, HeadTab tab, Operand xn, int R, int H) {
   if (H % 4 != 0 || P.ld % 4 != 0 || P.stride % 4 != 0 || tab.rows_per_head < 1) return cudaErrorInvalidValue;
-  DISPATCH_T(dtype, return launch_k(resblock_update_kernel<T>, dim3((H + 1023) / 1024, R), dim3(256), 0, L.st, L.pdl,
-                                    x, P, tab, (T *)xn.hi, (T *)xn.lo, H);)
+  if (P.sk_ctas != 0) return cudaErrorInvalidValue;
+  FOR_SPLIT(dtype, P, return launch_k(resblock_update_kernel<T, NS>, dim3((H + 1023) / 1024, R), dim3(256), 0, L.st,
+                                      L.pdl, x, P, tab, (T *)xn.hi, (T *)xn.lo, H);)
 }
 
 cudaError_t embed_update(Launch L, int dtype, const int32_t *tok, const void *E, const void *g, float *x,
@@ -901,8 +934,8 @@ cudaError_t embed_update(Launch L, int dtype, const int32_t *tok, const void *E,
 cudaError_t row_update(Launch L, int dtype, float *x, SplitIn P, const void *g, Operand xg, float *sumsq,
                        int R, int H) {
   if (H % 4 != 0 || P.ld % 4 != 0 || P.stride % 4 != 0) return cudaErrorInvalidValue;
-  DISPATCH_T(dtype, return launch_k(row_update_kernel<T>, dim3((H + 1023) / 1024, R), dim3(256), 0, L.st, L.pdl,
-                                    x, P, (const T *)g, (T *)xg.hi, (T *)xg.lo, sumsq, H);)
+  FOR_SPLIT(dtype, P, return launch_k(row_update_kernel<T, NS, SK>, dim3((H + 1023) / 1024, R), dim3(256), 0, L.st,
+                                      L.pdl, x, P, (const T *)g, (T *)xg.hi, (T *)xg.lo, sumsq, H);)
 }
 
 cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan plan, float *q_out,
@@ -910,13 +943,14 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
                           int head_dim, int S_max) {
   bf16 *qh = (bf16 *)q_pair.hi, *ql = (bf16 *)q_pair.lo;
   if (dtype == 0 || ql == nullptr) qh = ql = nullptr;      // the pair exists for bf16 storage only
-  if (head_dim % 4 == 0 && qkv.ld % 2 == 0 && qkv.stride % 2 == 0) {
+  const bool one_tile = qkv.sk_ctas == 0 || head_dim == 128;      // a head's columns have one number of partial sums
+  if (head_dim % 4 == 0 && qkv.ld % 2 == 0 && qkv.stride % 2 == 0 && one_tile) {
     const int work = n_heads * head_dim / 4;
     const int threads = work < 128 ? ((work + 31) / 32) * 32 : 128;
     const int slices = (work + threads - 1) / threads;
-    DISPATCH_T(dtype, return launch_k(rope_kv_vec_kernel<T>, dim3(R, slices), dim3(threads), 0, L.st, L.pdl, qkv, sc, plan,
-                                      q_out, qh, ql, (T *)k_cache, (T *)v_cache, rows_per_seq, n_heads, head_dim,
-                                      S_max);)
+    FOR_SPLIT(dtype, qkv, return launch_k(rope_kv_vec_kernel<T, NS, SK>, dim3(R, slices), dim3(threads), 0, L.st, L.pdl,
+                                          qkv, sc, plan, q_out, qh, ql, (T *)k_cache, (T *)v_cache, rows_per_seq,
+                                          n_heads, head_dim, S_max);)
   }
   DISPATCH_T(dtype, return launch_k(rope_kv_kernel<T>, dim3(R, n_heads), dim3(head_dim / 2), 0, L.st,
                                     L.pdl, qkv, sc, plan, q_out, qh, ql, (T *)k_cache, (T *)v_cache,
@@ -925,8 +959,8 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
 
 cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, int R, int F) {
   if (F % 4 == 0 && gu.ld % 4 == 0 && gu.stride % 4 == 0) {
-    DISPATCH_T(dtype, return launch_k(swiglu_vec_kernel<T>, dim3((F / 4 + 255) / 256, R), dim3(256), 0, L.st,
-                                      L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)
+    FOR_SPLIT(dtype, gu, return launch_k(swiglu_vec_kernel<T, NS, SK>, dim3((F / 4 + 255) / 256, R), dim3(256), 0, L.st,
+                                         L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)
   }
   DISPATCH_T(dtype, return launch_k(swiglu_kernel<T>, dim3((F + 255) / 256, R), dim3(256), 0, L.st,
                                     L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)
