@@ -118,9 +118,8 @@ __device__ __forceinline__ uint64_t tile_visibility(uint64_t m0, uint64_t m1, in
 struct AttnParams {
   RowPlan plan;
   bf16 *out, *out_lo;      // [R][n_heads * 128]
-  int rows_per_seq, n_heads, S_max, chunks;
+  int rows_per_seq, n_heads, S_max, chunks, chunk_bits;
   int longest_first;       // 1: grid slot y / n_heads takes the sequence with that rank in descending cache length
-  int l2_ahead;            // K/V tiles requested into L2 this many tiles ahead of the ring (0 = none)
   int dry_pass;            // 1: the row warps make a dry pass over the tile loop body before the dependency wait
   int *status;
 };
@@ -134,7 +133,10 @@ struct AttnParams {
 // 32..63; the row maximum is one more shuffle; at the end they swap halves of O_v, O_r the same
 // way and write dims 0..63 and 64..127.  Otherwise warp w owns rows 32w .. 32w+31 entirely and
 // the pair is two accumulating MMAs.
-template <bool DUP>
+// ONE: a single chunk (its end phase instead of the merge).  Both are template arguments because a launch
+// fetches its instructions anew and runs most of them once: 60 KB of code in one body were a third of
+// the fixed cost of a launch.
+template <bool DUP, bool ONE>
 __global__ void __launch_bounds__(THREADS, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_constant__ CUtensorMap tmQl,
                     const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -200,6 +202,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       const int nb = (int)gridDim.y / P.n_heads;              // <= 32 here
       const int len_l = lane < nb ? P.plan.kv_len[lane] : -1;
       int rank = 0;
+#pragma unroll 1
       for (int j = 0; j < nb; ++j) {
         const int len_j = __shfl_sync(0xffffffffu, len_l, j);
         rank += (len_j > len_l || (len_j == len_l && j < lane)) ? 1 : 0;
@@ -211,9 +214,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
     kv_len = P.plan.kv_len[b];
     kv_len = kv_len > P.S_max ? P.S_max : kv_len;
     const int n_tiles = (kv_len + TK - 1) / TK;
-    tile_lo = (int)(((long long)n_tiles * c) / P.chunks);
-    const int tile_hi = (int)(((long long)n_tiles * (c + 1)) / P.chunks);
-    T = tile_hi - tile_lo;
+    tile_lo = (n_tiles * c) >> P.chunk_bits;          // a power of two of chunks
+    T = ((n_tiles * (c + 1)) >> P.chunk_bits) - tile_lo;
   };
   // row ownership of warps 0..3
   const int half = DUP ? (lane >> 4) : 0;                   // DUP: residual lane; takes the second half of the keys / dims
@@ -225,24 +227,20 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
     if (DUP) {
       // of every 32 MMA rows the first 16 are the values of 16 queries, the other 16 their residuals
       mbar_expect_tx(&q_full, (uint32_t)(2 * QSUB));
-#pragma unroll
-      for (int hb = 0; hb < 2; ++hb)
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-#pragma unroll
-          for (int part = 0; part < 2; ++part)
-            tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + OFF_Q + hb * QSUB + (32 * g + 16 * part) * 128,
-                        h * DH + 64 * hb, b * P.rows_per_seq + 16 * g);
+#pragma unroll 1
+      for (int i = 0; i < 16; ++i) {
+        const int part = i & 1, hb = (i >> 1) & 1, g = i >> 2;
+        tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + OFF_Q + hb * QSUB + (32 * g + 16 * part) * 128,
+                    h * DH + 64 * hb, b * P.rows_per_seq + 16 * g);
+      }
     } else {
       mbar_expect_tx(&q_full, (uint32_t)(4 * QSUB));
-#pragma unroll
-      for (int part = 0; part < 2; ++part)
-#pragma unroll
-        for (int hb = 0; hb < 2; ++hb)
-#pragma unroll
-          for (int rh = 0; rh < 2; ++rh)
-            tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + OFF_Q + (part * 2 + hb) * QSUB + rh * (QSUB / 2),
-                        h * DH + 64 * hb, b * P.rows_per_seq + 64 * rh);
+#pragma unroll 1
+      for (int i = 0; i < 8; ++i) {
+        const int rh = i & 1, hb = (i >> 1) & 1, part = i >> 2;
+        tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + OFF_Q + (part * 2 + hb) * QSUB + rh * (QSUB / 2),
+                    h * DH + 64 * hb, b * P.rows_per_seq + 64 * rh);
+      }
     }
   }
   int r_glob = 0;
@@ -255,19 +253,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       const int y0 = (P.plan.cache_of(b) * P.n_heads + h) * P.S_max;
       bool ok = true;
       int issued = 0;
-      auto request_l2 = [&](int t) {
-        const int y = y0 + (tile_lo + t) * TK;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                       ::"l"(q < 2 ? &tmK : &tmV), "r"(64 * (q & 1)), "r"(y) : "memory");
-      };
-      // the cache is streamed from HBM by one CTA with a few tiles in flight: tiles beyond the ring
-      // are requested into L2 so that the ring's own loads find them there
-      for (int t = NST; t < NST + P.l2_ahead && t < T; ++t) request_l2(t);
+#pragma unroll 1
       for (int t = 0; t < T; ++t) {
         const int s = t % NST;
-        if (P.l2_ahead > 0 && t + NST + P.l2_ahead < T) request_l2(t + NST + P.l2_ahead);
         if (t >= NST) {
           ok = mbar_wait(&kv_empty[s], (uint32_t)((t / NST) - 1) & 1u);
           if (!ok) break;
@@ -275,10 +263,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         mbar_expect_tx(&kv_full[s], (uint32_t)KV_STAGE);
         unsigned char *dst = sm + OKV + s * KV_STAGE;
         const int y = y0 + (tile_lo + t) * TK;
-        tma_load_2d(&tmK, &kv_full[s], dst, 0, y);
-        tma_load_2d(&tmK, &kv_full[s], dst + SUB, 64, y);
-        tma_load_2d(&tmV, &kv_full[s], dst + 2 * SUB, 0, y);
-        tma_load_2d(&tmV, &kv_full[s], dst + 3 * SUB, 64, y);
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) tma_load_2d(i < 2 ? &tmK : &tmV, &kv_full[s], dst + i * SUB, 64 * (i & 1), y);
         issued = t + 1;
       }
       if (!ok) {
@@ -317,9 +303,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         return true;
       };
       bool ok = T > 0 ? mbar_wait(&q_full, 0) : true;
-      if (ok && T > 0) ok = issue_s(0);
-      for (int t = 0; t < T && ok; ++t) {
+#pragma unroll 1
+      for (int t = T > 0 ? -1 : 0; t < T && ok; ++t) {     // one place that issues S: the first one at t = -1
         if (t + 1 < T) { ok = issue_s(t + 1); if (!ok) break; }
+        if (t < 0) continue;
         ok = mbar_wait(&p_full[t & 1], (uint32_t)(t >> 1) & 1u);
         if (!ok) break;
         tc_fence_after();
@@ -493,8 +480,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   const int rs = wc + 4;                 // floats per received row: wc dims, m, l (first keys), l (other keys), pad
   constexpr int RR = DUP ? 64 : 128;     // rows per source chunk in the receive buffer
   float *recv = reinterpret_cast<float *>(sm + OKV);
-  if (P.chunks > 1) cluster_sync_all();  // the receive buffer reuses the K/V ring: every CTA of the cluster is done with its tiles
-  if (row_warp && P.chunks == 1) {
+  if constexpr (!ONE) cluster_sync_all();  // the receive buffer reuses the K/V ring: every CTA of the cluster is done with its tiles
+  if (ONE && row_warp) {
     // one chunk: nothing to merge - O out of tensor memory 16 dims at a time, normalised and stored
     tc_fence_after();
     const uint32_t o_lane = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)COL_O;   // this thread's lane, dim 0
@@ -542,7 +529,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         }
       }
     }
-  } else if (row_warp) {
+  } else if (!ONE && row_warp) {
     // the chunk's unnormalised O (relative to m_run) out of tensor memory, 16 dims at a time, each
     // group to the CTA that merges those dims
     tc_fence_after();
@@ -560,7 +547,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       }
       const int j = c0 / wc;
       const uint32_t a = mine + (uint32_t)(c0 - j * wc) * 4;
-      const uint32_t ra = P.chunks > 1 ? peer_addr(a, (uint32_t)j) : a;
+      const uint32_t ra = peer_addr(a, (uint32_t)j);
       if constexpr (DUP) {
         // the query's two lanes hold the two parts of the pair's product: add them (both lanes get
         // the sum) and let each lane store eight of the sixteen dims
@@ -586,15 +573,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
 #pragma unroll 1
       for (int j = 0; j < P.chunks; ++j) {
         const uint32_t a = mine + (uint32_t)wc * 4;
-        const uint32_t ra = P.chunks > 1 ? peer_addr(a, (uint32_t)j) : a;
+        const uint32_t ra = peer_addr(a, (uint32_t)j);
         if (half == 0) asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(ra), "f"(m_run), "f"(l_run) : "memory");
         else asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra + 8), "f"(l_run) : "memory");
         if (!DUP) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra + 8), "f"(0.f) : "memory");
       }
     }
   }
-  if (P.chunks > 1) cluster_sync_all(); else __syncthreads();
-  if (row_in && !failed && P.chunks > 1) {
+  if constexpr (!ONE) cluster_sync_all(); else __syncthreads();
+  if (!ONE && row_in && !failed) {
     const int ncol = DUP ? wc / 2 : wc;                    // this thread's share of the CTA's dims
     const int col0 = DUP ? half * ncol : 0;
     float mm = -INFINITY, l = 0.f;
@@ -647,14 +634,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
 
 int g_attn_tc_min_rows = 16;   // fewer query rows per sequence than this: the mma.sync kernel
 int g_attn_tc_chunks = 0;      // > 0: this many key chunks whatever the shape (A/B runs)
-int g_attn_tc_l2_ahead = 0;    // K/V tiles requested into L2 ahead of the ring
 int g_attn_tc_dry_pass = 1;
 
 }  // namespace
 
 void attn_tc_set_min_rows(int rows) { g_attn_tc_min_rows = rows; }
 void attn_tc_set_chunks(int chunks) { g_attn_tc_chunks = chunks; }
-void attn_tc_set_l2_ahead(int tiles) { g_attn_tc_l2_ahead = tiles < 0 ? 0 : tiles; }
 void attn_tc_set_dry_pass(int on) { g_attn_tc_dry_pass = on ? 1 : 0; }
 
 // Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the CTA
@@ -679,11 +664,14 @@ bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max) {
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
                               RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
                               int *status) {
-  static SmemOptIn optin_dup, optin_full;
+  static SmemOptIn optin[4];
   const size_t smem = (size_t)SMEM_BYTES + 1024;
-  cudaError_t e = optin_dup.ensure((const void *)tree_attn_tc_kernel<true>, smem);
-  if (e == cudaSuccess) e = optin_full.ensure((const void *)tree_attn_tc_kernel<false>, smem);
-  if (e != cudaSuccess) return e;
+  const void *forms[4] = {(const void *)tree_attn_tc_kernel<true, true>, (const void *)tree_attn_tc_kernel<true, false>,
+                          (const void *)tree_attn_tc_kernel<false, true>, (const void *)tree_attn_tc_kernel<false, false>};
+  for (int i = 0; i < 4; ++i) {
+    const cudaError_t e = optin[i].ensure(forms[i], smem);
+    if (e != cudaSuccess) return e;
+  }
   if (chunks != 1 && chunks != 2 && chunks != 4 && chunks != 8) return cudaErrorInvalidValue;
   if (q_pair.hi == nullptr || q_pair.lo == nullptr) return cudaErrorInvalidValue;
   const long long rows = (long long)cache_seqs * n_heads * S_max;
@@ -695,8 +683,8 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
       !tc_get_map(k_cache, (int)rows, DH, TK, &tmK) || !tc_get_map(v_cache, (int)rows, DH, TK, &tmV))
     return cudaErrorInvalidValue;
   const int longest_first = (B > 1 && B <= 32 && (long long)chunks * B * n_heads > tc_num_sms()) ? 1 : 0;
-  AttnParams P{plan, (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks, longest_first,
-               g_attn_tc_l2_ahead, g_attn_tc_dry_pass, status};
+  AttnParams P{plan, (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks, 31 - __builtin_clz((unsigned)chunks), longest_first,
+               g_attn_tc_dry_pass, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, n_heads * B);
   cfg.blockDim = dim3(THREADS);
@@ -712,8 +700,9 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
   cfg.attrs = attr;
   cfg.numAttrs = chunks > 1 ? 2 : 1;
   ++g_launches;
-  if (rows_per_seq <= 64) return cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<true>, tmQh, tmQl, tmK, tmV, P);
-  return cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<false>, tmQh, tmQl, tmK, tmV, P);
+  auto go = [&](auto *kern) { return cudaLaunchKernelEx(&cfg, kern, tmQh, tmQl, tmK, tmV, P); };
+  if (rows_per_seq <= 64) return chunks == 1 ? go(tree_attn_tc_kernel<true, true>) : go(tree_attn_tc_kernel<true, false>);
+  return chunks == 1 ? go(tree_attn_tc_kernel<false, true>) : go(tree_attn_tc_kernel<false, false>);
 }
 
 }  // namespace koala

@@ -139,6 +139,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
 
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
+#pragma unroll 1
     for (int s = 0; s < P.stages; ++s) {
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
@@ -425,6 +426,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
 
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
+#pragma unroll 1
     for (int s = 0; s < n_stages; ++s) {
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
@@ -482,6 +484,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       };
       // the first stages' weights do not depend on the kernel before this one
       int kb_first[PAIR_MAX_STAGES], tok_first[PAIR_MAX_STAGES];
+#pragma unroll 1
       for (int it = 0; it < pre; ++it) {
         kb_first[it] = kb;
         tok_first[it] = tok0;
@@ -489,10 +492,12 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
         next_unit();
       }
       pdl_wait();
+#pragma unroll 1
       for (int it = 0; it < pre; ++it) load_x(it, kb_first[it], tok_first[it]);
       bool ok = true;
       int s = pre % n_stages;
       uint32_t ph = (uint32_t)(pre / n_stages) & 1u;
+#pragma unroll 1
       for (int it = pre; it < n_units; ++it) {
         ok = mbar_wait(&empty_bar[s], ph ^ 1u);
         if (!ok) break;
@@ -769,13 +774,11 @@ int tc_init_driver(char *err, size_t errlen) {
 
 void attn_tc_set_min_rows(int rows);
 void attn_tc_set_chunks(int chunks);
-void attn_tc_set_l2_ahead(int tiles);
 void attn_tc_set_dry_pass(int on);
 void attn_mma_set_chunks(int chunks);
 void tc_set_tuning(int key, int value) {
   if (key == 9) attn_tc_set_min_rows(value);
   if (key == 12) attn_tc_set_chunks(value);
-  if (key == 19) attn_tc_set_l2_ahead(value);
   if (key == 20) attn_tc_set_dry_pass(value);
   if (key == 1) g_tune_stages = value;
   if (key == 10) g_tune_no_wave_split = value;

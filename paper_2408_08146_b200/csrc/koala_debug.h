@@ -27,8 +27,7 @@ extern "C" {
  * accumulator columns (the form used up to 128 tokens) instead of 256-token tiles with two accumulating
  * MMAs; keys 15 (256-row weight tiles) and 16 (128-row tiles) = 1, 2 or 4: that many epilogue warps per
  * 32 accumulator lanes instead of the default; key 17 = 1: no CTA-pair GEMM kernel, 2: not up to 128
- * rows; key 18 = fewest rows for it (default 113); key 19 = K/V tiles the
- * tcgen05 attention requests into L2 ahead of its ring (default 0); key 20 = 0: no dry pass over its
+ * rows; key 18 = fewest rows for it (default 113); key 20 = 0: no dry pass over its
  * tile loop before the dependency wait; key 21 = 0: no dry pass of the GEMM epilogue warps; key 22 =
  * key chunks of the mma.sync attention kernel (0 = by rule). */
 void koala_set_tuning(int key, int value);

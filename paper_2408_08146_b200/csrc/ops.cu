@@ -579,6 +579,7 @@ __device__ __forceinline__ ValIdx block_argmax(ValIdx x, ValIdx *red) {
   return x;
 }
 
+// Arg-max of rows wider than the kernel below takes.
 __global__ void argmax_rows_kernel(const float *logits, int32_t *__restrict__ out, float *spread, RowMap map, int V) {
   __shared__ ValIdx red[32];
   pdl_launch_dependents();
@@ -631,200 +632,163 @@ __global__ void topk_logp_kernel(const float *logits, int32_t *__restrict__ tok,
   }
 }
 
-__device__ __forceinline__ ValIdx warp_argmax(ValIdx x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ValIdx y;
-    y.v = __shfl_xor_sync(0xffffffffu, x.v, o);
-    y.i = __shfl_xor_sync(0xffffffffu, x.i, o);
-    x = better(x, y);
-  }
-  return x;
+// The same result for V <= 32768 and k <= 32, the row read once: one CTA per row up to 4096 columns, beyond
+// that eight as a thread-block cluster.  A CTA holds its part of the row, 16 strided elements per thread in
+// registers; every warp extracts the k best of its 512 elements, warp 0 merges the eight sorted lists, and
+// CTA 0 merges the parts' lists and (max, sum of exponentials) pairs through distributed shared memory.
+// Values are compared as order-preserving integers, so that a round is two warp-wide integer reductions
+// (largest key, then smallest id among equals) and only the winning lane looks at its elements again.
+// logp == nullptr: only the ids are wanted (the arg-max of a row is its top-1), no exponentials.
+// spread: the row is also copied to row map(r) of it.
+// (Rounds of five shuffle steps over (value, id) pairs with 16 comparisons in every lane took 20 us per call
+// at V = 32000, k = 10 in a running step, and a 32-element body for narrow rows 12 us at V = 1024.)
+constexpr int TKP = 8;            // CTAs per row of more than 256 * TKE columns
+constexpr int TKE = 16;           // elements per thread
+constexpr uint32_t NO_KEY = 0u;   // below every number's key
+constexpr uint32_t NO_ID = 0x7fffffffu;
+__device__ __forceinline__ uint32_t order_key(float v) {
+  const uint32_t b = __float_as_uint(v + 0.f);           // -0 counts as +0
+  return v == v ? b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u) : NO_KEY;
+}
+__device__ __forceinline__ float key_value(uint32_t k) {
+  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
 }
 
-// Same result for V <= 32768 and k <= 32 with two levels instead of k passes over the row: every
-// thread keeps its 32 strided elements in registers, every warp extracts the k best of its 1024
-// elements with shuffles only, and warp 0 extracts the k best of the 32 * k survivors.  (The k
-// best of the row are among the k best of each part; ties still go to the smaller id.)
-__global__ void __launch_bounds__(1024)
-topk_logp_fast_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp,
-                      int V, int k) {
-  __shared__ ValIdx cand[32 * 32];
-  __shared__ float redf[32];
-  __shared__ float s_mx;
-  pdl_launch_dependents();
-  pdl_wait();
-  const float *row = logits + (size_t)blockIdx.x * V;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  float vals[32];
-  float mx = -INFINITY;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const int i = tid + 1024 * j;
-    vals[j] = i < V ? row[i] : -INFINITY;
-    mx = fmaxf(mx, vals[j]);
-  }
-  mx = warp_max(mx);
-  if (lane == 0) redf[w] = mx;
-  __syncthreads();
-  if (w == 0) {
-    const float m2 = warp_max(redf[lane]);
-    if (lane == 0) s_mx = m2;
-  }
-  __syncthreads();
-  mx = s_mx;
-  float se = 0.f;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) se += expf(vals[j] - mx);       // exp(-inf) = 0 for the padding
-  const float lse = mx + logf(block_sum(se, redf));
-  for (int r = 0; r < k; ++r) {
-    ValIdx best{-INFINITY, 0x7fffffff};
-#pragma unroll
-    for (int j = 0; j < 32; ++j) best = better(best, ValIdx{vals[j], tid + 1024 * j});
-    best = warp_argmax(best);
-    if ((best.i & 1023) == tid) {
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (j == (best.i >> 10)) vals[j] = -INFINITY;
-    }
-    if (lane == 0) cand[w * k + r] = best;
-  }
-  __syncthreads();
-  if (w == 0) {
-    const int n = 32 * k;
-    for (int r = 0; r < k; ++r) {
-      ValIdx best{-INFINITY, 0x7fffffff};
-      int at = -1;
-      for (int c = lane; c < n; c += 32) {
-        const ValIdx x = cand[c];
-        if (x.v > best.v || (x.v == best.v && x.i < best.i)) { best = x; at = c; }
-      }
-      const ValIdx win = warp_argmax(best);
-      if (at >= 0 && best.i == win.i) cand[at] = ValIdx{-INFINITY, 0x7fffffff};
-      __syncwarp();
-      if (lane == 0) {
-        tok[(size_t)blockIdx.x * k + r] = win.i;
-        logp[(size_t)blockIdx.x * k + r] = win.v - lse;
-      }
-    }
-  }
-}
-
-// The same result on eight CTAs per row (a thread-block cluster): CTA p takes an eighth of the
-// row - 16 strided elements per thread in registers - and extracts its k best (every warp the k
-// best of its 512 elements with shuffles, warp 0 the k best of those 8 * k) together with its
-// (max, sum of exponentials); after a cluster barrier CTA 0 reads the eight candidate lists and
-// the eight (max, sum) pairs through distributed shared memory, takes the k best of the 8 * k
-// candidates (ties still go to the smaller id) and forms the log-sum-exp.  V <= 32768, k <= 32.
-constexpr int TKP = 8;            // CTAs per row
-__global__ void __launch_bounds__(256)
-topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp, float *spread, RowMap map, int V, int k) {
-  // logp == nullptr: only the ids are wanted (the arg-max of a row is its top-1), no exponentials
-  __shared__ ValIdx cand[8 * 32];
-  __shared__ ValIdx mine[32];     // this CTA's k best, read by CTA 0
-  __shared__ float s_ms[2];       // this CTA's (max, sum of exp(v - max))
-  __shared__ float redf[32];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int part = blockIdx.x, r = map(blockIdx.y);          // the row is read at blockIdx.y, its results go to r
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int chunk = (((V + TKP - 1) / TKP) + 255) & ~255;          // ids per CTA, a multiple of 256
-  const int base = part * chunk;
-  const float *row = logits + (size_t)blockIdx.y * V;
-  float vals[16];
-  float mx = -INFINITY;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int i = base + tid + 256 * j;
-    vals[j] = (tid + 256 * j < chunk && i < V) ? row[i] : -INFINITY;
-    mx = fmaxf(mx, vals[j]);
-    if (spread != nullptr && tid + 256 * j < chunk && i < V) spread[(size_t)r * V + i] = vals[j];
-  }
-  mx = warp_max(mx);
-  if (lane == 0) redf[w] = mx;
-  __syncthreads();
-  mx = warp_max(lane < 8 ? redf[lane] : -INFINITY);
-  __syncthreads();
-  float se = 0.f;
-  if (mx != -INFINITY && logp != nullptr) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) se += expf(vals[j] - mx);
-  }
-  se = warp_sum(se);
-  if (lane == 0) redf[w] = se;
-  __syncthreads();
-  se = warp_sum(lane < 8 ? redf[lane] : 0.f);
-  if (tid == 0) { s_ms[0] = mx; s_ms[1] = se; }
+// Merges `lists` lists of k (key, id) pairs, each sorted from best to worst, into dst[0..k): lane l of the
+// calling warp walks list l.
+__device__ __noinline__ void merge_lists(const uint2 *src, int lists, int k, uint2 *dst) {
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+  uint2 head = lane < lists ? src[lane * k] : make_uint2(NO_KEY, NO_ID);
+#pragma unroll 1
   for (int rnd = 0; rnd < k; ++rnd) {
-    ValIdx best{-INFINITY, 0x7fffffff};
-#pragma unroll
-    for (int j = 0; j < 16; ++j) best = better(best, ValIdx{vals[j], vals[j] == -INFINITY ? 0x7fffffff : base + tid + 256 * j});
-    best = warp_argmax(best);
-    if (best.i != 0x7fffffff && ((best.i - base) & 255) == tid) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (j == ((best.i - base) >> 8)) vals[j] = -INFINITY;
+    const uint32_t m = __reduce_max_sync(0xffffffffu, head.x);
+    const uint32_t id = __reduce_min_sync(0xffffffffu, head.x == m ? head.y : 0xffffffffu);
+    if (head.x == m && head.y == id) {
+      dst[rnd] = head;
+      ++at;
+      head = lane < lists && at < k ? src[lane * k + at] : make_uint2(NO_KEY, NO_ID);
     }
-    if (lane == 0) cand[w * k + rnd] = best;
   }
-  __syncthreads();
-  if (w == 0) {
-    const int n = 8 * k;
-    for (int rnd = 0; rnd < k; ++rnd) {
-      ValIdx best{-INFINITY, 0x7fffffff};
-      int at = -1;
-      for (int c = lane; c < n; c += 32) {
-        const ValIdx x = cand[c];
-        if (x.v > best.v || (x.v == best.v && x.i < best.i)) { best = x; at = c; }
+  __syncwarp();
+}
+
+__global__ void __launch_bounds__(256)
+topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *__restrict__ logp, float *spread,
+                         RowMap map, int V, int k) {
+  __shared__ __align__(8) uint2 cand[8 * 32];   // the warps' lists, then the parts'
+  __shared__ __align__(8) uint2 mine[32];       // this CTA's k best, read by CTA 0
+  __shared__ __align__(8) uint2 result[32];
+  __shared__ __align__(8) float s_ms[2];        // this CTA's (max, sum of exp(v - max))
+  __shared__ float redf[32];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int part = blockIdx.x, parts = gridDim.x, r = map(blockIdx.y);   // the row is read at blockIdx.y, its results go to r
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int chunk = (((V + parts - 1) / parts) + 255) & ~255;      // ids per CTA, a multiple of 256
+  const int base = part * chunk;
+  const int end = min(chunk, V - base);                            // this CTA's elements (may be <= 0)
+  const float *row = logits + (size_t)blockIdx.y * V + base;
+  float vals[TKE];
+  float mx = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < TKE; ++j) {
+    const int o = tid + 256 * j;
+    vals[j] = o < end ? row[o] : -INFINITY;
+    mx = fmaxf(mx, vals[j]);
+  }
+  if (spread != nullptr) {
+    float *to = spread + (size_t)r * V + base;
+#pragma unroll
+    for (int j = 0; j < TKE; ++j)
+      if (tid + 256 * j < end) to[tid + 256 * j] = vals[j];
+  }
+  if (logp != nullptr) {
+    mx = warp_max(mx);
+    if (lane == 0) redf[w] = mx;
+    __syncthreads();
+    mx = warp_max(lane < 8 ? redf[lane] : -INFINITY);
+    __syncthreads();
+    float se = 0.f;
+    if (mx != -INFINITY) {
+#pragma unroll 4
+      for (int j = 0; j < TKE; ++j) se += expf(vals[j] - mx);
+    }
+    se = warp_sum(se);
+    if (lane == 0) redf[w] = se;
+    __syncthreads();
+    se = warp_sum(lane < 8 ? redf[lane] : 0.f);
+    if (tid == 0) { s_ms[0] = mx; s_ms[1] = se; }
+  }
+  // this warp's k best
+  uint32_t keys[TKE];
+#pragma unroll
+  for (int j = 0; j < TKE; ++j) keys[j] = tid + 256 * j < end ? order_key(vals[j]) : NO_KEY;
+  uint32_t best = NO_KEY;
+  int at = TKE;                     // rescan first
+#pragma unroll 1
+  for (int rnd = 0, scan = 1; rnd < k; ++rnd) {
+    if (scan) {
+      best = NO_KEY;
+      int next = 0;
+#pragma unroll
+      for (int j = 0; j < TKE; ++j) {
+        if (j == at) keys[j] = NO_KEY;                   // taken in the round before
+        if (keys[j] > best) { best = keys[j]; next = j; }   // the first of equals: the smaller id
       }
-      const ValIdx win = warp_argmax(best);
-      if (at >= 0 && best.i == win.i && win.i != 0x7fffffff) cand[at] = ValIdx{-INFINITY, 0x7fffffff};
-      __syncwarp();
-      if (lane == 0) mine[rnd] = win;
+      at = next;
     }
+    const uint32_t id = best == NO_KEY ? NO_ID : (uint32_t)(base + tid + 256 * at);
+    const uint32_t m = __reduce_max_sync(0xffffffffu, best);
+    const uint32_t win = __reduce_min_sync(0xffffffffu, best == m ? id : 0xffffffffu);
+    if (lane == 0) cand[w * k + rnd] = make_uint2(m, win);
+    scan = m != NO_KEY && best == m && id == win;
   }
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (w == 0) merge_lists(cand, 8, k, parts > 1 ? mine : result);
+  if (parts > 1) {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
   if (part == 0 && w == 0) {
-    // lane l holds candidate l of every CTA (eight registers) and CTA (l % 8)'s (max, sum)
-    const uint32_t a_mine = (uint32_t)__cvta_generic_to_shared(&mine[lane < k ? lane : 0]);
-    const uint32_t a_ms = (uint32_t)__cvta_generic_to_shared(&s_ms[0]);
-    ValIdx c8[TKP];
+    float M = 0.f, S = 1.f;
+    if (logp != nullptr && parts == 1) { M = s_ms[0]; S = s_ms[1]; }
+    if (parts > 1) {
+      // every part's list and (max, sum) into this CTA, then the same merge
+      const uint32_t a_mine = (uint32_t)__cvta_generic_to_shared(&mine[lane < k ? lane : 0]);
+      const uint32_t a_ms = (uint32_t)__cvta_generic_to_shared(&s_ms[0]);
+      uint2 c8[TKP];
 #pragma unroll
-    for (int j = 0; j < TKP; ++j) {
-      uint32_t ra;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a_mine), "r"(j));
-      float v; int id;
-      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
-      asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(id) : "r"(ra + 4) : "memory");
-      c8[j] = lane < k ? ValIdx{v, id} : ValIdx{-INFINITY, 0x7fffffff};
-    }
-    uint32_t rb;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(a_ms), "r"(lane & 7));
-    float mj, sj;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(mj) : "r"(rb) : "memory");
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(sj) : "r"(rb + 4) : "memory");
-    const float M = warp_max(mj);
-    float part_sum = (lane < 8 && mj != -INFINITY) ? sj * expf(mj - M) : 0.f;
-    const float lse = M + logf(warp_sum(part_sum));
-    for (int rnd = 0; rnd < k; ++rnd) {
-      ValIdx best{-INFINITY, 0x7fffffff};
-#pragma unroll
-      for (int j = 0; j < TKP; ++j) best = better(best, c8[j]);
-      const ValIdx win = warp_argmax(best);
-#pragma unroll
-      for (int j = 0; j < TKP; ++j)
-        if (c8[j].i == win.i) c8[j] = ValIdx{-INFINITY, 0x7fffffff};
-      if (lane == 0) {
-        tok[(size_t)r * k + rnd] = win.i;
-        if (logp != nullptr) logp[(size_t)r * k + rnd] = win.v - lse;
+      for (int j = 0; j < TKP; ++j) {
+        uint32_t ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a_mine), "r"(j));
+        asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(c8[j].x), "=r"(c8[j].y) : "r"(ra) : "memory");
       }
+      if (logp != nullptr) {
+        uint32_t rb;
+        float mj, sj;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(a_ms), "r"(lane & 7));
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(mj), "=f"(sj) : "r"(rb) : "memory");
+        M = warp_max(mj);
+        S = warp_sum((lane < 8 && mj != -INFINITY) ? sj * expf(mj - M) : 0.f);
+      }
+      if (lane < k) {
+#pragma unroll
+        for (int j = 0; j < TKP; ++j) cand[j * k + lane] = c8[j];
+      }
+      __syncwarp();
+      merge_lists(cand, TKP, k, result);
+    }
+    if (lane < k) {
+      tok[(size_t)r * k + lane] = (int)result[lane].y;
+      if (logp != nullptr) logp[(size_t)r * k + lane] = key_value(result[lane].x) - (M + logf(S));
     }
   }
-  // no CTA leaves while CTA 0 may still read its shared memory
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (parts > 1) {
+    // no CTA leaves while CTA 0 may still read its shared memory
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
 }
 
 }  // namespace
@@ -986,7 +950,8 @@ cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_ca
 static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *tok, float *logp, float *spread, RowMap map,
                                        int R, int V, int k) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(TKP, R);
+  const int parts = V <= 256 * TKE ? 1 : TKP;      // a row that fits in one CTA's registers needs no cluster
+  cfg.gridDim = dim3(parts, R);
   cfg.blockDim = dim3(256);
   cfg.stream = L.st;
   cudaLaunchAttribute attr[2];
@@ -997,21 +962,19 @@ static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *t
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = parts > 1 ? 2 : 1;
   ++g_launches;
   return cudaLaunchKernelEx(&cfg, topk_logp_cluster_kernel, logits, tok, logp, spread, map, V, k);
 }
 
 cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, float *spread, RowMap map, int R, int V) {
-  // the arg-max (ties: smaller id) is the top-1; wide rows go to the eight-CTA kernel
-  if (V <= 32768 && V >= 4096) return topk_cluster_launch(L, logits, out, nullptr, spread, map, R, V, 1);
+  // the arg-max (ties: smaller id) is the top-1
+  if (V <= 256 * TKE * TKP) return topk_cluster_launch(L, logits, out, nullptr, spread, map, R, V, 1);
   return launch_k(argmax_rows_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, out, spread, map, V);
 }
 
 cudaError_t topk_logp(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k) {
-  if (V <= 32768 && k <= 32 && V >= 4096) return topk_cluster_launch(L, logits, tok, logp, nullptr, RowMap{0, 0}, R, V, k);
-  if (V <= 32768 && k <= 32)
-    return launch_k(topk_logp_fast_kernel, dim3(R), dim3(1024), 0, L.st, L.pdl, logits, tok, logp, V, k);
+  if (V <= 256 * TKE * TKP && k <= 32) return topk_cluster_launch(L, logits, tok, logp, nullptr, RowMap{0, 0}, R, V, k);
   const size_t smem = (size_t)V * sizeof(float);
   static SmemOptIn optin;
   {

@@ -381,3 +381,33 @@ def test_attention_of_one_row_ragged_batch():
         first = hid
     assert eng.device_status() == 0 and eng.check_guards()[1] == 0
     eng.close()
+
+
+@pytest.mark.parametrize("V,k", [(5, 5), (300, 16), (1024, 2), (4096, 10), (4097, 10), (9000, 1), (32000, 16), (32768, 3), (40000, 4)])
+def test_topk_of_rows_with_ties_and_extremes(V, k):
+    """Top-k over one CTA, a cluster of eight and the wide-row kernel: equal values (the smaller id wins, across
+    warps and parts), +-0, infinities, a row whose best are all in one warp; log-probabilities in float64."""
+    cfg = TINY_EAGLE.with_(V=V, topk=k, D=2, N=min(8, 1 + k), B=4, prompt_len=8, S_max=64)
+    eng, _, _ = make_pair(cfg)
+    eng.prefill(prompts(cfg), cfg.N)
+    eng.koala_draft(0)
+    rng = np.random.default_rng(V * 31 + k)
+    x = np.round(rng.normal(size=(4, V)) * 4).astype(np.float32) / 4          # many equal values
+    x[1] = 0.0
+    x[1, ::2] = -0.0                                                       # all equal
+    x[2, : min(V, 40)] = 9.0                                               # ids 0..39: neighbouring lanes
+    x[3, V // 2:] = -np.inf
+    eng.buffers()["draft_logits"].copy_(torch.from_numpy(x))
+    eng.set_expand_mode(1)
+    eng.koala_expand_tree(0)
+    bufs = eng.buffers()
+    tok, lp = bufs["topk_tok"].cpu().numpy(), bufs["topk_logp"].cpu().numpy()
+    for r in range(4):
+        want = np.argsort(-x[r], kind="stable")[:k]
+        if np.isfinite(x[r][want]).all():
+            assert tok[r].tolist() == want.tolist(), (r, tok[r], want)
+            d = x[r].astype(np.float64)
+            ref = d[want] - (d.max() + np.log(np.exp(d - d.max()).sum()))
+            assert np.abs(lp[r] - ref).max() <= 2e-6 * (1 + np.abs(ref).max())     # fp32 sum of V terms, log of it
+    assert eng.device_status() == 0
+    eng.close()
