@@ -382,19 +382,21 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
 }  // namespace
 
 // Key chunks per (sequence, head, row group) = cluster size: the largest of 1, 2, 4, 8 that keeps the
-// launch within what is resident at once (two CTAs of 96 KB per SM; clusters of eight do not fill every
-// GPC, hence seven eighths), never finer than 128 keys of capacity per chunk.
+// launch within about what is resident at once (two CTAs of 96 KB per SM, and a tenth more: the late
+// CTAs are short; clusters of eight do not fill every GPC, hence seven eighths there), at least one tile
+// of capacity per chunk.  (13B shape, four sequences, 160 sequence-head pairs, 2 x 5 launches per
+// iteration: 17.0 / 16.4 / 17.1 ms with 1 / 2 / 4 chunks; 7B, five rows, 36 launches: 4.30 / 4.13 /
+// 3.97 / 3.89 ms with 1 / 2 / 4 / 8.)
 int g_attn_mma_chunks = 0;     // > 0: this many key chunks whatever the shape (A/B runs)
 void attn_mma_set_chunks(int chunks) { g_attn_mma_chunks = chunks; }
 int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms) {
   const int rgs = (rows_per_seq + 15) / 16;
-  const int room = 2 * num_sms * 7 / 8;
   int c = 1;
   if (g_attn_mma_chunks > 0) {
     while (2 * c <= g_attn_mma_chunks && 2 * c <= 8 && 2 * c * 64 <= S_max) c *= 2;
     return c;
   }
-  while (c < 8 && 2 * c * rgs * B * n_heads <= room && 2 * c * 128 <= S_max) c *= 2;
+  while (c < 8 && 2 * c * rgs * B * n_heads <= (c == 4 ? 2 * num_sms * 7 / 8 : 2 * num_sms * 11 / 10) && 2 * c * 64 <= S_max) c *= 2;
   return c;
 }
 

@@ -38,24 +38,31 @@ namespace {
 
 constexpr int DH = 128;
 constexpr int TK = 64;                       // keys per tile
-constexpr int NKV = 3;                       // K/V stages (four with at most 64 rows, where Q takes half the room)
-constexpr int NKV_MAX = 4;
+constexpr int NKV_MAX = 3;
 constexpr int SUB = 64 * 64 * 2;             // one [64 keys][64 dims] block: 8 KB
 constexpr int QSUB = 128 * 64 * 2;           // one [128 rows][64 columns] block: 16 KB
-constexpr int OFF_Q = 0;                     // Q hi (2 blocks), Q lo (2 blocks)
-constexpr int OFF_KV = 4 * QSUB;             // stages of K (2 blocks) + V (2 blocks)
-constexpr int KV_STAGE = 4 * SUB;
-constexpr int OFF_P = OFF_KV + NKV * KV_STAGE;   // two buffers of P hi, P lo
-constexpr int P_BUF = 2 * QSUB;
-constexpr int SMEM_BYTES = OFF_P + 2 * P_BUF;    // 224 KB
+// Shared memory by form.  Up to 64 rows: Q 32 KB, two K and two V buffers of 16 KB, one P buffer of 16 KB =
+// 112 KB, so that two CTAs share an SM (their row warps' dependent chains overlap), or one CTA leaves
+// half an SM to the next kernel, whose weight loads then start while attention still runs.  More rows:
+// Q 64 KB, three K/V buffers, two P buffers = 224 KB.
+template <bool DUP> struct Lay {
+  static constexpr int NST = DUP ? 2 : 3;              // K and V buffers
+  static constexpr int NP = DUP ? 1 : 2;               // P buffers
+  static constexpr int PB = DUP ? QSUB : 2 * QSUB;     // bytes of one: value and residual rows in one operand, or two
+  static constexpr int Q = 0;
+  static constexpr int K = DUP ? 2 * QSUB : 4 * QSUB;
+  static constexpr int V = K + NST * 2 * SUB;
+  static constexpr int P = V + NST * 2 * SUB;
+  static constexpr int BYTES = P + NP * PB;
+};
 constexpr int THREADS = 192;
-constexpr int E_TIMEOUT = 6;
+constexpr int E_INVALID = 1, E_TIMEOUT = 6;
 constexpr int TMEM_COLS = 256;               // S: 2 x 64 columns, O: 128 columns
 constexpr int COL_S = 0, COL_O = 128;
 constexpr float RESCALE_STEP = 8.f;          // O is rescaled only when a row's maximum grows by more than 2^8
-// the chunk-merge buffer reuses the K/V ring once every CTA of the cluster is done with its tiles
-static_assert(8 * 128 * (DH / 8 + 4) * 4 <= NKV * KV_STAGE && 128 * (DH + 4) * 4 <= NKV * KV_STAGE,
-              "the chunk-merge buffer fits in the K/V ring");
+constexpr int OSTRIDE = DH + 4;              // floats of a row of the chunk's result: O[128], m, l, pad
+// the chunk's result goes where the K/V buffers were
+static_assert(64 * OSTRIDE * 4 <= 2 * 4 * SUB && 128 * OSTRIDE * 4 <= 3 * 4 * SUB, "the chunk's result fits");
 
 __device__ __forceinline__ void split_pack(float x, float y, uint32_t &hi, uint32_t &lo) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
@@ -86,8 +93,10 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t local_addr, uint32_t rank
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
   return ra;
 }
-__device__ __forceinline__ void st_cluster_v4(uint32_t ra, float a, float b, float c, float d) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ra), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t ra) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ra) : "memory");
+  return v;
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
@@ -120,6 +129,7 @@ struct AttnParams {
   bf16 *out, *out_lo;      // [R][n_heads * 128]
   int rows_per_seq, n_heads, S_max, chunks, chunk_bits;
   int longest_first;       // 1: grid slot y / n_heads takes the sequence with that rank in descending cache length
+  unsigned smem_bytes;     // dynamic shared memory of the launch
   int dry_pass;            // 1: the row warps make a dry pass over the tile loop body before the dependency wait
   int *status;
 };
@@ -137,16 +147,15 @@ struct AttnParams {
 // fetches its instructions anew and runs most of them once: 60 KB of code in one body were a third of
 // the fixed cost of a launch.
 template <bool DUP, bool ONE>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(THREADS, DUP ? 2 : 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_constant__ CUtensorMap tmQl,
                     const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const AttnParams P) {
   constexpr int NC = DUP ? 32 : 64;      // keys of a tile per thread
-  constexpr int PB = DUP ? QSUB : P_BUF; // bytes of one P buffer
-  constexpr int NST = DUP ? NKV + 1 : NKV;             // K/V stages
-  constexpr int OKV = DUP ? OFF_KV - KV_STAGE : OFF_KV; // the ring starts where the second half of Q would be
+  typedef Lay<DUP> LY;
+  constexpr int NST = LY::NST, NP = LY::NP;
   extern __shared__ unsigned char smem_raw[];
-  __shared__ uint64_t q_full, kv_full[NKV_MAX], kv_empty[NKV_MAX], s_full[2], p_full[2], pv_done[2], drain_bar;
+  __shared__ uint64_t q_full, k_full[NKV_MAX], k_empty[NKV_MAX], v_full[NKV_MAX], v_empty[NKV_MAX], s_full[2], p_full[2], pv_done[2], drain_bar;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int s_error;
 
@@ -154,6 +163,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char *sm = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   const uint32_t sb = smem_u32(sm);
+  // the launcher counts on the static variables and the alignment gap sharing 1 KB (see there)
+  if (sb + LY::BYTES > raw + P.smem_bytes) {
+    if (threadIdx.x == 0 && P.status) atomicMax(P.status, E_INVALID);
+    return;
+  }
   const int c = blockIdx.x;
   int b = blockIdx.y / P.n_heads;
   const int h = blockIdx.y % P.n_heads;
@@ -164,7 +178,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
     mbar_init(&q_full, 1);
-    for (int s = 0; s < NST; ++s) { mbar_init(&kv_full[s], 1); mbar_init(&kv_empty[s], 1); }
+    for (int s = 0; s < NST; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1); mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1); }
     mbar_init(&drain_bar, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1);
@@ -230,7 +244,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
 #pragma unroll 1
       for (int i = 0; i < 16; ++i) {
         const int part = i & 1, hb = (i >> 1) & 1, g = i >> 2;
-        tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + OFF_Q + hb * QSUB + (32 * g + 16 * part) * 128,
+        tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + LY::Q + hb * QSUB + (32 * g + 16 * part) * 128,
                     h * DH + 64 * hb, b * P.rows_per_seq + 16 * g);
       }
     } else {
@@ -238,7 +252,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
 #pragma unroll 1
       for (int i = 0; i < 8; ++i) {
         const int rh = i & 1, hb = (i >> 1) & 1, part = i >> 2;
-        tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + OFF_Q + (part * 2 + hb) * QSUB + rh * (QSUB / 2),
+        tma_load_2d(part ? &tmQl : &tmQh, &q_full, sm + LY::Q + (part * 2 + hb) * QSUB + rh * (QSUB / 2),
                     h * DH + 64 * hb, b * P.rows_per_seq + 64 * rh);
       }
     }
@@ -253,25 +267,28 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       const int y0 = (P.plan.cache_of(b) * P.n_heads + h) * P.S_max;
       bool ok = true;
       int issued = 0;
+      // K's buffer is free once S has been computed, V's only after P V: K runs ahead
 #pragma unroll 1
-      for (int t = 0; t < T; ++t) {
-        const int s = t % NST;
+      for (int i = 0; i < 2 * T; ++i) {
+        const int t = i >> 1, v = i & 1, s = t % NST;
+        uint64_t *full = v ? &v_full[s] : &k_full[s];
         if (t >= NST) {
-          ok = mbar_wait(&kv_empty[s], (uint32_t)((t / NST) - 1) & 1u);
+          ok = mbar_wait(v ? &v_empty[s] : &k_empty[s], (uint32_t)((t / NST) - 1) & 1u);
           if (!ok) break;
         }
-        mbar_expect_tx(&kv_full[s], (uint32_t)KV_STAGE);
-        unsigned char *dst = sm + OKV + s * KV_STAGE;
+        mbar_expect_tx(full, (uint32_t)(2 * SUB));
+        unsigned char *dst = sm + (v ? LY::V : LY::K) + s * 2 * SUB;
         const int y = y0 + (tile_lo + t) * TK;
-#pragma unroll 1
-        for (int i = 0; i < 4; ++i) tma_load_2d(i < 2 ? &tmK : &tmV, &kv_full[s], dst + i * SUB, 64 * (i & 1), y);
-        issued = t + 1;
+        const CUtensorMap *map = v ? &tmV : &tmK;
+        tma_load_2d(map, full, dst, 0, y);
+        tma_load_2d(map, full, dst + SUB, 64, y);
+        issued = i + 1;
       }
       if (!ok) {
         atomicExch(&s_error, 1);
         // let the copies already requested land before the block's memory goes away
-        for (int t = issued > NST ? issued - NST : 0; t < issued; ++t)
-          (void)mbar_wait(&kv_full[t % NST], (uint32_t)(t / NST) & 1u);
+        for (int i = issued > 2 * NST ? issued - 2 * NST : 0; i < issued; ++i)
+          (void)mbar_wait((i & 1) ? &v_full[(i >> 1) % NST] : &k_full[(i >> 1) % NST], (uint32_t)((i >> 1) / NST) & 1u);
       }
       if (T == 0 || !ok) (void)mbar_wait(&q_full, 0);      // nobody else waits for Q then
     }
@@ -284,15 +301,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
                                ((128u >> 4) << 24);
       auto issue_s = [&](int t) -> bool {
         const int s = t % NST;
-        if (!mbar_wait(&kv_full[s], (uint32_t)(t / NST) & 1u)) return false;
+        if (!mbar_wait(&k_full[s], (uint32_t)(t / NST) & 1u)) return false;
         tc_fence_after();
-        const uint32_t kb = sb + OKV + s * KV_STAGE;
+        const uint32_t kb = sb + LY::K + s * 2 * SUB;
         const uint32_t d = tmem + (uint32_t)(COL_S + (t & 1) * TK);
 #pragma unroll
         for (int part = 0; part < (DUP ? 1 : 2); ++part) { // Q value, then Q residual (DUP: both in one operand)
 #pragma unroll
           for (int hb = 0; hb < 2; ++hb) {                 // 64-dim block
-            const uint64_t da = smem_desc_sw128(sb + OFF_Q + (DUP ? hb : part * 2 + hb) * QSUB);
+            const uint64_t da = smem_desc_sw128(sb + LY::Q + (DUP ? hb : part * 2 + hb) * QSUB);
             const uint64_t db = smem_desc_sw128(kb + hb * SUB);
 #pragma unroll
             for (int k = 0; k < 4; ++k)
@@ -300,6 +317,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
           }
         }
         umma_commit(&s_full[t & 1]);
+        umma_commit(&k_empty[s]);
         return true;
       };
       bool ok = T > 0 ? mbar_wait(&q_full, 0) : true;
@@ -308,10 +326,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         if (t + 1 < T) { ok = issue_s(t + 1); if (!ok) break; }
         if (t < 0) continue;
         ok = mbar_wait(&p_full[t & 1], (uint32_t)(t >> 1) & 1u);
+        if (ok) ok = mbar_wait(&v_full[t % NST], (uint32_t)(t / NST) & 1u);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t vb = sb + OKV + (t % NST) * KV_STAGE + 2 * SUB;
-        const uint32_t pb = sb + OFF_P + (t & 1) * PB;
+        const uint32_t vb = sb + LY::V + (t % NST) * 2 * SUB;
+        const uint32_t pb = sb + LY::P + (t % NP) * LY::PB;
         const uint32_t d = tmem + (uint32_t)COL_O;
 #pragma unroll
         for (int part = 0; part < (DUP ? 1 : 2); ++part) { // P value, then P residual (DUP: both in one operand)
@@ -322,7 +341,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
             umma_bf16(d, da + (uint64_t)(2 * k), db, idesc_o, (t | part | k) ? 1u : 0u);   // O accumulates over the tiles
           }
         }
-        umma_commit(&kv_empty[t % NST]);
+        umma_commit(&v_empty[t % NST]);
         umma_commit(&pv_done[t & 1]);
       }
       if (!ok) atomicExch(&s_error, 1);
@@ -388,10 +407,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         // The last tile reaches past kv_len: those cache slots were never written and may hold
         // anything, NaN bit patterns included, and 0 x NaN in P V would poison every row.  Zero
         // the value rows from kv_len on (a row is 128 bytes of each 64-dim block; the swizzle
-        // only permutes inside the row).  The tile has landed: S, which this warp waited for, was
-        // issued after it.  Every row warp in use writes the same zeros.
-        const uint32_t vb = sb + OKV + (t % NST) * KV_STAGE + 2 * SUB;
-        for (int kr = kv_len - key0 + lane; kr < TK; kr += 32) {
+        // only permutes inside the row), once the tile has landed.  Every row warp in use writes the
+        // same zeros.
+        if (live) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&v_full[t % NST], (uint32_t)(t / NST) & 1u));
+          if (!ok) break;
+        }
+        const uint32_t vb = sb + LY::V + (live ? t % NST : 0) * 2 * SUB;
+        for (int kr = (live ? kv_len - key0 : TK) + lane; kr < TK; kr += 32) {
 #pragma unroll
           for (int blk = 0; blk < 2; ++blk)
 #pragma unroll
@@ -435,14 +458,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       } else if (t == 0) {
         l_run = 0.f;
       }
-      // the P buffer of tile t was last read by the P V of tile t - 2
-      if (t >= 2) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[t & 1], (uint32_t)((t - 2) >> 1) & 1u));
+      // the P buffer of tile t was last read by the P V of tile t - NP
+      if (t >= NP) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[(t - NP) & 1], (uint32_t)((t - NP) >> 1) & 1u));
         if (!ok) break;
       }
       const float mu = m_run == -INFINITY ? 0.f : m_run;
       float l_t = 0.f;
-      const uint32_t pb = sb + OFF_P + (uint32_t)((t & 1) * PB) + prow;
+      const uint32_t pb = sb + LY::P + (uint32_t)((t & (NP - 1)) * LY::PB) + prow;
 #pragma unroll
       for (int ch = 0; ch < NC / 8; ++ch) {
         uint32_t hi[4], lo[4];
@@ -473,14 +496,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   tc_fence_before();
   __syncthreads();                       // all tiles consumed
   const bool failed = s_error != 0;
-  // ---- merge over the chunks.  Every CTA receives, from every chunk j (itself included), the
-  // dims [c * wc, (c + 1) * wc) of all rows plus (m, l): recv[j][row][wc + 4].  The code from here
-  // on runs once per CTA, so it is written as short loops rather than unrolled over the 128 dims.
-  const int wc = DH / P.chunks;
-  const int rs = wc + 4;                 // floats per received row: wc dims, m, l (first keys), l (other keys), pad
-  constexpr int RR = DUP ? 64 : 128;     // rows per source chunk in the receive buffer
-  float *recv = reinterpret_cast<float *>(sm + OKV);
-  if constexpr (!ONE) cluster_sync_all();  // the receive buffer reuses the K/V ring: every CTA of the cluster is done with its tiles
+  // ---- the end phase runs once per CTA, so it is written as short loops rather than unrolled over the dims
   if (ONE && row_warp) {
     // one chunk: nothing to merge - O out of tensor memory 16 dims at a time, normalised and stored
     tc_fence_after();
@@ -529,95 +545,86 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         }
       }
     }
-  } else if (!ONE && row_warp) {
-    // the chunk's unnormalised O (relative to m_run) out of tensor memory, 16 dims at a time, each
-    // group to the CTA that merges those dims
-    tc_fence_after();
-    const uint32_t o_lane = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)COL_O;   // this thread's lane, dim 0
-    const uint32_t mine = smem_u32(recv + ((size_t)c * RR + row) * rs);
-#pragma unroll 1
-    for (int c0 = 0; c0 < DH; c0 += 16) {
-      uint32_t o[16];
-      if (have_o) {
-        tmem_ld16(o_lane + (uint32_t)c0, o);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) o[j] = 0u;
-      }
-      const int j = c0 / wc;
-      const uint32_t a = mine + (uint32_t)(c0 - j * wc) * 4;
-      const uint32_t ra = peer_addr(a, (uint32_t)j);
-      if constexpr (DUP) {
-        // the query's two lanes hold the two parts of the pair's product: add them (both lanes get
-        // the sum) and let each lane store eight of the sixteen dims
-        float x[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float lo8 = __uint_as_float(o[k]) + __shfl_xor_sync(0xffffffffu, __uint_as_float(o[k]), 16);
-          const float hi8 = __uint_as_float(o[8 + k]) + __shfl_xor_sync(0xffffffffu, __uint_as_float(o[8 + k]), 16);
-          x[k] = half ? hi8 : lo8;
-        }
-        if (row_in) {
-          st_cluster_v4(ra + (uint32_t)half * 32u, x[0], x[1], x[2], x[3]);
-          st_cluster_v4(ra + (uint32_t)half * 32u + 16u, x[4], x[5], x[6], x[7]);
-        }
-      } else if (row_in) {
-#pragma unroll
-        for (int k = 0; k < 16; k += 4)
-          st_cluster_v4(ra + (uint32_t)k * 4u, __uint_as_float(o[k]), __uint_as_float(o[k + 1]),
-                        __uint_as_float(o[k + 2]), __uint_as_float(o[k + 3]));
-      }
-    }
-    if (row_in) {
-#pragma unroll 1
-      for (int j = 0; j < P.chunks; ++j) {
-        const uint32_t a = mine + (uint32_t)wc * 4;
-        const uint32_t ra = peer_addr(a, (uint32_t)j);
-        if (half == 0) asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(ra), "f"(m_run), "f"(l_run) : "memory");
-        else asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra + 8), "f"(l_run) : "memory");
-        if (!DUP) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra + 8), "f"(0.f) : "memory");
-      }
-    }
   }
-  if constexpr (!ONE) cluster_sync_all(); else __syncthreads();
-  if (!ONE && row_in && !failed) {
-    const int ncol = DUP ? wc / 2 : wc;                    // this thread's share of the CTA's dims
-    const int col0 = DUP ? half * ncol : 0;
-    float mm = -INFINITY, l = 0.f;
+  if constexpr (!ONE) {
+    // Merge over the chunks: every CTA leaves its unnormalised O (relative to m), m and l per row in its own
+    // shared memory; after one cluster barrier CTA c finishes the dims [c * wc, (c + 1) * wc) of all rows,
+    // reading them from every CTA of the cluster, in chunk order.  (Pushing each peer's dims into its
+    // shared memory needed a barrier before and after and took 5.9 us per launch, 11.5 us with 128 rows.)
+    float *stage = reinterpret_cast<float *>(sm + LY::K);
+    if (row_warp) {
+      tc_fence_after();
+      const uint32_t o_lane = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)COL_O;   // this thread's lane, dim 0
+      float *mine = stage + (size_t)row * OSTRIDE;
 #pragma unroll 1
-    for (int j = 0; j < P.chunks; ++j) mm = fmaxf(mm, recv[((size_t)j * RR + row) * rs + wc]);
-    if (mm != -INFINITY) {
-#pragma unroll 1
-      for (int j = 0; j < P.chunks; ++j) {
-        const float4 ml = *reinterpret_cast<const float4 *>(recv + ((size_t)j * RR + row) * rs + wc);
-        if (ml.x != -INFINITY) l += exp2f(ml.x - mm) * (ml.y + ml.z);
+      for (int c0 = 0; c0 < DH; c0 += 16) {
+        uint32_t o[16];
+        if (have_o) {
+          tmem_ld16(o_lane + (uint32_t)c0, o);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) o[j] = 0u;
+        }
+        if constexpr (DUP) {
+          // the query's two lanes hold the two parts of the pair's product: add them; each lane stores eight dims
+          float x[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float lo8 = __uint_as_float(o[k]) + __shfl_xor_sync(0xffffffffu, __uint_as_float(o[k]), 16);
+            const float hi8 = __uint_as_float(o[8 + k]) + __shfl_xor_sync(0xffffffffu, __uint_as_float(o[8 + k]), 16);
+            x[k] = half ? hi8 : lo8;
+          }
+          float4 *to = reinterpret_cast<float4 *>(mine + c0 + 8 * half);
+          to[0] = make_float4(x[0], x[1], x[2], x[3]);
+          to[1] = make_float4(x[4], x[5], x[6], x[7]);
+        } else {
+          float4 *to = reinterpret_cast<float4 *>(mine + c0);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            to[k] = make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]), __uint_as_float(o[4 * k + 2]),
+                                __uint_as_float(o[4 * k + 3]));
+        }
       }
+      float l = l_run;
+      if (DUP) l += __shfl_xor_sync(0xffffffffu, l_run, 16);      // the query's other 32 keys of every tile
+      if (half == 0) *reinterpret_cast<float2 *>(mine + DH) = make_float2(m_run, l);
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    const size_t ob = (size_t)r_glob * H + h * DH + c * wc + col0;
+    cluster_sync_all();
+    if (!failed) {
+      const int wc = DH >> P.chunk_bits, per_row = wc >> 3;          // eight dims per thread and step
+      const uint32_t st0 = smem_u32(stage);
 #pragma unroll 1
-    for (int d0 = 0; d0 < ncol; d0 += 8) {
-      float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (mm != -INFINITY) {
-#pragma unroll 1
+      for (int e = threadIdx.x; e < P.rows_per_seq * per_row; e += THREADS) {
+        const int r = e / per_row, d = c * wc + (e - r * per_row) * 8;
+        const uint32_t at = st0 + (uint32_t)(r * OSTRIDE) * 4u;
+        float mm = -INFINITY;
+#pragma unroll 4
+        for (int j = 0; j < P.chunks; ++j) mm = fmaxf(mm, ld_cluster_v4(peer_addr(at + DH * 4u, (uint32_t)j)).x);
+        float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float l = 0.f;
+        const float mu = mm == -INFINITY ? 0.f : mm;
+#pragma unroll 4
         for (int j = 0; j < P.chunks; ++j) {               // in chunk order
-          const float *src = recv + ((size_t)j * RR + row) * rs;
-          const float mj = src[wc];
-          if (mj == -INFINITY) continue;
-          const float w = exp2f(mj - mm);
-          const float4 x0 = *reinterpret_cast<const float4 *>(src + col0 + d0);
-          const float4 x1 = *reinterpret_cast<const float4 *>(src + col0 + d0 + 4);
+          const uint32_t pa = peer_addr(at, (uint32_t)j);
+          const float4 ml = ld_cluster_v4(pa + DH * 4u);
+          const float4 x0 = ld_cluster_v4(pa + (uint32_t)d * 4u), x1 = ld_cluster_v4(pa + (uint32_t)d * 4u + 16u);
+          const float w = exp2f(ml.x - mu);                // exp2(-inf) = 0; such a chunk's O is zero
+          l += w * ml.y;
           o[0] += w * x0.x; o[1] += w * x0.y; o[2] += w * x0.z; o[3] += w * x0.w;
           o[4] += w * x1.x; o[5] += w * x1.y; o[6] += w * x1.z; o[7] += w * x1.w;
         }
-      }
-      uint32_t hi[4], lo[4];
+        const float inv = l > 0.f ? 1.f / l : 0.f;
+        uint32_t hi[4], lo[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) split_pack(o[2 * e] * inv, o[2 * e + 1] * inv, hi[e], lo[e]);
-      *reinterpret_cast<uint4 *>(P.out + ob + d0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      if (P.out_lo != nullptr) *reinterpret_cast<uint4 *>(P.out_lo + ob + d0) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        for (int k = 0; k < 4; ++k) split_pack(o[2 * k] * inv, o[2 * k + 1] * inv, hi[k], lo[k]);
+        const size_t ob = (size_t)(b * P.rows_per_seq + r) * H + h * DH + d;
+        *reinterpret_cast<uint4 *>(P.out + ob) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        if (P.out_lo != nullptr) *reinterpret_cast<uint4 *>(P.out_lo + ob) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      }
     }
+    // no CTA leaves while another may still read its shared memory
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   }
   if (warp == 5) {
     if (failed) {      // MMAs issued before a wait ran out may still be running: no free under them
@@ -630,6 +637,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
   }
   if (threadIdx.x == 0 && failed && P.status) atomicMax(P.status, E_TIMEOUT);
+  if constexpr (!ONE) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 int g_attn_tc_min_rows = 16;   // fewer query rows per sequence than this: the mma.sync kernel
@@ -642,10 +650,8 @@ void attn_tc_set_min_rows(int rows) { g_attn_tc_min_rows = rows; }
 void attn_tc_set_chunks(int chunks) { g_attn_tc_chunks = chunks; }
 void attn_tc_set_dry_pass(int on) { g_attn_tc_dry_pass = on ? 1 : 0; }
 
-// Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the CTA
-// count within the SMs (one CTA per SM is resident; measured: a second, partly filled round and the
-// co-scheduling of clusters cost more than shorter CTAs gain), each chunk with at least 128 keys of
-// capacity.
+// Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the CTA count
+// within the SMs, each chunk with at least 128 keys of capacity.
 int attn_tc_chunks(int B, int n_heads, int S_max, int num_sms) {
   int c = 1;
   if (g_attn_tc_chunks > 0) {
@@ -658,20 +664,13 @@ int attn_tc_chunks(int B, int n_heads, int S_max, int num_sms) {
 
 bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max) {
   return head_dim == DH && rows_per_seq >= g_attn_tc_min_rows && rows_per_seq <= 128 &&
-         tc_smem_optin() >= SMEM_BYTES + 1024 + 1280 && S_max >= 1;
+         tc_smem_optin() >= Lay<false>::BYTES + 1024 && S_max >= 1;
 }
 
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
                               RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
                               int *status) {
-  static SmemOptIn optin[4];
-  const size_t smem = (size_t)SMEM_BYTES + 1024;
-  const void *forms[4] = {(const void *)tree_attn_tc_kernel<true, true>, (const void *)tree_attn_tc_kernel<true, false>,
-                          (const void *)tree_attn_tc_kernel<false, true>, (const void *)tree_attn_tc_kernel<false, false>};
-  for (int i = 0; i < 4; ++i) {
-    const cudaError_t e = optin[i].ensure(forms[i], smem);
-    if (e != cudaSuccess) return e;
-  }
+  const bool dup = rows_per_seq <= 64;
   if (chunks != 1 && chunks != 2 && chunks != 4 && chunks != 8) return cudaErrorInvalidValue;
   if (q_pair.hi == nullptr || q_pair.lo == nullptr) return cudaErrorInvalidValue;
   const long long rows = (long long)cache_seqs * n_heads * S_max;
@@ -682,13 +681,12 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
   if (!tc_get_map(q_pair.hi, q_rows_alloc, H, q_box, &tmQh) || !tc_get_map(q_pair.lo, q_rows_alloc, H, q_box, &tmQl) ||
       !tc_get_map(k_cache, (int)rows, DH, TK, &tmK) || !tc_get_map(v_cache, (int)rows, DH, TK, &tmV))
     return cudaErrorInvalidValue;
-  const int longest_first = (B > 1 && B <= 32 && (long long)chunks * B * n_heads > tc_num_sms()) ? 1 : 0;
-  AttnParams P{plan, (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks, 31 - __builtin_clz((unsigned)chunks), longest_first,
-               g_attn_tc_dry_pass, status};
+  const int longest_first = (B > 1 && B <= 32 && (long long)chunks * B * n_heads > (dup ? 2 : 1) * tc_num_sms()) ? 1 : 0;
+  AttnParams P{plan, (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks,
+               31 - __builtin_clz((unsigned)chunks), longest_first, 0u, g_attn_tc_dry_pass, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, n_heads * B);
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = smem;
   cfg.stream = L.st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -699,10 +697,27 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chunks > 1 ? 2 : 1;
-  ++g_launches;
-  auto go = [&](auto *kern) { return cudaLaunchKernelEx(&cfg, kern, tmQh, tmQl, tmK, tmV, P); };
-  if (rows_per_seq <= 64) return chunks == 1 ? go(tree_attn_tc_kernel<true, true>) : go(tree_attn_tc_kernel<true, false>);
-  return chunks == 1 ? go(tree_attn_tc_kernel<false, true>) : go(tree_attn_tc_kernel<false, false>);
+  // Static variables (barriers) come first, then the gap up to a 1 KB boundary: the two share 1 KB, so that
+  // two CTAs of the 112 KB form fit on an SM to the byte.
+  static SmemOptIn optin[4];
+  static size_t static_bytes[4] = {};
+  auto go = [&](auto *kern, int form, size_t need) -> cudaError_t {
+    if (static_bytes[form] == 0) {                       // the same value whichever thread comes first
+      cudaFuncAttributes fa;
+      const cudaError_t e = cudaFuncGetAttributes(&fa, (const void *)kern);
+      if (e != cudaSuccess) return e;
+      static_bytes[form] = fa.sharedSizeBytes;
+    }
+    if (static_bytes[form] > 1024) return cudaErrorInvalidValue;
+    P.smem_bytes = (unsigned)(need + 1024 - static_bytes[form]);
+    cfg.dynamicSmemBytes = P.smem_bytes;
+    const cudaError_t e = optin[form].ensure((const void *)kern, P.smem_bytes);
+    if (e != cudaSuccess) return e;
+    ++g_launches;
+    return cudaLaunchKernelEx(&cfg, kern, tmQh, tmQl, tmK, tmV, P);
+  };
+  if (dup) return chunks == 1 ? go(tree_attn_tc_kernel<true, true>, 0, Lay<true>::BYTES) : go(tree_attn_tc_kernel<true, false>, 1, Lay<true>::BYTES);
+  return chunks == 1 ? go(tree_attn_tc_kernel<false, true>, 2, Lay<false>::BYTES) : go(tree_attn_tc_kernel<false, false>, 3, Lay<false>::BYTES);
 }
 
 }  // namespace koala
