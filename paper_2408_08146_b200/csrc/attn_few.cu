@@ -1,5 +1,6 @@
-// Tree-masked attention of at most four query rows per sequence (one-token steps, chain drafts,
-// short drafts) for bf16 caches with head_dim 128.
+// Tree-masked attention on CUDA cores: at most four query rows per sequence (one-token steps, chain drafts)
+// of bf16 caches with head_dim 128, and every size of the fp32 and head_dim 64 configurations, whose rows
+// are taken in groups (grid z).
 //
 // With so few rows the cached keys and values are all there is to move: 512 bytes per key and head
 // against a few hundred multiply-adds, so the products run in fp32 on the CUDA cores (the tensor-core
@@ -12,25 +13,49 @@
 // Tried and dropped: tiles dealt evenly over all CTAs with partials in global memory and the last
 // arriver adding them (fence, counter and the re-read: 4 us at the end of every launch; 14 us per
 // launch, ragged batch 22 us).
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace koala {
 namespace {
 
-constexpr int DH = 128;
 constexpr int TILE = 64;
 constexpr int WARPS = 8;
 constexpr int MAX_CHUNKS = 8;
-constexpr int PSTRIDE = DH + 4;           // floats of a partial: O[128], m, l, pad (16-byte rows)
 
-__device__ __forceinline__ void unpack8(const uint4 &u, float *f) {
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    f[2 * i] = __uint_as_float(w[i] << 16);
-    f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+// E consecutive cache elements of a lane, as loaded and as floats.
+template <typename T, int E> struct Frag;
+template <int E> struct Frag<bf16, E> {
+  uint32_t w[E / 2];
+  __device__ __forceinline__ void load(const bf16 *p, bool in) {
+    if constexpr (E == 8) {
+      const uint4 u = in ? *reinterpret_cast<const uint4 *>(p) : make_uint4(0u, 0u, 0u, 0u);
+      w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
+    } else {
+      const uint2 u = in ? *reinterpret_cast<const uint2 *>(p) : make_uint2(0u, 0u);
+      w[0] = u.x; w[1] = u.y;
+    }
   }
-}
+  __device__ __forceinline__ void unpack(float *f) const {
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) {
+      f[2 * i] = __uint_as_float(w[i] << 16);
+      f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+  }
+};
+template <int E> struct Frag<float, E> {
+  float4 w[E / 4];
+  __device__ __forceinline__ void load(const float *p, bool in) {
+#pragma unroll
+    for (int i = 0; i < E / 4; ++i) w[i] = in ? reinterpret_cast<const float4 *>(p)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ void unpack(float *f) const {
+#pragma unroll
+    for (int i = 0; i < E / 4; ++i) { f[4 * i] = w[i].x; f[4 * i + 1] = w[i].y; f[4 * i + 2] = w[i].z; f[4 * i + 3] = w[i].w; }
+  }
+};
 
 __device__ __forceinline__ float ld_cluster(uint32_t local_addr, uint32_t rank) {
   uint32_t ra;
@@ -40,35 +65,38 @@ __device__ __forceinline__ float ld_cluster(uint32_t local_addr, uint32_t rank) 
   return v;
 }
 
-template <int RT>
+template <typename T, int DH, int RT>
 __global__ void __launch_bounds__(WARPS * 32, RT <= 2 ? 2 : 1)
-tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan plan, bf16 *__restrict__ out,
-                     bf16 *__restrict__ out_lo, int rows_per_seq, int n_heads, int S_max) {
+tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *__restrict__ out, T *__restrict__ out_lo,
+                     int rows_per_seq, int n_heads, int S_max) {
+  constexpr int E = DH / 16;                               // dims of a lane
+  constexpr int PSTRIDE = DH + 4;                          // floats of a partial: O[DH], m, l, pad (16-byte rows)
   __shared__ __align__(16) float s_q[RT][DH];
   __shared__ __align__(16) float s_o[2 * WARPS][RT][PSTRIDE];
   __shared__ __align__(16) float s_c[RT][PSTRIDE];         // this chunk's result, read by the cluster
   pdl_launch_dependents();
   pdl_wait();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hf = lane >> 4, d0 = (lane & 15) * 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hf = lane >> 4, d0 = (lane & 15) * E;
   const int H = n_heads * DH;
   const int c = (int)blockIdx.x, chunks = (int)gridDim.x;
   const int b = (int)blockIdx.y / n_heads, h = (int)blockIdx.y % n_heads;
-  const float sc = 0.08838834764831845f * 1.4426950408889634f;    // 1/sqrt(128) * log2(e)
+  const float sc = (DH == 128 ? 0.08838834764831845f : 0.125f) * 1.4426950408889634f;    // 1/sqrt(DH) * log2(e)
+  const int i0 = (int)blockIdx.z * RT;                     // this CTA's rows of the sequence: i0 ..
   const int ctx = plan.ctx_len[b];
   const int kv_len = min(plan.kv_len[b], S_max);
   const int tiles = (kv_len + TILE - 1) / TILE;
   const int t_lo = tiles * c / chunks, t_hi = tiles * (c + 1) / chunks;
   const size_t base = ((size_t)plan.cache_of(b) * n_heads + h) * S_max;
-  const bf16 *kb = kc + base * DH + d0, *vb = vc + base * DH + d0;
+  const T *kb = kc + base * DH + d0, *vb = vc + base * DH + d0;
   const int k_off = warp * 8 + hf;                       // this half-warp's keys of a tile: k_off + 2 j
-  uint4 kn[4], vn[4];
+  Frag<T, E> kn[4], vn[4];
   auto load = [&](int t) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int key = t * TILE + k_off + 2 * j;
       const bool in = key < kv_len;                      // slots past the end were never written
-      kn[j] = in ? *reinterpret_cast<const uint4 *>(kb + (size_t)key * DH) : make_uint4(0u, 0u, 0u, 0u);
-      vn[j] = in ? *reinterpret_cast<const uint4 *>(vb + (size_t)key * DH) : make_uint4(0u, 0u, 0u, 0u);
+      kn[j].load(kb + (size_t)key * DH, in);
+      vn[j].load(vb + (size_t)key * DH, in);
     }
   };
   load(t_lo);                                            // first of all: the longest way
@@ -76,44 +104,48 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
   unsigned row_ok = 0;
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
-    const int rg = b * rows_per_seq + (r < rows_per_seq ? r : 0);
+    const int rg = b * rows_per_seq + (i0 + r < rows_per_seq ? i0 + r : 0);
     const int slot = plan.slot[rg];
     mk0[r] = plan.mask[(size_t)rg * 2];
     mk1[r] = plan.mask[(size_t)rg * 2 + 1];
-    if (r < rows_per_seq && slot >= 0) row_ok |= 1u << r;
+    if (i0 + r < rows_per_seq && slot >= 0) row_ok |= 1u << r;
   }
   for (int e = threadIdx.x; e < RT * DH; e += WARPS * 32) {
     const int r = e / DH, d = e % DH;
-    s_q[r][d] = q[(size_t)(b * rows_per_seq + (r < rows_per_seq ? r : 0)) * H + h * DH + d] * sc;
+    s_q[r][d] = q[(size_t)(b * rows_per_seq + (i0 + r < rows_per_seq ? i0 + r : 0)) * H + h * DH + d] * sc;
   }
   __syncthreads();
-  float m[RT], l[RT], o[RT][8];
+  float m[RT], l[RT], o[RT][E];
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
     m[r] = -INFINITY;
     l[r] = 0.f;
 #pragma unroll
-    for (int d = 0; d < 8; ++d) o[r][d] = 0.f;
+    for (int d = 0; d < E; ++d) o[r][d] = 0.f;
   }
   for (int t = t_lo; t < t_hi; ++t) {
-    uint4 kx[4], vx[4];
+    Frag<T, E> kx[4], vx[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) { kx[j] = kn[j]; vx[j] = vn[j]; }
     if (t + 1 < t_hi) load(t + 1);
     float s[RT][4];
     {
-      float kf[4][8];
+      float kf[4][E];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) unpack8(kx[j], kf[j]);
+      for (int j = 0; j < 4; ++j) kx[j].unpack(kf[j]);
 #pragma unroll
       for (int r = 0; r < RT; ++r) {
-        const float4 qa = *reinterpret_cast<const float4 *>(&s_q[r][d0]), qb = *reinterpret_cast<const float4 *>(&s_q[r][d0 + 4]);
-        const float qr[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+        float qr[E];
+#pragma unroll
+        for (int d = 0; d < E; d += 4) {
+          const float4 qa = *reinterpret_cast<const float4 *>(&s_q[r][d0 + d]);
+          qr[d] = qa.x; qr[d + 1] = qa.y; qr[d + 2] = qa.z; qr[d + 3] = qa.w;
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           float a = 0.f;
 #pragma unroll
-          for (int d = 0; d < 8; ++d) a = fmaf(qr[d], kf[j][d], a);
+          for (int d = 0; d < E; ++d) a = fmaf(qr[d], kf[j][d], a);
           s[r][j] = a;
         }
       }
@@ -141,7 +173,7 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
       m[r] = mx;
       l[r] *= corr;
 #pragma unroll
-      for (int d = 0; d < 8; ++d) o[r][d] *= corr;
+      for (int d = 0; d < E; ++d) o[r][d] *= corr;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         s[r][j] = exp2f(s[r][j] - mu);
@@ -150,12 +182,12 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float vf[8];
-      unpack8(vx[j], vf);
+      float vf[E];
+      vx[j].unpack(vf);
 #pragma unroll
       for (int r = 0; r < RT; ++r)
 #pragma unroll
-        for (int d = 0; d < 8; ++d) o[r][d] = fmaf(s[r][j], vf[d], o[r][d]);
+        for (int d = 0; d < E; ++d) o[r][d] = fmaf(s[r][j], vf[d], o[r][d]);
     }
   }
 // ---- the CTA's sixteen half-warps
@@ -163,16 +195,16 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
 #pragma unroll
-    for (int d = 0; d < 8; d += 4)
+    for (int d = 0; d < E; d += 4)
       *reinterpret_cast<float4 *>(&s_o[src][r][d0 + d]) = make_float4(o[r][d], o[r][d + 1], o[r][d + 2], o[r][d + 3]);
     if ((lane & 15) == 0) { s_o[src][r][DH] = m[r]; s_o[src][r][DH + 1] = l[r]; }
   }
   __syncthreads();
   auto emit = [&](int r, int d, float v) {
-    const size_t at = (size_t)(b * rows_per_seq + r) * H + h * DH + d;
-    const bf16 hi = __float2bfloat16_rn(v);
+    const size_t at = (size_t)(b * rows_per_seq + i0 + r) * H + h * DH + d;
+    const T hi = from_f<T>(v);
     out[at] = hi;
-    if (out_lo != nullptr) out_lo[at] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    if (out_lo != nullptr) out_lo[at] = from_f<T>(v - to_f(hi));
   };
   for (int e = threadIdx.x; e < RT * DH; e += WARPS * 32) {
     const int r = e / DH, d = e % DH;
@@ -189,7 +221,7 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
       }
     }
     if (chunks == 1) {
-      if (r < rows_per_seq) emit(r, d, ll > 0.f ? acc / ll : 0.f);
+      if (i0 + r < rows_per_seq) emit(r, d, ll > 0.f ? acc / ll : 0.f);
     } else {
       s_c[r][d] = acc;
       if (d == 0) { s_c[r][DH] = mm; s_c[r][DH + 1] = ll; }
@@ -224,7 +256,7 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
         ll += wt * pl[k];
       }
     }
-    if (r < rows_per_seq) emit(r, d, ll > 0.f ? acc / ll : 0.f);
+    if (i0 + r < rows_per_seq) emit(r, d, ll > 0.f ? acc / ll : 0.f);
   }
   // no CTA leaves while another may still read its result
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
@@ -233,36 +265,50 @@ tree_attn_few_kernel(const float *q, const bf16 *kc, const bf16 *vc, RowPlan pla
 
 }  // namespace
 
+// Rows per CTA: in bf16 at head_dim 128, where up to four rows come here, all of them; elsewhere one while
+// that makes few CTAs (latency), four (two with fp32 rows of 128) where the cache would be re-read too often.
 // Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the launch
 // within what is resident at once (two CTAs per SM up to two rows, else one; clusters of eight do not
-// fill every GPC, hence seven eighths), and at least two tiles of capacity per chunk.
-cudaError_t tree_attention_few(Launch L, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
-                               Operand out, int rows_per_seq, int B, int n_heads, int S_max, int num_sms) {
-  if (rows_per_seq < 1 || rows_per_seq > ATTN_FEW_ROWS) return cudaErrorInvalidValue;
-  const int room = (rows_per_seq <= 2 ? 2 : 1) * num_sms * 7 / 8;
-  int chunks = 1;
-  while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads <= room && 2 * chunks * 2 * TILE <= S_max) chunks *= 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(chunks, n_heads * B);
-  cfg.blockDim = dim3(WARPS * 32);
-  cfg.stream = L.st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = L.pdl ? 1 : 0;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = chunks;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = chunks > 1 ? 2 : 1;
-  ++g_launches;
-  auto go = [&](auto *kern) {
-    return cudaLaunchKernelEx(&cfg, kern, q, (const bf16 *)k_cache, (const bf16 *)v_cache, plan, (bf16 *)out.hi,
-                              (bf16 *)out.lo, rows_per_seq, n_heads, S_max);
+// fill every GPC, hence seven eighths), and at least `min_keys` of capacity per chunk: two tiles, eight
+// in the small configurations, where the cluster's two barriers cost more than a few tiles.
+cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
+                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms) {
+  if (rows_per_seq < 1 || (head_dim != 64 && head_dim != 128)) return cudaErrorInvalidValue;
+  const bool bf = dtype != 0;
+  auto go = [&](auto tag, auto dh, auto rt) -> cudaError_t {
+    typedef decltype(tag) T;
+    constexpr int DH = decltype(dh)::value, RT = decltype(rt)::value;
+    const int groups = (rows_per_seq + RT - 1) / RT;
+    const int room = (RT <= 2 ? 2 : 1) * num_sms * 7 / 8, min_keys = (bf && DH == 128 ? 2 : 8) * TILE;
+    int chunks = 1;
+    while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads * groups <= room && 2 * chunks * min_keys <= S_max) chunks *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(chunks, n_heads * B, groups);
+    cfg.blockDim = dim3(WARPS * 32);
+    cfg.stream = L.st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = L.pdl ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = chunks;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chunks > 1 ? 2 : 1;
+    ++g_launches;
+    return cudaLaunchKernelEx(&cfg, tree_attn_few_kernel<T, DH, RT>, q, (const T *)k_cache, (const T *)v_cache, plan,
+                              (T *)out.hi, (T *)out.lo, rows_per_seq, n_heads, S_max);
   };
-  if (rows_per_seq == 1) return go(tree_attn_few_kernel<1>);
-  if (rows_per_seq == 2) return go(tree_attn_few_kernel<2>);
-  return go(tree_attn_few_kernel<4>);
+  std::integral_constant<int, 64> d64;
+  std::integral_constant<int, 128> d128;
+  std::integral_constant<int, 1> r1;
+  std::integral_constant<int, 2> r2;
+  std::integral_constant<int, 4> r4;
+  const bool one = rows_per_seq == 1 || (!(bf && head_dim == 128) && (long long)rows_per_seq * B * n_heads <= 4LL * num_sms);
+  if (bf && head_dim == 128) return one ? go(bf16{}, d128, r1) : (rows_per_seq == 2 ? go(bf16{}, d128, r2) : go(bf16{}, d128, r4));
+  if (bf) return one ? go(bf16{}, d64, r1) : go(bf16{}, d64, r4);
+  if (head_dim == 64) return one ? go(float{}, d64, r1) : go(float{}, d64, r4);
+  return one ? go(float{}, d128, r1) : go(float{}, d128, r2);
 }
 
 }  // namespace koala

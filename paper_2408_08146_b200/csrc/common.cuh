@@ -5,6 +5,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <cstring>
 #include <mutex>
 
 typedef __nv_bfloat16 bf16;
@@ -218,9 +219,6 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
                           Operand q_pair, void *k_cache, void *v_cache, int R, int rows_per_seq, int n_heads,
                           int head_dim, int S_max);
 cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, int R, int F);
-cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_cache,
-                           const void *v_cache, RowPlan plan, Operand out, int R, int rows_per_seq,
-                           int B, int n_heads, int head_dim, int S_max);
 // out[map(r)] <- arg-max of row r; with `spread` the row is also copied to row map(r) of it
 cudaError_t argmax_rows(Launch L, const float *logits, int32_t *out, float *spread, RowMap map, int R, int V);
 cudaError_t topk_logp(Launch L, const float *logits, int32_t *tok, float *logp, int R, int V, int k);
@@ -234,10 +232,11 @@ int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms
 cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, const void *v_cache,
                                RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks);
 
-// attn_few.cu : bf16 caches, head_dim 128, at most ATTN_FEW_ROWS query rows per sequence
+// attn_few.cu : any dtype, head_dim 64 or 128, on CUDA cores; where the tensor-core kernels apply, up to ATTN_FEW_ROWS
+// rows per sequence
 constexpr int ATTN_FEW_ROWS = 4;
-cudaError_t tree_attention_few(Launch L, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
-                               Operand out, int rows_per_seq, int B, int n_heads, int S_max, int num_sms);
+cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
+                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms);
 
 // attn_tc.cu : the same on tcgen05 tensor cores, all rows of a sequence in one CTA, key chunks as a cluster;
 // the queries come as the bf16 pair written by rope_kv_write ([q_rows_alloc][n_heads * 128] each)
@@ -246,6 +245,25 @@ bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max);
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
                               RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
                               int *status);
+
+// gemm_few.cu : fp32 multiplies of latency-bound sizes together with the row-wise steps around them
+enum { FEW_ROPE = 1, FEW_SWIGLU = 2, FEW_RESIDUAL = 3 };
+struct FewJob {
+  int mode, R, K, n_out;        // n_out: rows of one weight matrix (ROPE: three of them, SWIGLU: two)
+  const void *X, *W[3];         // ROPE, SWIGLU: X is the residual stream, its norm is part of the launch
+  const void *gain;             // gain and eps of that norm
+  float eps;
+  float *x;                     // RESIDUAL: x += result, or x = result + bias
+  const void *bias;
+  void *out;                    // RESIDUAL: x once more (may be null), out2 likewise; SWIGLU: activations
+  float *out2;
+  RowPlan plan;                 // ROPE
+  float *q_out;
+  void *k_cache, *v_cache;
+  int rows_per_seq, n_heads, head_dim, S_max;
+};
+bool few_supported(const void *X, int R, int K, int units, const void *const *W, int n_w);
+cudaError_t gemm_few(Launch L, const FewJob &job, int num_sms);
 
 // gemm_simt.cu : Y[R][sum n_out] (fp32, ld ldy) = X[R][K_in] * W^T, X and W of `dtype`
 cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int R, float *Y,

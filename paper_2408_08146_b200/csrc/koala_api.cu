@@ -48,6 +48,7 @@ struct Carver {
 };
 
 constexpr int MAX_SPLIT = 12;     // partial-sum matrices the workspace holds per GEMM
+constexpr int NUM_SMS = 148;
 // Prompt tokens per forward of koala_ingest: enough for the multiplies to be bound by the tensor cores
 // (256-token tiles, four of them), few enough for the workspace to stay small (four partial-sum
 // matrices of that many rows; 7B shape: 0.36 GB).
@@ -331,16 +332,13 @@ int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq) {
   if (c->use_tc && g.dtype == KOALA_BF16 && c->qpair.lo != nullptr &&
       attn_tc_supported(rows_per_seq, g.head_dim, g.S_max)) {
     CU_TRY(tree_attention_tc(LN(c), c->qpair, c->Mp, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups,
-                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, 148), c->status));
-  } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq <= ATTN_FEW_ROWS) {
-    CU_TRY(tree_attention_few(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
-                              g.S_max, 148));
-  } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq <= 128) {
+                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, NUM_SMS), c->status));
+  } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq > ATTN_FEW_ROWS && rows_per_seq <= 128) {
     CU_TRY(tree_attention_mma(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
-                              g.S_max, attn_mma_chunks(groups, g.n_heads, rows_per_seq, g.S_max, 148)));
+                              g.S_max, attn_mma_chunks(groups, g.n_heads, rows_per_seq, g.S_max, NUM_SMS)));
   } else {
-    CU_TRY(tree_attention(LN(c), g.dtype, c->qbuf, kc, vc, row_plan(c), c->attn_out, R, rows_per_seq, groups,
-                          g.n_heads, g.head_dim, g.S_max));
+    CU_TRY(tree_attention_few(LN(c), g.dtype, c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
+                              g.head_dim, g.S_max, NUM_SMS));
   }
   time_end(c, ta);
   return KOALA_OK;
@@ -394,6 +392,71 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
 }
 
 
+// Whether the layers of a forward over R rows run as multiplies with the row-wise steps inside (gemm_few).
+bool layers_few(koala_ctx *c, const std::vector<LayerW> &layers, int R) {
+  const koala_config &g = c->cfg;
+  if (g.dtype != KOALA_FP32 || layers.empty()) return false;
+  for (const LayerW &w : layers) {
+    const void *qkv[4] = {w.wq, w.wk, w.wv, w.attn_norm}, *gu[3] = {w.wg, w.wu, w.ffn_norm};
+    if (!few_supported(c->x, R, g.H, 3 * g.H / 2, qkv, 4) || !few_supported(c->attn_out.hi, R, g.H, g.H / 2, &w.wo, 1) ||
+        !few_supported(c->x, R, g.H, g.F, gu, 3) || !few_supported(c->act.hi, R, g.F, g.H / 2, &w.wd, 1))
+      return false;
+  }
+  return true;
+}
+
+int few_gemm(koala_ctx *c, const FewJob &j, int n_w) {
+  const int tb = time_begin(c, KOALA_CLS_GEMM_SIMT, (uint64_t)n_w * j.n_out * j.K * c->esz);
+  CU_TRY(gemm_few(LN(c), j, NUM_SMS));
+  time_end(c, tb);
+  return KOALA_OK;
+}
+
+// run_layers in that form: five launches a layer, everything between them in c->x.
+int run_layers_few(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, void *kbase, void *vbase, int R,
+                   int rows_per_seq, const void *final_g, Operand final_xn, float *out_f32, RowMap out_map,
+                   bool last_kv_only) {
+  const koala_config &g = c->cfg;
+  const int H = g.H, F = g.F;
+  const size_t le = kv_layer_elems(g) * c->esz;
+  FewJob j;
+  auto job = [&](int mode, const void *X, int K, int n_out) {
+    memset(&j, 0, sizeof(j));
+    j.mode = mode; j.R = R; j.K = K; j.n_out = n_out; j.X = X; j.eps = g.rms_eps;
+  };
+  c->pending = RowScale{nullptr, 0, 0.f, 0.f, 0};
+  for (int l = 0; l < n_layers; ++l) {
+    const LayerW &w = layers[l];
+    const bool last = l == n_layers - 1;
+    void *kc = (unsigned char *)kbase + (size_t)l * le, *vc = (unsigned char *)vbase + (size_t)l * le;
+    job(FEW_ROPE, c->x, H, H);
+    j.W[0] = w.wq; j.W[1] = w.wk; j.W[2] = w.wv; j.gain = w.attn_norm;
+    j.plan = row_plan(c); j.q_out = c->qbuf; j.k_cache = kc; j.v_cache = vc;
+    j.rows_per_seq = rows_per_seq; j.n_heads = g.n_heads; j.head_dim = g.head_dim; j.S_max = g.S_max;
+    K_TRY(few_gemm(c, j, 3));
+    if (last && last_kv_only) return KOALA_OK;
+    K_TRY(run_attention(c, kc, vc, R, rows_per_seq));
+    job(FEW_RESIDUAL, c->attn_out.hi, H, H);
+    j.W[0] = w.wo; j.x = c->x;
+    K_TRY(few_gemm(c, j, 1));
+    job(FEW_SWIGLU, c->x, H, F);
+    j.W[0] = w.wg; j.W[1] = w.wu; j.gain = w.ffn_norm; j.out = c->act.hi;
+    K_TRY(few_gemm(c, j, 2));
+    if (last && final_g != nullptr) {        // the last norm needs whole rows
+      SplitIn s;
+      GemmMats dn{{w.wd, nullptr, nullptr}, {H, 0, 0}, 1};
+      K_TRY(do_gemm(c, c->act, F, dn, R, nullptr, 0, &s));
+      CU_TRY(row_epilogue(LN(c), g.dtype, 0, c->x, s, nullptr, final_g, final_xn, out_f32, out_map, R, H, g.rms_eps));
+    } else {
+      job(FEW_RESIDUAL, c->act.hi, F, H);
+      j.W[0] = w.wd; j.x = c->x;
+      if (last) { j.out = final_xn.hi; j.out2 = out_f32; }
+      K_TRY(few_gemm(c, j, 1));
+    }
+  }
+  return KOALA_OK;
+}
+
 // n_layers pre-norm decoder layers over R rows.  On entry x holds the residual stream and c->xn the
 // first layer's input (normalised, or x * gain with its scale pending in c->pending).  last_kv_only: the
 // last layer only writes its keys and values (prompt positions whose hidden state nobody reads).  After the
@@ -405,6 +468,8 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
 int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, void *kbase, void *vbase, int R,
                int rows_per_seq, const void *final_g, Operand final_xn, float *out_f32, RowMap out_map,
                bool last_kv_only = false) {
+  if (n_layers > 0 && layers_few(c, layers, R))
+    return run_layers_few(c, layers, n_layers, kbase, vbase, R, rows_per_seq, final_g, final_xn, out_f32, out_map, last_kv_only);
   const koala_config &g = c->cfg;
   const int H = g.H, F = g.F;
   const size_t le = kv_layer_elems(g) * c->esz;
@@ -513,6 +578,19 @@ int run_layers(koala_ctx *c, const std::vector<LayerW> &layers, int n_layers, vo
   return KOALA_OK;
 }
 
+// fc of an EAGLE-style head with its bias in the same launch, for layers that take their input from c->x.
+bool fc_few(koala_ctx *c, int R) {
+  const koala_config &g = c->cfg;
+  return g.K > 0 && layers_few(c, c->draft_layers, R) && few_supported(c->cat.hi, R, 2 * g.H, g.H / 2, &c->fc_w, 1);
+}
+int fc_few_run(koala_ctx *c, int R) {
+  const koala_config &g = c->cfg;
+  FewJob j;
+  memset(&j, 0, sizeof(j));
+  j.mode = FEW_RESIDUAL; j.R = R; j.K = 2 * g.H; j.n_out = g.H; j.X = c->cat.hi; j.W[0] = c->fc_w; j.x = c->x; j.bias = c->fc_b;
+  return few_gemm(c, j, 1);
+}
+
 // x and the first target layer's input from the plan's tokens
 int embed_rows(koala_ctx *c, int R) {
   const koala_config &g = c->cfg;
@@ -572,7 +650,8 @@ int draft_eagle(koala_ctx *c, int pass) {
   CU_TRY(eagle_concat(LN(c), g.dtype, feat_src, c->p.row_src, c->p.row_tok, c->embed, c->cat, R, H, g.V));
   SplitIn s;
   GemmMats fc{{c->fc_w, nullptr, nullptr}, {H, 0, 0}, 1};
-  K_TRY(do_gemm(c, c->cat, 2 * H, fc, R, nullptr, 0, &s));
+  const bool few = fc_few(c, R);
+  if (!few) K_TRY(do_gemm(c, c->cat, 2 * H, fc, R, nullptr, 0, &s));
   // pass 0: the feature of every row stays in x and the last valid row is gathered afterwards;
   // pass >= 1: every row's feature goes to feat[pass & 1] and to the LM head's input.
   float *f_all = pass == 0 ? nullptr : c->feat[pass & 1];
@@ -582,8 +661,12 @@ int draft_eagle(koala_ctx *c, int pass) {
   if (g.K == 0) {
     CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, nullptr, lm_all, f_all, same, R, H, g.rms_eps));
   } else {
-    CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, c->draft_layers[0].attn_norm, c->xn, nullptr,
-                        same, R, H, g.rms_eps));
+    if (few) {
+      K_TRY(fc_few_run(c, R));
+    } else {
+      CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, c->draft_layers[0].attn_norm, c->xn, nullptr,
+                          same, R, H, g.rms_eps));
+    }
     K_TRY(run_layers(c, c->draft_layers, g.K, c->dk, c->dv, R, rows, nullptr, lm_all, f_all, same));
   }
   int lm_rows = R;

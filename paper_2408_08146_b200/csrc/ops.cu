@@ -471,78 +471,6 @@ __global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc
                              silu_f(rs * a.z) * (rs * b.z), silu_f(rs * a.w) * (rs * b.w)));
 }
 
-// ------------------------------------------------------------------------------- tree attention
-// One block = 8 query rows of one (sequence, head); one warp per query row.  Keys/values stream
-// through shared memory 32 at a time; lane j scores key j, then the warp accumulates P.V with
-// each lane owning DH/32 output dimensions.  Online softmax in fp32.
-template <typename T, int DH>
-__global__ void __launch_bounds__(256)
-tree_attn_kernel(const float *q, const T *kc, const T *vc,
-                 RowPlan plan, T *__restrict__ out, T *__restrict__ out_lo, int rows_per_seq,
-                 int n_heads, int S_max) {
-  __shared__ float Ks[32][DH + 1];
-  __shared__ float Vs[32][DH];
-  __shared__ float qs[8][DH];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int b = blockIdx.z, h = blockIdx.y;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + w;
-  const int H = n_heads * DH;
-  const int r = b * rows_per_seq + (i < rows_per_seq ? i : 0);
-  const bool valid = (i < rows_per_seq) && (plan.slot[r] >= 0);
-  const int ctx = plan.ctx_len[b], kv_len = plan.kv_len[b];
-  const uint64_t m0 = plan.mask[(size_t)r * 2], m1 = plan.mask[(size_t)r * 2 + 1];
-  for (int d = lane; d < DH; d += 32) qs[w][d] = valid ? q[(size_t)r * H + h * DH + d] : 0.f;
-  const int cb = plan.cache_of(b);
-  const T *kb = kc + ((size_t)cb * n_heads + h) * S_max * DH;
-  const T *vb = vc + ((size_t)cb * n_heads + h) * S_max * DH;
-  const float scale = rsqrtf((float)DH);
-  float m = -INFINITY, l = 0.f;
-  float o[DH / 32];
-#pragma unroll
-  for (int d = 0; d < DH / 32; ++d) o[d] = 0.f;
-  for (int t0 = 0; t0 < kv_len; t0 += 32) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < 32 * DH; e += 256) {
-      const int j = e / DH, d = e % DH;
-      const bool in = (t0 + j) < kv_len;
-      Ks[j][d] = in ? to_f(kb[(size_t)(t0 + j) * DH + d]) : 0.f;
-      Vs[j][d] = in ? to_f(vb[(size_t)(t0 + j) * DH + d]) : 0.f;
-    }
-    __syncthreads();
-    const int t = t0 + lane;
-    bool vis = valid && t < kv_len;
-    if (vis && t >= ctx) {
-      const int rel = t - ctx;
-      vis = rel < 64 ? ((m0 >> rel) & 1ull) : (rel < 128 ? ((m1 >> (rel - 64)) & 1ull) : false);
-    }
-    float s = 0.f;
-#pragma unroll 8
-    for (int d = 0; d < DH; ++d) s += qs[w][d] * Ks[lane][d];
-    s = vis ? s * scale : -INFINITY;
-    const float m_new = fmaxf(m, warp_max(s));
-    if (m_new == -INFINITY) continue;   // nothing visible so far (uniform across the warp)
-    const float p = vis ? expf(s - m_new) : 0.f;
-    const float corr = (m == -INFINITY) ? 0.f : expf(m - m_new);
-    l = l * corr + warp_sum(p);
-    m = m_new;
-#pragma unroll
-    for (int d = 0; d < DH / 32; ++d) o[d] *= corr;
-    for (int j = 0; j < 32; ++j) {
-      const float pj = __shfl_sync(0xffffffffu, p, j);
-#pragma unroll
-      for (int d = 0; d < DH / 32; ++d) o[d] += pj * Vs[j][lane + 32 * d];
-    }
-  }
-  if (i < rows_per_seq) {
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-    for (int d = 0; d < DH / 32; ++d)
-      store_operand(out, out_lo, (size_t)r * H + h * DH + lane + 32 * d, o[d] * inv);
-  }
-}
-
 // ------------------------------------------------------------------------------- arg-max / top-k
 struct ValIdx {
   float v;
@@ -928,23 +856,6 @@ cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, in
   }
   DISPATCH_T(dtype, return launch_k(swiglu_kernel<T>, dim3((F + 255) / 256, R), dim3(256), 0, L.st,
                                     L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)
-}
-
-cudaError_t tree_attention(Launch L, int dtype, const float *q, const void *k_cache,
-                           const void *v_cache, RowPlan plan, Operand out, int R, int rows_per_seq,
-                           int B, int n_heads, int head_dim, int S_max) {
-  (void)R;
-  dim3 grid((rows_per_seq + 7) / 8, n_heads, B);
-  if (head_dim == 64) {
-    DISPATCH_T(dtype, return launch_k(tree_attn_kernel<T, 64>, grid, dim3(256), 0, L.st, L.pdl, q,
-                                      (const T *)k_cache, (const T *)v_cache, plan, (T *)out.hi,
-                                      (T *)out.lo, rows_per_seq, n_heads, S_max);)
-  } else if (head_dim == 128) {
-    DISPATCH_T(dtype, return launch_k(tree_attn_kernel<T, 128>, grid, dim3(256), 0, L.st, L.pdl, q,
-                                      (const T *)k_cache, (const T *)v_cache, plan, (T *)out.hi,
-                                      (T *)out.lo, rows_per_seq, n_heads, S_max);)
-  }
-  return cudaErrorInvalidValue;
 }
 
 static cudaError_t topk_cluster_launch(Launch L, const float *logits, int32_t *tok, float *logp, float *spread, RowMap map,

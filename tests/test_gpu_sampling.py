@@ -131,6 +131,8 @@ def test_draws_over_vocabularies_that_do_not_fill_the_segments(V):
     eng.prefill(pr, cfg.N)
     orc.prefill(pr, cfg.N)
     for it in range(3):
-        _iteration(cfg, eng, orc, 300 + it, True)
+        # (seeds 300.. put one draw of V = 3100 at 2e-6 of the mass from a boundary, inside the margin _margin_ok
+        #  asks for on account of fp32 probabilities: rounding of V terms, at most V * 2^-24 relative)
+        _iteration(cfg, eng, orc, 400 + it, True)
     assert eng.device_status() == 0
     eng.close()
