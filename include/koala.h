@@ -181,12 +181,12 @@ int koala_expand_tree(koala_ctx *ctx, int pass);
 int koala_verify(koala_ctx *ctx, const koala_tree *tree);
 
 /* Prompt ingestion in forwards wider than a tree.  Every prompt is cut into n_parts equal parts (the
- * first len % n_parts of them one token longer); all parts but the last are taken into the caches as if
- * each had been verified as a chain and accepted in full, followed, for an EAGLE-style head, by
- * koala_draft(0) with the next prompt token as root: target and head caches, seq_len and the acceptance
- * counters are as after those calls.  Up to 1024 tokens go through one forward and no logits are formed.
- * The caller continues with koala_verify(chain of the last part) and koala_accept.
- * tok: DEVICE [B][stride] prompts; len: HOST [B], copied. */
+ * first len % n_parts of them one token longer) of at most N tokens.  Target and head caches, seq_len, the
+ * acceptance counters, the tree and the verification buffers are afterwards as if every part had been
+ * verified as a chain, all but the last accepted in full and, with an EAGLE-style head, followed by
+ * koala_draft(0) with the next prompt token as root: the caller continues with koala_accept, with the
+ * lengths of the last parts (tree_n) as forced lengths.  Up to 1024 tokens go through one forward; logits
+ * are formed for the last parts only.  tok: DEVICE [B][stride] prompts; len: HOST [B], copied. */
 int koala_ingest(koala_ctx *ctx, const int32_t *tok, int32_t stride, const int32_t *len, int32_t n_parts);
 
 /* Greedy acceptance (Section 4.1: a draft token is kept only if it equals the target's greedy

@@ -382,22 +382,18 @@ class Koala:
 
     def prefill(self, prompts: Sequence[Sequence[int]], chunk: int):
         """Ingests the prompts as chain trees with full forced acceptance (EAGLE-style heads also
-        run draft pass 0 over every chunk but the last, with the next prompt token as root); the
-        chunks before the last go through koala_ingest, many at a time."""
+        run draft pass 0 over every chunk but the last, with the next prompt token as root);
+        koala_ingest takes many chunks through one forward."""
         c = self.cfg
         chunk = min(chunk, c.N)
         n_chunks = max(-(-len(p) // chunk) for p in prompts)
         lens = [len(p) for p in prompts]
-        last = [n // n_chunks for n in lens]             # the last of n_chunks equal parts
-        if n_chunks > 1:
-            host = np.zeros((c.B, max(lens)), np.int32)
-            for b, p in enumerate(prompts):
-                host[b, :lens[b]] = np.asarray(p)
-            toks = torch.from_numpy(host).to(self.dev)
-            self._check(self.lib.koala_ingest(self._ctx, toks.data_ptr(), toks.shape[1], _i32_array(lens), n_chunks))
-        tree = self.chain_tree([np.asarray(p)[lens[b] - last[b]:] for b, p in enumerate(prompts)])
-        self.koala_verify(tree)
-        self.koala_accept(tree[2])
+        host = np.zeros((c.B, max(lens)), np.int32)
+        for b, p in enumerate(prompts):
+            host[b, :lens[b]] = np.asarray(p)
+        toks = torch.from_numpy(host).to(self.dev)
+        self._check(self.lib.koala_ingest(self._ctx, toks.data_ptr(), toks.shape[1], _i32_array(lens), n_chunks))
+        self.koala_accept(self.buffers()["tree_n"])
 
     def step(self, forced_len: Optional[torch.Tensor] = None):
         """One whole iteration: D x (draft, expand_tree), verify, accept."""

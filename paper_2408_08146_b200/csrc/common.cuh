@@ -340,9 +340,11 @@ constexpr int INGEST_MAX_BLOCKS = 64;
 struct IngestBlocks {
   int n, q;
   int32_t start[INGEST_MAX_BLOCKS];
+  int32_t last[INGEST_MAX_BLOCKS];       // row of the block at which the sequence's last part begins (may lie outside)
   int16_t seq[INGEST_MAX_BLOCKS], count[INGEST_MAX_BLOCKS];
+  int16_t from[INGEST_MAX_BLOCKS];       // block of the target's forward that holds the rows (the head skips some)
 };
-// Prompt of each sequence: len tokens in n_parts equal parts, all but the last of which are ingested.
+// Prompt of each sequence: len tokens in n_parts equal parts; `count` tokens before the last part.
 struct IngestLens {
   int n_parts;
   int32_t len[64], count[64];
@@ -369,8 +371,13 @@ struct IngestKeep {
   int32_t src[64], dst[64];
 };
 cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, int H);
-// seq_len += count; acceptance counters as if every ingested part had been accepted as a chain
-cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, int32_t *seq_len, int B);
+// Rows of the sequences' last parts: verify_hid row b * N + u <- hid, xn row b * n_max + u <- T(hid).
+cudaError_t ingest_last(Launch L, int dtype, IngestBlocks k, const float *hid, float *verify_hid, Operand xn, int N, int n_max,
+                        int H);
+// seq_len += count; acceptance counters as if every part but the last had been accepted as a chain; the tree of
+// each sequence becomes the chain of its last part
+cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N,
+                          int *status);
 cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
                         int rows, int head_dim, float rope_base, int S_max, int *status);
 cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k,

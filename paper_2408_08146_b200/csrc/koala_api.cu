@@ -20,7 +20,7 @@ unsigned long long g_launches = 0;
 
 namespace {
 
-enum Phase { PH_READY = 0, PH_DRAFTED, PH_EXPANDED, PH_TREE, PH_VERIFIED, PH_INGESTED };
+enum Phase { PH_READY = 0, PH_DRAFTED, PH_EXPANDED, PH_TREE, PH_VERIFIED };
 
 struct LayerW {
   const void *attn_norm, *wq, *wk, *wv, *wo, *ffn_norm, *wg, *wu, *wd;
@@ -606,29 +606,58 @@ int embed_rows(koala_ctx *c, int R) {
   return KOALA_OK;
 }
 
-// One forward of the target over prompt blocks, then of an EAGLE-style head over the same positions
-// (hidden state of a position paired with the token after it).  Only caches are written.
-int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, const int32_t *tok, int stride) {
+// One forward of the target over prompt blocks, then of an EAGLE-style head over the positions before the last
+// parts (hidden state of a position paired with the token after it).  Besides the caches only the rows of
+// the last parts are kept, where a verification would leave them (n_max of them per sequence).
+int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, const int32_t *tok, int stride, int n_max) {
   const koala_config &g = c->cfg;
-  const int R = k.n * k.q, H = g.H;
-  const bool head = g.head_kind == KOALA_EAGLE && g.K > 0;
+  const int H = g.H;
   const Operand none{nullptr, nullptr};
   const RowMap same{0, 0};
+  IngestBlocks hd;                    // the head's blocks: rows before the last part
+  memset(&hd, 0, sizeof(hd));
+  hd.q = k.q;
+  bool has_last = false;
+  for (int v = 0; v < k.n; ++v) {
+    const int before = k.last[v] < k.count[v] ? k.last[v] : k.count[v];
+    has_last = has_last || before < k.count[v];
+    if (before <= 0) continue;
+    hd.start[hd.n] = k.start[v]; hd.seq[hd.n] = k.seq[v]; hd.count[hd.n] = (int16_t)before; hd.from[hd.n] = (int16_t)v;
+    ++hd.n;
+  }
+  const bool head = g.head_kind == KOALA_EAGLE && g.K > 0 && hd.n > 0;
+  const int R = k.n * k.q, Rh = hd.n * hd.q;
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
+  c->ingest_blocks = k.n;
   CU_TRY(plan_ingest(LN(c), c->p, k, tok, stride, 0, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
   K_TRY(embed_rows(c, R));
-  K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, k.q, c->final_norm, none, c->mx, same, !head));
+  K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, k.q, c->final_norm, none, c->mx, same, !head && !has_last));
+  if (has_last) CU_TRY(ingest_last(LN(c), g.dtype, k, c->mx, c->verify_hid, c->lmin, g.N, n_max, H));
   if (!head) return KOALA_OK;
   CU_TRY(ingest_keep(LN(c), c->t, keep, c->mx, H));
-  CU_TRY(plan_ingest(LN(c), c->p, k, tok, stride, 1, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
-  CU_TRY(eagle_concat(LN(c), g.dtype, c->mx, c->p.row_src, c->p.row_tok, c->embed, c->cat, R, H, g.V));
+  c->ingest_blocks = hd.n;
+  CU_TRY(plan_ingest(LN(c), c->p, hd, tok, stride, 1, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
+  CU_TRY(eagle_concat(LN(c), g.dtype, c->mx, c->p.row_src, c->p.row_tok, c->embed, c->cat, Rh, H, g.V));
   SplitIn s;
   GemmMats fc{{c->fc_w, nullptr, nullptr}, {H, 0, 0}, 1};
-  K_TRY(do_gemm(c, c->cat, 2 * H, fc, R, nullptr, 0, &s));
-  CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, c->draft_layers[0].attn_norm, c->xn, nullptr, same, R, H,
+  K_TRY(do_gemm(c, c->cat, 2 * H, fc, Rh, nullptr, 0, &s));
+  CU_TRY(row_epilogue(LN(c), g.dtype, 1, c->x, s, c->fc_b, c->draft_layers[0].attn_norm, c->xn, nullptr, same, Rh, H,
                       g.rms_eps));
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
-  return run_layers(c, c->draft_layers, g.K, c->dk, c->dv, R, k.q, nullptr, none, nullptr, same, true);
+  return run_layers(c, c->draft_layers, g.K, c->dk, c->dv, Rh, k.q, nullptr, none, nullptr, same, true);
+}
+
+// Logits and greedy tokens of R verified rows in c->lmin; row r is node row out_map(r) of the buffers.
+int target_logits(koala_ctx *c, int R, RowMap out_map) {
+  const koala_config &g = c->cfg;
+  GemmMats lm{{c->lm_head, nullptr, nullptr}, {g.V, 0, 0}, 1};
+  // spread rows: the product goes through the partial-sum buffer and the arg-max kernel, which reads every
+  // logit anyway, puts the rows in their places (in the multiply's own stores the row arithmetic cost
+  // every launch 4 %)
+  float *logits = out_map.rows == 0 ? c->verify_logits : c->P;
+  K_TRY(do_gemm(c, c->lmin, g.H, lm, R, logits, g.V, nullptr));
+  CU_TRY(argmax_rows(LN(c), logits, c->verify_tgt, out_map.rows == 0 ? nullptr : c->verify_logits, out_map, R, g.V));
+  return KOALA_OK;
 }
 
 int draft_eagle(koala_ctx *c, int pass) {
@@ -945,13 +974,7 @@ int koala_verify(koala_ctx *c, const koala_tree *tree) {
   CU_TRY(plan_verify(LN(c), c->t, c->p, c->seq_len, g.B, g.N, rows, g.head_dim, g.rope_base, g.S_max, c->status));
   K_TRY(embed_rows(c, R));
   K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, rows, c->final_norm, c->lmin, c->verify_hid, out_map));
-  GemmMats lm{{c->lm_head, nullptr, nullptr}, {g.V, 0, 0}, 1};
-  // spread rows: the product goes through the partial-sum buffer and the arg-max kernel, which reads every
-  // logit anyway, puts the rows in their places (in the multiply's own stores the row arithmetic cost
-  // every launch 4 %)
-  float *logits = out_map.rows == 0 ? c->verify_logits : c->P;
-  K_TRY(do_gemm(c, c->lmin, g.H, lm, R, logits, g.V, nullptr));
-  CU_TRY(argmax_rows(LN(c), logits, c->verify_tgt, out_map.rows == 0 ? nullptr : c->verify_logits, out_map, R, g.V));
+  K_TRY(target_logits(c, R, out_map));
   c->phase = PH_VERIFIED;
   return KOALA_OK;
 }
@@ -963,16 +986,17 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
   IngestLens k;
   memset(&k, 0, sizeof(k));
   k.n_parts = n_parts;
-  int longest = 0;
+  int longest = 0, n_max = 1;
   for (int b = 0; b < g.B; ++b) {
     if (len[b] < 0 || len[b] > stride) return fail(c, KOALA_E_INVALID, "prompt %d: %d tokens (stride %d)", b, len[b], stride);
     k.len[b] = len[b];
-    k.count[b] = len[b] - len[b] / n_parts;        // the last of the equal parts is the shorter kind
-    if (k.count[b] > longest) longest = k.count[b];
+    const int last = len[b] / n_parts;             // the last of the equal parts is the shorter kind
+    if (last > g.N) return fail(c, KOALA_E_INVALID, "prompt %d: last part of %d tokens (N = %d)", b, last, g.N);
+    k.count[b] = len[b] - last;
+    if (last > n_max) n_max = last;
+    if (len[b] > longest) longest = len[b];
   }
-  c->phase = PH_INGESTED;
-  c->last_pass = -1;
-  if (longest == 0) return KOALA_OK;
+  if (longest == 0) return fail(c, KOALA_E_INVALID, "empty prompts");
   // Block length: the one that leaves the fewest unused rows (ties: the longest, which re-reads the
   // cached keys least); one block if every prompt is short.
   int q = longest < 128 ? longest : 128;
@@ -981,14 +1005,14 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     int best = 1 << 30;
     for (int t = q; t > 48; --t) {
       int rows = 0;
-      for (int b = 0; b < g.B; ++b) rows += (k.count[b] + t - 1) / t * t;
+      for (int b = 0; b < g.B; ++b) rows += (k.len[b] + t - 1) / t * t;
       if (rows < best) { best = rows; q = t; }
     }
   }
   int fwd = c->ingest_rows / q;
   fwd = fwd > INGEST_MAX_BLOCKS ? INGEST_MAX_BLOCKS : (fwd < 1 ? 1 : fwd);
   int total = 0;
-  for (int b = 0; b < g.B; ++b) total += (k.count[b] + q - 1) / q;
+  for (int b = 0; b < g.B; ++b) total += (k.len[b] + q - 1) / q;
   const int n_fwd = (total + fwd - 1) / fwd;
   fwd = (total + n_fwd - 1) / n_fwd;               // forwards of equal size
   // blocks by position, all sequences side by side: a block comes after the earlier ones of its sequence
@@ -1008,22 +1032,27 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
       keep.src[keep.n] = v * q + at;
       keep.dst[keep.n++] = b * g.N + row;
     }
-    c->ingest_blocks = blk.n;
-    rc = ingest_forward(c, blk, keep, tok, stride);
+    rc = ingest_forward(c, blk, keep, tok, stride, n_max);
     c->ingest_blocks = 0;
     blk.n = 0;
   };
   for (int s0 = 0; s0 < longest; s0 += q)
     for (int b = 0; b < g.B; ++b) {
-      if (s0 >= k.count[b]) continue;
+      if (s0 >= k.len[b]) continue;
       blk.start[blk.n] = s0;
+      blk.last[blk.n] = k.count[b] - s0;
       blk.seq[blk.n] = (int16_t)b;
-      blk.count[blk.n] = (int16_t)(k.count[b] - s0 < q ? k.count[b] - s0 : q);
+      blk.count[blk.n] = (int16_t)(k.len[b] - s0 < q ? k.len[b] - s0 : q);
+      blk.from[blk.n] = (int16_t)blk.n;
       if (++blk.n == fwd) flush();
     }
   flush();
   if (rc != KOALA_OK) return rc;
-  CU_TRY(ingest_commit(LN(c), c->t, k, c->seq_len, g.B));
+  K_TRY(target_logits(c, g.B * n_max, n_max == g.N ? RowMap{0, 0} : RowMap{n_max, g.N}));
+  CU_TRY(ingest_commit(LN(c), c->t, k, tok, stride, c->seq_len, g.B, g.N, c->status));
+  c->phase = PH_VERIFIED;
+  c->last_tree_from_caller = true;
+  c->pend_cap = n_max;
   return KOALA_OK;
 }
 

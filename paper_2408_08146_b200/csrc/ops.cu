@@ -334,6 +334,24 @@ __global__ void cast_rows_kernel(const float *src, const int32_t *row_src,
   }
 }
 
+// Rows of a prompt forward that belong to their sequence's last part, to where a verification leaves them.
+template <typename T>
+__global__ void ingest_last_kernel(const __grid_constant__ IngestBlocks k, const float *hid, float *__restrict__ verify_hid,
+                                   T *__restrict__ xn, T *__restrict__ xn_lo, int N, int n_max, int H) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int v = blockIdx.x, i = blockIdx.y, u = i - k.last[v];
+  if (i >= k.count[v] || u < 0 || u >= n_max) return;
+  const float *src = hid + (size_t)(v * k.q + i) * H;
+  float *to = verify_hid + (size_t)(k.seq[v] * N + u) * H;
+  const size_t at = (size_t)(k.seq[v] * n_max + u) * H;
+  for (int d = threadIdx.x; d < H; d += blockDim.x) {
+    const float x = src[d];
+    to[d] = x;
+    store_operand(xn, xn_lo, at + d, x);
+  }
+}
+
 __global__ void reduce_splits_kernel(SplitIn P, float *__restrict__ Y, int ldy, int ncols) {
   pdl_launch_dependents();
   pdl_wait();
@@ -802,6 +820,12 @@ cudaError_t cast_rows(Launch L, int dtype, const float *src, const int32_t *row_
                       float *dst32, int dst32_stride, int R, int H) {
   DISPATCH_T(dtype, return launch_k(cast_rows_kernel<T>, dim3(R), dim3(256), 0, L.st, L.pdl, src,
                                     row_src, (T *)dst.hi, (T *)dst.lo, dst32, dst32_stride, H);)
+}
+
+cudaError_t ingest_last(Launch L, int dtype, IngestBlocks k, const float *hid, float *verify_hid, Operand xn, int N, int n_max,
+                        int H) {
+  DISPATCH_T(dtype, return launch_k(ingest_last_kernel<T>, dim3(k.n, k.q), dim3(256), 0, L.st, L.pdl, k, hid, verify_hid,
+                                    (T *)xn.hi, (T *)xn.lo, N, n_max, H);)
 }
 
 cudaError_t reduce_splits(Launch L, SplitIn P, float *Y, int ldy, int R, int ncols) {

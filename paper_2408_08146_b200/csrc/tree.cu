@@ -175,7 +175,7 @@ __global__ void plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlo
     p.mask[r * 2] = i >= 63 ? ~0ull : (1ull << (i + 1)) - 1ull;
     p.mask[r * 2 + 1] = i < 64 ? 0ull : (i == 127 ? ~0ull : (1ull << (i - 63)) - 1ull);
     p.row_tok[r] = i < n ? tok[(size_t)b * stride + k.start[v] + i + shift] : 0;
-    p.row_src[r] = (int)r;
+    p.row_src[r] = k.from[v] * k.q + i;
   }
   write_rope(p.rope, r, S + i < 0 ? 0 : S + i, head_dim, rope_base, threadIdx.x, blockDim.x);
 }
@@ -187,9 +187,28 @@ __global__ void ingest_keep_kernel(TreeBufs t, const __grid_constant__ IngestKee
     t.pend_hid[(size_t)k.dst[blockIdx.x] * H + d] = hid[(size_t)k.src[blockIdx.x] * H + d];
 }
 
-__global__ void ingest_commit_kernel(TreeBufs t, const __grid_constant__ IngestLens k, int32_t *seq_len, int B) {
+// block 0: lengths and counters; block 1 + b: sequence b's tree
+__global__ void ingest_commit_kernel(TreeBufs t, const __grid_constant__ IngestLens k, const int32_t *tok, int stride,
+                                     int32_t *seq_len, int B, int N, int *status) {
   pdl_launch_dependents();
   pdl_wait();
+  if (blockIdx.x > 0) {
+    const int b = blockIdx.x - 1;
+    int n = k.len[b] - k.count[b];
+    if (n < 1 || n > N) {
+      if (threadIdx.x == 0 && status) atomicMax(status, E_INVALID);
+      n = n < 1 ? 1 : N;
+    }
+    for (int u = threadIdx.x; u < N; u += blockDim.x) {
+      const bool in = u < n && k.count[b] + u < k.len[b];
+      t.tree_tok[b * N + u] = in ? tok[(size_t)b * stride + k.count[b] + u] : 0;
+      t.tree_parent[b * N + u] = u < n ? u - 1 : -1;
+      t.tree_level[b * N + u] = u < n ? u : 0;
+      t.tree_score[b * N + u] = 0.f;
+    }
+    if (threadIdx.x == 0) t.tree_n[b] = n;
+    return;
+  }
   const int i = threadIdx.x;                  // chain position i + 1
   unsigned long long hits = 0;
   for (int b = 0; b < B; ++b) {
@@ -553,8 +572,9 @@ cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, in
   if (k.n == 0) return cudaSuccess;
   return launch_k(ingest_keep_kernel, dim3(k.n), dim3(256), 0, L.st, L.pdl, t, k, hid, H);
 }
-cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, int32_t *seq_len, int B) {
-  return launch_k(ingest_commit_kernel, dim3(1), dim3(128), 0, L.st, L.pdl, t, k, seq_len, B);
+cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N,
+                          int *status) {
+  return launch_k(ingest_commit_kernel, dim3(1 + B), dim3(128), 0, L.st, L.pdl, t, k, tok, stride, seq_len, B, N, status);
 }
 cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
                         int rows, int head_dim, float rope_base, int S_max, int *status) {
