@@ -209,9 +209,6 @@ struct HeadTab {
   int rows_per_head;
 };
 cudaError_t resblock_update(Launch L, int dtype, float *x, SplitIn P, HeadTab tab, Operand xn, int R, int H);
-// x <- E[tok]; xg <- T(x * g) (not normalised); sumsq as in row_update.  H % 4 == 0.
-cudaError_t embed_update(Launch L, int dtype, const int32_t *tok, const void *E, const void *g, float *x,
-                         Operand xg, float *sumsq, int R, int H, int V);
 cudaError_t row_update(Launch L, int dtype, float *x, SplitIn P, const void *g, Operand xg, float *sumsq,
                        int R, int H);
 // q_out: rotated queries in fp32; q_pair (bf16 only, may be null): the same as a bf16 pair
@@ -322,7 +319,6 @@ cudaError_t selftest_timeout(Launch L, int *status, long long limit_cycles);
 struct TreeBufs {
   int32_t *tree_tok, *tree_parent, *tree_level, *tree_n;
   float *tree_score;
-  uint64_t *tree_anc;      // [B][N][2]
   int32_t *cand_tok, *cand_parent, *cand_level, *cand_rank;
   float *cand_score;
   int32_t *frontier;       // [B][k] candidate ids
@@ -357,14 +353,26 @@ struct PlanBufs {
 };
 cudaError_t tree_from_caller(Launch L, TreeBufs t, const int32_t *tok, const int32_t *parent,
                              const int32_t *n_nodes, int stride, int B, int N, int *status);
-cudaError_t tree_ancestors(Launch L, TreeBufs t, int B, int N);
+// rope_base ^ (-2 i / head_dim), computed once on the host
+struct RopeInv {
+  double v[64];
+};
+// What a plan kernel fills its rows with (E null: nothing; the caller launches that separately).
+struct RowFill {
+  int dtype, H, V;
+  const void *E;                    // embedding
+  const void *gain;                 // target: x <- E[tok], out <- x * gain, sumsq [rows][ROW_SUMS]
+  float *x, *sumsq;
+  const float *feat;                // head: out <- [feat[src] ; E[tok]]
+  Operand out;
+};
 // rows <= N: plan rows per sequence (row b * rows + u is node u of sequence b)
-cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows,
-                        int head_dim, float rope_base, int S_max, int *status);
+cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows, int head_dim,
+                        const RopeInv &inv, const RowFill &fill, int S_max, int *status);
 // Plan of a forward over prompt blocks (chains on top of their own earlier tokens); row_tok = the token
 // `shift` places further on (0: the row's own; 1: the one the draft head pairs with it).
 cudaError_t plan_ingest(Launch L, PlanBufs p, IngestBlocks k, const int32_t *tok, int stride, int shift,
-                        const int32_t *seq_len, int head_dim, float rope_base, int S_max, int *status);
+                        const int32_t *seq_len, int head_dim, const RopeInv &inv, const RowFill &fill, int S_max, int *status);
 // Rows of a forward whose hidden state stays in the pending buffer: pend_hid row dst[i] <- hid row src[i].
 struct IngestKeep {
   int n;
@@ -378,26 +386,25 @@ cudaError_t ingest_last(Launch L, int dtype, IngestBlocks k, const float *hid, f
 // each sequence becomes the chain of its last part
 cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N,
                           int *status);
-cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
-                        int rows, int head_dim, float rope_base, int S_max, int *status);
-cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k,
-                         int pool, int pass, int head_dim, float rope_base, int S_max, int *status);
+cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows, int head_dim,
+                        const RopeInv &inv, const RowFill &fill, int S_max, int *status);
+cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k, int pool, int pass,
+                         int head_dim, const RopeInv &inv, const RowFill &fill, int S_max, int *status);
 cudaError_t expand_dynamic(Launch L, TreeBufs t, int B, int k, int pool, int pass, int D, int N);
 cudaError_t expand_static(Launch L, TreeBufs t, const int32_t *s_parent, const int32_t *s_level,
                           const int32_t *s_rank, int B, int N, int k);
 cudaError_t plan_medusa(Launch L, TreeBufs t, PlanBufs p, int B, int N, int heads);
-cudaError_t accept_walk(Launch L, TreeBufs t, const int32_t *verify_tgt, const float *verify_hid,
-                        const int32_t *forced_len, int32_t *seq_len, int32_t *out_tokens,
-                        int out_stride, int32_t *out_len, int B, int N, int H);
-cudaError_t kv_compact(Launch L, int dtype, TreeBufs t, void *k_cache, void *v_cache, int L_layers,
+cudaError_t accept_walk(Launch L, TreeBufs t, const int32_t *verify_tgt, const int32_t *forced_len, int32_t *seq_len,
+                        int32_t *out_tokens, int out_stride, int32_t *out_len, int B, int N);
+// moves the accepted nodes' cache rows into place and their hidden states to the pending buffer
+cudaError_t kv_compact(Launch L, int dtype, TreeBufs t, const float *hid, void *k_cache, void *v_cache, int L_layers,
                        int B, int N, int n_heads, int head_dim, int S_max);
 
 // sampling.cu : speculative sampling on chain drafts (one row / one chain per sequence)
 cudaError_t sample_rows(Launch L, const float *logits, const float *u, int u_stride, int u_off, int32_t *tok,
                         float *logp, float *probs, int R, int V);
-cudaError_t accept_sampled(Launch L, TreeBufs t, const float *verify_logits, const float *verify_hid,
-                           const float *chain_d, const float *u_accept, const float *u_bonus, int32_t *seq_len,
-                           int32_t *out_tokens, int out_stride, int32_t *out_len, int B, int N, int H, int V, int D,
+cudaError_t accept_sampled(Launch L, TreeBufs t, const float *verify_logits, const float *chain_d, const float *u_accept, const float *u_bonus, int32_t *seq_len,
+                           int32_t *out_tokens, int out_stride, int32_t *out_len, int B, int N, int V, int D,
                            int *status);
 
 }  // namespace koala

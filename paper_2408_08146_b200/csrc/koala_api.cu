@@ -1,5 +1,6 @@
 // C ABI of libkoala: context, workspace carving and the kernel sequence of each step.
 // Host code only enqueues kernels on the caller's stream; it never synchronises.
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -92,6 +93,7 @@ struct koala_ctx {
   Phase phase;
   int last_pass, pend_cap, draft_rows, expand_mode;
   bool last_tree_from_caller;
+  RopeInv rope_inv;
   int ingest_blocks;      // > 0 while koala_ingest enqueues a forward: its groups of rows (else one group per sequence)
   int *host_status;       // pinned
   cudaEvent_t poll_ev;
@@ -221,7 +223,6 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   t.tree_level = w.take<int32_t>(M);
   t.tree_n = w.take<int32_t>(B);
   t.tree_score = w.take<float>(M);
-  t.tree_anc = w.take<uint64_t>((size_t)M * 2);
   t.cand_tok = w.take<int32_t>((size_t)B * pool);
   t.cand_parent = w.take<int32_t>((size_t)B * pool);
   t.cand_level = w.take<int32_t>((size_t)B * pool);
@@ -591,18 +592,30 @@ int fc_few_run(koala_ctx *c, int R) {
   return few_gemm(c, j, 1);
 }
 
-// x and the first target layer's input from the plan's tokens
-int embed_rows(koala_ctx *c, int R) {
+// What the plan kernels fill their rows with; rows that are not whole groups of four go by kernels of their own.
+bool fill_rows(const koala_config &g) { return (g.H % 4) == 0 && g.H <= 8192; }
+RowFill fill_target(koala_ctx *c) {
   const koala_config &g = c->cfg;
-  if ((g.H % 4) == 0 && g.H <= 8192) {
-    // the embedding rows in the deferred form: their RMSNorm scale is applied by the first layer's consumer
-    CU_TRY(embed_update(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, c->sumsq[1],
-                        R, g.H, g.V));
+  return RowFill{g.dtype, g.H, g.V, fill_rows(g) ? c->embed : nullptr, c->layers[0].attn_norm, c->x, c->sumsq[1], nullptr, c->xn};
+}
+RowFill fill_head(koala_ctx *c, const float *feat) {
+  const koala_config &g = c->cfg;
+  return RowFill{g.dtype, g.H, g.V, fill_rows(g) ? c->embed : nullptr, nullptr, nullptr, nullptr, feat, c->cat};
+}
+// After the plan of a target forward: x and the first layer's input stand.
+int target_rows(koala_ctx *c, int R) {
+  const koala_config &g = c->cfg;
+  if (fill_rows(g)) {      // the deferred form: the RMSNorm scale is applied by the first layer's consumer
     c->pending = RowScale{c->sumsq[1], (g.H + 1023) / 1024, 1.f / (float)g.H, g.rms_eps, ROW_SUMS};
-  } else {
-    CU_TRY(embed_norm(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, R, g.H, g.V,
-                      g.rms_eps));
+    return KOALA_OK;
   }
+  CU_TRY(embed_norm(LN(c), g.dtype, c->p.row_tok, c->embed, c->layers[0].attn_norm, c->x, c->xn, R, g.H, g.V, g.rms_eps));
+  return KOALA_OK;
+}
+int head_rows(koala_ctx *c, const float *feat, int R) {
+  const koala_config &g = c->cfg;
+  if (!fill_rows(g))
+    CU_TRY(eagle_concat(LN(c), g.dtype, feat, c->p.row_src, c->p.row_tok, c->embed, c->cat, R, g.H, g.V));
   return KOALA_OK;
 }
 
@@ -629,15 +642,16 @@ int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, 
   const int R = k.n * k.q, Rh = hd.n * hd.q;
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
   c->ingest_blocks = k.n;
-  CU_TRY(plan_ingest(LN(c), c->p, k, tok, stride, 0, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
-  K_TRY(embed_rows(c, R));
+  CU_TRY(plan_ingest(LN(c), c->p, k, tok, stride, 0, c->seq_len, g.head_dim, c->rope_inv, fill_target(c), g.S_max, c->status));
+  K_TRY(target_rows(c, R));
   K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, k.q, c->final_norm, none, c->mx, same, !head && !has_last));
   if (has_last) CU_TRY(ingest_last(LN(c), g.dtype, k, c->mx, c->verify_hid, c->lmin, g.N, n_max, H));
   if (!head) return KOALA_OK;
   CU_TRY(ingest_keep(LN(c), c->t, keep, c->mx, H));
   c->ingest_blocks = hd.n;
-  CU_TRY(plan_ingest(LN(c), c->p, hd, tok, stride, 1, c->seq_len, g.head_dim, g.rope_base, g.S_max, c->status));
-  CU_TRY(eagle_concat(LN(c), g.dtype, c->mx, c->p.row_src, c->p.row_tok, c->embed, c->cat, Rh, H, g.V));
+  CU_TRY(plan_ingest(LN(c), c->p, hd, tok, stride, 1, c->seq_len, g.head_dim, c->rope_inv, fill_head(c, c->mx), g.S_max,
+                     c->status));
+  K_TRY(head_rows(c, c->mx, Rh));
   SplitIn s;
   GemmMats fc{{c->fc_w, nullptr, nullptr}, {H, 0, 0}, 1};
   K_TRY(do_gemm(c, c->cat, 2 * H, fc, Rh, nullptr, 0, &s));
@@ -666,17 +680,15 @@ int draft_eagle(koala_ctx *c, int pass) {
   const int rows = pass == 0 ? c->pend_cap : k;
   const int R = B * rows;
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
-  const float *feat_src;
+  const float *feat = pass == 0 ? c->t.pend_hid : c->feat[(pass - 1) & 1];
   if (pass == 0) {
-    CU_TRY(plan_draft0(LN(c), c->t, c->p, c->seq_len, B, g.N, rows, g.head_dim, g.rope_base, g.S_max,
+    CU_TRY(plan_draft0(LN(c), c->t, c->p, c->seq_len, B, g.N, rows, g.head_dim, c->rope_inv, fill_head(c, feat), g.S_max,
                        c->status));
-    feat_src = c->t.pend_hid;
   } else {
-    CU_TRY(plan_draft_p(LN(c), c->t, c->p, c->seq_len, B, k, c->pool, pass, g.head_dim, g.rope_base,
+    CU_TRY(plan_draft_p(LN(c), c->t, c->p, c->seq_len, B, k, c->pool, pass, g.head_dim, c->rope_inv, fill_head(c, feat),
                         g.S_max, c->status));
-    feat_src = c->feat[(pass - 1) & 1];
   }
-  CU_TRY(eagle_concat(LN(c), g.dtype, feat_src, c->p.row_src, c->p.row_tok, c->embed, c->cat, R, H, g.V));
+  K_TRY(head_rows(c, feat, R));
   SplitIn s;
   GemmMats fc{{c->fc_w, nullptr, nullptr}, {H, 0, 0}, 1};
   const bool few = fc_few(c, R);
@@ -898,6 +910,7 @@ int koala_init(const koala_config *cfg, const koala_weights *w, const koala_stat
   memset(c->t_launches, 0, sizeof(c->t_launches));
   c->last_tree_from_caller = false;
   c->ingest_blocks = 0;
+  for (int i = 0; i < 64; ++i) c->rope_inv.v[i] = std::pow((double)g.rope_base, -2.0 * (double)i / (double)g.head_dim);
   return KOALA_OK;
 }
 
@@ -970,9 +983,9 @@ int koala_verify(koala_ctx *c, const koala_tree *tree) {
   const int R = g.B * rows;
   const RowMap out_map = rows == g.N ? RowMap{0, 0} : RowMap{rows, g.N};
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
-  CU_TRY(tree_ancestors(LN(c), c->t, g.B, g.N));
-  CU_TRY(plan_verify(LN(c), c->t, c->p, c->seq_len, g.B, g.N, rows, g.head_dim, g.rope_base, g.S_max, c->status));
-  K_TRY(embed_rows(c, R));
+  CU_TRY(plan_verify(LN(c), c->t, c->p, c->seq_len, g.B, g.N, rows, g.head_dim, c->rope_inv, fill_target(c), g.S_max,
+                     c->status));
+  K_TRY(target_rows(c, R));
   K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, rows, c->final_norm, c->lmin, c->verify_hid, out_map));
   K_TRY(target_logits(c, R, out_map));
   c->phase = PH_VERIFIED;
@@ -1062,9 +1075,8 @@ int koala_accept(koala_ctx *c, const int32_t *forced_len, int32_t *out_tokens, i
   const koala_config &g = c->cfg;
   if (!out_tokens || !out_len || out_stride < 1) return fail(c, KOALA_E_INVALID, "null outputs");
   if (c->phase != PH_VERIFIED) return fail(c, KOALA_E_STATE, "koala_accept must follow koala_verify");
-  CU_TRY(accept_walk(LN(c), c->t, c->verify_tgt, c->verify_hid, forced_len, c->seq_len, out_tokens,
-                     out_stride, out_len, g.B, g.N, g.H));
-  CU_TRY(kv_compact(LN(c), g.dtype, c->t, c->tk, c->tv, g.L, g.B, g.N, g.n_heads, g.head_dim, g.S_max));
+  CU_TRY(accept_walk(LN(c), c->t, c->verify_tgt, forced_len, c->seq_len, out_tokens, out_stride, out_len, g.B, g.N));
+  CU_TRY(kv_compact(LN(c), g.dtype, c->t, c->verify_hid, c->tk, c->tv, g.L, g.B, g.N, g.n_heads, g.head_dim, g.S_max));
   c->phase = PH_READY;
   c->last_pass = -1;
   return KOALA_OK;
@@ -1087,9 +1099,9 @@ int koala_accept_sampled(koala_ctx *c, const float *u_accept, const float *u_bon
     return fail(c, KOALA_E_STATE, "koala_accept_sampled needs sampled chain drafts (koala_set_sampling)");
   if (c->phase != PH_VERIFIED || c->last_tree_from_caller)
     return fail(c, KOALA_E_STATE, "koala_accept_sampled must follow koala_verify of the drafted chain");
-  CU_TRY(accept_sampled(LN(c), c->t, c->verify_logits, c->verify_hid, c->chain_d, u_accept, u_bonus, c->seq_len,
-                        out_tokens, out_stride, out_len, g.B, g.N, g.H, g.V, g.D, c->status));
-  CU_TRY(kv_compact(LN(c), g.dtype, c->t, c->tk, c->tv, g.L, g.B, g.N, g.n_heads, g.head_dim, g.S_max));
+  CU_TRY(accept_sampled(LN(c), c->t, c->verify_logits, c->chain_d, u_accept, u_bonus, c->seq_len, out_tokens, out_stride,
+                        out_len, g.B, g.N, g.V, g.D, c->status));
+  CU_TRY(kv_compact(LN(c), g.dtype, c->t, c->verify_hid, c->tk, c->tv, g.L, g.B, g.N, g.n_heads, g.head_dim, g.S_max));
   c->phase = PH_READY;
   c->last_pass = -1;
   return KOALA_OK;

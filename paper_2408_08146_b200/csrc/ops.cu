@@ -2,39 +2,14 @@
 // epilogues, RoPE + KV-cache write, SwiGLU, tree-masked attention (CUDA-core version),
 // arg-max and top-k with log-probabilities.  All statistics are fp32.
 #include "common.cuh"
+#include "row_ops.cuh"
 
 namespace koala {
 
 namespace {
 
-__device__ __forceinline__ float block_sum(float v, float *red) {
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  float t = (threadIdx.x < nw) ? red[threadIdx.x] : 0.f;
-  if (w == 0) {
-    t = warp_sum(t);
-    if (lane == 0) red[0] = t;
-  }
-  __syncthreads();
-  t = red[0];
-  __syncthreads();
-  return t;
-}
-
 // (not inlined: an exponential and a division, used a dozen times by kernels that run their instructions once)
 __device__ __noinline__ float silu_f(float v) { return v / (1.f + expf(-v)); }
-
-// Stores v as a matrix-multiply operand.  bf16 operands are kept as a pair hi + lo (lo = the
-// rounding residual of hi, itself rounded to bf16), which carries 16 significant bits into the
-// tensor cores; fp32 operands are exact and have no lo part.
-template <typename T>
-__device__ __forceinline__ void store_operand(T *hi, T *lo, size_t i, float v) {
-  const T h = from_f<T>(v);
-  hi[i] = h;
-  if (lo != nullptr) lo[i] = from_f<T>(v - to_f(h));
-}
 
 // ------------------------------------------------------------------------------- embedding + norm
 template <typename T>
@@ -117,34 +92,6 @@ __device__ __forceinline__ float4 split_sum4(const SplitIn &P, int r, int c, int
   for (int s = 1; s < NS; ++s) { v.x += u[s].x; v.y += u[s].y; v.z += u[s].z; v.w += u[s].w; }
   return v;
 }
-template <typename T> __device__ __forceinline__ float4 load4(const T *p);
-template <> __device__ __forceinline__ float4 load4<float>(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-template <> __device__ __forceinline__ float4 load4<bf16>(const bf16 *p) {
-  const uint2 u = *reinterpret_cast<const uint2 *>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
-  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
-  return make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ void store_operand4(float *hi, float *lo, size_t i, float4 v) {
-  (void)lo;
-  *reinterpret_cast<float4 *>(hi + i) = v;
-}
-__device__ __forceinline__ void store_operand4(bf16 *hi, bf16 *lo, size_t i, float4 v) {
-  const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
-  uint2 u;
-  u.x = *reinterpret_cast<const uint32_t *>(&h0);
-  u.y = *reinterpret_cast<const uint32_t *>(&h1);
-  *reinterpret_cast<uint2 *>(hi + i) = u;
-  if (lo != nullptr) {
-    const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
-    const __nv_bfloat162 l0 = __floats2bfloat162_rn(v.x - f0.x, v.y - f0.y);
-    const __nv_bfloat162 l1 = __floats2bfloat162_rn(v.z - f1.x, v.w - f1.y);
-    u.x = *reinterpret_cast<const uint32_t *>(&l0);
-    u.y = *reinterpret_cast<const uint32_t *>(&l1);
-    *reinterpret_cast<uint2 *>(lo + i) = u;
-  }
-}
-
 template <typename T, int VPT, int NS, bool SK>
 __global__ void __launch_bounds__(1024)
 row_epilogue_vec_kernel(int mode, float *__restrict__ x, SplitIn P, const T *__restrict__ bias,
@@ -251,31 +198,6 @@ resblock_update_kernel(float *__restrict__ x, SplitIn P, HeadTab tab, T *__restr
   store_operand4(xn, xn_lo, (size_t)r * H + c, o);
 }
 
-// The first rows of a forward in the same deferred form: x <- E[tok]; xg <- T(x * g) (not
-// normalised); sumsq[r][chunk] <- partial sums of x^2.  grid (ceil(H / 1024), R), 256 threads.
-template <typename T>
-__global__ void __launch_bounds__(256)
-embed_update_kernel(const int32_t *tok, const T *__restrict__ E, const T *__restrict__ g, float *__restrict__ x,
-                    T *__restrict__ xg, T *__restrict__ xg_lo, float *__restrict__ sumsq, int H, int V) {
-  __shared__ float red[32];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int r = blockIdx.y;
-  const int c = (blockIdx.x * 256 + threadIdx.x) * 4;
-  float ss = 0.f;
-  if (c < H) {
-    int t = tok[r];
-    t = t < 0 ? 0 : (t >= V ? V - 1 : t);
-    const float4 gg = load4<T>(g + c);
-    const float4 o = load4<T>(E + (size_t)t * H + c);
-    *reinterpret_cast<float4 *>(x + (size_t)r * H + c) = o;
-    ss = o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w;
-    store_operand4(xg, xg_lo, (size_t)r * H + c, make_float4(o.x * gg.x, o.y * gg.y, o.z * gg.z, o.w * gg.w));
-  }
-  const float tot = block_sum(ss, red);
-  if (threadIdx.x == 0) sumsq[(size_t)r * ROW_SUMS + blockIdx.x] = tot;
-}
-
 // ------------------------------------------------------------------------------- EAGLE fc input
 template <typename T>
 __global__ void eagle_concat_kernel(const float *feat_src,
@@ -296,27 +218,6 @@ __global__ void eagle_concat_kernel(const float *feat_src,
     cat[base + H + i] = e[i];
     if (cat_lo != nullptr) cat_lo[base + H + i] = from_f<T>(0.f);
   }
-}
-
-// The same with four elements per thread and the row spread over grid.y CTAs (H % 4 == 0): one
-// trip to memory per thread instead of a loop of dependent ones.
-template <typename T>
-__global__ void eagle_concat_vec_kernel(const float *feat_src, const int32_t *row_src, const int32_t *row_tok,
-                                        const T *__restrict__ E, T *__restrict__ cat, T *__restrict__ cat_lo,
-                                        int H, int V) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int r = blockIdx.x;
-  const int i = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
-  if (i >= H) return;
-  const int src = row_src[r];
-  int t = row_tok[r];
-  t = t < 0 ? 0 : (t >= V ? V - 1 : t);
-  const float4 f = *reinterpret_cast<const float4 *>(feat_src + (size_t)src * H + i);
-  const float4 e = load4<T>(E + (size_t)t * H + i);
-  const size_t base = (size_t)r * 2 * H;
-  store_operand4(cat, cat_lo, base + i, f);
-  store_operand4(cat, cat_lo, base + H + i, e);      // the embedding is exact in T: its residual is zero
 }
 
 template <typename T>
@@ -805,12 +706,6 @@ cudaError_t row_epilogue(Launch L, int dtype, int mode, float *x, SplitIn P, con
 
 cudaError_t eagle_concat(Launch L, int dtype, const float *feat_src, const int32_t *row_src,
                          const int32_t *row_tok, const void *E, Operand cat, int R, int H, int V) {
-  if ((H & 3) == 0) {
-    const int threads = 128;
-    DISPATCH_T(dtype, return launch_k(eagle_concat_vec_kernel<T>, dim3(R, (H / 4 + threads - 1) / threads),
-                                      dim3(threads), 0, L.st, L.pdl, feat_src, row_src, row_tok, (const T *)E,
-                                      (T *)cat.hi, (T *)cat.lo, H, V);)
-  }
   DISPATCH_T(dtype, return launch_k(eagle_concat_kernel<T>, dim3(R), dim3(256), 0, L.st, L.pdl,
                                     feat_src, row_src, row_tok, (const T *)E, (T *)cat.hi, (T *)cat.lo, H,
                                     V);)
@@ -838,13 +733,6 @@ cudaError_t resblock_update(Launch L, int dtype, float *x, SplitIn P, HeadTab ta
   if (P.sk_ctas != 0) return cudaErrorInvalidValue;
   FOR_SPLIT(dtype, P, return launch_k(resblock_update_kernel<T, NS>, dim3((H + 1023) / 1024, R), dim3(256), 0, L.st,
                                       L.pdl, x, P, tab, (T *)xn.hi, (T *)xn.lo, H);)
-}
-
-cudaError_t embed_update(Launch L, int dtype, const int32_t *tok, const void *E, const void *g, float *x,
-                         Operand xg, float *sumsq, int R, int H, int V) {
-  if (H % 4 != 0) return cudaErrorInvalidValue;
-  DISPATCH_T(dtype, return launch_k(embed_update_kernel<T>, dim3((H + 1023) / 1024, R), dim3(256), 0, L.st, L.pdl,
-                                    tok, (const T *)E, (const T *)g, x, (T *)xg.hi, (T *)xg.lo, sumsq, H, V);)
 }
 
 cudaError_t row_update(Launch L, int dtype, float *x, SplitIn P, const void *g, Operand xg, float *sumsq,

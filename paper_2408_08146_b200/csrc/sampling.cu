@@ -146,9 +146,9 @@ sample_rows_kernel(const float *logits, const float *u, int u_stride, int u_off,
 
 // grid B, block 1024, dynamic shared memory V floats.
 __global__ void __launch_bounds__(NT)
-accept_sampled_kernel(TreeBufs t, const float *verify_logits, const float *hid, const float *chain_d,
+accept_sampled_kernel(TreeBufs t, const float *verify_logits, const float *chain_d,
                       const float *u_accept, const float *u_bonus, int32_t *seq_len, int32_t *out_tokens,
-                      int out_stride, int32_t *out_len, int N, int H, int V, int D, int *status) {
+                      int out_stride, int32_t *out_len, int N, int V, int D, int *status) {
   extern __shared__ float srow[];
   __shared__ Scratch sc;
   __shared__ int s_tok[128];
@@ -233,11 +233,6 @@ accept_sampled_kernel(TreeBufs t, const float *verify_logits, const float *hid, 
       if (len < n) atomicAdd(&t.alpha_trials[len - 1], 1ull);
     }
   }
-  for (int i = 0; i < len; ++i) {
-    const float *src = hid + ((size_t)b * N + i) * H;
-    float *dst = t.pend_hid + ((size_t)b * N + i) * H;
-    for (int dd = threadIdx.x; dd < H; dd += NT) dst[dd] = src[dd];
-  }
 }
 
 }  // namespace
@@ -252,16 +247,15 @@ cudaError_t sample_rows(Launch L, const float *logits, const float *u, int u_str
                   probs, V);
 }
 
-cudaError_t accept_sampled(Launch L, TreeBufs t, const float *verify_logits, const float *verify_hid,
-                           const float *chain_d, const float *u_accept, const float *u_bonus, int32_t *seq_len,
-                           int32_t *out_tokens, int out_stride, int32_t *out_len, int B, int N, int H, int V, int D,
-                           int *status) {
+cudaError_t accept_sampled(Launch L, TreeBufs t, const float *verify_logits, const float *chain_d,
+                           const float *u_accept, const float *u_bonus, int32_t *seq_len,
+                           int32_t *out_tokens, int out_stride, int32_t *out_len, int B, int N, int V, int D, int *status) {
   static SmemOptIn optin;
   const size_t smem = (size_t)V * sizeof(float);
   cudaError_t e = optin.ensure((const void *)accept_sampled_kernel, smem);
   if (e != cudaSuccess) return e;
-  return launch_k(accept_sampled_kernel, dim3(B), dim3(NT), smem, L.st, L.pdl, t, verify_logits, verify_hid, chain_d,
-                  u_accept, u_bonus, seq_len, out_tokens, out_stride, out_len, N, H, V, D, status);
+  return launch_k(accept_sampled_kernel, dim3(B), dim3(NT), smem, L.st, L.pdl, t, verify_logits, chain_d,
+                  u_accept, u_bonus, seq_len, out_tokens, out_stride, out_len, N, V, D, status);
 }
 
 }  // namespace koala

@@ -2,6 +2,7 @@
 // forwards, dynamic / static expansion, greedy acceptance and KV compaction.
 // One thread block per sequence unless stated otherwise; all of it is latency-bound.
 #include "common.cuh"
+#include "row_ops.cuh"
 
 namespace koala {
 namespace {
@@ -13,15 +14,13 @@ __device__ __forceinline__ void set_bit(uint64_t *m, int bit) {
   else if (bit < 128) m[1] |= 1ull << (bit - 64);
 }
 
-__device__ __forceinline__ void write_rope(float2 *rope, size_t row, int pos, int head_dim,
-                                           float rope_base, int lane, int nthreads) {
-  const int half = head_dim >> 1;
-  for (int i = lane; i < half; i += nthreads) {
-    const double inv = pow((double)rope_base, -2.0 * (double)i / (double)head_dim);
-    double s, c;
-    sincos((double)pos * inv, &s, &c);
-    rope[row * half + i] = make_float2((float)c, (float)s);
-  }
+// `first`: the thread that takes column 0 (the other threads of the block have other work)
+__device__ __forceinline__ void write_rope(float2 *rope, size_t row, int pos, int head_dim, const RopeInv &inv, int first) {
+  const int half = head_dim >> 1, i = (int)threadIdx.x - first;
+  if (i < 0 || i >= half) return;
+  double s, c;
+  sincos((double)pos * inv.v[i], &s, &c);
+  rope[row * half + i] = make_float2((float)c, (float)s);
 }
 
 // ------------------------------------------------------------------------------- caller tree
@@ -66,59 +65,44 @@ __global__ void tree_from_caller_kernel(TreeBufs t, const int32_t *tok,
   }
 }
 
-__global__ void tree_ancestors_kernel(TreeBufs t, int N) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int b = blockIdx.x;
-  const int n = t.tree_n[b];
-  for (int u = threadIdx.x; u < N; u += blockDim.x) {
-    uint64_t m[2] = {0ull, 0ull};
-    if (u < n) {
-      int v = u, steps = 0;
-      while (v >= 0 && steps <= N) {
-        set_bit(m, v);
-        v = t.tree_parent[b * N + v];
-        ++steps;
-      }
-    }
-    t.tree_anc[((size_t)b * N + u) * 2] = m[0];
-    t.tree_anc[((size_t)b * N + u) * 2 + 1] = m[1];
-  }
-}
-
 // ------------------------------------------------------------------------------- plans
-__global__ void plan_verify_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len,
-                                   int N, int rows, int head_dim, float rope_base, int S_max, int *status) {
+// grid (B, rows): a block plans row b * rows + u (node u of sequence b) and fills it with its embedding.
+template <typename T>
+__global__ void __launch_bounds__(ROW_THREADS)
+plan_verify_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len, int N, int rows, int head_dim,
+                   const __grid_constant__ RopeInv inv, const __grid_constant__ RowFill fill, int S_max, int *status) {
+  __shared__ int s_par[128];
   pdl_launch_dependents();
   pdl_wait();
-  const int b = blockIdx.x;
-  const int S = seq_len[b];
-  const int n = t.tree_n[b];
+  const int b = blockIdx.x, u = blockIdx.y;
+  const size_t node = (size_t)b * N + u, r = (size_t)b * rows + u;
+  const int S = seq_len[b], n = t.tree_n[b], tok = t.tree_tok[node], lvl = t.tree_level[node];
+  for (int v = threadIdx.x; v <= u && v < 128; v += blockDim.x) s_par[v] = t.tree_parent[(size_t)b * N + v];
   const bool fits = S >= 0 && S + n <= S_max;
-  if (!fits && threadIdx.x == 0 && status) atomicMax(status, E_CAPACITY);
+  __syncthreads();
   if (threadIdx.x == 0) {
-    p.ctx_len[b] = fits ? S : 0;
-    p.kv_len[b] = fits ? S + n : 0;
-  }
-  {
-    const int u = blockIdx.y;
-    const size_t node = (size_t)b * N + u, r = (size_t)b * rows + u;
-    const int lvl = t.tree_level[node];
-    if (threadIdx.x == 0) {
-      p.pos[r] = S + lvl;
-      p.slot[r] = (fits && u < n) ? S + u : -1;
-      p.mask[r * 2] = t.tree_anc[node * 2];
-      p.mask[r * 2 + 1] = t.tree_anc[node * 2 + 1];
-      p.row_tok[r] = t.tree_tok[node];
+    if (u == 0) {
+      if (!fits && status) atomicMax(status, E_CAPACITY);
+      p.ctx_len[b] = fits ? S : 0;
+      p.kv_len[b] = fits ? S + n : 0;
     }
-    write_rope(p.rope, r, S + lvl, head_dim, rope_base, threadIdx.x, blockDim.x);
+    uint64_t m[2] = {0ull, 0ull};          // the node's ancestors and itself
+    for (int v = u < n ? u : -1, steps = 0; v >= 0 && steps <= N; v = s_par[v], ++steps) set_bit(m, v);
+    p.pos[r] = S + lvl;
+    p.slot[r] = (fits && u < n) ? S + u : -1;
+    p.mask[r * 2] = m[0];
+    p.mask[r * 2 + 1] = m[1];
+    p.row_tok[r] = tok;
   }
+  write_rope(p.rope, r, S + lvl, head_dim, inv, 128);
+  if (fill.E != nullptr) fill_embedding<T>(fill, r, tok);
 }
 
 // Draft pass 0 (EAGLE-style): the positions accepted last, as a chain on top of the head's cache.
-__global__ void plan_draft0_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len,
-                                   int N, int rows, int head_dim, float rope_base, int S_max,
-                                   int *status) {
+template <typename T>
+__global__ void __launch_bounds__(ROW_THREADS)
+plan_draft0_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len, int N, int rows, int head_dim,
+                   const __grid_constant__ RopeInv inv, const __grid_constant__ RowFill fill, int S_max, int *status) {
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
@@ -136,6 +120,7 @@ __global__ void plan_draft0_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_le
     const int i = blockIdx.y;
     const size_t r = (size_t)b * rows + i;
     const int pos = S - n + i;
+    const int tok = (i < n - 1) ? t.pend_tok[b * N + i] : t.root_tok[b], src = b * N + (i < N ? i : N - 1);
     if (threadIdx.x == 0) {
       p.pos[r] = pos;
       p.slot[r] = i < n ? pos : -1;
@@ -144,18 +129,21 @@ __global__ void plan_draft0_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_le
       else { m[0] = ~0ull; m[1] = (i == 127) ? ~0ull : ((1ull << (i - 63)) - 1); }
       p.mask[r * 2] = m[0];
       p.mask[r * 2 + 1] = m[1];
-      p.row_tok[r] = (i < n - 1) ? t.pend_tok[b * N + i] : t.root_tok[b];
-      p.row_src[r] = b * N + (i < N ? i : N - 1);
+      p.row_tok[r] = tok;
+      p.row_src[r] = src;
     }
-    write_rope(p.rope, r, pos < 0 ? 0 : pos, head_dim, rope_base, threadIdx.x, blockDim.x);
+    write_rope(p.rope, r, pos < 0 ? 0 : pos, head_dim, inv, 128);
+    if (fill.E != nullptr) fill_concat<T>(fill, r, src, tok);
   }
 }
 
 // Prompt ingestion: row i of block v is the token at start + i of its sequence, as a chain on top of
 // everything before it.  grid (blocks, q).
-__global__ void plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlocks k, const int32_t *tok, int stride,
-                                   int shift, const int32_t *seq_len, int head_dim, float rope_base, int S_max,
-                                   int *status) {
+template <typename T>
+__global__ void __launch_bounds__(ROW_THREADS)
+plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlocks k, const int32_t *tok, int stride, int shift,
+                   const int32_t *seq_len, int head_dim, const __grid_constant__ RopeInv inv,
+                   const __grid_constant__ RowFill fill, int S_max, int *status) {
   pdl_launch_dependents();
   pdl_wait();
   const int v = blockIdx.x, i = blockIdx.y;
@@ -163,6 +151,7 @@ __global__ void plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlo
   const int S = seq_len[b] + k.start[v];
   const bool fits = S >= 0 && S + n <= S_max;
   const size_t r = (size_t)v * k.q + i;
+  const int tk = i < n ? tok[(size_t)b * stride + k.start[v] + i + shift] : 0, src = k.from[v] * k.q + i;
   if (threadIdx.x == 0) {
     if (i == 0) {
       if (!fits && status) atomicMax(status, E_CAPACITY);
@@ -174,10 +163,13 @@ __global__ void plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlo
     p.slot[r] = (fits && i < n) ? S + i : -1;
     p.mask[r * 2] = i >= 63 ? ~0ull : (1ull << (i + 1)) - 1ull;
     p.mask[r * 2 + 1] = i < 64 ? 0ull : (i == 127 ? ~0ull : (1ull << (i - 63)) - 1ull);
-    p.row_tok[r] = i < n ? tok[(size_t)b * stride + k.start[v] + i + shift] : 0;
-    p.row_src[r] = k.from[v] * k.q + i;
+    p.row_tok[r] = tk;
+    p.row_src[r] = src;
   }
-  write_rope(p.rope, r, S + i < 0 ? 0 : S + i, head_dim, rope_base, threadIdx.x, blockDim.x);
+  write_rope(p.rope, r, S + i < 0 ? 0 : S + i, head_dim, inv, 128);
+  if (fill.E == nullptr) return;
+  if (shift == 0) fill_embedding<T>(fill, r, tk);
+  else fill_concat<T>(fill, r, src, tk);
 }
 
 __global__ void ingest_keep_kernel(TreeBufs t, const __grid_constant__ IngestKeep k, const float *hid, int H) {
@@ -238,9 +230,10 @@ __global__ void plan_medusa_kernel(TreeBufs t, PlanBufs p, int B, int N, int hea
 }
 
 // Draft pass p >= 1: the k frontier candidates of level p.
-__global__ void plan_draft_p_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len,
-                                    int k, int pool, int pass, int head_dim, float rope_base,
-                                    int S_max, int *status) {
+template <typename T>
+__global__ void __launch_bounds__(ROW_THREADS)
+plan_draft_p_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_len, int k, int pool, int pass, int head_dim,
+                    const __grid_constant__ RopeInv inv, const __grid_constant__ RowFill fill, int S_max, int *status) {
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
@@ -255,19 +248,20 @@ __global__ void plan_draft_p_kernel(TreeBufs t, PlanBufs p, const int32_t *seq_l
     const int i = blockIdx.y;
     const size_t r = (size_t)b * k + i;
     const int pos = S + pass - 1;
+    const int cid = t.frontier[b * k + i];
+    const int par = t.cand_parent[(size_t)b * pool + cid], tok = t.cand_tok[(size_t)b * pool + cid];
+    // the parent's predicted feature: row (slot of the parent in the previous pass)
+    const int src = b * k + (par < 0 ? 0 : t.front_row[(size_t)b * pool + par] - (pass - 2) * k);
     if (threadIdx.x == 0) {
-      const int cid = t.frontier[b * k + i];
-      const int par = t.cand_parent[(size_t)b * pool + cid];
       p.pos[r] = pos;
       p.slot[r] = fits ? S + (pass - 1) * k + i : -1;
       p.mask[r * 2] = t.front_mask[r * 2];
       p.mask[r * 2 + 1] = t.front_mask[r * 2 + 1];
-      p.row_tok[r] = t.cand_tok[(size_t)b * pool + cid];
-      // the parent's predicted feature: row (slot of the parent in the previous pass)
-      const int pslot = par < 0 ? 0 : t.front_row[(size_t)b * pool + par] - (pass - 2) * k;
-      p.row_src[r] = b * k + pslot;
+      p.row_tok[r] = tok;
+      p.row_src[r] = src;
     }
-    write_rope(p.rope, r, pos, head_dim, rope_base, threadIdx.x, blockDim.x);
+    write_rope(p.rope, r, pos, head_dim, inv, 128);
+    if (fill.E != nullptr) fill_concat<T>(fill, r, src, tok);
   }
 }
 
@@ -432,11 +426,8 @@ __global__ void expand_static_kernel(TreeBufs t, const int32_t *__restrict__ s_p
 }
 
 // ------------------------------------------------------------------------------- acceptance
-__global__ void accept_walk_kernel(TreeBufs t, const int32_t *tgt,
-                                   const float *hid,
-                                   const int32_t *forced_len, int32_t *seq_len,
-                                   int32_t *out_tokens, int out_stride, int32_t *out_len, int N,
-                                   int H) {
+__global__ void accept_walk_kernel(TreeBufs t, const int32_t *tgt, const int32_t *forced_len, int32_t *seq_len,
+                                   int32_t *out_tokens, int out_stride, int32_t *out_len, int N) {
   __shared__ int s_path[128];
   __shared__ int s_len;
   __shared__ int s_par[128], s_tok[128], s_tgt[128];
@@ -515,30 +506,29 @@ __global__ void accept_walk_kernel(TreeBufs t, const int32_t *tgt,
     t.root_tok[b] = bonus;
     seq_len[b] = S + len;
   }
-  __syncthreads();
-  const int len = s_len;
-  for (int i = 0; i < len; ++i) {
-    const float *src = hid + ((size_t)b * N + s_path[i]) * H;
-    float *dst = t.pend_hid + ((size_t)b * N + i) * H;
-    if ((H & 3) == 0) {
-      for (int d = threadIdx.x; d < (H >> 2); d += blockDim.x)
-        reinterpret_cast<float4 *>(dst)[d] = reinterpret_cast<const float4 *>(src)[d];
-    } else {
-      for (int d = threadIdx.x; d < H; d += blockDim.x) dst[d] = src[d];
-    }
-  }
 }
 
-// grid (layers * 2, B, n_heads), block head_dim: thread d moves column d of the accepted rows,
-// in path order (path[i] >= i and increasing, so a source is never overwritten before it is read).
+// grid (layers * 2 + HID_BLOCKS, B, n_heads), block head_dim: thread d moves column d of the accepted rows,
+// in path order (path[i] >= i and increasing, so a source is never overwritten before it is read).  The
+// last HID_BLOCKS of x copy the accepted rows' hidden states to the pending buffer instead, a head's columns
+// each.  (The acceptance walk's one block per sequence copied them row after row: 160 us after a
+// prompt part of 56 tokens.)
+constexpr int HID_BLOCKS = 8;
 template <typename T>
-__global__ void kv_compact_kernel(TreeBufs t, T *__restrict__ k_cache, T *__restrict__ v_cache,
+__global__ void kv_compact_kernel(TreeBufs t, const float *hid, T *__restrict__ k_cache, T *__restrict__ v_cache, int n_layers,
                                   int B, int N, int n_heads, int head_dim, int S_max) {
   pdl_launch_dependents();
   pdl_wait();
   const int layer = blockIdx.x >> 1, b = blockIdx.y, h = blockIdx.z, d = threadIdx.x;
-  T *cache = (blockIdx.x & 1) ? v_cache : k_cache;
   const int len = t.acc_len[b], S = t.acc_S[b];
+  if (layer >= n_layers) {
+    const int H = n_heads * head_dim, col = h * head_dim + d;
+#pragma unroll 4
+    for (int i = (int)blockIdx.x - 2 * n_layers; i < len; i += HID_BLOCKS)
+      t.pend_hid[((size_t)b * N + i) * H + col] = hid[((size_t)b * N + t.acc_path[b * N + i]) * H + col];
+    return;
+  }
+  T *cache = (blockIdx.x & 1) ? v_cache : k_cache;
   T *base = cache + ((((size_t)layer * B + b) * n_heads + h) * S_max) * head_dim;
   for (int i = 0; i < len; ++i) {
     const int p = t.acc_path[b * N + i];
@@ -555,18 +545,16 @@ cudaError_t tree_from_caller(Launch L, TreeBufs t, const int32_t *tok, const int
   return launch_k(tree_from_caller_kernel, dim3(B), dim3(128), 0, L.st, L.pdl, t, tok, parent,
                   n_nodes, stride, N, status);
 }
-cudaError_t tree_ancestors(Launch L, TreeBufs t, int B, int N) {
-  return launch_k(tree_ancestors_kernel, dim3(B), dim3(128), 0, L.st, L.pdl, t, N);
-}
-cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows,
-                        int head_dim, float rope_base, int S_max, int *status) {
-  return launch_k(plan_verify_kernel, dim3(B, rows), dim3(64), 0, L.st, L.pdl, t, p, seq_len, N, rows, head_dim,
-                  rope_base, S_max, status);
+#define PLAN_DISPATCH(kern, grid, ...)                                                                       \
+  (fill.dtype == 0 ? launch_k(kern<float>, grid, dim3(ROW_THREADS), 0, L.st, L.pdl, __VA_ARGS__)              \
+                   : launch_k(kern<bf16>, grid, dim3(ROW_THREADS), 0, L.st, L.pdl, __VA_ARGS__))
+cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows, int head_dim,
+                        const RopeInv &inv, const RowFill &fill, int S_max, int *status) {
+  return PLAN_DISPATCH(plan_verify_kernel, dim3(B, rows), t, p, seq_len, N, rows, head_dim, inv, fill, S_max, status);
 }
 cudaError_t plan_ingest(Launch L, PlanBufs p, IngestBlocks k, const int32_t *tok, int stride, int shift,
-                        const int32_t *seq_len, int head_dim, float rope_base, int S_max, int *status) {
-  return launch_k(plan_ingest_kernel, dim3(k.n, k.q), dim3(64), 0, L.st, L.pdl, p, k, tok, stride, shift, seq_len,
-                  head_dim, rope_base, S_max, status);
+                        const int32_t *seq_len, int head_dim, const RopeInv &inv, const RowFill &fill, int S_max, int *status) {
+  return PLAN_DISPATCH(plan_ingest_kernel, dim3(k.n, k.q), p, k, tok, stride, shift, seq_len, head_dim, inv, fill, S_max, status);
 }
 cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, int H) {
   if (k.n == 0) return cudaSuccess;
@@ -576,15 +564,13 @@ cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok
                           int *status) {
   return launch_k(ingest_commit_kernel, dim3(1 + B), dim3(128), 0, L.st, L.pdl, t, k, tok, stride, seq_len, B, N, status);
 }
-cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N,
-                        int rows, int head_dim, float rope_base, int S_max, int *status) {
-  return launch_k(plan_draft0_kernel, dim3(B, rows), dim3(64), 0, L.st, L.pdl, t, p, seq_len, N, rows,
-                  head_dim, rope_base, S_max, status);
+cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows, int head_dim,
+                        const RopeInv &inv, const RowFill &fill, int S_max, int *status) {
+  return PLAN_DISPATCH(plan_draft0_kernel, dim3(B, rows), t, p, seq_len, N, rows, head_dim, inv, fill, S_max, status);
 }
-cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k,
-                         int pool, int pass, int head_dim, float rope_base, int S_max, int *status) {
-  return launch_k(plan_draft_p_kernel, dim3(B, k), dim3(64), 0, L.st, L.pdl, t, p, seq_len, k, pool,
-                  pass, head_dim, rope_base, S_max, status);
+cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k, int pool, int pass,
+                         int head_dim, const RopeInv &inv, const RowFill &fill, int S_max, int *status) {
+  return PLAN_DISPATCH(plan_draft_p_kernel, dim3(B, k), t, p, seq_len, k, pool, pass, head_dim, inv, fill, S_max, status);
 }
 cudaError_t plan_medusa(Launch L, TreeBufs t, PlanBufs p, int B, int N, int heads) {
   return launch_k(plan_medusa_kernel, dim3(1), dim3(((heads * B + 31) / 32) * 32), 0, L.st, L.pdl, t, p,
@@ -603,20 +589,19 @@ cudaError_t expand_static(Launch L, TreeBufs t, const int32_t *s_parent, const i
   return launch_k(expand_static_kernel, dim3(B), dim3(128), 0, L.st, L.pdl, t, s_parent, s_level,
                   s_rank, B, N, k);
 }
-cudaError_t accept_walk(Launch L, TreeBufs t, const int32_t *verify_tgt, const float *verify_hid,
-                        const int32_t *forced_len, int32_t *seq_len, int32_t *out_tokens,
-                        int out_stride, int32_t *out_len, int B, int N, int H) {
-  return launch_k(accept_walk_kernel, dim3(B), dim3(256), 0, L.st, L.pdl, t, verify_tgt, verify_hid,
-                  forced_len, seq_len, out_tokens, out_stride, out_len, N, H);
+cudaError_t accept_walk(Launch L, TreeBufs t, const int32_t *verify_tgt, const int32_t *forced_len, int32_t *seq_len,
+                        int32_t *out_tokens, int out_stride, int32_t *out_len, int B, int N) {
+  return launch_k(accept_walk_kernel, dim3(B), dim3(128), 0, L.st, L.pdl, t, verify_tgt, forced_len, seq_len, out_tokens,
+                  out_stride, out_len, N);
 }
-cudaError_t kv_compact(Launch L, int dtype, TreeBufs t, void *k_cache, void *v_cache, int L_layers,
+cudaError_t kv_compact(Launch L, int dtype, TreeBufs t, const float *hid, void *k_cache, void *v_cache, int L_layers,
                        int B, int N, int n_heads, int head_dim, int S_max) {
-  dim3 grid(L_layers * 2, B, n_heads);
+  dim3 grid(L_layers * 2 + HID_BLOCKS, B, n_heads);
   if (dtype == 0)
-    return launch_k(kv_compact_kernel<float>, grid, dim3(head_dim), 0, L.st, L.pdl, t,
-                    (float *)k_cache, (float *)v_cache, B, N, n_heads, head_dim, S_max);
-  return launch_k(kv_compact_kernel<bf16>, grid, dim3(head_dim), 0, L.st, L.pdl, t, (bf16 *)k_cache,
-                  (bf16 *)v_cache, B, N, n_heads, head_dim, S_max);
+    return launch_k(kv_compact_kernel<float>, grid, dim3(head_dim), 0, L.st, L.pdl, t, hid,
+                    (float *)k_cache, (float *)v_cache, L_layers, B, N, n_heads, head_dim, S_max);
+  return launch_k(kv_compact_kernel<bf16>, grid, dim3(head_dim), 0, L.st, L.pdl, t, hid, (bf16 *)k_cache,
+                  (bf16 *)v_cache, L_layers, B, N, n_heads, head_dim, S_max);
 }
 
 }  // namespace koala
