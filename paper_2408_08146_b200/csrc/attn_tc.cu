@@ -265,6 +265,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       const int y0 = (P.plan.cache_of(b) * P.n_heads + h) * P.S_max;
+      const uint64_t policy = stream_policy(P.plan.seq == nullptr);     // prompt blocks share their sequence's keys
       bool ok = true;
       int issued = 0;
       // K's buffer is free once S has been computed, V's only after P V: K runs ahead
@@ -280,8 +281,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         unsigned char *dst = sm + (v ? LY::V : LY::K) + s * 2 * SUB;
         const int y = y0 + (tile_lo + t) * TK;
         const CUtensorMap *map = v ? &tmV : &tmK;
-        tma_load_2d(map, full, dst, 0, y);
-        tma_load_2d(map, full, dst + SUB, 64, y);
+        tma_load_2d_hint(map, full, dst, 0, y, policy);
+        tma_load_2d_hint(map, full, dst + SUB, 64, y, policy);
         issued = i + 1;
       }
       if (!ok) {
