@@ -7,7 +7,7 @@
 // K = 16, both operands K-major in shared memory with the 128-byte swizzle that TMA writes.
 // The fp32 accumulator [128 x tokens] lives in tensor memory.  Warp 0 streams weight and
 // activation tiles with TMA through a ring of shared-memory stages (mbarrier full/empty pairs),
-// warp 1 issues the MMAs, eight or sixteen epilogue warps read the accumulator back (tcgen05.ld)
+// warp 1 issues the MMAs, four or sixteen epilogue warps read the accumulator back (tcgen05.ld)
 // and store it.
 // The weight stream does not depend on the previous kernel, so under programmatic dependent
 // launch the first stages are requested before waiting for the producer of X.
@@ -43,7 +43,7 @@ constexpr int BM = 128;             // weight rows per CTA (MMA M)
 constexpr int BK = 64;              // K elements per stage: 128 bytes of bf16 = one swizzle row
 constexpr int UMMA_K = 16;
 constexpr int THREADS_WIDE = 576;   // most threads a launch uses: producer warp, MMA warp and sixteen epilogue
-                                    // warps (256-row weight tiles); 128-row tiles launch 320 threads
+                                    // warps (256-row weight tiles); 128-row tiles launch 192 threads
 constexpr int W_STAGE_BYTES = BM * BK * 2;
 constexpr int E_TIMEOUT = 6;
 constexpr int MAX_STAGES = 12;
@@ -817,7 +817,7 @@ bool tc_supported(const GemmMats &m, int K_in) {
 // every split keeps at least 8 K-blocks and the fp32 partial sums written and re-read
 // (split x tokens x 4 bytes per output) stay below about half of the weight bytes.
 static int split_cap(int kblocks, int tokens) {
-  int s = 8;
+  int s = 12;
   const int by_k = kblocks / 8;
   const int by_traffic = (kblocks * 64) / (g_tune_traffic_div * (tokens > 0 ? tokens : 1));
   if (s > by_k) s = by_k;
@@ -1095,10 +1095,10 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   }
   // Epilogue warps per 32 accumulator lanes.  256-row tiles keep one accumulator set, so the MMAs
   // of a CTA's next tile wait for the epilogue: sixteen warps (13B-shaped verification of 256 rows:
-  // 18.3 ms with four, 16.8 with eight, 16.3 with sixteen).  128-row tiles: eight warps (per 7B
-  // verification, against four: 16 to 48 rows 2-3 % faster, 60 and 64 rows 1 %, 100 rows 0.8 %,
-  // 80 rows 0.5 % slower; the draft passes 2 % faster).
-  int groups = wide ? 4 : 2;
+  // 18.3 ms with four, 16.8 with eight, 16.3 with sixteen).  128-row tiles: four warps (eight: 7B
+  // Medusa iteration of 64 rows + 1.5 %, EAGLE iteration + 0.8 %, sampled chain + 1.5 %, one-token
+  // step + 0.1 %; sixteen + 20 %).
+  int groups = wide ? 4 : 1;
   const int forced = wide ? g_tune_epi : g_tune_epi_narrow;
   if (forced == 1 || forced == 2 || forced == 4) groups = forced;
   auto go = [&](auto *kern) {
