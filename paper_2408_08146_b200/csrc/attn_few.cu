@@ -68,14 +68,14 @@ __device__ __forceinline__ float ld_cluster(uint32_t local_addr, uint32_t rank) 
 template <typename T, int DH, int RT>
 __global__ void __launch_bounds__(WARPS * 32, RT <= 2 ? 2 : 1)
 tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *__restrict__ out, T *__restrict__ out_lo,
-                     int rows_per_seq, int n_heads, int S_max) {
+                     int rows_per_seq, int n_heads, int S_max, int early) {
   constexpr int E = DH / 16;                               // dims of a lane
   constexpr int PSTRIDE = DH + 4;                          // floats of a partial: O[DH], m, l, pad (16-byte rows)
   __shared__ __align__(16) float s_q[RT][DH];
   __shared__ __align__(16) float s_o[2 * WARPS][RT][PSTRIDE];
   __shared__ __align__(16) float s_c[RT][PSTRIDE];         // this chunk's result, read by the cluster
   pdl_launch_dependents();
-  pdl_wait();
+  if (!early) pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hf = lane >> 4, d0 = (lane & 15) * E;
   const int H = n_heads * DH;
   const int c = (int)blockIdx.x, chunks = (int)gridDim.x;
@@ -99,7 +99,15 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
       vn[j].load(vb + (size_t)key * DH, in);
     }
   };
-  load(t_lo);                                            // first of all: the longest way
+  if (early) {
+    // a tile of nothing but context does not depend on the kernel before
+    const bool context = (t_lo + 1) * TILE <= ctx;
+    if (context) load(t_lo);
+    pdl_wait();
+    if (!context) load(t_lo);
+  } else {
+    load(t_lo);                                          // first of all: the longest way
+  }
   uint64_t mk0[RT], mk1[RT];
   unsigned row_ok = 0;
 #pragma unroll
@@ -272,7 +280,7 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
 // fill every GPC, hence seven eighths), and at least `min_keys` of capacity per chunk: two tiles, eight
 // in the small configurations, where the cluster's two barriers cost more than a few tiles.
 cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
-                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms) {
+                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early) {
   if (rows_per_seq < 1 || (head_dim != 64 && head_dim != 128)) return cudaErrorInvalidValue;
   const bool bf = dtype != 0;
   auto go = [&](auto tag, auto dh, auto rt) -> cudaError_t {
@@ -297,7 +305,7 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
     cfg.numAttrs = chunks > 1 ? 2 : 1;
     ++g_launches;
     return cudaLaunchKernelEx(&cfg, tree_attn_few_kernel<T, DH, RT>, q, (const T *)k_cache, (const T *)v_cache, plan,
-                              (T *)out.hi, (T *)out.lo, rows_per_seq, n_heads, S_max);
+                              (T *)out.hi, (T *)out.lo, rows_per_seq, n_heads, S_max, early ? 1 : 0);
   };
   std::integral_constant<int, 64> d64;
   std::integral_constant<int, 128> d128;

@@ -89,10 +89,10 @@ constexpr int MSTRIDE = DH + 4;          // floats per merged row in shared memo
 __global__ void __launch_bounds__(128)
 tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
                      RowPlan plan, bf16 *__restrict__ out, bf16 *__restrict__ out_lo,
-                     int rows_per_seq, int n_heads, int S_max, int chunks) {
+                     int rows_per_seq, int n_heads, int S_max, int chunks, int early) {
   extern __shared__ __align__(1024) unsigned char smem[];     // [NST][K tile | V tile]
   pdl_launch_dependents();
-  pdl_wait();
+  if (!early) pdl_wait();
   const int c = blockIdx.x, rg = blockIdx.y;
   const int b = blockIdx.z / n_heads, h = blockIdx.z % n_heads;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -122,6 +122,17 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
     }
   };
 
+  if (early) {
+    // tiles of nothing but context do not depend on the kernel before
+    bool waited = false;
+#pragma unroll 1
+    for (int sidx = 0; sidx < NST - 1; ++sidx) {
+      if (!waited && (tile_lo + sidx + 1) * TILE > ctx) { pdl_wait(); waited = true; }
+      if (tile_lo + sidx < tile_hi) load_tile(tile_lo + sidx, sidx);
+      cp_async_commit();
+    }
+    if (!waited) pdl_wait();
+  }
   const int i0 = rg * 16 + g, i1 = i0 + 8;
   const bool in0 = i0 < rows_per_seq, in1 = i1 < rows_per_seq;
   const int r0 = b * rows_per_seq + (in0 ? i0 : 0), r1 = b * rows_per_seq + (in1 ? i1 : 0);
@@ -142,10 +153,12 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
     }
   }
 
-#pragma unroll
-  for (int sidx = 0; sidx < NST - 1; ++sidx) {
-    if (tile_lo + sidx < tile_hi) load_tile(tile_lo + sidx, sidx);
-    cp_async_commit();
+  if (!early) {
+#pragma unroll 1
+    for (int sidx = 0; sidx < NST - 1; ++sidx) {
+      if (tile_lo + sidx < tile_hi) load_tile(tile_lo + sidx, sidx);
+      cp_async_commit();
+    }
   }
 
   const bool ok0 = in0 && slot0 >= 0, ok1 = in1 && slot1 >= 0;
@@ -401,7 +414,7 @@ int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms
 }
 
 cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, const void *v_cache,
-                               RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks) {
+                               RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks, bool early) {
   static SmemOptIn optin;
   const size_t smem = (size_t)NST * 2 * TILE_BYTES;
   static_assert((size_t)5 * 16 * MSTRIDE * sizeof(float) <= (size_t)NST * 2 * TILE_BYTES, "merge buffer fits");
@@ -427,7 +440,7 @@ cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, co
   cfg.numAttrs = chunks > 1 ? 2 : 1;
   ++g_launches;
   return cudaLaunchKernelEx(&cfg, tree_attn_mma_kernel, q, (const bf16 *)k_cache, (const bf16 *)v_cache, plan,
-                            (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks);
+                            (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks, early ? 1 : 0);
 }
 
 }  // namespace koala

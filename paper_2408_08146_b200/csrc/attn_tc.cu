@@ -130,6 +130,7 @@ struct AttnParams {
   int rows_per_seq, n_heads, S_max, chunks, chunk_bits;
   int longest_first;       // 1: grid slot y / n_heads takes the sequence with that rank in descending cache length
   unsigned smem_bytes;     // dynamic shared memory of the launch
+  int early;               // 1: the plan and the cached context may be read before the dependency wait
   int dry_pass;            // 1: the row warps make a dry pass over the tile loop body before the dependency wait
   int *status;
 };
@@ -207,8 +208,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   // comes after the dependency wait in read_plan().  The row warps call it inside their tile loop,
   // after a dry pass over the loop body (see there); the other threads here.
   int ctx = 0, kv_len = 0, tile_lo = 0, T = 0;
-  auto read_plan = [&]() {
-    pdl_wait();
+  auto read_plan = [&](bool wait) {
+    if (wait) pdl_wait();
     if (P.longest_first) {
       // More CTAs than SMs: the CTAs beyond the first round start when the first ones finish, so the
       // sequences are taken longest first and the late CTAs belong to the shortest one.  Lane l holds
@@ -236,8 +237,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   const int row = DUP ? warp * 16 + (lane & 15) : warp * 32 + lane;
   const bool row_warp = warp < 4 && warp < n_q;
   const bool row_in = row_warp && row < P.rows_per_seq;
-  if (!row_warp) read_plan();
-  if (threadIdx.x == 128) {        // warp 4 lane 0: the queries do not depend on the plan
+  if (!row_warp) read_plan(!P.early);
+  auto load_q = [&]() {            // warp 4 lane 0, after the dependency wait
     if (DUP) {
       // of every 32 MMA rows the first 16 are the values of 16 queries, the other 16 their residuals
       mbar_expect_tx(&q_full, (uint32_t)(2 * QSUB));
@@ -256,7 +257,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
                     h * DH + 64 * hb, b * P.rows_per_seq + 64 * rh);
       }
     }
-  }
+  };
   int r_glob = 0;
   float m_run = -INFINITY, l_run = 0.f;
   bool have_o = false;             // this warp's O in tensor memory is complete (warp-uniform)
@@ -269,14 +270,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       bool ok = true;
       int issued = 0;
       // K's buffer is free once S has been computed, V's only after P V: K runs ahead
-#pragma unroll 1
-      for (int i = 0; i < 2 * T; ++i) {
+      auto load_kv = [&](int i) {
         const int t = i >> 1, v = i & 1, s = t % NST;
         uint64_t *full = v ? &v_full[s] : &k_full[s];
-        if (t >= NST) {
-          ok = mbar_wait(v ? &v_empty[s] : &k_empty[s], (uint32_t)((t / NST) - 1) & 1u);
-          if (!ok) break;
-        }
         mbar_expect_tx(full, (uint32_t)(2 * SUB));
         unsigned char *dst = sm + (v ? LY::V : LY::K) + s * 2 * SUB;
         const int y = y0 + (tile_lo + t) * TK;
@@ -284,7 +280,22 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         tma_load_2d_hint(map, full, dst, 0, y, policy);
         tma_load_2d_hint(map, full, dst + SUB, 64, y, policy);
         issued = i + 1;
+      };
+      // before the wait: the first tiles, as far as they hold nothing but context
+      const int n_pre = P.early ? 2 * min(min(NST, T), max(0, ctx / TK - tile_lo)) : 0;
+      bool waited = !P.early;
+      if (waited) load_q();
+#pragma unroll 1
+      for (int i = 0; i < 2 * T; ++i) {
+        if (!waited && i == n_pre) { waited = true; pdl_wait(); load_q(); }
+        const int t = i >> 1;
+        if (t >= NST) {
+          ok = mbar_wait((i & 1) ? &v_empty[t % NST] : &k_empty[t % NST], (uint32_t)((t / NST) - 1) & 1u);
+          if (!ok) break;
+        }
+        load_kv(i);
       }
+      if (!waited) { pdl_wait(); load_q(); }
       if (!ok) {
         atomicExch(&s_error, 1);
         // let the copies already requested land before the block's memory goes away
@@ -370,7 +381,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
     int T_run = 1;
     for (int t = P.dry_pass ? -1 : 0; t < T_run; ++t) {
       if (t == 0) {
-        read_plan();
+        read_plan(true);
         T_run = T;
         r_glob = b * P.rows_per_seq + (row_in ? row : 0);    // also needed by a chunk without tiles: it still merges and stores its dims
         if (T == 0) break;
@@ -670,7 +681,7 @@ bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max) {
 
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
                               RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
-                              int *status) {
+                              bool early, int *status) {
   const bool dup = rows_per_seq <= 64;
   if (chunks != 1 && chunks != 2 && chunks != 4 && chunks != 8) return cudaErrorInvalidValue;
   if (q_pair.hi == nullptr || q_pair.lo == nullptr) return cudaErrorInvalidValue;
@@ -684,7 +695,7 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
     return cudaErrorInvalidValue;
   const int longest_first = (B > 1 && B <= 32 && (long long)chunks * B * n_heads > (dup ? 2 : 1) * tc_num_sms()) ? 1 : 0;
   AttnParams P{plan, (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks,
-               31 - __builtin_clz((unsigned)chunks), longest_first, 0u, g_attn_tc_dry_pass, status};
+               31 - __builtin_clz((unsigned)chunks), longest_first, 0u, early ? 1 : 0, g_attn_tc_dry_pass, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, n_heads * B);
   cfg.blockDim = dim3(THREADS);

@@ -224,16 +224,19 @@ cudaError_t cast_rows(Launch L, int dtype, const float *src, const int32_t *row_
                       float *dst32, int dst32_stride, int R, int H);
 cudaError_t reduce_splits(Launch L, SplitIn P, float *Y, int ldy, int R, int ncols);
 
+// Attention kernels, `early`: the kernel before is rope_kv_write's, so the plan and the cached context may be read
+// before the dependency wait.
 // attn_mma.cu : bf16 caches, head_dim 128, tensor cores, split over key chunks
 int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms);
 cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, const void *v_cache,
-                               RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks);
+                               RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int S_max, int chunks,
+                               bool early);
 
 // attn_few.cu : any dtype, head_dim 64 or 128, on CUDA cores; where the tensor-core kernels apply, up to ATTN_FEW_ROWS
 // rows per sequence
 constexpr int ATTN_FEW_ROWS = 4;
 cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
-                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms);
+                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early);
 
 // attn_tc.cu : the same on tcgen05 tensor cores, all rows of a sequence in one CTA, key chunks as a cluster;
 // the queries come as the bf16 pair written by rope_kv_write ([q_rows_alloc][n_heads * 128] each)
@@ -241,7 +244,7 @@ int attn_tc_chunks(int B, int n_heads, int S_max, int num_sms);
 bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max);
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
                               RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,
-                              int *status);
+                              bool early, int *status);
 
 // gemm_few.cu : fp32 multiplies of latency-bound sizes together with the row-wise steps around them
 enum { FEW_ROPE = 1, FEW_SWIGLU = 2, FEW_RESIDUAL = 3 };

@@ -326,20 +326,20 @@ int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct,
 
 // Tree-masked attention of one layer over R rows: reads the rotated queries (fp32 and pair) and the
 // cache, writes the O projection's operand pair.
-int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq) {
+int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq, bool early = false) {
   const koala_config &g = c->cfg;
   const int groups = c->ingest_blocks > 0 ? c->ingest_blocks : g.B;
   const int ta = time_begin(c, KOALA_CLS_ATTENTION, 0);
   if (c->use_tc && g.dtype == KOALA_BF16 && c->qpair.lo != nullptr &&
       attn_tc_supported(rows_per_seq, g.head_dim, g.S_max)) {
     CU_TRY(tree_attention_tc(LN(c), c->qpair, c->Mp, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups,
-                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, NUM_SMS), c->status));
+                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, NUM_SMS), early, c->status));
   } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq > ATTN_FEW_ROWS && rows_per_seq <= 128) {
     CU_TRY(tree_attention_mma(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
-                              g.S_max, attn_mma_chunks(groups, g.n_heads, rows_per_seq, g.S_max, NUM_SMS)));
+                              g.S_max, attn_mma_chunks(groups, g.n_heads, rows_per_seq, g.S_max, NUM_SMS), early));
   } else {
     CU_TRY(tree_attention_few(LN(c), g.dtype, c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
-                              g.head_dim, g.S_max, NUM_SMS));
+                              g.head_dim, g.S_max, NUM_SMS, early));
   }
   time_end(c, ta);
   return KOALA_OK;
@@ -368,7 +368,8 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
                        g.head_dim, g.S_max));
   c->pending = none;
   if (kv_only) return KOALA_OK;
-  K_TRY(run_attention(c, kc, vc, R, rows_per_seq));
+  // (the context of a prompt block includes rows of the same forward: nothing of it may be read early)
+  K_TRY(run_attention(c, kc, vc, R, rows_per_seq, c->ingest_blocks == 0));
   GemmMats o{{w.wo, nullptr, nullptr}, {H, 0, 0}, 1};
   K_TRY(do_gemm(c, c->attn_out, H, o, R, nullptr, 0, &s));
   RowScale ffn = none;
