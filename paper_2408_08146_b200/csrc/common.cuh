@@ -240,7 +240,7 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
 
 // attn_tc.cu : the same on tcgen05 tensor cores, all rows of a sequence in one CTA, key chunks as a cluster;
 // the queries come as the bf16 pair written by rope_kv_write ([q_rows_alloc][n_heads * 128] each)
-int attn_tc_chunks(int B, int n_heads, int S_max, int num_sms);
+int attn_tc_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms);
 bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max);
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
                               RowPlan plan, Operand out, int rows_per_seq, int B, int cache_seqs, int n_heads, int S_max, int chunks,

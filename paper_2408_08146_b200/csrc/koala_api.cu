@@ -333,7 +333,7 @@ int run_attention(koala_ctx *c, void *kc, void *vc, int R, int rows_per_seq, boo
   if (c->use_tc && g.dtype == KOALA_BF16 && c->qpair.lo != nullptr &&
       attn_tc_supported(rows_per_seq, g.head_dim, g.S_max)) {
     CU_TRY(tree_attention_tc(LN(c), c->qpair, c->Mp, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups,
-                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, g.S_max, NUM_SMS), early, c->status));
+                             g.B, g.n_heads, g.S_max, attn_tc_chunks(groups, g.n_heads, rows_per_seq, g.S_max, NUM_SMS), early, c->status));
   } else if (c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && rows_per_seq > ATTN_FEW_ROWS && rows_per_seq <= 128) {
     CU_TRY(tree_attention_mma(LN(c), c->qbuf, kc, vc, row_plan(c), c->attn_out, rows_per_seq, groups, g.n_heads,
                               g.S_max, attn_mma_chunks(groups, g.n_heads, rows_per_seq, g.S_max, NUM_SMS), early));
