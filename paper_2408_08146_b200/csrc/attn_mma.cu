@@ -82,7 +82,8 @@ __device__ __forceinline__ float2 ld_cluster2(uint32_t local_addr, uint32_t rank
 // grid (chunks, row groups of 16, n_heads * B); block = 4 warps.  All four warps serve the same
 // 16 query rows; warp w takes keys [16w, 16w + 16) of every 64-key tile and keeps its own running
 // (max, sum, O); the four are merged through shared memory at the end.  With chunks == 1 the CTA
-// writes the normalised output operand itself; otherwise it writes an unnormalised partial.
+// writes the normalised output operand itself; otherwise the chunks form a cluster and every CTA
+// finishes its share of the output from all of their merged parts.
 constexpr int NST = 3;                   // cp.async stages
 constexpr int MSTRIDE = DH + 4;          // floats per merged row in shared memory (keeps 16-byte alignment)
 

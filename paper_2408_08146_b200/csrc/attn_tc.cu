@@ -14,14 +14,13 @@
 // t into P (two S buffers in tensor memory, two P buffers in shared memory).  Q and P enter the
 // MMAs as bf16 pairs (value + rounding residual: two accumulating MMAs), so only the cached K and V
 // carry bf16 rounding.  Q (written as a pair by the rotary-embedding kernel) and the K/V tiles
-// arrive by TMA with the 128-byte swizzle, K/V in a three-stage ring.
+// arrive by TMA with the 128-byte swizzle, K/V in a ring of two (up to 64 rows) or three stages.
 // Warps 0..3 own the rows, warp 4 lane 0 issues the copies, warp 5 lane 0 the MMAs.
-// With several chunks the CTAs of one (head, sequence) form a thread-block cluster: every CTA
-// pushes, into each peer's shared memory, that peer's slice of the head dimension of its
-// unnormalised (O, m, l); after a cluster barrier every CTA merges its slice over the chunks in
-// chunk order from its own shared memory and writes it as a matrix-multiply operand pair.  (The
-// receive buffer reuses the K/V ring, so a first cluster barrier makes sure that every peer is done
-// with its tiles.)
+// With several chunks the CTAs of one (head, sequence) form a thread-block cluster: every CTA leaves
+// its unnormalised (O, m, l) in its own shared memory (the K/V ring is free by then); after a cluster
+// barrier every CTA reads its slice of the head dimension from all of them, merges it in chunk order
+// and writes it as a matrix-multiply operand pair; a second barrier keeps the CTAs alive until all
+// have read.
 // The mask is: slots below ctx_len visible to every row; slot ctx_len + j visible to a row iff
 // bit j of its 128-bit mask; slots from kv_len on invisible.
 // Every wait is bounded: on expiry the kernel records a timeout in *status and returns.
