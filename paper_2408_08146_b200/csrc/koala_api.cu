@@ -183,7 +183,7 @@ size_t carve(koala_ctx *c, const koala_config &cfg, unsigned char *base) {
   c->x = w.take<float>((size_t)Mp * H);
   c->qbuf = w.take<float>((size_t)Mp * H);
   c->p_floats = (size_t)(MAX_SPLIT * Mt > INGEST_SPLIT * wide ? MAX_SPLIT * Mt : INGEST_SPLIT * wide) * pcols;
-  if (B > 1 && c->p_floats < (size_t)M * V) c->p_floats = (size_t)M * V;       // a short tree's logits pass through it
+  if (B > 1 && c->p_floats < (size_t)M * V) c->p_floats = (size_t)M * V;       // a batch's short trees' logits pass through it
   c->P = w.take<float>(c->p_floats);
   c->verify_logits = w.take<float>((size_t)Mt * V);
   c->draft_logits = w.take<float>((size_t)(draft_rows + 16) * V);
@@ -663,9 +663,16 @@ int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, 
   return run_layers(c, c->draft_layers, g.K, c->dk, c->dv, Rh, k.q, nullptr, none, nullptr, same, true);
 }
 
+// Node rows of a forward over `rows` rows per sequence (with one sequence they are where they belong already).
+RowMap node_rows(const koala_config &g, int rows) {
+  return g.B == 1 || rows == g.N ? RowMap{0, 0} : RowMap{rows, g.N};
+}
+
 // Logits and greedy tokens of R verified rows in c->lmin; row r is node row out_map(r) of the buffers.
 int target_logits(koala_ctx *c, int R, RowMap out_map) {
   const koala_config &g = c->cfg;
+  if (out_map.rows != 0 && (size_t)R * g.V > c->p_floats)      // carve() makes room for B * N of them
+    return fail(c, KOALA_E_CAPACITY, "%d rows of logits do not fit in the partial-sum buffer", R);
   GemmMats lm{{c->lm_head, nullptr, nullptr}, {g.V, 0, 0}, 1};
   // spread rows: the product goes through the partial-sum buffer and the arg-max kernel, which reads every
   // logit anyway, puts the rows in their places (in the multiply's own stores the row arithmetic cost
@@ -983,7 +990,7 @@ int koala_verify(koala_ctx *c, const koala_tree *tree) {
   // steps of four sequences on an engine for 64-node trees ran all 256 rows before: 8.1 -> 3.7 ms.)
   const int rows = tree ? tree->n_max : g.N;
   const int R = g.B * rows;
-  const RowMap out_map = rows == g.N ? RowMap{0, 0} : RowMap{rows, g.N};
+  const RowMap out_map = node_rows(g, rows);
   c->pending = RowScale{nullptr, 0, 0.f, 0.f};
   CU_TRY(plan_verify(LN(c), c->t, c->p, c->seq_len, g.B, g.N, rows, g.head_dim, c->rope_inv, fill_target(c), g.S_max,
                      c->status));
@@ -1063,7 +1070,7 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     }
   flush();
   if (rc != KOALA_OK) return rc;
-  K_TRY(target_logits(c, g.B * n_max, n_max == g.N ? RowMap{0, 0} : RowMap{n_max, g.N}));
+  K_TRY(target_logits(c, g.B * n_max, node_rows(g, n_max)));
   CU_TRY(ingest_commit(LN(c), c->t, k, tok, stride, c->seq_len, g.B, g.N, c->status));
   c->phase = PH_VERIFIED;
   c->last_tree_from_caller = true;

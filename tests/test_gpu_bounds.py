@@ -1,0 +1,49 @@
+"""Sizes and arguments at the edge of what a call may be given: models whose vocabulary is wide against
+their hidden size, and caller trees and prompts that do not keep to their own bounds."""
+import numpy as np
+import pytest
+import torch
+
+from tests.harness import make_pair
+from tests.parity import assert_close, check_argmax
+from workloads import T7_EAGLE, TINY_EAGLE, reduced
+from workloads.generate import prompts
+
+pytestmark = pytest.mark.gpu
+
+
+def _to(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to("cuda:0")
+
+
+# (N - 1) rows of logits take more floats than the partial sums of any multiply of these models
+WIDE = {"fp32": TINY_EAGLE.with_(N=15, V=40000, S_max=64, prompt_len=20, seed=41),
+        "bf16": reduced(T7_EAGLE, 1, K=1, H=512, n_heads=4, F=1376, V=50000, N=64, S_max=256, prompt_len=100, seed=42)}
+
+
+@pytest.mark.parametrize("model", WIDE)
+@pytest.mark.parametrize("B", [1, 2])
+def test_short_trees_and_prompts_under_a_wide_vocabulary(model, B):
+    cfg = WIDE[model].with_(B=B)
+    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float64 if model == "fp32" else np.float32, cache_host=model == "fp32")
+    N, n_max = cfg.N, cfg.N - 1
+    pr = prompts(cfg)
+    eng.prefill(pr, n_max)                       # the last parts are shorter than N
+    orc.prefill(pr, n_max)
+
+    def check(n, what):
+        bufs = eng.buffers()
+        for b in range(B):
+            assert_close(bufs["verify_logits"][b * N:b * N + n].cpu().numpy(), orc.verify_logits[b][:n], cfg.dtype, f"{what} {b}")
+            check_argmax(bufs["verify_tgt"][b * N:b * N + n].cpu().numpy(), orc.verify_logits[b], f"{what} {b}")
+
+    check(len(np.array_split(pr[0], -(-len(pr[0]) // n_max))[-1]), "prompt")
+    rng = np.random.default_rng(n_max)
+    tok = rng.integers(0, cfg.V, (B, n_max))
+    par = np.asarray([[-1] + [int(rng.integers(0, u)) for u in range(1, n_max)] for _ in range(B)])
+    eng.koala_verify((_to(tok), _to(par), _to(np.full(B, n_max)), n_max))
+    orc.verify([(list(map(int, tok[b])), list(map(int, par[b]))) for b in range(B)])
+    check(n_max, "tree")
+    assert eng.device_status() == 0
+    assert eng.check_guards()[1] == 0
+    eng.close()
