@@ -663,6 +663,49 @@ int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, 
   return run_layers(c, c->draft_layers, g.K, c->dk, c->dv, Rh, k.q, nullptr, none, nullptr, same, true);
 }
 
+// Cuts the prompts into blocks and hands them out as forwards of at most `ingest_rows` rows, run(blocks) each;
+// the first code other than KOALA_OK that run returns ends it.
+template <typename Run>
+int deal_blocks(const IngestLens &k, int B, int ingest_rows, Run run) {
+  int longest = 0;
+  for (int b = 0; b < B; ++b) longest = k.len[b] > longest ? k.len[b] : longest;
+  // Block length: the one that leaves the fewest unused rows (ties: the longest, which re-reads the
+  // cached keys least); one block if every prompt is short.
+  int q = longest < 128 ? longest : 128;
+  if (q > ingest_rows) q = ingest_rows;            // a prompt beyond the cache's capacity: reported by the plan
+  if (q > 48) {
+    int best = 1 << 30;
+    for (int t = q; t > 48; --t) {
+      int rows = 0;
+      for (int b = 0; b < B; ++b) rows += (k.len[b] + t - 1) / t * t;
+      if (rows < best) { best = rows; q = t; }
+    }
+  }
+  int fwd = ingest_rows / q;
+  fwd = fwd > INGEST_MAX_BLOCKS ? INGEST_MAX_BLOCKS : (fwd < 1 ? 1 : fwd);
+  int total = 0;
+  for (int b = 0; b < B; ++b) total += (k.len[b] + q - 1) / q;
+  const int n_fwd = (total + fwd - 1) / fwd;
+  fwd = (total + n_fwd - 1) / n_fwd;               // forwards of equal size
+  // blocks by position, all sequences side by side: a block comes after the earlier ones of its sequence
+  IngestBlocks blk;
+  memset(&blk, 0, sizeof(blk));
+  blk.q = q;
+  for (int s0 = 0; s0 < longest; s0 += q)
+    for (int b = 0; b < B; ++b) {
+      if (s0 >= k.len[b]) continue;
+      blk.start[blk.n] = s0;
+      blk.last[blk.n] = k.count[b] - s0;
+      blk.seq[blk.n] = (int16_t)b;
+      blk.count[blk.n] = (int16_t)(k.len[b] - s0 < q ? k.len[b] - s0 : q);
+      blk.from[blk.n] = (int16_t)blk.n;
+      if (++blk.n < fwd) continue;
+      K_TRY(run(blk));
+      blk.n = 0;
+    }
+  return blk.n > 0 ? run(blk) : KOALA_OK;
+}
+
 // Node rows of a forward over `rows` rows per sequence (with one sequence they are where they belong already).
 RowMap node_rows(const koala_config &g, int rows) {
   return g.B == 1 || rows == g.N ? RowMap{0, 0} : RowMap{rows, g.N};
@@ -1019,31 +1062,7 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     if (len[b] > longest) longest = len[b];
   }
   if (longest == 0) return fail(c, KOALA_E_INVALID, "empty prompts");
-  // Block length: the one that leaves the fewest unused rows (ties: the longest, which re-reads the
-  // cached keys least); one block if every prompt is short.
-  int q = longest < 128 ? longest : 128;
-  if (q > c->ingest_rows) q = c->ingest_rows;      // a prompt beyond the cache's capacity: reported by the plan
-  if (q > 48) {
-    int best = 1 << 30;
-    for (int t = q; t > 48; --t) {
-      int rows = 0;
-      for (int b = 0; b < g.B; ++b) rows += (k.len[b] + t - 1) / t * t;
-      if (rows < best) { best = rows; q = t; }
-    }
-  }
-  int fwd = c->ingest_rows / q;
-  fwd = fwd > INGEST_MAX_BLOCKS ? INGEST_MAX_BLOCKS : (fwd < 1 ? 1 : fwd);
-  int total = 0;
-  for (int b = 0; b < g.B; ++b) total += (k.len[b] + q - 1) / q;
-  const int n_fwd = (total + fwd - 1) / fwd;
-  fwd = (total + n_fwd - 1) / n_fwd;               // forwards of equal size
-  // blocks by position, all sequences side by side: a block comes after the earlier ones of its sequence
-  IngestBlocks blk;
-  memset(&blk, 0, sizeof(blk));
-  blk.q = q;
-  int rc = KOALA_OK;
-  auto flush = [&]() {
-    if (blk.n == 0 || rc != KOALA_OK) return;
+  K_TRY(deal_blocks(k, g.B, c->ingest_rows, [&](const IngestBlocks &blk) {
     // The pending rows of a sequence are those of its last part; where earlier parts were one token
     // longer, the row after them still holds the last token of the last longer part.
     IngestKeep keep;
@@ -1051,25 +1070,13 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     for (int v = 0; v < blk.n; ++v) {
       const int b = blk.seq[v], row = k.len[b] / n_parts, at = (k.len[b] % n_parts) * (row + 1) - 1 - blk.start[v];
       if (at < 0 || at >= blk.count[v] || row >= g.N) continue;
-      keep.src[keep.n] = v * q + at;
+      keep.src[keep.n] = v * blk.q + at;
       keep.dst[keep.n++] = b * g.N + row;
     }
-    rc = ingest_forward(c, blk, keep, tok, stride, n_max);
+    const int rc = ingest_forward(c, blk, keep, tok, stride, n_max);
     c->ingest_blocks = 0;
-    blk.n = 0;
-  };
-  for (int s0 = 0; s0 < longest; s0 += q)
-    for (int b = 0; b < g.B; ++b) {
-      if (s0 >= k.len[b]) continue;
-      blk.start[blk.n] = s0;
-      blk.last[blk.n] = k.count[b] - s0;
-      blk.seq[blk.n] = (int16_t)b;
-      blk.count[blk.n] = (int16_t)(k.len[b] - s0 < q ? k.len[b] - s0 : q);
-      blk.from[blk.n] = (int16_t)blk.n;
-      if (++blk.n == fwd) flush();
-    }
-  flush();
-  if (rc != KOALA_OK) return rc;
+    return rc;
+  }));
   K_TRY(target_logits(c, g.B * n_max, node_rows(g, n_max)));
   CU_TRY(ingest_commit(LN(c), c->t, k, tok, stride, c->seq_len, g.B, g.N, c->status));
   c->phase = PH_VERIFIED;
@@ -1201,6 +1208,24 @@ int koala_selftest_timeout(koala_ctx *c, int limit_cycles) {
   if (limit_cycles < 1 || limit_cycles > 100000000) return fail(c, KOALA_E_INVALID, "limit_cycles outside 1..1e8");
   CU_TRY(koala::selftest_timeout(LN(c), c->status, (long long)limit_cycles));
   return KOALA_OK;
+}
+
+int koala_debug_deal_blocks(int B, const int32_t *len, int ingest_rows, int fail_at, int *n_blocks, int *n_tokens) {
+  if (B < 1 || B > 64 || !len || ingest_rows < 1 || !n_blocks || !n_tokens) return KOALA_E_INVALID;
+  IngestLens k;
+  memset(&k, 0, sizeof(k));
+  k.n_parts = 1;
+  for (int b = 0; b < B; ++b) {
+    if (len[b] < 1) return KOALA_E_INVALID;
+    k.len[b] = len[b];
+  }
+  *n_blocks = *n_tokens = 0;
+  int call = 0;
+  return deal_blocks(k, B, ingest_rows, [&](const IngestBlocks &blk) {
+    *n_blocks += blk.n;
+    for (int v = 0; v < blk.n; ++v) *n_tokens += blk.count[v];
+    return call++ == fail_at ? KOALA_E_CUDA : KOALA_OK;
+  });
 }
 
 int koala_debug_check_guards(koala_ctx *c, int *n_guards, int *n_damaged) {

@@ -49,6 +49,11 @@ int koala_selftest_timeout(koala_ctx *ctx, int limit_cycles);
  * n_damaged: host ints. */
 int koala_debug_check_guards(koala_ctx *ctx, int *n_guards, int *n_damaged);
 
+/* How koala_ingest deals the blocks of B prompts of len[b] tokens to forwards of at most ingest_rows rows,
+ * without enqueueing anything: *n_blocks and *n_tokens handed out until the forward with index fail_at
+ * (< 0: none) reports KOALA_E_CUDA, which ends the dealing and is returned.  Host memory only. */
+int koala_debug_deal_blocks(int B, const int32_t *len, int ingest_rows, int fail_at, int *n_blocks, int *n_tokens);
+
 #ifdef __cplusplus
 }
 #endif
