@@ -114,7 +114,8 @@ typedef struct {
 typedef struct {
   const int32_t *tok;     /* [B][stride] */
   const int32_t *parent;  /* [B][stride], root -1, parent < child */
-  const int32_t *n_nodes; /* [B], 1 <= n_nodes[b] <= n_max */
+  const int32_t *n_nodes; /* [B], 1 <= n_nodes[b] <= n_max; anything else sets the device status to
+                             KOALA_E_INVALID and the tree is cut to the nearest of the two */
   int32_t stride;
   int32_t n_max;          /* host-known bound on n_nodes, <= N */
 } koala_tree;

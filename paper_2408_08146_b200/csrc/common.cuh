@@ -355,7 +355,7 @@ struct PlanBufs {
   float2 *rope;
 };
 cudaError_t tree_from_caller(Launch L, TreeBufs t, const int32_t *tok, const int32_t *parent,
-                             const int32_t *n_nodes, int stride, int B, int N, int *status);
+                             const int32_t *n_nodes, int stride, int n_max, int B, int N, int *status);
 // rope_base ^ (-2 i / head_dim), computed once on the host
 struct RopeInv {
   double v[64];

@@ -1019,8 +1019,8 @@ int koala_verify(koala_ctx *c, const koala_tree *tree) {
     if (tree->n_max < 1 || tree->n_max > g.N || tree->stride < tree->n_max)
       return fail(c, KOALA_E_INVALID, "tree n_max %d / stride %d out of range (N = %d)", tree->n_max,
                   tree->stride, g.N);
-    CU_TRY(tree_from_caller(LN(c), c->t, tree->tok, tree->parent, tree->n_nodes, tree->stride, g.B, g.N,
-                            c->status));
+    CU_TRY(tree_from_caller(LN(c), c->t, tree->tok, tree->parent, tree->n_nodes, tree->stride, tree->n_max, g.B,
+                            g.N, c->status));
     c->last_tree_from_caller = true;
     c->pend_cap = tree->n_max;
   } else {

@@ -26,15 +26,15 @@ __device__ __forceinline__ void write_rope(float2 *rope, size_t row, int pos, in
 // ------------------------------------------------------------------------------- caller tree
 __global__ void tree_from_caller_kernel(TreeBufs t, const int32_t *tok,
                                         const int32_t *parent,
-                                        const int32_t *n_nodes, int stride, int N,
+                                        const int32_t *n_nodes, int stride, int n_max, int N,
                                         int *status) {
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
   int n = n_nodes[b];
-  if (n < 1 || n > N) {
+  if (n < 1 || n > n_max) {            // the forward has n_max rows per sequence: no others are computed
     if (threadIdx.x == 0 && status) atomicMax(status, E_INVALID);
-    n = n < 1 ? 1 : N;
+    n = n < 1 ? 1 : n_max;
   }
   for (int u = threadIdx.x; u < N; u += blockDim.x) {
     int p = -1, tk = 0;
@@ -541,9 +541,9 @@ __global__ void kv_compact_kernel(TreeBufs t, const float *hid, T *__restrict__ 
 }  // namespace
 
 cudaError_t tree_from_caller(Launch L, TreeBufs t, const int32_t *tok, const int32_t *parent,
-                             const int32_t *n_nodes, int stride, int B, int N, int *status) {
+                             const int32_t *n_nodes, int stride, int n_max, int B, int N, int *status) {
   return launch_k(tree_from_caller_kernel, dim3(B), dim3(128), 0, L.st, L.pdl, t, tok, parent,
-                  n_nodes, stride, N, status);
+                  n_nodes, stride, n_max, N, status);
 }
 #define PLAN_DISPATCH(kern, grid, ...)                                                                       \
   (fill.dtype == 0 ? launch_k(kern<float>, grid, dim3(ROW_THREADS), 0, L.st, L.pdl, __VA_ARGS__)              \

@@ -47,3 +47,30 @@ def test_short_trees_and_prompts_under_a_wide_vocabulary(model, B):
     assert eng.device_status() == 0
     assert eng.check_guards()[1] == 0
     eng.close()
+
+
+@pytest.mark.parametrize("N,n_max", [(15, 4), (15, 14), (15, 15)])
+def test_a_tree_larger_than_its_bound_is_reported_and_cut(N, n_max):
+    """n_nodes[b] = n_max + 1 where the arrays hold that node: the forward has no row for it, so the sequence's
+    tree ends at n_max nodes (as if the caller had said so) and the status says that it was cut."""
+    cfg = TINY_EAGLE.with_(B=2, N=N, prompt_len=30, S_max=128, seed=43)
+    eng, orc, _ = make_pair(cfg)
+    pr = prompts(cfg)
+    eng.prefill(pr, cfg.N)
+    orc.prefill(pr, cfg.N)
+    rng = np.random.default_rng(n_max)
+    tok = rng.integers(0, cfg.V, (2, n_max + 1))
+    par = np.asarray([[-1] + list(range(n_max))] * 2)                     # chains
+    eng.koala_verify((_to(tok), _to(par), _to([n_max, n_max + 1]), n_max))
+    orc.verify([(list(map(int, tok[b, :n_max])), list(map(int, par[b, :n_max]))) for b in range(2)])
+    forced = _to([n_max + 1, n_max + 1])                                   # as far as the tree goes
+    got, n = eng.koala_accept(forced)
+    assert n.cpu().tolist() == [n_max, n_max]
+    assert eng.seq_len.cpu().tolist() == [30 + n_max, 30 + n_max]
+    for b in range(2):
+        logits = eng.buffers()["verify_logits"][b * N:b * N + n_max].cpu().numpy()
+        assert_close(logits, orc.verify_logits[b], cfg.dtype, f"logits {b}")
+        check_argmax(got[b, n_max - 1:n_max].cpu().numpy(), orc.verify_logits[b][n_max - 1:], f"bonus {b}")
+    assert eng.device_status() == 1
+    assert eng.check_guards()[1] == 0
+    eng.close()
