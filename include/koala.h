@@ -187,7 +187,8 @@ int koala_verify(koala_ctx *ctx, const koala_tree *tree);
  * verified as a chain, all but the last accepted in full and, with an EAGLE-style head, followed by
  * koala_draft(0) with the next prompt token as root: the caller continues with koala_accept, with the
  * lengths of the last parts (tree_n) as forced lengths.  Up to 1024 tokens go through one forward; logits
- * are formed for the last parts only.  tok: DEVICE [B][stride] prompts; len: HOST [B], copied. */
+ * are formed for the last parts only.  tok: DEVICE [B][stride] prompts; len: HOST [B], copied,
+ * n_parts <= len[b] <= stride (no part is empty). */
 int koala_ingest(koala_ctx *ctx, const int32_t *tok, int32_t stride, const int32_t *len, int32_t n_parts);
 
 /* Greedy acceptance (Section 4.1: a draft token is kept only if it equals the target's greedy

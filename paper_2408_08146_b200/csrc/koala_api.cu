@@ -1051,17 +1051,16 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
   IngestLens k;
   memset(&k, 0, sizeof(k));
   k.n_parts = n_parts;
-  int longest = 0, n_max = 1;
+  int n_max = 1;
   for (int b = 0; b < g.B; ++b) {
-    if (len[b] < 0 || len[b] > stride) return fail(c, KOALA_E_INVALID, "prompt %d: %d tokens (stride %d)", b, len[b], stride);
+    if (len[b] < n_parts || len[b] > stride)       // a part without tokens has no row to be pending
+      return fail(c, KOALA_E_INVALID, "prompt %d: %d tokens in %d parts (stride %d)", b, len[b], n_parts, stride);
     k.len[b] = len[b];
     const int last = len[b] / n_parts;             // the last of the equal parts is the shorter kind
     if (last > g.N) return fail(c, KOALA_E_INVALID, "prompt %d: last part of %d tokens (N = %d)", b, last, g.N);
     k.count[b] = len[b] - last;
     if (last > n_max) n_max = last;
-    if (len[b] > longest) longest = len[b];
   }
-  if (longest == 0) return fail(c, KOALA_E_INVALID, "empty prompts");
   K_TRY(deal_blocks(k, g.B, c->ingest_rows, [&](const IngestBlocks &blk) {
     // The pending rows of a sequence are those of its last part; where earlier parts were one token
     // longer, the row after them still holds the last token of the last longer part.

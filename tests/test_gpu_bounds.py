@@ -4,7 +4,8 @@ import numpy as np
 import pytest
 import torch
 
-from tests.harness import make_pair
+from paper_2408_08146_b200 import KoalaError
+from tests.harness import make_pair, tok_list
 from tests.parity import assert_close, check_argmax
 from workloads import T7_EAGLE, TINY_EAGLE, reduced
 from workloads.generate import prompts
@@ -73,4 +74,25 @@ def test_a_tree_larger_than_its_bound_is_reported_and_cut(N, n_max):
         check_argmax(got[b, n_max - 1:n_max].cpu().numpy(), orc.verify_logits[b][n_max - 1:], f"bonus {b}")
     assert eng.device_status() == 1
     assert eng.check_guards()[1] == 0
+    eng.close()
+
+
+def test_a_prompt_shorter_than_its_number_of_parts_is_refused():
+    """Five tokens cannot be six parts: refused before anything is enqueued, nothing of the batch has moved."""
+    cfg = TINY_EAGLE.with_(B=2, prompt_len=60, S_max=128, seed=44)
+    eng, orc, _ = make_pair(cfg)
+    rng = np.random.default_rng(44)
+    long, short = rng.integers(0, cfg.V, 60), rng.integers(0, cfg.V, 5)
+    launches = eng.launch_count()
+    with pytest.raises(KoalaError) as e:
+        eng.prefill([long, short], 10)
+    assert e.value.code == 1 and eng.launch_count() == launches
+    assert eng.seq_len.cpu().tolist() == [0, 0]
+    eng.prefill([long, short], 15)               # four parts: 2 + 1 + 1 + 1 tokens
+    orc.prefill([long, short], 15)
+    for _ in range(2):
+        tk, ln = tok_list(*eng.step())
+        rt, rl = orc.step()
+        assert [list(x) for x in tk] == [list(x) for x in rt] and list(ln) == list(rl)
+    assert eng.device_status() == 0
     eng.close()
