@@ -387,8 +387,7 @@ cudaError_t ingest_last(Launch L, int dtype, IngestBlocks k, const float *hid, f
                         int H);
 // seq_len += count; acceptance counters as if every part but the last had been accepted as a chain; the tree of
 // each sequence becomes the chain of its last part
-cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N,
-                          int *status);
+cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N);
 cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows, int head_dim,
                         const RopeInv &inv, const RowFill &fill, int S_max, int *status);
 cudaError_t plan_draft_p(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int k, int pool, int pass,

@@ -1056,8 +1056,8 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     if (len[b] < n_parts || len[b] > stride)       // a part without tokens has no row to be pending
       return fail(c, KOALA_E_INVALID, "prompt %d: %d tokens in %d parts (stride %d)", b, len[b], n_parts, stride);
     k.len[b] = len[b];
-    const int last = len[b] / n_parts;             // the last of the equal parts is the shorter kind
-    if (last > g.N) return fail(c, KOALA_E_INVALID, "prompt %d: last part of %d tokens (N = %d)", b, last, g.N);
+    const int last = len[b] / n_parts, longest = last + (len[b] % n_parts ? 1 : 0);
+    if (longest > g.N) return fail(c, KOALA_E_INVALID, "prompt %d: a part of %d tokens (N = %d)", b, longest, g.N);
     k.count[b] = len[b] - last;
     if (last > n_max) n_max = last;
   }
@@ -1077,7 +1077,7 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     return rc;
   }));
   K_TRY(target_logits(c, g.B * n_max, node_rows(g, n_max)));
-  CU_TRY(ingest_commit(LN(c), c->t, k, tok, stride, c->seq_len, g.B, g.N, c->status));
+  CU_TRY(ingest_commit(LN(c), c->t, k, tok, stride, c->seq_len, g.B, g.N));
   c->phase = PH_VERIFIED;
   c->last_tree_from_caller = true;
   c->pend_cap = n_max;

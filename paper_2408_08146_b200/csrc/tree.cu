@@ -181,19 +181,13 @@ __global__ void ingest_keep_kernel(TreeBufs t, const __grid_constant__ IngestKee
 
 // block 0: lengths and counters; block 1 + b: sequence b's tree
 __global__ void ingest_commit_kernel(TreeBufs t, const __grid_constant__ IngestLens k, const int32_t *tok, int stride,
-                                     int32_t *seq_len, int B, int N, int *status) {
+                                     int32_t *seq_len, int B, int N) {
   pdl_launch_dependents();
   pdl_wait();
   if (blockIdx.x > 0) {
-    const int b = blockIdx.x - 1;
-    int n = k.len[b] - k.count[b];
-    if (n < 1 || n > N) {
-      if (threadIdx.x == 0 && status) atomicMax(status, E_INVALID);
-      n = n < 1 ? 1 : N;
-    }
+    const int b = blockIdx.x - 1, n = k.len[b] - k.count[b];       // 1 .. N (host)
     for (int u = threadIdx.x; u < N; u += blockDim.x) {
-      const bool in = u < n && k.count[b] + u < k.len[b];
-      t.tree_tok[b * N + u] = in ? tok[(size_t)b * stride + k.count[b] + u] : 0;
+      t.tree_tok[b * N + u] = u < n ? tok[(size_t)b * stride + k.count[b] + u] : 0;
       t.tree_parent[b * N + u] = u < n ? u - 1 : -1;
       t.tree_level[b * N + u] = u < n ? u : 0;
       t.tree_score[b * N + u] = 0.f;
@@ -204,7 +198,7 @@ __global__ void ingest_commit_kernel(TreeBufs t, const __grid_constant__ IngestL
   const int i = threadIdx.x;                  // chain position i + 1
   unsigned long long hits = 0;
   for (int b = 0; b < B; ++b) {
-    // the first len % n_parts parts have one token more; the last part is not ingested here
+    // the first len % n_parts parts have one token more; the last part is left to koala_accept
     const int base = k.len[b] / k.n_parts, longer = k.len[b] % k.n_parts, parts = k.n_parts - 1;
     const int n_long = longer < parts ? longer : parts;
     if (base + 1 > i + 1) hits += (unsigned long long)n_long;
@@ -560,9 +554,8 @@ cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, in
   if (k.n == 0) return cudaSuccess;
   return launch_k(ingest_keep_kernel, dim3(k.n), dim3(256), 0, L.st, L.pdl, t, k, hid, H);
 }
-cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N,
-                          int *status) {
-  return launch_k(ingest_commit_kernel, dim3(1 + B), dim3(128), 0, L.st, L.pdl, t, k, tok, stride, seq_len, B, N, status);
+cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N) {
+  return launch_k(ingest_commit_kernel, dim3(1 + B), dim3(128), 0, L.st, L.pdl, t, k, tok, stride, seq_len, B, N);
 }
 cudaError_t plan_draft0(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len, int B, int N, int rows, int head_dim,
                         const RopeInv &inv, const RowFill &fill, int S_max, int *status) {

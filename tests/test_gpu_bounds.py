@@ -1,5 +1,7 @@
 """Sizes and arguments at the edge of what a call may be given: models whose vocabulary is wide against
 their hidden size, and caller trees and prompts that do not keep to their own bounds."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -94,5 +96,25 @@ def test_a_prompt_shorter_than_its_number_of_parts_is_refused():
         tk, ln = tok_list(*eng.step())
         rt, rl = orc.step()
         assert [list(x) for x in tk] == [list(x) for x in rt] and list(ln) == list(rl)
+    assert eng.device_status() == 0
+    eng.close()
+
+
+def test_a_part_of_more_than_n_tokens_is_refused():
+    """2 N + 1 tokens in two parts: the first would have N + 1, a chain that no tree holds."""
+    cfg = TINY_EAGLE.with_(prompt_len=31, S_max=128, seed=45)
+    eng, orc, _ = make_pair(cfg)
+    pr = prompts(cfg)
+    tok = _to([pr[0]])
+    ingest = lambda parts: eng.lib.koala_ingest(eng._ctx, tok.data_ptr(), 31, (C.c_int32 * 1)(31), parts)
+    assert cfg.N == 15 and ingest(2) == 1
+    assert eng.seq_len.cpu().tolist() == [0] and eng.koala_accept_stats(20) == ([0] * 20, [0] * 20)
+    assert ingest(3) == 0
+    eng.koala_accept(eng.buffers()["tree_n"])
+    orc.prefill(pr, 15)
+    assert eng.seq_len.cpu().tolist() == orc.seq_len
+    rt, rl = orc.step()
+    tk, ln = tok_list(*eng.step())
+    assert [list(x) for x in tk] == [list(x) for x in rt] and list(ln) == list(rl)
     assert eng.device_status() == 0
     eng.close()
