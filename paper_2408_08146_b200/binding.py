@@ -387,10 +387,10 @@ class Koala:
         c = self.cfg
         chunk = min(chunk, c.N)
         n_chunks = max(-(-len(p) // chunk) for p in prompts)
-        lens = [len(p) for p in prompts]
+        lens = [len(prompts[b]) for b in range(c.B)]
         host = np.zeros((c.B, max(lens)), np.int32)
-        for b, p in enumerate(prompts):
-            host[b, :lens[b]] = np.asarray(p)
+        for b in range(c.B):
+            host[b, :lens[b]] = np.asarray(prompts[b])
         toks = torch.from_numpy(host).to(self.dev)
         self._check(self.lib.koala_ingest(self._ctx, toks.data_ptr(), toks.shape[1], _i32_array(lens), n_chunks))
         self.koala_accept(self.buffers()["tree_n"])
