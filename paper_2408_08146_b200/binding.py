@@ -392,6 +392,8 @@ class Koala:
         for b in range(c.B):
             host[b, :lens[b]] = np.asarray(prompts[b])
         toks = torch.from_numpy(host).to(self.dev)
+        if toks.is_cuda:
+            toks.record_stream(self.stream)     # the caller's current stream may be another one than the engine's
         self._check(self.lib.koala_ingest(self._ctx, toks.data_ptr(), toks.shape[1], _i32_array(lens), n_chunks))
         self.koala_accept(self.buffers()["tree_n"])
 

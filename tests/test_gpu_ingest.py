@@ -82,3 +82,28 @@ def test_a_prompt_beyond_the_capacity_is_reported():
     assert eng.device_status() == 3
     assert eng.check_guards()[1] == 0
     eng.close()
+
+
+def test_prompts_of_an_engine_on_another_stream():
+    """The engine's stream is busy when prefill returns, and the caller's stream takes up freed memory at once: the
+    prompt's tokens stay until the engine has read them."""
+    cfg = TINY_EAGLE.with_(S_max=256, prompt_len=200, seed=33)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        eng, orc, _ = make_pair(cfg)
+    side.synchronize()
+    pr = prompts(cfg)
+    eng.prefill([pr[0][::-1]], 15)                          # kernels loaded: the next call does not wait for the device
+    torch.cuda.synchronize()
+    eng.seq_len.zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(200_000_000)                      # about 0.1 s
+    eng.prefill(pr, 15)                                     # the current stream is the default one
+    other = [torch.full((1, 200), 7, dtype=torch.int32, device="cuda:0") for _ in range(8)]
+    torch.cuda.synchronize()
+    assert all(int(t.sum()) == 1400 for t in other)
+    orc.prefill(pr, 15)
+    _check(eng, orc, cfg, [200], np.float64)
+    assert eng.device_status() == 0
+    eng.close()
