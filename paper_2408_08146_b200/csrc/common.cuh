@@ -274,10 +274,11 @@ int tc_init_driver(char *err, size_t errlen);   // 0 on success
 bool tc_supported(const GemmMats &m, int K_in);
 int tc_default_split(int n_tiles, int kblocks, int tokens);
 // split >= 1: classic split-K; split == 0: automatic (stream-K where it applies).  `max_slots`
-// bounds the partial matrices written; *out describes them for the consumer.
+// bounds the partial matrices written; *out describes them for the consumer.  short_sums: no sum inside the
+// tensor core is longer than with 64 rows, whatever R.
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
                     float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
-                    SplitIn *out);
+                    SplitIn *out, bool short_sums = false);
 
 // layer_tc.cu : several GEMMs of a decoder layer and the row-wise steps between them in one
 // persistent launch (bf16, activations as pairs, at most 128 rows, head_dim 128 for the rotary step)

@@ -391,7 +391,23 @@ constexpr int PAIR_PART_BYTES = BM * BK * 2;          // 16 KB: 128 rows of one 
 constexpr int PAIR_MAX_STAGES = 4;
 constexpr int PAIR_ROWS = 4 * BM;                     // weight rows per cluster tile
 
-__global__ void __launch_bounds__(PAIR_THREADS, 1)
+// CHAIN: the tensor core adds into its fp32 accumulators by truncation, so the error of a sum grows with the
+// number of MMAs that went into it (towards zero; K = 4096 as value and residual, 512 MMAs: 9.2e-6 of the
+// result, as much as four times what the pairs leave out).  Where a product has several token tiles its
+// partial sums are too large to be cut along K into global memory as with few rows (where the longest sum is
+// 64 to 256 MMAs; hidden state after 32 layers of the 7B shape, 509 prompt tokens, against float64: 1.7e-3 in
+// parts of 64 rows, 2.7e-3 with 512-MMA sums, 1.4e-3 in this form); instead every CHAIN_KB K blocks the MMAs
+// change to the other accumulator set, and the epilogue warps add the finished one to sums in registers,
+// rounding to nearest, while it fills: 32 MMAs per sum, 5.6e-7.  256 weight rows per cluster, one
+// accumulator of up to 256 tokens: two sets in tensor memory, 128 sums per thread of eight warps.  (512 rows x
+// 128 tokens, the same loads, read more of shared memory per MMA: 7B prompt of 509 tokens 17.0 ms against
+// 14.3; chains of 8 K blocks: the same time, twice the error.)
+constexpr int CHAIN_KB = 4;
+constexpr int CHAIN_THREADS = 320;
+constexpr int CHAIN_ROWS = 2 * BM;                    // weight rows per cluster tile
+
+template <bool CHAIN>
+__global__ void __launch_bounds__(CHAIN ? CHAIN_THREADS : PAIR_THREADS, 1)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
                     const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmX,
                     const __grid_constant__ CUtensorMap tmXlo, const TcParams P) {
@@ -414,15 +430,17 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
   const unsigned u_hi = (cid + 1u) * P.sk_units / (unsigned)P.sk_ctas;
   const int n_units = (int)(u_hi - u_lo);
   const int n_epi = (int)(blockDim.x >> 5) - 2;
+  constexpr int PARTS = CHAIN ? 1 : 2;                   // accumulators of 256 weight rows
+  constexpr int ROWS = CHAIN ? CHAIN_ROWS : PAIR_ROWS;
   const int tt = P.tt;                                   // tokens per tile: a multiple of 32, at most 256
   const int x_part = (tt >> 1) * BK * 2;                  // this CTA's tokens, value or residual rows
-  const int stage_bytes = 2 * PAIR_PART_BYTES + 2 * x_part;
+  const int stage_bytes = PARTS * PAIR_PART_BYTES + 2 * x_part;
   const int n_stages = P.stages;
 
   auto tile_map = [&](int tile, int &row0) -> const CUtensorMap * {
-    if (tile >= P.tiles1) { row0 = (tile - P.tiles1) * PAIR_ROWS; return &tmW2; }
-    if (tile >= P.tiles0) { row0 = (tile - P.tiles0) * PAIR_ROWS; return &tmW1; }
-    row0 = tile * PAIR_ROWS;
+    if (tile >= P.tiles1) { row0 = (tile - P.tiles1) * ROWS; return &tmW2; }
+    if (tile >= P.tiles0) { row0 = (tile - P.tiles0) * ROWS; return &tmW1; }
+    row0 = tile * ROWS;
     return &tmW0;
   };
   const int pre = n_units < n_stages ? n_units : n_stages;
@@ -479,10 +497,10 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
         unsigned char *dst = tiles + (size_t)s * stage_bytes;
         if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * (uint32_t)stage_bytes);
         tma_load_2d_pair_hint(tmW, full_even[s], dst, kb * BK, row0 + (int)rank * BM, policy);
-        tma_load_2d_pair_hint(tmW, full_even[s], dst + PAIR_PART_BYTES, kb * BK, row0 + 2 * BM + (int)rank * BM, policy);
+        if (!CHAIN) tma_load_2d_pair_hint(tmW, full_even[s], dst + PAIR_PART_BYTES, kb * BK, row0 + 2 * BM + (int)rank * BM, policy);
       };
       auto load_x = [&](int s, int kbx, int tokx) {
-        unsigned char *dst = tiles + (size_t)s * stage_bytes + 2 * PAIR_PART_BYTES;
+        unsigned char *dst = tiles + (size_t)s * stage_bytes + PARTS * PAIR_PART_BYTES;
         tma_load_2d_pair(&tmX, full_even[s], dst, kbx * BK, tokx + (int)rank * (tt >> 1));
         tma_load_2d_pair(&tmXlo, full_even[s], dst + x_part, kbx * BK, tokx + (int)rank * (tt >> 1));
       };
@@ -519,7 +537,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tt >> 3) << 17) |
                              ((uint32_t)(256 >> 4) << 24);
       bool ok = true;
-      int seg = 0;
+      int seg = 0, links = 0;              // CHAIN: a "segment" here is what goes into one accumulator set
       bool seg_start = true;
       int kb = (int)(u_lo % KB), s = 0, buf = 0;
       uint32_t ph = 0;
@@ -535,19 +553,25 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
         const uint32_t wa = smem_u32(tiles + (size_t)s * stage_bytes);
         const uint64_t da0 = smem_desc_sw128(wa);
         const uint64_t da1 = smem_desc_sw128(wa + PAIR_PART_BYTES);
-        const uint64_t dbh = smem_desc_sw128(wa + 2 * PAIR_PART_BYTES);
-        const uint64_t dbl = smem_desc_sw128(wa + 2 * PAIR_PART_BYTES + (uint32_t)x_part);
-        const uint32_t d0 = tmem_acc + (uint32_t)(buf * 2 * tt), d1 = d0 + (uint32_t)tt;
+        const uint64_t dbh = smem_desc_sw128(wa + PARTS * PAIR_PART_BYTES);
+        const uint64_t dbl = smem_desc_sw128(wa + PARTS * PAIR_PART_BYTES + (uint32_t)x_part);
+        const uint32_t d0 = tmem_acc + (uint32_t)(buf * PARTS * tt), d1 = d0 + (uint32_t)tt;
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; ++k) {
           const uint32_t acc = (!seg_start || k > 0) ? 1u : 0u;
           umma2_bf16(d0, da0 + (uint64_t)(2 * k), dbh + (uint64_t)(2 * k), idesc, acc);
           umma2_bf16(d0, da0 + (uint64_t)(2 * k), dbl + (uint64_t)(2 * k), idesc, 1u);
-          umma2_bf16(d1, da1 + (uint64_t)(2 * k), dbh + (uint64_t)(2 * k), idesc, acc);
-          umma2_bf16(d1, da1 + (uint64_t)(2 * k), dbl + (uint64_t)(2 * k), idesc, 1u);
+          if (!CHAIN) {
+            umma2_bf16(d1, da1 + (uint64_t)(2 * k), dbh + (uint64_t)(2 * k), idesc, acc);
+            umma2_bf16(d1, da1 + (uint64_t)(2 * k), dbl + (uint64_t)(2 * k), idesc, 1u);
+          }
         }
         umma2_commit_to(&empty_bar[s], 3);
-        const bool seg_end = (kb == KB - 1) || it == n_units - 1;
+        bool seg_end = (kb == KB - 1) || it == n_units - 1;
+        if (CHAIN) {
+          seg_end = ++links == CHAIN_KB || seg_end;
+          if (seg_end) links = 0;
+        }
         if (seg_end) {
           umma2_commit_to(&acc_full[buf], 3);
           ++seg;
@@ -568,7 +592,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
     const int c_hi = min(c_lo + c_per, tt);
     const uint32_t acc_empty_even[2] = {cluster_addr_of(smem_u32(&acc_empty[0]), 0),
                                         cluster_addr_of(smem_u32(&acc_empty[1]), 0)};
-    bool dry = P.epi_dry != 0;           // a dry pass over the loop body first (nothing stored, nothing waited for)
+    bool dry = !CHAIN && P.epi_dry != 0; // a dry pass over the loop body first (nothing stored, nothing waited for)
     bool ok = true;
     int seg = 0;
     unsigned u = u_lo;
@@ -576,47 +600,82 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       const int tile = (int)(u / KB);
       unsigned seg_hi = (unsigned)(tile + 1) * KB;
       if (seg_hi > u_hi) seg_hi = u_hi;
-      const int buf = seg % P.nbuf;
-      if (!dry) {
-        ok = mbar_wait(&acc_full[buf], (uint32_t)(seg / P.nbuf) & 1u);
-        if (!ok) break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       int row0, col_off = 0, n_rows = P.n0;
       const int wt = tile / P.ztiles, tok0 = (tile % P.ztiles) * tt;
-      if (wt >= P.tiles1) { row0 = (wt - P.tiles1) * PAIR_ROWS; col_off = P.n0 + P.n1; n_rows = P.n2; }
-      else if (wt >= P.tiles0) { row0 = (wt - P.tiles0) * PAIR_ROWS; col_off = P.n0; n_rows = P.n1; }
-      else row0 = wt * PAIR_ROWS;
+      if (wt >= P.tiles1) { row0 = (wt - P.tiles1) * ROWS; col_off = P.n0 + P.n1; n_rows = P.n2; }
+      else if (wt >= P.tiles0) { row0 = (wt - P.tiles0) * ROWS; col_off = P.n0; n_rows = P.n1; }
+      else row0 = wt * ROWS;
       if (dry) n_rows = 0;
       // partial-sum slot = rank of this cluster among the tile's contributors
       const int slot = (int)cid - (int)sk_owner((unsigned)tile * KB, (unsigned)P.sk_ctas, P.sk_units);
-#pragma unroll 1
-      for (int a = 0; a < 2; ++a) {
+      auto store16 = [&](int a, int c0, auto value) {
         const int feat = row0 + a * 2 * BM + (int)rank * BM + quarter * 32 + lane;
-        float *Yp = P.Y + (size_t)slot * P.split_stride + col_off + feat;
-        const uint32_t lane_base = tmem_acc + (uint32_t)((buf * 2 + a) * tt) + ((uint32_t)(quarter * 32) << 16);
-#pragma unroll 1
-        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {       // rolled, as in the one-CTA kernel
-          uint32_t va[16];
-          tmem_ld16(lane_base + (uint32_t)c0, va);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          const int left = feat < n_rows ? P.R - (tok0 + c0) : 0;
-          float *yp = Yp + (size_t)(tok0 + c0) * P.ldy;
+        const int left = feat < n_rows ? P.R - (tok0 + c0) : 0;
+        float *yp = P.Y + (size_t)slot * P.split_stride + col_off + feat + (size_t)(tok0 + c0) * P.ldy;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            if (j < left) *yp = __uint_as_float(va[j]);
-            yp += P.ldy;
+        for (int j = 0; j < 16; ++j) {
+          if (j < left) *yp = value(j);
+          yp += P.ldy;
+        }
+      };
+      if constexpr (CHAIN) {
+        constexpr int GROUPS = 8;                          // steps of 16 columns per warp
+        float sum[GROUPS][16];
+#pragma unroll
+        for (int i = 0; i < GROUPS; ++i)
+#pragma unroll
+          for (int j = 0; j < 16; ++j) sum[i][j] = 0.f;
+#pragma unroll 1
+        for (unsigned v = u; v < seg_hi; v += CHAIN_KB, ++seg) {
+          const int buf = seg & 1;
+          ok = mbar_wait(&acc_full[buf], (uint32_t)(seg >> 1) & 1u);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t from = tmem_acc + (uint32_t)(buf * tt + c_lo) + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+          for (int i = 0; i < GROUPS; ++i) {
+            if (c_lo + 16 * i >= c_hi) break;
+            uint32_t va[16];
+            tmem_ld16(from + 16u * i, va);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[i][j] += __uint_as_float(va[j]);
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(acc_empty_even[buf]);
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int i = 0; i < GROUPS; ++i)
+          if (c_lo + 16 * i < c_hi) store16(0, c_lo + 16 * i, [&](int j) { return sum[i][j]; });
+      } else {
+        const int buf = seg % P.nbuf;
+        if (!dry) {
+          ok = mbar_wait(&acc_full[buf], (uint32_t)(seg / P.nbuf) & 1u);
+          if (!ok) break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+        for (int a = 0; a < 2; ++a) {
+          const uint32_t lane_base = tmem_acc + (uint32_t)((buf * 2 + a) * tt) + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+          for (int c0 = c_lo; c0 < c_hi; c0 += 16) {       // rolled, as in the one-CTA kernel
+            uint32_t va[16];
+            tmem_ld16(lane_base + (uint32_t)c0, va);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            store16(a, c0, [&](int j) { return __uint_as_float(va[j]); });
           }
         }
+        if (dry) {                         // the same segment again, for real
+          dry = false;
+          continue;
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acc_empty_even[buf]);
+        ++seg;
       }
-      if (dry) {                         // the same segment again, for real
-        dry = false;
-        continue;
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(acc_empty_even[buf]);
-      ++seg;
       u = seg_hi;
     }
     if (!ok) atomicExch(&s_error, 1);
@@ -681,6 +740,7 @@ int g_tune_epi_narrow = 0;  // 1, 2, 4: epilogue warps per lane quarter for 128-
 int g_tune_no_pair2 = 0;    // 1 = no CTA-pair kernel; 2 = not for 65 to 128 tokens
 int g_tune_pair_min = 0;    // > 0: fewest rows for the CTA-pair kernel
 int g_tune_epi_dry = 1;
+int g_tune_short_sums = 0;  // 1 = the CTA-pair kernel always sums in short chains, from 65 rows up
 int g_tune_no_wide = 0;      // 1 = 128 weight rows per CTA also for wide token tiles
 int g_tune_traffic_div = 8; // split <= K_in / (div * tokens)
 
@@ -753,7 +813,8 @@ int tc_init_driver(char *err, size_t errlen) {
     const size_t smem = (size_t)d.smem_optin - 1024;       // as many stages as fit, see gemm_tc()
     d.pair_clusters = 0;
     if ((size_t)d.smem_optin >= (size_t)3 * (2 * PAIR_PART_BYTES + 256 * BK * 2) + 2048 &&
-        cudaFuncSetAttribute(gemm_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
+        cudaFuncSetAttribute(gemm_tc_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+        cudaFuncSetAttribute(gemm_tc_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(2 * (d.num_sms / 2));
       cfg.blockDim = dim3(PAIR_THREADS);
@@ -766,7 +827,7 @@ int tc_init_driver(char *err, size_t errlen) {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel, &cfg) == cudaSuccess && n > 0)
+      if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<false>, &cfg) == cudaSuccess && n > 0)
         d.pair_clusters = n < d.num_sms / 2 ? n : d.num_sms / 2;
       (void)cudaGetLastError();
     }
@@ -794,6 +855,7 @@ void tc_set_tuning(int key, int value) {
   if (key == 18) g_tune_pair_min = value;
   if (key == 21) g_tune_epi_dry = value;
   if (key == 22) attn_mma_set_chunks(value);
+  if (key == 23) g_tune_short_sums = value;
   if (key == 2) g_tune_max_split = value;
   if (key == 3) g_tune_no_streamk = value;
   if (key == 6) g_tune_late_w = value;
@@ -879,7 +941,7 @@ int tc_streamk_ctas(int n_tiles, int kblocks, int tokens, int max_slots, int *sl
 
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
                     float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
-                    SplitIn *out) {
+                    SplitIn *out, bool short_sums) {
   if (!use_current_device()) return cudaErrorInitializationError;
   if (!tc_supported(m, K_in) || R < 1 || ((uintptr_t)X.hi & 15u) || ((uintptr_t)X.lo & 15u))
     return cudaErrorInvalidValue;
@@ -921,18 +983,35 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   // 5.53 against 5.43, 80 rows 5.25 against 4.48, where the one-CTA form uses an 80-token tile;
   // with 32- and 64-token tiles the pair form measured 13-15 % slower at 16 to 64 rows, where two
   // independent CTAs per SM overlap each other's start and end).
-  const int pair_min_rows = g_tune_pair_min > 0 ? g_tune_pair_min : 113;
+  short_sums = short_sums || g_tune_short_sums != 0;
+  const int pair_min_rows = short_sums ? 65 : (g_tune_pair_min > 0 ? g_tune_pair_min : 113);
   if (pair && R >= pair_min_rows && !(g_tune_no_pair2 & 1) && g_pair_clusters > 0 && split == 0 &&
-      out != nullptr && max_slots >= 2 && m.n <= 3 && (R > 128 || !(g_tune_no_pair2 & 2))) {
-    const int q0 = (m.n_out[0] + PAIR_ROWS - 1) / PAIR_ROWS, q1 = m.n > 1 ? (m.n_out[1] + PAIR_ROWS - 1) / PAIR_ROWS : 0,
-              q2 = m.n > 2 ? (m.n_out[2] + PAIR_ROWS - 1) / PAIR_ROWS : 0;
+      out != nullptr && max_slots >= 2 && m.n <= 3 && (R > 128 || short_sums || !(g_tune_no_pair2 & 2))) {
+    const int zt = (R + 255) / 256, KB = K_in / BK;
+    // Short chains: prompt forwards, which take the place of forwards of 64 rows; and where several token tiles
+    // would sum over more of K than with one CTA per tile, whose split factor makes more parts (300 rows,
+    // 27648 x 5120: 9.4e-6 against 5.7e-6, 0.6e-6 in chains).
+    auto tiles_of = [&](int rows) {
+      int n = 0;
+      for (int i = 0; i < m.n; ++i) n += (m.n_out[i] + rows - 1) / rows;
+      return n;
+    };
+    bool chain = short_sums;
+    if (R > 256 && !chain) {
+      const int one = wide ? wave_split(tiles_of(2 * BM) * ztiles, KB, R, 1, g_num_sms)
+                           : wave_split(tiles_of(BM) * ztiles, KB, R, tc_default_split(tiles_of(BM), KB, R), 2 * g_num_sms);
+      const int run = (tiles_of(PAIR_ROWS) * zt * KB + g_pair_clusters - 1) / g_pair_clusters;
+      chain = (run < KB ? run : KB) > (KB + one - 1) / one;
+    }
+    const int rows = chain ? CHAIN_ROWS : PAIR_ROWS;
+    const int q0 = (m.n_out[0] + rows - 1) / rows, q1 = m.n > 1 ? (m.n_out[1] + rows - 1) / rows : 0,
+              q2 = m.n > 2 ? (m.n_out[2] + rows - 1) / rows : 0;
     // Token tiles: equal up to 32 rows (the MMA's N follows the tile, so 300 rows cost 320 and not 512),
     // all in one launch, the token tiles of a weight tile next to one another in the deal of units:
     // the clusters that share a weight tile then read it at about the same time.
-    const int zt = (R + 255) / 256;
     int ptt = ((R + zt - 1) / zt + 31) / 32 * 32;
-    if (ptt < 128) ptt = 128;
-    const int n_tiles = (q0 + q1 + q2) * zt, KB = K_in / BK;
+    if (ptt < 128 && !chain) ptt = 128;
+    const int n_tiles = (q0 + q1 + q2) * zt;
     const long long units = (long long)n_tiles * KB;
     long long g = g_pair_clusters;
     if (g > units / 8) g = units / 8;
@@ -951,7 +1030,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
       P.kblocks = KB;
       P.tt = ptt;
       P.bn = ptt;
-      P.nbuf = ptt <= 128 ? 2 : 1;
+      P.nbuf = chain || ptt <= 128 ? 2 : 1;
       P.ztiles = zt;
       P.sk_ctas = (int)g;
       P.sk_units = (unsigned)units;
@@ -964,11 +1043,11 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
         const int j = i < m.n ? i : 0;
         if (!get_map(m.W[j], m.n_out[j], K_in, BM, &mw[i])) return cudaErrorInvalidValue;
       }
-      SplitIn si{Y, slots_of(g), split_stride, ldy, (unsigned)g, (unsigned)units, (unsigned)KB, 2u};
+      SplitIn si{Y, slots_of(g), split_stride, ldy, (unsigned)g, (unsigned)units, (unsigned)KB, chain ? 1u : 2u};
       si.sk_zt = (unsigned)zt;
       si.sk_tt = (unsigned)ptt;
       bool ragged = false;
-      for (int i = 0; i + 1 < m.n; ++i) ragged = ragged || (m.n_out[i] % PAIR_ROWS) != 0;
+      for (int i = 0; i + 1 < m.n; ++i) ragged = ragged || (m.n_out[i] % rows) != 0;
       if (ragged) {
         si.sk_m0 = (unsigned)P.n0;
         si.sk_m1 = m.n > 2 ? (unsigned)(P.n0 + P.n1) : 0xFFFFFFFFu;
@@ -976,14 +1055,14 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
         si.sk_t1 = (unsigned)(q0 + q1);
       }
       *out = si;
-      const int stage = 2 * PAIR_PART_BYTES + ptt * BK * 2;
+      const int stage = (chain ? 1 : 2) * PAIR_PART_BYTES + ptt * BK * 2;
       P.stages = (g_smem_optin - 2048) / stage < PAIR_MAX_STAGES ? (g_smem_optin - 2048) / stage : PAIR_MAX_STAGES;
       CUtensorMap mx, mxlo;
       if (!get_map(X.hi, x_rows_alloc, K_in, ptt / 2, &mx)) return cudaErrorInvalidValue;
       if (!get_map(X.lo, x_rows_alloc, K_in, ptt / 2, &mxlo)) return cudaErrorInvalidValue;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)(2 * g));
-      cfg.blockDim = dim3(PAIR_THREADS);
+      cfg.blockDim = dim3(chain ? CHAIN_THREADS : PAIR_THREADS);
       cfg.dynamicSmemBytes = (size_t)P.stages * stage + 1024;
       cfg.stream = L.st;
       cudaLaunchAttribute attr[2];
@@ -996,7 +1075,8 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
       cfg.attrs = attr;
       cfg.numAttrs = 2;
       ++g_launches;
-      return cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel, mw[0], mw[1], mw[2], mx, mxlo, P);
+      return chain ? cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<true>, mw[0], mw[1], mw[2], mx, mxlo, P)
+                   : cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<false>, mw[0], mw[1], mw[2], mx, mxlo, P);
     }
     memset(&P, 0, sizeof(P));
     P.tt = tt; P.ztiles = ztiles; P.Y = Y; P.ldy = ldy; P.R = R; P.bn = bn; P.tmem_cols = cols;

@@ -307,7 +307,8 @@ int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct,
     const int slots = fit < (size_t)MAX_SPLIT ? (int)fit : MAX_SPLIT;
     const int tb = time_begin(c, KOALA_CLS_GEMM_TC, wbytes);
     SplitIn res;
-    CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, direct ? 1 : 0, stride, c->status, slots, &res));
+    CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, direct ? 1 : 0, stride, c->status, slots, &res,
+                   c->ingest_blocks > 0));
     time_end(c, tb);
     if (out) *out = res;
   } else {
