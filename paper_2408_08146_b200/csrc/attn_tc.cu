@@ -30,7 +30,6 @@
 namespace koala {
 
 bool tc_get_map(const void *ptr, int rows, int K_in, int box_rows, CUtensorMap *out);
-int tc_smem_optin();
 int tc_num_sms();
 
 namespace {
@@ -54,6 +53,15 @@ template <bool DUP> struct Lay {
   static constexpr int P = V + NST * 2 * SUB;
   static constexpr int BYTES = P + NP * PB;
 };
+// The kernel's only static shared variables.  They come first, then the gap up to the 1 KB boundary that the
+// buffers start at: the two share 1 KB, so that two CTAs of the 112 KB form fit on an SM to the byte.
+struct alignas(16) SyncVars {
+  uint64_t q_full, k_full[NKV_MAX], k_empty[NKV_MAX], v_full[NKV_MAX], v_empty[NKV_MAX], s_full[2], p_full[2], pv_done[2], drain_bar;
+  uint32_t tmem_base_slot;
+  int s_error;
+};
+static_assert(sizeof(SyncVars) <= 1024, "the static variables and the alignment gap share 1 KB");
+template <bool DUP> constexpr unsigned SMEM_BYTES = Lay<DUP>::BYTES + 1024 - (unsigned)sizeof(SyncVars);
 constexpr int THREADS = 192;
 constexpr int E_INVALID = 1, E_TIMEOUT = 6;
 constexpr int TMEM_COLS = 256;               // S: 2 x 64 columns, O: 128 columns
@@ -128,7 +136,6 @@ struct AttnParams {
   bf16 *out, *out_lo;      // [R][n_heads * 128]
   int rows_per_seq, n_heads, S_max, chunks, chunk_bits;
   int longest_first;       // 1: grid slot y / n_heads takes the sequence with that rank in descending cache length
-  unsigned smem_bytes;     // dynamic shared memory of the launch
   int early;               // 1: the plan and the cached context may be read before the dependency wait
   int dry_pass;            // 1: the row warps make a dry pass over the tile loop body before the dependency wait
   int *status;
@@ -155,16 +162,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   typedef Lay<DUP> LY;
   constexpr int NST = LY::NST, NP = LY::NP;
   extern __shared__ unsigned char smem_raw[];
-  __shared__ uint64_t q_full, k_full[NKV_MAX], k_empty[NKV_MAX], v_full[NKV_MAX], v_empty[NKV_MAX], s_full[2], p_full[2], pv_done[2], drain_bar;
-  __shared__ uint32_t tmem_base_slot;
-  __shared__ int s_error;
+  __shared__ SyncVars sync;
+  auto &q_full = sync.q_full, &drain_bar = sync.drain_bar;
+  auto &k_full = sync.k_full, &k_empty = sync.k_empty, &v_full = sync.v_full, &v_empty = sync.v_empty;
+  auto &s_full = sync.s_full, &p_full = sync.p_full, &pv_done = sync.pv_done;
+  auto &tmem_base_slot = sync.tmem_base_slot;
+  auto &s_error = sync.s_error;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t raw = smem_u32(smem_raw);
   unsigned char *sm = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   const uint32_t sb = smem_u32(sm);
-  // the launcher counts on the static variables and the alignment gap sharing 1 KB (see there)
-  if (sb + LY::BYTES > raw + P.smem_bytes) {
+  if (sb + LY::BYTES > raw + SMEM_BYTES<DUP>) {       // the static variables are not where SyncVars counts on them
     if (threadIdx.x == 0 && P.status) atomicMax(P.status, E_INVALID);
     return;
   }
@@ -677,8 +686,7 @@ int attn_tc_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms)
 }
 
 bool attn_tc_supported(int rows_per_seq, int head_dim, int S_max) {
-  return head_dim == DH && rows_per_seq >= g_attn_tc_min_rows && rows_per_seq <= 128 &&
-         tc_smem_optin() >= Lay<false>::BYTES + 1024 && S_max >= 1;
+  return head_dim == DH && rows_per_seq >= g_attn_tc_min_rows && rows_per_seq <= 128 && S_max >= 1;
 }
 
 cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const void *k_cache, const void *v_cache,
@@ -697,7 +705,7 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
     return cudaErrorInvalidValue;
   const int longest_first = (B > 1 && B <= 32 && (long long)chunks * B * n_heads > (dup ? 2 : 1) * tc_num_sms()) ? 1 : 0;
   AttnParams P{plan, (bf16 *)out.hi, (bf16 *)out.lo, rows_per_seq, n_heads, S_max, chunks,
-               31 - __builtin_clz((unsigned)chunks), longest_first, 0u, early ? 1 : 0, g_attn_tc_dry_pass, status};
+               31 - __builtin_clz((unsigned)chunks), longest_first, early ? 1 : 0, g_attn_tc_dry_pass, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, n_heads * B);
   cfg.blockDim = dim3(THREADS);
@@ -711,27 +719,28 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chunks > 1 ? 2 : 1;
-  // Static variables (barriers) come first, then the gap up to a 1 KB boundary: the two share 1 KB, so that
-  // two CTAs of the 112 KB form fit on an SM to the byte.
-  static SmemOptIn optin[4];
-  static size_t static_bytes[4] = {};
-  auto go = [&](auto *kern, int form, size_t need) -> cudaError_t {
-    if (static_bytes[form] == 0) {                       // the same value whichever thread comes first
-      cudaFuncAttributes fa;
-      const cudaError_t e = cudaFuncGetAttributes(&fa, (const void *)kern);
-      if (e != cudaSuccess) return e;
-      static_bytes[form] = fa.sharedSizeBytes;
-    }
-    if (static_bytes[form] > 1024) return cudaErrorInvalidValue;
-    P.smem_bytes = (unsigned)(need + 1024 - static_bytes[form]);
-    cfg.dynamicSmemBytes = P.smem_bytes;
-    const cudaError_t e = optin[form].ensure((const void *)kern, P.smem_bytes);
-    if (e != cudaSuccess) return e;
+  auto go = [&](auto *kern, unsigned smem) -> cudaError_t {
+    cfg.dynamicSmemBytes = smem;
     ++g_launches;
     return cudaLaunchKernelEx(&cfg, kern, tmQh, tmQl, tmK, tmV, P);
   };
-  if (dup) return chunks == 1 ? go(tree_attn_tc_kernel<true, true>, 0, Lay<true>::BYTES) : go(tree_attn_tc_kernel<true, false>, 1, Lay<true>::BYTES);
-  return chunks == 1 ? go(tree_attn_tc_kernel<false, true>, 2, Lay<false>::BYTES) : go(tree_attn_tc_kernel<false, false>, 3, Lay<false>::BYTES);
+  if (dup) return chunks == 1 ? go(tree_attn_tc_kernel<true, true>, SMEM_BYTES<true>) : go(tree_attn_tc_kernel<true, false>, SMEM_BYTES<true>);
+  return chunks == 1 ? go(tree_attn_tc_kernel<false, true>, SMEM_BYTES<false>) : go(tree_attn_tc_kernel<false, false>, SMEM_BYTES<false>);
+}
+
+// Once per device (tc_init_driver): whether the kernels can run as laid out, and their shared-memory limit.
+bool attn_tc_prepare(int smem_optin) {
+  if (smem_optin < Lay<false>::BYTES + 1024) return false;
+  const void *kern[4] = {(const void *)tree_attn_tc_kernel<true, true>, (const void *)tree_attn_tc_kernel<true, false>,
+                         (const void *)tree_attn_tc_kernel<false, true>, (const void *)tree_attn_tc_kernel<false, false>};
+  for (int i = 0; i < 4; ++i) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern[i]) != cudaSuccess || fa.sharedSizeBytes != sizeof(SyncVars)) return false;
+    if (cudaFuncSetAttribute(kern[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(i < 2 ? SMEM_BYTES<true> : SMEM_BYTES<false>)) != cudaSuccess)
+      return false;
+  }
+  return true;
 }
 
 }  // namespace koala

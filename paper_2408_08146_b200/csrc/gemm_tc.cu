@@ -774,6 +774,7 @@ bool tc_get_map(const void *ptr, int rows, int K_in, int box_rows, CUtensorMap *
 }
 int tc_smem_optin() { return use_current_device() ? g_smem_optin : 0; }
 int tc_num_sms() { return use_current_device() ? g_num_sms : 0; }
+bool attn_tc_prepare(int smem_optin);
 
 // Prepares the calling thread's current device (once per device) and remembers it for the
 // launchers that follow on this thread.
@@ -831,6 +832,10 @@ int tc_init_driver(char *err, size_t errlen) {
         d.pair_clusters = n < d.num_sms / 2 ? n : d.num_sms / 2;
       (void)cudaGetLastError();
     }
+  }
+  if (!attn_tc_prepare(d.smem_optin)) {
+    snprintf(err, errlen, "the attention kernels' shared memory is not laid out as they count on");
+    return 1;
   }
   d.ready = true;
   g_dev[dev] = d;
