@@ -12,7 +12,9 @@ constexpr int FPW = 4;       // output features per warp
 constexpr int ROWS = 16;     // X rows per block
 constexpr int KC = 512;      // K elements staged per step
 constexpr int WARPS = 8;
-constexpr double SMALL_MACS = 4e8;   // multiply-adds up to which the small kernel is taken
+// Multiply-adds up to which the small kernel is taken (see gemm_simt).
+constexpr int FEW_ROWS = 16;
+constexpr double SMALL_MACS_FEW_ROWS = 4e8, SMALL_MACS = 1e8;
 
 template <typename T>
 __global__ void __launch_bounds__(WARPS * 32)
@@ -169,14 +171,16 @@ cudaError_t gemm_simt(Launch L, int dtype, Operand X, GemmMats m, int K_in, int 
                       int ldy) {
   const int n0 = m.n_out[0], n1 = m.n > 1 ? m.n_out[1] : 0, n2 = m.n > 2 ? m.n_out[2] : 0;
   const int ntot = n0 + n1 + n2;
-  // The small kernel reads a weight row once per RT rows of X and X once per block of eight features,
-  // all from L1 / L2; it is taken while that traffic is a few hundred KB per SM (the tiny configurations,
-  // batches of them, short heads); beyond that the staged kernel's reuse wins.
+  // The small kernel reads a weight row once per RT rows of X and X once per block of eight features, all from
+  // L1 / L2; up to 16 rows it is taken while that is a few hundred KB per SM, with more rows, where the staged
+  // kernel's tile of 16 rows is full and its reuse counts, only for the smallest matrices.  (bf16 forwards whose
+  // F is no multiple of 64, small against staged: hidden 1024, 128 rows 700 / 391 us; 1536, 40 rows 557 / 388;
+  // 2048, 24 rows 611 / 502; 4096, 8 rows 841 / 970.)
   const size_t esz = dtype == 0 ? 4 : 2;
   const bool aligned = (K_in & 3) == 0 && ((uintptr_t)X.hi % (4 * esz)) == 0 && ((uintptr_t)X.lo % (4 * esz)) == 0 &&
                        ((uintptr_t)m.W[0] % (4 * esz)) == 0 && (m.n < 2 || ((uintptr_t)m.W[1] % (4 * esz)) == 0) &&
                        (m.n < 3 || ((uintptr_t)m.W[2] % (4 * esz)) == 0);
-  if (aligned && (double)R * K_in * ntot <= SMALL_MACS) {
+  if (aligned && (double)R * K_in * ntot <= (R <= FEW_ROWS ? SMALL_MACS_FEW_ROWS : SMALL_MACS)) {
     auto go = [&](auto tag, auto rt) {
       typedef decltype(tag) T;
       constexpr int RT = decltype(rt)::value;

@@ -133,3 +133,11 @@ def test_cuda_core_gemm_of_few_rows(shape, pair):
     torch.cuda.synchronize()
     ref = full.cpu().numpy() @ w.double().cpu().numpy().T
     assert np.abs(y.cpu().numpy() - ref).max() <= 2e-5 * np.sqrt(K) + 1e-6
+
+
+@pytest.mark.parametrize("shape", [(16, 4096, 4096), (17, 4096, 4096), (17, 1024, 4096), (24, 1001, 4100), (128, 512, 1024), (128, 1000, 1028)])
+def test_cuda_core_gemm_on_both_sides_of_the_small_kernel(shape):
+    M, N, K = shape
+    x, w, ref = _inputs(M, N, K)
+    err = np.abs(koala_gemm_bf16(x, w, False).cpu().numpy() - ref).max()
+    assert err <= 2e-5 * np.sqrt(K) + 1e-6, f"max err {err}"      # fp32 accumulation of K products
