@@ -1,6 +1,6 @@
-// Tree-masked attention on CUDA cores: at most four query rows per sequence (one-token steps, chain drafts)
-// of bf16 caches with head_dim 128, and every size of the fp32 and head_dim 64 configurations, whose rows
-// are taken in groups (grid z).
+// Tree-masked attention on CUDA cores: one or two query rows per sequence (one-token steps) of bf16 caches
+// with head_dim 128, and every size of the fp32 and head_dim 64 configurations, whose rows are taken in
+// groups (grid z).
 //
 // With so few rows the cached keys and values are all there is to move: 512 bytes per key and head
 // against a few hundred multiply-adds, so the products run in fp32 on the CUDA cores (the tensor-core
@@ -273,8 +273,8 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
 
 }  // namespace
 
-// Rows per CTA: in bf16 at head_dim 128, where up to four rows come here, all of them; elsewhere one while
-// that makes few CTAs (latency), four (two with fp32 rows of 128) where the cache would be re-read too often.
+// Rows per CTA: in bf16 at head_dim 128 one, two or (tensor cores switched off) groups of four; elsewhere one
+// while that makes few CTAs (latency), four (two with fp32 rows of 128) where the cache would be re-read too often.
 // Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the launch
 // within what is resident at once (two CTAs per SM up to two rows, else one; clusters of eight do not
 // fill every GPC, hence seven eighths), and at least `min_keys` of capacity per chunk: two tiles, eight

@@ -233,8 +233,10 @@ cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, co
                                bool early);
 
 // attn_few.cu : any dtype, head_dim 64 or 128, on CUDA cores; where the tensor-core kernels apply, up to ATTN_FEW_ROWS
-// rows per sequence
-constexpr int ATTN_FEW_ROWS = 4;
+// rows per sequence (eight layers, context 2000, CUDA cores / mma.sync, us per forward: 32 heads, one sequence 1 row
+// 780 / 788, 2 rows 795 / 788, 3 rows 860 / 793; four sequences 979 / 927, 997 / 933, 1251 / 940; 40 heads, four
+// sequences 1335 / 1380, 1307 / 1385, 1855 / 1378: with three rows a CTA holds four and has an SM to itself)
+constexpr int ATTN_FEW_ROWS = 2;
 cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
                                Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early);
 

@@ -411,3 +411,14 @@ def test_topk_of_rows_with_ties_and_extremes(V, k):
             assert np.abs(lp[r] - ref).max() <= 2e-6 * (1 + np.abs(ref).max())     # fp32 sum of V terms, log of it
     assert eng.device_status() == 0
     eng.close()
+
+
+@pytest.mark.parametrize("N,B,n_heads,context,S_max", [
+    (3, 1, 32, 900, 1024), (4, 4, 32, 500, 640),      # just past the rows that the CUDA cores take
+    (1, 5, 32, 1400, 2048), (2, 5, 32, 700, 1024),    # one row, more (sequence, head) pairs than SMs: two key chunks
+    (5, 5, 32, 1900, 2048), (5, 5, 32, 900, 1024),    # mma.sync a tenth past two CTAs per SM: two chunks from 2048 keys
+    (6, 10, 32, 1000, 4096),                          # beyond that from 4096
+    (33, 5, 32, 600, 1024), (32, 5, 32, 600, 1024),   # tcgen05: two chunks there with more than 32 rows
+])
+def test_attention_chunks_beyond_one_round_of_ctas(N, B, n_heads, context, S_max):
+    _attention_case(N, B, n_heads, context, S_max)
