@@ -278,7 +278,11 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
 // Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the launch
 // within what is resident at once (two CTAs per SM up to two rows, else one; clusters of eight do not
 // fill every GPC, hence seven eighths), and at least `min_keys` of capacity per chunk: two tiles, eight
-// in the small configurations, where the cluster's two barriers cost more than a few tiles.
+// in the small configurations, where the cluster's two barriers cost more than a few tiles.  Single rows of bf16
+// caches take two chunks of at least 1024 keys also where not all are resident at once: one chunk leaves most
+// SMs a single CTA, which cannot draw the SM's share of the bandwidth (160 pairs, four layers: context 2000
+// 602 -> 544 us with equal, 515 -> 475 with ragged lengths, context 4000 776 -> 656 and 627 -> 552; 256 pairs
+// 609 -> 584, 563 -> 526; two rows: 1 % either way with equal lengths).
 cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
                                Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early) {
   if (rows_per_seq < 1 || (head_dim != 64 && head_dim != 128)) return cudaErrorInvalidValue;
@@ -290,6 +294,7 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
     const int room = (RT <= 2 ? 2 : 1) * num_sms * 7 / 8, min_keys = (bf && DH == 128 ? 2 : 8) * TILE;
     int chunks = 1;
     while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads * groups <= room && 2 * chunks * min_keys <= S_max) chunks *= 2;
+    if (bf && DH == 128 && RT == 1 && chunks == 1 && S_max >= 2048) chunks = 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(chunks, n_heads * B, groups);
     cfg.blockDim = dim3(WARPS * 32);
