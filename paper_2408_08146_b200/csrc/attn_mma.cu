@@ -3,7 +3,7 @@
 // One CTA = one (key chunk, group of 16 query rows, head, sequence) with four warps that split
 // every 64-key tile among themselves.  The sequence's keys are cut into `chunks` ranges of whole
 // tiles from the device-side length, so the grid is fixed by host-known sizes while the work
-// follows the real context length; short contexts use a single chunk and need no second kernel.
+// follows the real context length.
 // K and V tiles stream through shared memory with cp.async (three stages,
 // 16-byte vector loads, XOR-swizzled rows); scores S = Q K^T and the update O += P V run on
 // mma.sync m16n8k16 with fp32 accumulators.  Q and P enter the MMAs as bf16 pairs (value +
@@ -395,12 +395,15 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
 
 }  // namespace
 
-// Key chunks per (sequence, head, row group) = cluster size: the largest of 1, 2, 4, 8 that keeps the
-// launch within about what is resident at once (two CTAs of 96 KB per SM, and a tenth more: the late
-// CTAs are short; clusters of eight do not fill every GPC, hence seven eighths there), at least one tile
-// of capacity per chunk.  (13B shape, four sequences, 160 sequence-head pairs, 2 x 5 launches per
-// iteration: 17.0 / 16.4 / 17.1 ms with 1 / 2 / 4 chunks; 7B, five rows, 36 launches: 4.30 / 4.13 /
-// 3.97 / 3.89 ms with 1 / 2 / 4 / 8.)
+// Key chunks per (sequence, head, row group) = cluster size: the largest of 1, 2, 4, 8 that keeps the launch
+// within what is resident at once (two CTAs of 96 KB per SM; clusters of eight do not fill every GPC, hence
+// seven eighths there), at least one tile of capacity per chunk.  One sequence of 32 heads, context 2000, four
+// layers: 528 / 460 / 430 / 418 us with 1 / 2 / 4 / 8.  Past that more chunks pay where lengths are ragged (the host
+// does not know them) and chunks long: a tenth more CTAs from 2048 keys of capacity, and two chunks of whatever
+// fits in one round from 4096.  Fewer / more chunks, five rows, four layers, equal and ragged lengths: 80 pairs
+// at context 2000 318 / 339 and 300 / 282 us, at 600 253 / 281 and 244 / 258; 160 pairs at 2000 568 / 592 and
+// 553 / 490, at 600 (eight layers) 966 / 1050 and 986 / 1008; 192 pairs at 4000 735 / 785 and 705 / 583, at 2000
+// 568 / 613 and 554 / 507; 320 pairs at 4000 1055 / 935 and 712 / 707.
 int g_attn_mma_chunks = 0;     // > 0: this many key chunks whatever the shape (A/B runs)
 void attn_mma_set_chunks(int chunks) { g_attn_mma_chunks = chunks; }
 int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms) {
@@ -410,7 +413,10 @@ int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms
     while (2 * c <= g_attn_mma_chunks && 2 * c <= 8 && 2 * c * 64 <= S_max) c *= 2;
     return c;
   }
-  while (c < 8 && 2 * c * rgs * B * n_heads <= (c == 4 ? 2 * num_sms * 7 / 8 : 2 * num_sms * 11 / 10) && 2 * c * 64 <= S_max) c *= 2;
+  const int ctas = rgs * B * n_heads, room = 2 * num_sms;
+  auto limit = [&](int chunks) { return chunks == 8 ? room * 7 / 8 : (S_max >= 2048 ? room * 11 / 10 : room); };
+  while (c < 8 && 2 * c * ctas <= limit(2 * c) && 2 * c * 64 <= S_max) c *= 2;
+  if (c == 1 && ctas <= room * 11 / 10 && S_max >= 4096) c = 2;
   return c;
 }
 

@@ -415,10 +415,30 @@ def test_topk_of_rows_with_ties_and_extremes(V, k):
 
 @pytest.mark.parametrize("N,B,n_heads,context,S_max", [
     (3, 1, 32, 900, 1024), (4, 4, 32, 500, 640),      # just past the rows that the CUDA cores take
-    (1, 5, 32, 1400, 2048), (2, 5, 32, 700, 1024),    # one row, more (sequence, head) pairs than SMs: two key chunks
+    (2, 5, 32, 700, 1024),                            # two rows, more (sequence, head) pairs than SMs
     (5, 5, 32, 1900, 2048), (5, 5, 32, 900, 1024),    # mma.sync a tenth past two CTAs per SM: two chunks from 2048 keys
     (6, 10, 32, 1000, 4096),                          # beyond that from 4096
     (33, 5, 32, 600, 1024), (32, 5, 32, 600, 1024),   # tcgen05: two chunks there with more than 32 rows
 ])
 def test_attention_chunks_beyond_one_round_of_ctas(N, B, n_heads, context, S_max):
     _attention_case(N, B, n_heads, context, S_max)
+
+
+def test_one_row_of_more_pairs_than_sms_in_two_key_chunks():
+    cfg = reduced(T7_EAGLE, 1, K=1, N=1, D=1, topk=1, B=5, H=4096, n_heads=32, F=2048, V=2048, S_max=2048, prompt_len=1900)
+    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
+    eng.target_k.copy_(random_kv(cfg, "target_k", cfg.L, DEV))
+    eng.target_v.copy_(random_kv(cfg, "target_v", cfg.L, DEV))
+    lens = [1900, 1, 64, 700, 1023]
+    for b in range(cfg.B):
+        orc.target_k[0][b][...] = kv_to_oracle(eng.target_k, 0, b, np.float32)
+        orc.target_v[0][b][...] = kv_to_oracle(eng.target_v, 0, b, np.float32)
+        orc.seq_len[b] = lens[b]
+    eng.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    toks = [[3 + b] for b in range(cfg.B)]
+    eng.koala_verify(_tree_arrays(eng, toks, [[-1]] * cfg.B))
+    orc.verify([(t, [-1]) for t in toks])
+    for b in range(cfg.B):
+        assert_close(eng.buffers()["verify_hid"][b:b + 1].cpu().numpy(), orc.verify_hid[b][:1], cfg.dtype, f"hidden {b}")
+    assert eng.device_status() == 0 and eng.check_guards()[1] == 0
+    eng.close()
