@@ -671,9 +671,13 @@ void attn_tc_set_chunks(int chunks) { g_attn_tc_chunks = chunks; }
 void attn_tc_set_dry_pass(int on) { g_attn_tc_dry_pass = on ? 1 : 0; }
 
 // Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the CTA count
-// within the SMs, each chunk with at least 128 keys of capacity.  Up to 64 rows, where two CTAs share an SM:
-// two chunks where one would leave the SMs half empty (13B shape, four sequences, 160 pairs: 17.9 -> 17.7 ms
-// per iteration; more chunks where they fit twice over are slower, 7B at batch 1 5.09 -> 5.29 with eight).
+// within the SMs, each chunk with at least 128 keys of capacity.  From 33 to 64 rows, where two CTAs share an
+// SM, two chunks up to a tenth more pairs than SMs: a few SMs with two whole sequences' CTAs are what the
+// launch waits for then.  One / two chunks, 64 rows, context 2000, eight layers, equal and ragged lengths: 156
+// pairs 3695 / 3803 and 3553 / 3522 us, 160 pairs 3258 / 3356 and 3220 / 3116 (40 heads), 2904 / 3010 and
+// 2865 / 2782 (32 heads); 176 pairs 2060 / 2160 and 1959 / 1954, 200 pairs 4214 / 4321 and 4097 / 4102; 32 rows,
+// 160 pairs 1824 / 1949 and 1803 / 1901.  13B shape, four ragged sequences: 17.9 -> 17.5 ms per iteration.
+// (More chunks where they fit twice over are slower, 7B at batch 1 5.09 -> 5.29 ms with eight.)
 int attn_tc_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms) {
   int c = 1;
   if (g_attn_tc_chunks > 0) {
@@ -681,7 +685,7 @@ int attn_tc_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms)
     return c;
   }
   while (c < 8 && 2 * c * B * n_heads <= num_sms && 2 * c * 128 <= S_max) c *= 2;
-  if (c == 1 && rows_per_seq <= 64 && 20 * B * n_heads <= 22 * num_sms && 256 <= S_max) c = 2;
+  if (c == 1 && rows_per_seq > 32 && rows_per_seq <= 64 && 20 * B * n_heads <= 22 * num_sms && 256 <= S_max) c = 2;
   return c;
 }
 
