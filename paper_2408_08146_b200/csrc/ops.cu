@@ -671,7 +671,6 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
       if ((P).n == 3) SPLIT_CASE(3, false, __VA_ARGS__)                           \
       if ((P).n <= 5) SPLIT_CASE(5, false, __VA_ARGS__)                           \
       if ((P).n <= 8) SPLIT_CASE(8, false, __VA_ARGS__)                           \
-      if ((P).n == 9) SPLIT_CASE(9, false, __VA_ARGS__)                           \
       SPLIT_CASE(12, false, __VA_ARGS__)                                          \
     }                                                                             \
     if ((P).n <= 3) SPLIT_CASE(3, true, __VA_ARGS__)                              \
