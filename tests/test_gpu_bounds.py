@@ -118,3 +118,24 @@ def test_a_part_of_more_than_n_tokens_is_refused():
     assert [list(x) for x in tk] == [list(x) for x in rt] and list(ln) == list(rl)
     assert eng.device_status() == 0
     eng.close()
+
+
+@pytest.mark.parametrize("dtype", [0, 1], ids=["fp32", "bf16"])
+def test_rows_wider_than_the_vectorised_kernels_take(dtype):
+    """A hidden size above 8192 goes by the row-wise kernels of any width: prompt, draft pass and verification."""
+    cfg = reduced(T7_EAGLE, 1, dtype=dtype, K=1, H=8320, n_heads=65, F=256, V=512, D=1, topk=2, N=3, S_max=128, prompt_len=6, seed=46)
+    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
+    pr = prompts(cfg)
+    eng.prefill(pr, 3)
+    orc.prefill(pr, 3)
+    eng.koala_draft(0)
+    orc.draft(0)
+    assert_close(eng.buffers()["draft_logits"][:1].cpu().numpy(), orc.draft_logits[0][:1], dtype, "draft logits")
+    eng.koala_expand_tree(0)
+    eng.koala_verify(None)
+    b = eng.buffers()
+    n = int(b["tree_n"][0])
+    orc.verify([(b["tree_tok"][0, :n].cpu().numpy(), b["tree_parent"][0, :n].cpu().numpy())])
+    assert_close(b["verify_logits"][:n].cpu().numpy(), orc.verify_logits[0], dtype, "logits")
+    assert eng.device_status() == 0 and eng.check_guards()[1] == 0
+    eng.close()
