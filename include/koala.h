@@ -148,7 +148,9 @@ typedef struct {
   int32_t draft_rows;    /* rows of draft_logits currently meaningful */
 } koala_buffer_table;
 
-/* Bytes of workspace koala_init() needs for this configuration (0 if the configuration is invalid). */
+/* Bytes of workspace koala_init() needs for this configuration (0 if the configuration is invalid).  Of it the
+ * operands and partial sums of a prompt forward of min(1024, B * S_max) rows are held by every context, whether
+ * it ingests prompts or not: some 0.4 GB at the 7B shape, batch 1. */
 size_t koala_workspace_bytes(const koala_config *cfg);
 
 /* Section 2.2 set-up: validates shapes, carves the workspace, encodes the TMA descriptors of the
@@ -186,9 +188,10 @@ int koala_verify(koala_ctx *ctx, const koala_tree *tree);
  * acceptance counters, the tree and the verification buffers are afterwards as if every part had been
  * verified as a chain, all but the last accepted in full and, with an EAGLE-style head, followed by
  * koala_draft(0) with the next prompt token as root: the caller continues with koala_accept, with the
- * lengths of the last parts (tree_n) as forced lengths.  Up to 1024 tokens go through one forward; logits
- * are formed for the last parts only.  tok: DEVICE [B][stride] prompts; len: HOST [B], copied,
- * n_parts <= len[b] <= stride (no part is empty). */
+ * lengths of the last parts (tree_n) as forced lengths.  "As if" holds up to the rounding of sums: up to 1024
+ * tokens go through one forward, whose sums are cut differently (against float64 they are at least as exact as
+ * with parts of 64 rows); logits are formed for the last parts only.  tok: DEVICE [B][stride] prompts, kept until
+ * the stream has read them; len: HOST [B], copied, n_parts <= len[b] <= stride (no part is empty). */
 int koala_ingest(koala_ctx *ctx, const int32_t *tok, int32_t stride, const int32_t *len, int32_t n_parts);
 
 /* Greedy acceptance (Section 4.1: a draft token is kept only if it equals the target's greedy

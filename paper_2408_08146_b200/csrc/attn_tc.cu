@@ -212,9 +212,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   tc_fence_after();
   const uint32_t tmem = tmem_base_slot;
 
-  // Q, the tree rows of K/V and the row plan come from earlier kernels: everything that reads them
-  // comes after the dependency wait in read_plan().  The row warps call it inside their tile loop,
-  // after a dry pass over the loop body (see there); the other threads here.
+  // Q and the K/V rows of this forward come from the kernel before: what reads them comes after the dependency
+  // wait.  With `early` the plan and the cached context are older and are read before it, except by the row warps,
+  // which call read_plan inside their tile loop, after a dry pass over the loop body (see there).
   int ctx = 0, kv_len = 0, tile_lo = 0, T = 0;
   auto read_plan = [&](bool wait) {
     if (wait) pdl_wait();
@@ -660,7 +660,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   if constexpr (!ONE) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-int g_attn_tc_min_rows = 16;   // fewer query rows per sequence than this: the mma.sync kernel
+// Fewer query rows per sequence than this: the mma.sync kernel.  (tcgen05 / mma.sync, 32 heads, eight layers, us per
+// forward: one sequence at context 2000 12 rows 829 / 808, 16 rows 834 / 817, 20 rows 843 / 879; four sequences at
+// 500 8 rows 810 / 835, 15 rows 915 / 966.  Batches would gain from eight rows on, one sequence lose.)
+int g_attn_tc_min_rows = 16;
 int g_attn_tc_chunks = 0;      // > 0: this many key chunks whatever the shape (A/B runs)
 int g_attn_tc_dry_pass = 1;
 

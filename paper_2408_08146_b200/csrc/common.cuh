@@ -197,8 +197,6 @@ cudaError_t row_epilogue(Launch L, int dtype, int mode, float *x, SplitIn P, con
                          const void *g, Operand xn, float *out_f32, RowMap out_map, int R, int H, float eps);
 cudaError_t eagle_concat(Launch L, int dtype, const float *feat_src, const int32_t *row_src,
                          const int32_t *row_tok, const void *E, Operand cat, int R, int H, int V);
-// x <- x + sum(P); xg <- T(x * g) (not normalised); sumsq[r][chunk] <- partial sums of x^2 over
-// chunks of 1024 columns (chunks = ceil(H / 1024)).  H % 4 == 0.
 // Residual SiLU-Linear blocks of several independent heads in one launch (Medusa-style heads):
 // rows [h * rows_per_head, (h + 1) * rows_per_head) belong to head h, whose partial sums start at
 // P.p = p[h] (row index local to the head) and whose bias is bias[h]:
@@ -209,6 +207,8 @@ struct HeadTab {
   int rows_per_head;
 };
 cudaError_t resblock_update(Launch L, int dtype, float *x, SplitIn P, HeadTab tab, Operand xn, int R, int H);
+// x <- x + sum(P); xg <- T(x * g) (not normalised); sumsq[r][chunk] <- partial sums of x^2 over
+// chunks of 1024 columns (chunks = ceil(H / 1024)).  H % 4 == 0.
 cudaError_t row_update(Launch L, int dtype, float *x, SplitIn P, const void *g, Operand xg, float *sumsq,
                        int R, int H);
 // q_out: rotated queries in fp32; q_pair (bf16 only, may be null): the same as a bf16 pair

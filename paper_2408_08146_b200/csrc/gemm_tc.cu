@@ -19,8 +19,8 @@
 // accumulator columns, so a tile holds up to 256 tokens and the weights are passed over once.  With
 // 256 tokens a CTA takes 256 weight rows: four MMAs per K step share the activation tile and fill two
 // accumulators (all 512 tensor-memory columns); a stage is 32 KB of weights + 64 KB of activations,
-// two stages, one CTA per SM.  From 113 rows up (as a pair) gemm_tc_pair_kernel takes over where it
-// applies: two CTAs of a cluster as one MMA unit, see there.
+// two stages, one CTA per SM.  From 113 rows up (as a pair; prompt forwards from 65) gemm_tc_pair_kernel takes over
+// where it applies: two CTAs of a cluster as one MMA unit, see there.
 // Split-K: grid.y CTAs share a weight tile and write separate partial outputs that the consumer
 // kernel sums in a fixed order (deterministic).
 // Every wait is bounded: on expiry the kernel records KOALA_E_TIMEOUT in *status, drains, frees
@@ -313,8 +313,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       const int feat = row0 + hw * BM + quarter * 32 + lane;
       float *Yp = P.Y + (size_t)slot * P.split_stride + col_off + feat;
       const uint32_t lane_base = tmem_acc + (uint32_t)((buf + hw) * P.tmem_cols) + ((uint32_t)(quarter * 32) << 16);
-      // 16 token columns per step, in a rolled loop: with eight or sixteen warps the accumulator reads
-      // of one hide behind the stores of the others, and the loop's instructions are fetched once.
+      // 16 token columns per step, in a rolled loop: the accumulator reads of one warp hide behind the stores
+      // of the others, and the loop's instructions are fetched once.
 #pragma unroll 1
       for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
         uint32_t va[16];
@@ -372,15 +372,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
 }
 
 // ------------------------------------------------------------------------------- CTA pairs
-// More than 64 tokens as a pair of activations, two CTAs of a cluster as one MMA unit
-// (cta_group::2), token tile tt = 128 or 256.  With one CTA per tile these forms are bound by what
-// L2 delivers into shared memory (128 tokens: 48 KB per 128 weight rows and K block, three times the
+// 113 tokens and more as a pair of activations, two CTAs of a cluster as one MMA unit (cta_group::2), token
+// tiles of tt = 128 to 256 rows, a multiple of 32 (several of them in one launch above 256 rows).  With one CTA
+// per tile these forms are bound by what L2 delivers into shared memory (128 tokens: 48 KB per 128 weight rows and K block, three times the
 // weight bytes; 256 tokens: 96 KB per 256 weight rows).  Here a pair of CTAs owns 512 weight rows:
 // every MMA has M = 256 (128 weight rows from each CTA) and N = tt tokens, of which each CTA loads
 // only its half (value rows and residual rows).  Per CTA and stage: weight rows
 // [a*256 + rank*128, +128) for the accumulators a = 0, 1 (2 x 16 KB) and tokens [rank*tt/2, +tt/2)
-// as value and residual rows (2 x tt/2 x 128 B): 48 KB (four stages) or 64 KB (three).  With 128
-// tokens the two accumulators take 256 tensor-memory columns and there are two sets, so the
+// as value and residual rows (2 x tt/2 x 128 B): 48 KB (four stages) at 128 tokens, 64 KB (three) at 256.  With
+// 128 tokens the two accumulators take 256 tensor-memory columns and there are two sets, so the
 // epilogue of one segment overlaps the MMAs of the next.  Every load of both CTAs is counted on
 // the even CTA's full barrier; that CTA's MMA thread issues for the pair and its commits arrive on
 // the empty / accumulator barriers of both CTAs; each CTA's epilogue warps read its own 128

@@ -1,6 +1,5 @@
 // Row-wise kernels of the decoder layers and heads: embedding gather, RMSNorm / residual
-// epilogues, RoPE + KV-cache write, SwiGLU, tree-masked attention (CUDA-core version),
-// arg-max and top-k with log-probabilities.  All statistics are fp32.
+// epilogues, RoPE + KV-cache write, SwiGLU, arg-max and top-k with log-probabilities.  All statistics are fp32.
 #include "common.cuh"
 #include "row_ops.cuh"
 

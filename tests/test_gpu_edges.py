@@ -94,7 +94,7 @@ def test_eagle_head_without_layers():
 @pytest.mark.parametrize("context", [1000, 3900])
 def test_long_context_many_key_tiles_and_chunks(context):
     """bf16, head_dim 128, one 7B-shaped layer: the attention kernel walks dozens of key tiles and,
-    at the longer context, several key chunks merged by the second kernel."""
+    at the longer context, several key chunks merged inside a cluster."""
     cfg = reduced(T7_EAGLE, 1, K=1, N=60, S_max=4096, prompt_len=context)
     eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
     eng.target_k.copy_(random_kv(cfg, "target_k", cfg.L, DEV))
@@ -345,20 +345,20 @@ def test_short_caller_trees_of_a_batch_run_only_their_rows(base, B, N, n_max):
     (4, 9, 8, 200, 512),         # more (sequence, head) pairs than parts
     (2, 1, 1, 2000, 2048),       # a single head
     (3, 5, 16, 130, 256),
-    (5, 1, 32, 777, 1024),       # five to eight rows
+    (5, 1, 32, 777, 1024),       # three to fifteen rows: mma.sync
     (8, 3, 8, 500, 1024),
     (7, 1, 2, 1900, 2048),
-    (9, 1, 32, 1000, 1024),      # nine to fifteen rows: mma.sync, chunks merged by the last arriver
+    (9, 1, 32, 1000, 1024),
     (15, 2, 8, 600, 2048),
 ])
 @pytest.mark.parametrize("kind", ["plain", "poison", "growing"])
 def test_attention_of_few_rows(N, B, n_heads, context, S_max, kind):
-    """At most eight rows per sequence: tiles dealt evenly to the CTAs, parts merged by the last arriver."""
+    """Up to fifteen rows per sequence: the CUDA-core kernel (one or two rows) and mma.sync, key chunks as a cluster."""
     _attention_case(N, B, n_heads, context, S_max, poison=kind == "poison", growing=kind == "growing")
 
 
 def test_attention_of_one_row_ragged_batch():
-    """One-node trees of a ragged batch, twice on the same engine (the arrival counters are left at zero)."""
+    """One-node trees of a ragged batch, twice on the same engine."""
     cfg = reduced(T7_EAGLE, 1, K=1, N=1, D=1, topk=1, B=4, H=1024, n_heads=8, F=2048, V=2048, S_max=1536, prompt_len=1400)
     eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
     eng.target_k.copy_(random_kv(cfg, "target_k", cfg.L, DEV))
