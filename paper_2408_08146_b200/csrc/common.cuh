@@ -379,6 +379,12 @@ cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len
 // `shift` places further on (0: the row's own; 1: the one the draft head pairs with it).
 cudaError_t plan_ingest(Launch L, PlanBufs p, IngestBlocks k, const int32_t *tok, int stride, int shift,
                         const int32_t *seq_len, int head_dim, const RopeInv &inv, const RowFill &fill, int S_max, int *status);
+// Rows of a forward whose hidden state stays in the pending buffer: pend_hid row dst[i] <- hid row src[i].
+struct IngestKeep {
+  int n;
+  int32_t src[64], dst[64];
+};
+cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, int H);
 // Rows of the sequences' last parts: verify_hid row b * N + u <- hid, xn row b * n_max + u <- T(hid).
 cudaError_t ingest_last(Launch L, int dtype, IngestBlocks k, const float *hid, float *verify_hid, Operand xn, int N, int n_max,
                         int H);

@@ -622,7 +622,7 @@ int head_rows(koala_ctx *c, const float *feat, int R) {
 // One forward of the target over prompt blocks, then of an EAGLE-style head over the positions before the last
 // parts (hidden state of a position paired with the token after it).  Besides the caches only the rows of
 // the last parts are kept, where a verification would leave them (n_max of them per sequence).
-int ingest_forward(koala_ctx *c, const IngestBlocks &k, const int32_t *tok, int stride, int n_max) {
+int ingest_forward(koala_ctx *c, const IngestBlocks &k, const IngestKeep &keep, const int32_t *tok, int stride, int n_max) {
   const koala_config &g = c->cfg;
   const int H = g.H;
   const Operand none{nullptr, nullptr};
@@ -647,6 +647,7 @@ int ingest_forward(koala_ctx *c, const IngestBlocks &k, const int32_t *tok, int 
   K_TRY(run_layers(c, c->layers, g.L, c->tk, c->tv, R, k.q, c->final_norm, none, c->mx, same, !head && !has_last));
   if (has_last) CU_TRY(ingest_last(LN(c), g.dtype, k, c->mx, c->verify_hid, c->lmin, g.N, n_max, H));
   if (!head) return KOALA_OK;
+  CU_TRY(ingest_keep(LN(c), c->t, keep, c->mx, H));
   c->ingest_blocks = hd.n;
   CU_TRY(plan_ingest(LN(c), c->p, hd, tok, stride, 1, c->seq_len, g.head_dim, c->rope_inv, fill_head(c, c->mx), g.S_max,
                      c->status));
@@ -1062,7 +1063,17 @@ int koala_ingest(koala_ctx *c, const int32_t *tok, int32_t stride, const int32_t
     if (last > n_max) n_max = last;
   }
   K_TRY(deal_blocks(k, g.B, c->ingest_rows, [&](const IngestBlocks &blk) {
-    const int rc = ingest_forward(c, blk, tok, stride, n_max);
+    // The pending rows of a sequence are those of its last part; where earlier parts were one token
+    // longer, the row after them still holds the last token of the last longer part.
+    IngestKeep keep;
+    keep.n = 0;
+    for (int v = 0; v < blk.n; ++v) {
+      const int b = blk.seq[v], row = k.len[b] / n_parts, at = (k.len[b] % n_parts) * (row + 1) - 1 - blk.start[v];
+      if (at < 0 || at >= blk.count[v] || row >= g.N) continue;
+      keep.src[keep.n] = v * blk.q + at;
+      keep.dst[keep.n++] = b * g.N + row;
+    }
+    const int rc = ingest_forward(c, blk, keep, tok, stride, n_max);
     c->ingest_blocks = 0;
     return rc;
   }));

@@ -172,6 +172,13 @@ plan_ingest_kernel(PlanBufs p, const __grid_constant__ IngestBlocks k, const int
   else fill_concat<T>(fill, r, src, tk);
 }
 
+__global__ void ingest_keep_kernel(TreeBufs t, const __grid_constant__ IngestKeep k, const float *hid, int H) {
+  pdl_launch_dependents();
+  pdl_wait();
+  for (int d = threadIdx.x; d < H; d += blockDim.x)
+    t.pend_hid[(size_t)k.dst[blockIdx.x] * H + d] = hid[(size_t)k.src[blockIdx.x] * H + d];
+}
+
 // block 0: lengths and counters; block 1 + b: sequence b's tree
 __global__ void ingest_commit_kernel(TreeBufs t, const __grid_constant__ IngestLens k, const int32_t *tok, int stride,
                                      int32_t *seq_len, int B, int N) {
@@ -542,6 +549,10 @@ cudaError_t plan_verify(Launch L, TreeBufs t, PlanBufs p, const int32_t *seq_len
 cudaError_t plan_ingest(Launch L, PlanBufs p, IngestBlocks k, const int32_t *tok, int stride, int shift,
                         const int32_t *seq_len, int head_dim, const RopeInv &inv, const RowFill &fill, int S_max, int *status) {
   return PLAN_DISPATCH(plan_ingest_kernel, dim3(k.n, k.q), p, k, tok, stride, shift, seq_len, head_dim, inv, fill, S_max, status);
+}
+cudaError_t ingest_keep(Launch L, TreeBufs t, IngestKeep k, const float *hid, int H) {
+  if (k.n == 0) return cudaSuccess;
+  return launch_k(ingest_keep_kernel, dim3(k.n), dim3(256), 0, L.st, L.pdl, t, k, hid, H);
 }
 cudaError_t ingest_commit(Launch L, TreeBufs t, IngestLens k, const int32_t *tok, int stride, int32_t *seq_len, int B, int N) {
   return launch_k(ingest_commit_kernel, dim3(1 + B), dim3(128), 0, L.st, L.pdl, t, k, tok, stride, seq_len, B, N);
