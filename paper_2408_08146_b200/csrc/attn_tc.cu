@@ -674,13 +674,16 @@ void attn_tc_set_chunks(int chunks) { g_attn_tc_chunks = chunks; }
 void attn_tc_set_dry_pass(int on) { g_attn_tc_dry_pass = on ? 1 : 0; }
 
 // Key chunks (= cluster size) per (sequence, head): the largest of 1, 2, 4, 8 that keeps the CTA count
-// within the SMs, each chunk with at least 128 keys of capacity.  From 33 to 64 rows, where two CTAs share an
-// SM, two chunks up to a tenth more pairs than SMs: a few SMs with two whole sequences' CTAs are what the
-// launch waits for then.  One / two chunks, 64 rows, context 2000, eight layers, equal and ragged lengths: 156
-// pairs 3695 / 3803 and 3553 / 3522 us, 160 pairs 3258 / 3356 and 3220 / 3116 (40 heads), 2904 / 3010 and
-// 2865 / 2782 (32 heads); 176 pairs 2060 / 2160 and 1959 / 1954, 200 pairs 4214 / 4321 and 4097 / 4102; 32 rows,
-// 160 pairs 1824 / 1949 and 1803 / 1901.  13B shape, four ragged sequences: 17.9 -> 17.5 ms per iteration.
-// (More chunks where they fit twice over are slower, 7B at batch 1 5.09 -> 5.29 ms with eight.)
+// within the SMs, each chunk with at least 128 keys of capacity.  Up to 64 rows two CTAs share an SM: two chunks
+// while they fit so (144 pairs, eight layers, context 1000, one / two chunks: 32 rows 1126 / 1099 us, 16 rows 892 /
+// 858), and up to a tenth more pairs than SMs, where a few SMs with two whole sequences are what the launch waits
+// for.  There ragged lengths, which the host does not know, gain and equal ones lose.  Equal and ragged lengths, 64
+// rows, context 2000: 156 pairs 3695 / 3803 and 3553 / 3522 us, 160 pairs 3258 / 3356 and 3220 / 3116 (40 heads),
+// 2904 / 3010 and 2865 / 2782 (32 heads); 176 pairs 2060 / 2160 and 1959 / 1954, 200 pairs 4214 / 4321 and 4097 /
+// 4102; 16 rows, four layers, 160 pairs at context 4000 720 / 783 and 706 / 611, at 2000 594 / 640 and 585 / 555;
+// 32 rows at context 1000 1824 / 1949 and 1803 / 1901: up to 32 rows only from 2048 keys of capacity.  13B
+// shape, four ragged sequences: 17.9 -> 17.5 ms per iteration.  (More chunks where they fit twice over are
+// slower, 7B at batch 1 5.09 -> 5.29 ms with eight.)
 int attn_tc_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms) {
   int c = 1;
   if (g_attn_tc_chunks > 0) {
@@ -688,7 +691,8 @@ int attn_tc_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms)
     return c;
   }
   while (c < 8 && 2 * c * B * n_heads <= num_sms && 2 * c * 128 <= S_max) c *= 2;
-  if (c == 1 && rows_per_seq > 32 && rows_per_seq <= 64 && 20 * B * n_heads <= 22 * num_sms && 256 <= S_max) c = 2;
+  const int pairs = B * n_heads, longest = rows_per_seq > 32 || pairs <= num_sms ? 256 : 2048;
+  if (c == 1 && rows_per_seq <= 64 && 10 * pairs <= 11 * num_sms && S_max >= longest) c = 2;
   return c;
 }
 
