@@ -399,11 +399,11 @@ tree_attn_mma_kernel(const float *q, const bf16 *kc, const bf16 *vc,
 // within what is resident at once (two CTAs of 96 KB per SM; clusters of eight do not fill every GPC, hence
 // seven eighths there), at least one tile of capacity per chunk.  One sequence of 32 heads, context 2000, four
 // layers: 528 / 460 / 430 / 418 us with 1 / 2 / 4 / 8.  Past that more chunks pay where lengths are ragged (the host
-// does not know them) and chunks long: a tenth more CTAs from 2048 keys of capacity, and two chunks of whatever
-// fits in one round from 4096.  Fewer / more chunks, five rows, four layers, equal and ragged lengths: 80 pairs
+// does not know them) and chunks long: a tenth more CTAs from 2048 keys of capacity; and from 4096 two chunks
+// where one leaves a second round nearly empty.  Fewer / more chunks, five rows, four layers, equal and ragged lengths: 80 pairs
 // at context 2000 318 / 339 and 300 / 282 us, at 600 253 / 281 and 244 / 258; 160 pairs at 2000 568 / 592 and
-// 553 / 490, at 600 (eight layers) 966 / 1050 and 986 / 1008; 192 pairs at 4000 735 / 785 and 705 / 583, at 2000
-// 568 / 613 and 554 / 507; 320 pairs at 4000 1055 / 935 and 712 / 707.
+// 553 / 490, at 600 (eight layers) 966 / 1050 and 986 / 1008; 192 pairs at 4000 735 / 785 and 705 / 583 (one); 320
+// pairs at 4000 1055 / 935 and 712 / 707.
 int g_attn_mma_chunks = 0;     // > 0: this many key chunks whatever the shape (A/B runs)
 void attn_mma_set_chunks(int chunks) { g_attn_mma_chunks = chunks; }
 int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms) {
@@ -416,7 +416,7 @@ int attn_mma_chunks(int B, int n_heads, int rows_per_seq, int S_max, int num_sms
   const int ctas = rgs * B * n_heads, room = 2 * num_sms;
   auto limit = [&](int chunks) { return chunks == 8 ? room * 7 / 8 : (S_max >= 2048 ? room * 11 / 10 : room); };
   while (c < 8 && 2 * c * ctas <= limit(2 * c) && 2 * c * 64 <= S_max) c *= 2;
-  if (c == 1 && ctas <= room * 11 / 10 && S_max >= 4096) c = 2;
+  if (c == 1 && ctas > room && ctas <= room * 11 / 10 && S_max >= 4096) c = 2;
   return c;
 }
 
