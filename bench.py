@@ -51,11 +51,12 @@ HEADLINE = T13_EAGLE
 # DRAM traffic of the dominant launch from its ncu capture (one launch of gemm_tc_pair_kernel on the
 # 13B gate+up shape at 256 tokens, a 1.4 GB case: dram__bytes_read.sum + dram__bytes_write.sum), used
 # to scale the step's weight bytes per GEMM launch to DRAM bytes per launch: the traffic is the
-# weights once (1.03 x) plus one write-back of the fp32 partial sums, both proportional to the matrix.
-NCU_DRAM_BYTES = 291.5e6 + 28.2e6
+# weights once (1.03 x) plus what is written back of the fp32 partial sums (the weight loads are
+# evict-first, most of the sums stay in L2), both proportional to the matrix.
+NCU_DRAM_BYTES = 291.0e6 + 10.9e6
 NCU_ALGORITHMIC_BYTES = 283.1e6
 NCU_SOURCE = ("scaled from one ncu capture of the dominant launch (gemm_tc_pair_kernel, 13B gate+up at 256 tokens: "
-              "319.7 MB of DRAM traffic for 283.1 MB of weights; profiles/ncu_gemm_tc_pair_kernel_t13_gateup_256tokens.md) "
+              "301.9 MB of DRAM traffic for 283.1 MB of weights) "
               "by the weight bytes per launch of this step")
 
 
