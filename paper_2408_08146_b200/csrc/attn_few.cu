@@ -282,8 +282,9 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
 // caches take two chunks of at least 1024 keys also where not all are resident at once: one chunk leaves most
 // SMs a single CTA, which cannot draw the SM's share of the bandwidth (160 pairs, four layers: context 2000
 // 602 -> 544 us with equal, 515 -> 475 with ragged lengths, context 4000 776 -> 656 and 627 -> 552; 256 pairs
-// 609 -> 584, 563 -> 526).  Two rows do up to a tenth more pairs than SMs (160 pairs, context 4000 697 -> 665 and
-// 632 -> 549; 192 pairs 702 -> 727 and 662 -> 594: left at one).
+// 609 -> 584, 563 -> 526), up to as many pairs as two CTAs per SM take (320 pairs 477 -> 456 and 322 -> 333).  Two
+// rows do up to a tenth more pairs than SMs (160 pairs, context 4000 697 -> 665 and 632 -> 549; 192 pairs 702 ->
+// 727 and 662 -> 594: left at one).
 cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
                                Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early) {
   if (rows_per_seq < 1 || (head_dim != 64 && head_dim != 128)) return cudaErrorInvalidValue;
@@ -295,7 +296,7 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
     const int room = (RT <= 2 ? 2 : 1) * num_sms * 7 / 8, min_keys = (bf && DH == 128 ? 2 : 8) * TILE;
     int chunks = 1;
     while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads * groups <= room && 2 * chunks * min_keys <= S_max) chunks *= 2;
-    const bool halve = RT == 1 || (RT == 2 && 10 * B * n_heads <= 11 * num_sms);
+    const bool halve = RT <= 2 && 10 * B * n_heads <= (RT == 1 ? 20 : 11) * num_sms;
     if (bf && DH == 128 && halve && chunks == 1 && S_max >= 2048) chunks = 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(chunks, n_heads * B, groups);

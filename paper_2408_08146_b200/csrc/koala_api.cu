@@ -52,8 +52,8 @@ constexpr int MAX_SPLIT = 12;     // partial-sum matrices the workspace holds pe
 constexpr int NUM_SMS = 148;
 // Prompt tokens per forward of koala_ingest: enough for the multiplies to be bound by the tensor cores
 // (256-token tiles, four of them), few enough for the workspace to stay small (four partial-sum
-// matrices of that many rows; 7B shape: 0.36 GB).  13B batch of four prompts: 134 ms, with 512 tokens 138.5,
-// with 768 141.
+// matrices of that many rows; 7B shape: 0.36 GB).  13B batch of four prompts 140.0 ms, with 512 tokens 137.2, with 768
+// 147.0; 7B shape, eight layers, 600 tokens 4.1 ms, with 512 4.55, 1000 tokens 6.5 and 7.3.
 constexpr int INGEST_ROWS = 1024;
 constexpr int INGEST_SPLIT = 4;
 
