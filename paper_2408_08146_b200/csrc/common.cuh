@@ -62,14 +62,14 @@ struct SplitIn {
   // several matrices side by side whose widths are not whole tiles (0 = not the case): the columns
   // at which the second and third matrix start, and the tiles before them
   unsigned sk_m0, sk_m1, sk_t0, sk_t1;
-  // several token tiles of sk_tt rows dealt in the same launch: tile = weight tile * sk_zt + row / sk_tt
-  unsigned sk_zt, sk_tt;
+  // several token tiles of sk_tt rows dealt in the same launch (0 = one): tile = weight tile * sk_zt + row / sk_tt * sk_wt
+  unsigned sk_zt, sk_tt, sk_wt;
   // Stream-K tile that column c (of row r) belongs to.
   __device__ __forceinline__ unsigned tile_of(int r, int c) const {
     const unsigned sh = 7u + sk_wide, uc = (unsigned)c;
     unsigned tile = uc >> sh;
     if (sk_m0 != 0 && uc >= sk_m0) tile = uc < sk_m1 ? sk_t0 + ((uc - sk_m0) >> sh) : sk_t1 + ((uc - sk_m1) >> sh);
-    if (sk_zt > 1) tile = tile * sk_zt + (unsigned)r / sk_tt;
+    if (sk_tt != 0) tile = tile * sk_zt + (unsigned)r / sk_tt * sk_wt;
     return tile;
   }
   __device__ __forceinline__ int count(int r, int c) const {

@@ -55,6 +55,7 @@ struct TcParams {
   int bn;             // MMA N = rows of the activation tile in shared memory, multiple of 16, <= 256
   int tt;             // tokens per tile: bn, or bn / 2 when the activations are a hi/lo pair
   int ztiles;         // token tiles (classic mode; fastest-varying part of blockIdx.x)
+  int wtiles;         // CTA pairs in chains: weight tiles
   int tmem_cols;      // power of two >= max(32, bn), per accumulator buffer
   int nbuf;           // accumulator buffers in tensor memory (2 when they fit in 256 columns)
   int tiles0, tiles1; // weight tiles of matrix 0 and of matrices 0+1 (cumulative)
@@ -443,6 +444,12 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
     row0 = tile * ROWS;
     return &tmW0;
   };
+  // The deal of tiles.  Up to 512 rows the token tiles of a weight tile lie next to one another; in chains, with
+  // several tiles per cluster, a cluster would take them one after the other and the weights come from DRAM
+  // once for each (1024 rows of the 7B gate and up: 755 MB for 180): there the weight tiles of a token tile do, and
+  // groups of clusters, one per token tile, go through the weights side by side.
+  auto weight_of = [&](int tile) { return CHAIN ? tile % P.wtiles : tile / P.ztiles; };
+  auto tok_of = [&](int tile) { return CHAIN ? tile / P.wtiles : tile % P.ztiles; };
   const int pre = n_units < n_stages ? n_units : n_stages;
 
   pdl_launch_dependents();
@@ -483,14 +490,14 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       uint32_t full_even[PAIR_MAX_STAGES];
       for (int s = 0; s < PAIR_MAX_STAGES; ++s) full_even[s] = cluster_addr_of(smem_u32(&full_bar[s]), 0);
       int tile = (int)(u_lo / KB), kb = (int)(u_lo % KB), row0;
-      int tok0 = (tile % P.ztiles) * tt;
-      const CUtensorMap *tmW = tile_map(tile / P.ztiles, row0);
+      int tok0 = tok_of(tile) * tt;
+      const CUtensorMap *tmW = tile_map(weight_of(tile), row0);
       auto next_unit = [&]() {
         if (++kb == KB) {
           kb = 0;
           ++tile;
-          tok0 = (tile % P.ztiles) * tt;
-          tmW = tile_map(tile / P.ztiles, row0);
+          tok0 = tok_of(tile) * tt;
+          tmW = tile_map(weight_of(tile), row0);
         }
       };
       auto load_w = [&](int s) {
@@ -601,7 +608,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_const
       unsigned seg_hi = (unsigned)(tile + 1) * KB;
       if (seg_hi > u_hi) seg_hi = u_hi;
       int row0, col_off = 0, n_rows = P.n0;
-      const int wt = tile / P.ztiles, tok0 = (tile % P.ztiles) * tt;
+      const int wt = weight_of(tile), tok0 = tok_of(tile) * tt;
       if (wt >= P.tiles1) { row0 = (wt - P.tiles1) * ROWS; col_off = P.n0 + P.n1; n_rows = P.n2; }
       else if (wt >= P.tiles0) { row0 = (wt - P.tiles0) * ROWS; col_off = P.n0; n_rows = P.n1; }
       else row0 = wt * ROWS;
@@ -1011,9 +1018,8 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
     const int rows = chain ? CHAIN_ROWS : PAIR_ROWS;
     const int q0 = (m.n_out[0] + rows - 1) / rows, q1 = m.n > 1 ? (m.n_out[1] + rows - 1) / rows : 0,
               q2 = m.n > 2 ? (m.n_out[2] + rows - 1) / rows : 0;
-    // Token tiles: equal up to 32 rows (the MMA's N follows the tile, so 300 rows cost 320 and not 512),
-    // all in one launch, the token tiles of a weight tile next to one another in the deal of units:
-    // the clusters that share a weight tile then read it at about the same time.
+    // Token tiles: equal up to 32 rows (the MMA's N follows the tile, so 300 rows cost 320 and not 512), all in one
+    // launch.
     int ptt = ((R + zt - 1) / zt + 31) / 32 * 32;
     if (ptt < 128 && !chain) ptt = 128;
     const int n_tiles = (q0 + q1 + q2) * zt;
@@ -1037,6 +1043,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
       P.bn = ptt;
       P.nbuf = chain || ptt <= 128 ? 2 : 1;
       P.ztiles = zt;
+      P.wtiles = q0 + q1 + q2;
       P.sk_ctas = (int)g;
       P.sk_units = (unsigned)units;
       P.split = 1;
@@ -1049,8 +1056,11 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
         if (!get_map(m.W[j], m.n_out[j], K_in, BM, &mw[i])) return cudaErrorInvalidValue;
       }
       SplitIn si{Y, slots_of(g), split_stride, ldy, (unsigned)g, (unsigned)units, (unsigned)KB, chain ? 1u : 2u};
-      si.sk_zt = (unsigned)zt;
-      si.sk_tt = (unsigned)ptt;
+      if (zt > 1) {
+        si.sk_tt = (unsigned)ptt;
+        si.sk_zt = chain ? 1u : (unsigned)zt;
+        si.sk_wt = chain ? (unsigned)P.wtiles : 1u;
+      }
       bool ragged = false;
       for (int i = 0; i + 1 < m.n; ++i) ragged = ragged || (m.n_out[i] % rows) != 0;
       if (ragged) {
