@@ -15,7 +15,7 @@
 // MMAs as bf16 pairs (value + rounding residual: two accumulating MMAs), so only the cached K and V
 // carry bf16 rounding.  Q (written as a pair by the rotary-embedding kernel) and the K/V tiles
 // arrive by TMA with the 128-byte swizzle, K/V in a ring of two (up to 64 rows) or three stages.
-// Warps 0..3 own the rows, warp 4 lane 0 issues the copies, warp 5 lane 0 the MMAs.
+// Warps 0..3 own the rows, warp 4 lane 0 issues the copies, warp 5 lane 0 the MMAs (more than 64 rows: warp 6 lane 0 those of S).
 // With several chunks the CTAs of one (head, sequence) form a thread-block cluster: every CTA leaves
 // its unnormalised (O, m, l) in its own shared memory (the K/V ring is free by then); after a cluster
 // barrier every CTA reads its slice of the head dimension from all of them, merges it in chunk order
@@ -62,7 +62,7 @@ struct alignas(16) SyncVars {
 };
 static_assert(sizeof(SyncVars) <= 1024, "the static variables and the alignment gap share 1 KB");
 template <bool DUP> constexpr unsigned SMEM_BYTES = Lay<DUP>::BYTES + 1024 - (unsigned)sizeof(SyncVars);
-constexpr int THREADS = 192;
+template <bool DUP> constexpr int THREADS = DUP ? 192 : 224;
 constexpr int E_INVALID = 1, E_TIMEOUT = 6;
 constexpr int TMEM_COLS = 256;               // S: 2 x 64 columns, O: 128 columns
 constexpr int COL_S = 0, COL_O = 128;
@@ -154,7 +154,7 @@ struct AttnParams {
 // fetches its instructions anew and runs most of them once: 60 KB of code in one body were a third of
 // the fixed cost of a launch.
 template <bool DUP, bool ONE>
-__global__ void __launch_bounds__(THREADS, DUP ? 2 : 1)
+__global__ void __launch_bounds__(THREADS<DUP>, DUP ? 2 : 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_constant__ CUtensorMap tmQl,
                     const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const AttnParams P) {
@@ -188,7 +188,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
   if (threadIdx.x == 0) {
     mbar_init(&q_full, 1);
     for (int s = 0; s < NST; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1); mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1); }
-    mbar_init(&drain_bar, 1);
+    mbar_init(&drain_bar, DUP ? 1 : 2);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s_full[i], 1);
       mbar_init(&p_full[i], (uint32_t)n_arrive);
@@ -312,57 +312,65 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       }
       if (T == 0 || !ok) (void)mbar_wait(&q_full, 0);      // nobody else waits for Q then
     }
-  } else if (warp == 5) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      // D fp32, A and B bf16; S: N = 64, both K-major; O_t: N = 128, B MN-major
-      const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TK >> 3) << 17) | ((128u >> 4) << 24);
-      const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(DH >> 3) << 17) |
-                               ((128u >> 4) << 24);
-      auto issue_s = [&](int t) -> bool {
-        const int s = t % NST;
-        if (!mbar_wait(&k_full[s], (uint32_t)(t / NST) & 1u)) return false;
-        tc_fence_after();
-        const uint32_t kb = sb + LY::K + s * 2 * SUB;
-        const uint32_t d = tmem + (uint32_t)(COL_S + (t & 1) * TK);
+  } else if (warp >= 5) {
+    // ------------------------------------------------------------------ MMA issuers
+    // A thread hands over an MMA of these sizes every 50 to 100 cycles, about as fast as they execute, and prepares nothing
+    // meanwhile.  With more than 64 rows (16 MMAs of S and 8 of P V per tile) one thread for both was what a tile took,
+    // 2700 cycles of which the rows worked 1700: S and P V have a thread each there (128 rows, context 3989, 32 heads:
+    // 38.2 -> 32.9 us per launch).  Up to 64 rows it is half as many MMAs, and a second thread gained nothing.
+    // D fp32, A and B bf16; S: N = 64, both K-major; O: N = 128, B MN-major
+    const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TK >> 3) << 17) | ((128u >> 4) << 24);
+    const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(DH >> 3) << 17) | ((128u >> 4) << 24);
+    auto issue_s = [&](int t) -> bool {
+      const int s = t % NST;
+      // the rows have read S of tile t - 2 out of this buffer (one thread for both has waited for that before its P V)
+      if (!DUP && t >= 2 && !mbar_wait(&p_full[t & 1], (uint32_t)((t - 2) >> 1) & 1u)) return false;
+      if (!mbar_wait(&k_full[s], (uint32_t)(t / NST) & 1u)) return false;
+      tc_fence_after();
+      const uint32_t kb = sb + LY::K + s * 2 * SUB;
+      const uint32_t d = tmem + (uint32_t)(COL_S + (t & 1) * TK);
 #pragma unroll
-        for (int part = 0; part < (DUP ? 1 : 2); ++part) { // Q value, then Q residual (DUP: both in one operand)
+      for (int part = 0; part < (DUP ? 1 : 2); ++part) {   // Q value, then Q residual (DUP: both in one operand)
 #pragma unroll
-          for (int hb = 0; hb < 2; ++hb) {                 // 64-dim block
-            const uint64_t da = smem_desc_sw128(sb + LY::Q + (DUP ? hb : part * 2 + hb) * QSUB);
-            const uint64_t db = smem_desc_sw128(kb + hb * SUB);
+        for (int hb = 0; hb < 2; ++hb) {                   // 64-dim block
+          const uint64_t da = smem_desc_sw128(sb + LY::Q + (DUP ? hb : part * 2 + hb) * QSUB);
+          const uint64_t db = smem_desc_sw128(kb + hb * SUB);
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              umma_bf16(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc_s, (part | hb | k) ? 1u : 0u);
-          }
+          for (int k = 0; k < 4; ++k)
+            umma_bf16(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc_s, (part | hb | k) ? 1u : 0u);
         }
-        umma_commit(&s_full[t & 1]);
-        umma_commit(&k_empty[s]);
-        return true;
-      };
-      bool ok = T > 0 ? mbar_wait(&q_full, 0) : true;
+      }
+      umma_commit(&s_full[t & 1]);
+      umma_commit(&k_empty[s]);
+      return true;
+    };
+    auto issue_pv = [&](int t) -> bool {
+      if (!mbar_wait(&p_full[t & 1], (uint32_t)(t >> 1) & 1u)) return false;
+      if (!mbar_wait(&v_full[t % NST], (uint32_t)(t / NST) & 1u)) return false;
+      tc_fence_after();
+      const uint32_t vb = sb + LY::V + (t % NST) * 2 * SUB;
+      const uint32_t pb = sb + LY::P + (t % NP) * LY::PB;
+      const uint32_t d = tmem + (uint32_t)COL_O;
+#pragma unroll
+      for (int part = 0; part < (DUP ? 1 : 2); ++part) {   // P value, then P residual (DUP: both in one operand)
+        const uint64_t da = smem_desc_sw128(pb + part * QSUB);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {                      // 16 keys per MMA
+          const uint64_t db = smem_desc_mn_sw128(vb + k * 2048, SUB, 1024);
+          umma_bf16(d, da + (uint64_t)(2 * k), db, idesc_o, (t | part | k) ? 1u : 0u);   // O accumulates over the tiles
+        }
+      }
+      umma_commit(&v_empty[t % NST]);
+      umma_commit(&pv_done[t & 1]);
+      return true;
+    };
+    if (lane == 0) {
+      const bool do_s = DUP || warp == 6, do_pv = DUP || warp == 5;
+      bool ok = T > 0 && do_s ? mbar_wait(&q_full, 0) : true;
 #pragma unroll 1
       for (int t = T > 0 ? -1 : 0; t < T && ok; ++t) {     // one place that issues S: the first one at t = -1
-        if (t + 1 < T) { ok = issue_s(t + 1); if (!ok) break; }
-        if (t < 0) continue;
-        ok = mbar_wait(&p_full[t & 1], (uint32_t)(t >> 1) & 1u);
-        if (ok) ok = mbar_wait(&v_full[t % NST], (uint32_t)(t / NST) & 1u);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t vb = sb + LY::V + (t % NST) * 2 * SUB;
-        const uint32_t pb = sb + LY::P + (t % NP) * LY::PB;
-        const uint32_t d = tmem + (uint32_t)COL_O;
-#pragma unroll
-        for (int part = 0; part < (DUP ? 1 : 2); ++part) { // P value, then P residual (DUP: both in one operand)
-          const uint64_t da = smem_desc_sw128(pb + part * QSUB);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {                    // 16 keys per MMA
-            const uint64_t db = smem_desc_mn_sw128(vb + k * 2048, SUB, 1024);
-            umma_bf16(d, da + (uint64_t)(2 * k), db, idesc_o, (t | part | k) ? 1u : 0u);   // O accumulates over the tiles
-          }
-        }
-        umma_commit(&v_empty[t % NST]);
-        umma_commit(&pv_done[t & 1]);
+        if (do_s && t + 1 < T) ok = issue_s(t + 1);
+        if (do_pv && t >= 0 && ok) ok = issue_pv(t);
       }
       if (!ok) atomicExch(&s_error, 1);
     }
@@ -398,7 +406,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         mk1 = ok_row ? P.plan.mask[(size_t)r_glob * 2 + 1] : 0ull;
       }
       const bool live = t >= 0;
-      if (live) {
+      if (live && (DUP || t == 0)) {
         ok = __all_sync(0xffffffffu, mbar_wait(&s_full[t & 1], (uint32_t)(t >> 1) & 1u));   // warp-uniform
         if (!ok) break;
       }
@@ -441,15 +449,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
             for (int q = 0; q < 8; ++q) st_shared_v4(vb + blk * SUB + kr * 128 + q * 16, 0u, 0u, 0u, 0u);
         }
       }
-      uint64_t vis = ok_row ? tile_visibility(mk0, mk1, key0, ctx, kv_len) : 0ull;
-      if (DUP) vis >>= 32 * half;
-      float m_t = -INFINITY;
+      // (more than 64 rows, where a thread has 64 keys: a tile that every row in use sees whole is not masked key by key)
+      const bool open = !DUP && key0 + TK <= ctx && __all_sync(0xffffffffu, ok_row || !row_in);
+      if (!open) {
+        uint64_t vis = ok_row ? tile_visibility(mk0, mk1, key0, ctx, kv_len) : 0ull;
+        if (DUP) vis >>= 32 * half;
 #pragma unroll
-      for (int j = 0; j < NC; ++j) {
-        const float s = ((vis >> j) & 1ull) ? __uint_as_float(v[j]) * sc : -INFINITY;
-        v[j] = __float_as_uint(s);
-        m_t = fmaxf(m_t, s);
+        for (int j = 0; j < NC; ++j) v[j] = ((vis >> j) & 1ull) ? v[j] : 0xff800000u;      // -inf
       }
+      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+      for (int j = 0; j < NC; ++j) m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(v[j]));
+      float m_t = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sc;
       if (DUP) m_t = fmaxf(m_t, __shfl_xor_sync(0xffffffffu, m_t, 16));   // over all 64 keys: both lanes keep the same reference
       // raise the reference maximum?  (the first visible key sets it; O holds nothing of this row yet then)
       float factor = 1.f;
@@ -491,8 +502,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         uint32_t hi[4], lo[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float p0 = ex2_fast(__uint_as_float(v[ch * 8 + 2 * e]) - mu);
-          const float p1 = ex2_fast(__uint_as_float(v[ch * 8 + 2 * e + 1]) - mu);
+          const float p0 = ex2_fast(fmaf(__uint_as_float(v[ch * 8 + 2 * e]), sc, -mu));
+          const float p1 = ex2_fast(fmaf(__uint_as_float(v[ch * 8 + 2 * e + 1]), sc, -mu));
           l_t += p0 + p1;
           split_pack_trunc(p0, p1, hi[e], lo[e]);
         }
@@ -502,6 +513,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
         st_shared_v4(pb + (DUP ? 16 * 128 : QSUB) + off, lo[0], lo[1], lo[2], lo[3]);
       }
       l_run += l_t;
+      // S of the next tile was asked for a tile ago.  With a thread of its own for S its barrier is looked at here, before P
+      // is handed over: P V's operands then take all of the shared memory's bandwidth, and a try of a barrier 600 cycles.
+      if (!DUP && live && t + 1 < T_run) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&s_full[(t + 1) & 1], (uint32_t)((t + 1) >> 1) & 1u));
+        if (!ok) break;
+      }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_fence_before();
       __syncwarp();
@@ -615,24 +632,39 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
       const int wc = DH >> P.chunk_bits, per_row = wc >> 3;          // eight dims per thread and step
       const uint32_t st0 = smem_u32(stage);
 #pragma unroll 1
-      for (int e = threadIdx.x; e < P.rows_per_seq * per_row; e += THREADS) {
+      for (int e = threadIdx.x; e < P.rows_per_seq * per_row; e += THREADS<DUP>) {
         const int r = e / per_row, d = c * wc + (e - r * per_row) * 8;
         const uint32_t at = st0 + (uint32_t)(r * OSTRIDE) * 4u;
-        float mm = -INFINITY;
-#pragma unroll 4
-        for (int j = 0; j < P.chunks; ++j) mm = fmaxf(mm, ld_cluster_v4(peer_addr(at + DH * 4u, (uint32_t)j)).x);
+        float mm = -INFINITY, l = 0.f;
         float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        float l = 0.f;
-        const float mu = mm == -INFINITY ? 0.f : mm;
-#pragma unroll 4
-        for (int j = 0; j < P.chunks; ++j) {               // in chunk order
-          const uint32_t pa = peer_addr(at, (uint32_t)j);
-          const float4 ml = ld_cluster_v4(pa + DH * 4u);
-          const float4 x0 = ld_cluster_v4(pa + (uint32_t)d * 4u), x1 = ld_cluster_v4(pa + (uint32_t)d * 4u + 16u);
-          const float w = exp2f(ml.x - mu);                // exp2(-inf) = 0; such a chunk's O is zero
-          l += w * ml.y;
-          o[0] += w * x0.x; o[1] += w * x0.y; o[2] += w * x0.z; o[3] += w * x0.w;
-          o[4] += w * x1.x; o[5] += w * x1.y; o[6] += w * x1.z; o[7] += w * x1.w;
+#pragma unroll 1
+        for (int j0 = 0; j0 < P.chunks; j0 += 4) {           // four chunks at a time, all requested before the first is used
+          float4 ml[4], x0[4], x1[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            ml[j] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+            x0[j] = x1[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j0 + j >= P.chunks) continue;
+            const uint32_t pa = peer_addr(at, (uint32_t)(j0 + j));
+            ml[j] = ld_cluster_v4(pa + DH * 4u);
+            x0[j] = ld_cluster_v4(pa + (uint32_t)d * 4u);
+            x1[j] = ld_cluster_v4(pa + (uint32_t)d * 4u + 16u);
+          }
+          float mn = mm;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mn = fmaxf(mn, ml[j].x);
+          const float mu = mn == -INFINITY ? 0.f : mn, back = exp2f(mm - mu);      // exp2(-inf) = 0; such a chunk's O is zero
+          mm = mn;
+          l *= back;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) o[k] *= back;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {                      // in chunk order
+            const float w = exp2f(ml[j].x - mu);
+            l += w * ml[j].y;
+            o[0] += w * x0[j].x; o[1] += w * x0[j].y; o[2] += w * x0[j].z; o[3] += w * x0[j].w;
+            o[4] += w * x1[j].x; o[5] += w * x1[j].y; o[6] += w * x1[j].z; o[7] += w * x1[j].w;
+          }
         }
         const float inv = l > 0.f ? 1.f / l : 0.f;
         uint32_t hi[4], lo[4];
@@ -646,14 +678,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
     // no CTA leaves while another may still read its shared memory
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   }
+  // MMAs issued before a wait ran out may still be running: no free under them
+  if (failed && warp >= 5 && lane == 0) umma_commit(&drain_bar);
   if (warp == 5) {
-    if (failed) {      // MMAs issued before a wait ran out may still be running: no free under them
-      if (lane == 0) {
-        umma_commit(&drain_bar);
-        (void)mbar_wait(&drain_bar, 0);
-      }
-      __syncwarp();
-    }
+    if (failed) (void)mbar_wait(&drain_bar, 0);
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
   }
   if (threadIdx.x == 0 && failed && P.status) atomicMax(P.status, E_TIMEOUT);
@@ -719,7 +748,7 @@ cudaError_t tree_attention_tc(Launch L, Operand q_pair, int q_rows_alloc, const 
                31 - __builtin_clz((unsigned)chunks), longest_first, early ? 1 : 0, g_attn_tc_dry_pass, status};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, n_heads * B);
-  cfg.blockDim = dim3(THREADS);
+  cfg.blockDim = dim3(dup ? THREADS<true> : THREADS<false>);
   cfg.stream = L.st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
