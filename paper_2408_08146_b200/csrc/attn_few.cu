@@ -65,10 +65,14 @@ __device__ __forceinline__ float ld_cluster(uint32_t local_addr, uint32_t rank) 
   return v;
 }
 
-template <typename T, int DH, int RT>
+// ROPE: the queries come as the partial sums of the Q/K/V multiply, as do the new keys and values: the CTA whose tiles
+// hold a new row's slot writes it to the cache and reads it back with the tile.  A launch less per layer, whose 5 us
+// were one trip to the partial sums and back (rule and figures at attn_few_takes_sums).
+constexpr int ROPE_PARTS = 4;                              // partial sums that are requested side by side
+template <typename T, int DH, int RT, bool ROPE>
 __global__ void __launch_bounds__(WARPS * 32, RT <= 2 ? 2 : 1)
-tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *__restrict__ out, T *__restrict__ out_lo,
-                     int rows_per_seq, int n_heads, int S_max, int early) {
+tree_attn_few_kernel(const float *q, T *kc, T *vc, RowPlan plan, T *__restrict__ out, T *__restrict__ out_lo,
+                     int rows_per_seq, int n_heads, int S_max, int early, SplitIn qkv, RowScale scale) {
   constexpr int E = DH / 16;                               // dims of a lane
   constexpr int PSTRIDE = DH + 4;                          // floats of a partial: O[DH], m, l, pad (16-byte rows)
   __shared__ __align__(16) float s_q[RT][DH];
@@ -104,7 +108,7 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
     const bool context = (t_lo + 1) * TILE <= ctx;
     if (context) load(t_lo);
     pdl_wait();
-    if (!context) load(t_lo);
+    if (!ROPE && !context) load(t_lo);
   } else {
     load(t_lo);                                          // first of all: the longest way
   }
@@ -118,11 +122,47 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
     mk1[r] = plan.mask[(size_t)rg * 2 + 1];
     if (i0 + r < rows_per_seq && slot >= 0) row_ok |= 1u << r;
   }
+  if constexpr (ROPE) {
+    constexpr int HALF = DH / 2;
+#pragma unroll
+    for (int e = threadIdx.x; e < RT * 3 * HALF; e += WARPS * 32) {      // (row, Q / K / V, pair of dims)
+      const int r = e / (3 * HALF), mat = e / HALF % 3, i = e % HALF;
+      const int rg = b * rows_per_seq + (i0 + r < rows_per_seq ? i0 + r : 0), slot = plan.slot[rg];
+      if (mat > 0) {
+        const int tile = min(slot / TILE, tiles - 1);      // the chunk that holds the row's slot writes it
+        if (i0 + r >= rows_per_seq || slot < 0 || slot >= S_max || tile < t_lo || tile >= t_hi) continue;
+      }
+      const float *p = qkv.p + (size_t)rg * qkv.ld + mat * H + h * DH + i;
+      float ua[ROPE_PARTS], ub[ROPE_PARTS];
+#pragma unroll
+      for (int s = 0; s < ROPE_PARTS; ++s) {
+        ua[s] = s < qkv.n ? p[(size_t)s * qkv.stride] : 0.f;
+        ub[s] = s < qkv.n ? p[(size_t)s * qkv.stride + HALF] : 0.f;
+      }
+      const float rs = scale.of(rg);
+      const float2 cs = plan.rope[(size_t)rg * HALF + i];
+      float a = ua[0], c2 = ub[0];
+#pragma unroll
+      for (int s = 1; s < ROPE_PARTS; ++s) { a += ua[s]; c2 += ub[s]; }
+      a *= rs;
+      c2 *= rs;
+      const float ra = a * cs.x - c2 * cs.y, rb = c2 * cs.x + a * cs.y;
+      if (mat == 0) {
+        s_q[r][i] = ra * sc;
+        s_q[r][i + HALF] = rb * sc;
+      } else {
+        T *to = (mat == 1 ? kc : vc) + (base + slot) * DH + i;
+        to[0] = from_f<T>(mat == 1 ? ra : a);
+        to[HALF] = from_f<T>(mat == 1 ? rb : c2);
+      }
+    }
+  } else
   for (int e = threadIdx.x; e < RT * DH; e += WARPS * 32) {
     const int r = e / DH, d = e % DH;
     s_q[r][d] = q[(size_t)(b * rows_per_seq + (i0 + r < rows_per_seq ? i0 + r : 0)) * H + h * DH + d] * sc;
   }
   __syncthreads();
+  if (ROPE && (t_lo + 1) * TILE > ctx) load(t_lo);         // its new rows stand now
   float m[RT], l[RT], o[RT][E];
 #pragma unroll
   for (int r = 0; r < RT; ++r) {
@@ -285,19 +325,23 @@ tree_attn_few_kernel(const float *q, const T *kc, const T *vc, RowPlan plan, T *
 // 609 -> 584, 563 -> 526), up to as many pairs as two CTAs per SM take (320 pairs 477 -> 456 and 322 -> 333).  Two
 // rows do up to a tenth more pairs than SMs (160 pairs, context 4000 697 -> 665 and 632 -> 549; 192 pairs 702 ->
 // 727 and 662 -> 594: left at one).
-cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
-                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early) {
+static int few_chunks(bool bf128, int rt, int B, int n_heads, int groups, int S_max, int num_sms) {
+  const int room = (rt <= 2 ? 2 : 1) * num_sms * 7 / 8, min_keys = (bf128 ? 2 : 8) * TILE;
+  int chunks = 1;
+  while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads * groups <= room && 2 * chunks * min_keys <= S_max) chunks *= 2;
+  const bool halve = rt <= 2 && 10 * B * n_heads <= (rt == 1 ? 20 : 11) * num_sms;
+  return bf128 && halve && chunks == 1 && S_max >= 2048 ? 2 : chunks;
+}
+
+static cudaError_t attention_few(Launch L, int dtype, const float *q, const SplitIn *qkv, RowScale sc, void *k_cache, void *v_cache,
+                                 RowPlan plan, Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early) {
   if (rows_per_seq < 1 || (head_dim != 64 && head_dim != 128)) return cudaErrorInvalidValue;
   const bool bf = dtype != 0;
-  auto go = [&](auto tag, auto dh, auto rt) -> cudaError_t {
+  auto go = [&](auto tag, auto dh, auto rt, auto rope) -> cudaError_t {
     typedef decltype(tag) T;
     constexpr int DH = decltype(dh)::value, RT = decltype(rt)::value;
     const int groups = (rows_per_seq + RT - 1) / RT;
-    const int room = (RT <= 2 ? 2 : 1) * num_sms * 7 / 8, min_keys = (bf && DH == 128 ? 2 : 8) * TILE;
-    int chunks = 1;
-    while (chunks < MAX_CHUNKS && 2 * chunks * B * n_heads * groups <= room && 2 * chunks * min_keys <= S_max) chunks *= 2;
-    const bool halve = RT <= 2 && 10 * B * n_heads <= (RT == 1 ? 20 : 11) * num_sms;
-    if (bf && DH == 128 && halve && chunks == 1 && S_max >= 2048) chunks = 2;
+    const int chunks = few_chunks(bf && DH == 128, RT, B, n_heads, groups, S_max, num_sms);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(chunks, n_heads * B, groups);
     cfg.blockDim = dim3(WARPS * 32);
@@ -312,8 +356,8 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
     cfg.attrs = attr;
     cfg.numAttrs = chunks > 1 ? 2 : 1;
     ++g_launches;
-    return cudaLaunchKernelEx(&cfg, tree_attn_few_kernel<T, DH, RT>, q, (const T *)k_cache, (const T *)v_cache, plan,
-                              (T *)out.hi, (T *)out.lo, rows_per_seq, n_heads, S_max, early ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, tree_attn_few_kernel<T, DH, RT, decltype(rope)::value>, q, (T *)k_cache, (T *)v_cache, plan,
+                              (T *)out.hi, (T *)out.lo, rows_per_seq, n_heads, S_max, early ? 1 : 0, qkv != nullptr ? *qkv : SplitIn{}, sc);
   };
   std::integral_constant<int, 64> d64;
   std::integral_constant<int, 128> d128;
@@ -321,10 +365,34 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
   std::integral_constant<int, 2> r2;
   std::integral_constant<int, 4> r4;
   const bool one = rows_per_seq == 1 || (!(bf && head_dim == 128) && (long long)rows_per_seq * B * n_heads <= 4LL * num_sms);
-  if (bf && head_dim == 128) return one ? go(bf16{}, d128, r1) : (rows_per_seq == 2 ? go(bf16{}, d128, r2) : go(bf16{}, d128, r4));
-  if (bf) return one ? go(bf16{}, d64, r1) : go(bf16{}, d64, r4);
-  if (head_dim == 64) return one ? go(float{}, d64, r1) : go(float{}, d64, r4);
-  return one ? go(float{}, d128, r1) : go(float{}, d128, r2);
+  std::false_type plain;
+  if (qkv != nullptr) return one ? go(bf16{}, d128, r1, std::true_type{}) : go(bf16{}, d128, r2, std::true_type{});
+  if (bf && head_dim == 128) return one ? go(bf16{}, d128, r1, plain) : (rows_per_seq == 2 ? go(bf16{}, d128, r2, plain) : go(bf16{}, d128, r4, plain));
+  if (bf) return one ? go(bf16{}, d64, r1, plain) : go(bf16{}, d64, r4, plain);
+  if (head_dim == 64) return one ? go(float{}, d64, r1, plain) : go(float{}, d64, r4, plain);
+  return one ? go(float{}, d128, r1, plain) : go(float{}, d128, r2, plain);
+}
+
+cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
+                               Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early) {
+  return attention_few(L, dtype, q, nullptr, RowScale{}, const_cast<void *>(k_cache), const_cast<void *>(v_cache), plan, out, rows_per_seq, B,
+                       n_heads, head_dim, S_max, num_sms, early);
+}
+
+// Whether a forward of so many rows takes the partial sums itself.  The rotary launch it saves is a time in which the O
+// projection's first weights arrive; where a CTA has many keys to walk they arrive at the attention's expense instead.
+// Six layers of the 7B shape, us per one-token pass, keys of capacity per chunk: one sequence 160 598 -> 583, 528 676
+// -> 653; two 416 630 -> 631, 1056 714 -> 736; four 256 609 -> 591, 448 650 -> 629, 832 (ragged) 659 -> 664; eight 621 -> 604.
+bool attn_few_takes_sums(int rows_per_seq, int B, int n_heads, int S_max, int num_sms) {
+  return rows_per_seq >= 1 && rows_per_seq <= ATTN_FEW_ROWS &&
+         S_max <= 640 * few_chunks(true, rows_per_seq, B, n_heads, 1, S_max, num_sms);
+}
+bool attn_few_rope_supported(const SplitIn &qkv) { return qkv.sk_ctas == 0 && qkv.n <= ROPE_PARTS; }
+
+cudaError_t tree_attention_few_rope(Launch L, SplitIn qkv, RowScale sc, void *k_cache, void *v_cache, RowPlan plan, Operand out,
+                                    int rows_per_seq, int B, int n_heads, int S_max, int num_sms) {
+  if (rows_per_seq > ATTN_FEW_ROWS || !attn_few_rope_supported(qkv)) return cudaErrorInvalidValue;
+  return attention_few(L, 1, nullptr, &qkv, sc, k_cache, v_cache, plan, out, rows_per_seq, B, n_heads, 128, S_max, num_sms, true);
 }
 
 }  // namespace koala

@@ -239,6 +239,13 @@ cudaError_t tree_attention_mma(Launch L, const float *q, const void *k_cache, co
 constexpr int ATTN_FEW_ROWS = 2;
 cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *k_cache, const void *v_cache, RowPlan plan,
                                Operand out, int rows_per_seq, int B, int n_heads, int head_dim, int S_max, int num_sms, bool early);
+// The same straight from the Q/K/V multiply's partial sums (bf16 caches, head_dim 128, up to ATTN_FEW_ROWS rows per
+// sequence): rotates its queries, writes the new rows of the cache.  The plan and the cached context are read before the
+// dependency wait: the multiply must have been launched with late_dependents.
+bool attn_few_takes_sums(int rows_per_seq, int B, int n_heads, int S_max, int num_sms);
+bool attn_few_rope_supported(const SplitIn &qkv);
+cudaError_t tree_attention_few_rope(Launch L, SplitIn qkv, RowScale sc, void *k_cache, void *v_cache, RowPlan plan, Operand out,
+                                    int rows_per_seq, int B, int n_heads, int S_max, int num_sms);
 
 // attn_tc.cu : the same on tcgen05 tensor cores, all rows of a sequence in one CTA, key chunks as a cluster;
 // the queries come as the bf16 pair written by rope_kv_write ([q_rows_alloc][n_heads * 128] each)
@@ -280,7 +287,7 @@ int tc_default_split(int n_tiles, int kblocks, int tokens);
 // tensor core is longer than with 64 rows, whatever R.
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
                     float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
-                    SplitIn *out, bool short_sums = false);
+                    SplitIn *out, bool short_sums = false, bool late_dependents = false);
 
 // layer_tc.cu : several GEMMs of a decoder layer and the row-wise steps between them in one
 // persistent launch (bf16, activations as pairs, at most 128 rows, head_dim 128 for the rotary step)

@@ -67,6 +67,7 @@ struct TcParams {
   size_t split_stride;
   int stages;
   int early_w;        // how many of the first stages' weight tiles are requested before the dependency wait
+  int late_dep;       // 1: the next kernel may start only once everything before this one is complete (one-CTA form)
   int epi_dry;        // 1: the epilogue warps make a dry pass over their loop body (nothing stored) at kernel start
   int *status;
 };
@@ -141,7 +142,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
   };
   const int pre = n_units < P.stages ? n_units : P.stages;
 
-  pdl_launch_dependents();
+  if (!P.late_dep) pdl_launch_dependents();
   if (threadIdx.x == 0) {
 #pragma unroll 1
     for (int s = 0; s < P.stages; ++s) {
@@ -187,6 +188,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       int tile, kb, row0;
       const CUtensorMap *tmW;
       pdl_wait();
+      if (P.late_dep) pdl_launch_dependents();
       const int lo_off = P.tt * BK * 2;          // the lo rows follow the hi rows of the tile
       tile = (int)(u_lo / KB);
       kb = (int)(u_lo % KB);
@@ -953,7 +955,7 @@ int tc_streamk_ctas(int n_tiles, int kblocks, int tokens, int max_slots, int *sl
 
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
                     float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
-                    SplitIn *out, bool short_sums) {
+                    SplitIn *out, bool short_sums, bool late_dependents) {
   if (!use_current_device()) return cudaErrorInitializationError;
   if (!tc_supported(m, K_in) || R < 1 || ((uintptr_t)X.hi & 15u) || ((uintptr_t)X.lo & 15u))
     return cudaErrorInvalidValue;
@@ -1163,6 +1165,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   P.status = status;
   P.nbuf = (sk && 2 * cols <= 256) ? 2 : 1;
   P.epi_dry = g_tune_epi_dry;
+  P.late_dep = late_dependents ? 1 : 0;
   const int stage_bytes = (wide ? 2 : 1) * W_STAGE_BYTES + x_bytes;
   int stages = (g_smem_optin - 2048) / stage_bytes;
   if (stages > MAX_STAGES) stages = MAX_STAGES;

@@ -295,7 +295,7 @@ RowPlan row_plan(koala_ctx *c) {
 // Y = X * [W...]^T as a (possibly split) fp32 result in the partial buffer, or directly into
 // `direct` (ld = ld_direct) when given.
 int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct, int ld_direct,
-            SplitIn *out) {
+            SplitIn *out, bool late_dependents = false) {
   int ncols = 0;
   for (int i = 0; i < m.n; ++i) ncols += m.n_out[i];
   float *Y = direct ? direct : c->P + c->p_off;
@@ -308,7 +308,7 @@ int do_gemm(koala_ctx *c, Operand X, int K_in, GemmMats m, int R, float *direct,
     const int tb = time_begin(c, KOALA_CLS_GEMM_TC, wbytes);
     SplitIn res;
     CU_TRY(gemm_tc(LN(c), X, c->Mp, m, K_in, R, Y, ld, direct ? 1 : 0, stride, c->status, slots, &res,
-                   c->ingest_blocks > 0));
+                   c->ingest_blocks > 0, late_dependents));
     time_end(c, tb);
     if (out) *out = res;
   } else {
@@ -362,13 +362,23 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
   const RowMap same{0, 0};
   SplitIn s;
   GemmMats qkv{{w.wq, w.wk, w.wv}, {H, H, H}, 3};
-  K_TRY(do_gemm(c, c->xn, H, qkv, R, nullptr, 0, &s));
-  CU_TRY(rope_kv_write(LN(c), g.dtype, s, c->pending, row_plan(c), c->qbuf, c->qpair, kc, vc, R, rows_per_seq, g.n_heads,
-                       g.head_dim, g.S_max));
-  c->pending = none;
-  if (kv_only) return KOALA_OK;
-  // (the context of a prompt block includes rows of the same forward: nothing of it may be read early)
-  K_TRY(run_attention(c, kc, vc, R, rows_per_seq, c->ingest_blocks == 0));
+  // with a row or two per sequence the attention may take the multiply's partial sums itself
+  const bool few = c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && c->ingest_blocks == 0 && !kv_only && tc_supported(qkv, H) &&
+                   attn_few_takes_sums(rows_per_seq, g.B, g.n_heads, g.S_max, NUM_SMS);
+  K_TRY(do_gemm(c, c->xn, H, qkv, R, nullptr, 0, &s, few));
+  if (few && attn_few_rope_supported(s)) {
+    const int ta = time_begin(c, KOALA_CLS_ATTENTION, 0);
+    CU_TRY(tree_attention_few_rope(LN(c), s, c->pending, kc, vc, row_plan(c), c->attn_out, rows_per_seq, g.B, g.n_heads, g.S_max, NUM_SMS));
+    time_end(c, ta);
+    c->pending = none;
+  } else {
+    CU_TRY(rope_kv_write(LN(c), g.dtype, s, c->pending, row_plan(c), c->qbuf, c->qpair, kc, vc, R, rows_per_seq, g.n_heads,
+                         g.head_dim, g.S_max));
+    c->pending = none;
+    if (kv_only) return KOALA_OK;
+    // (the context of a prompt block includes rows of the same forward: nothing of it may be read early)
+    K_TRY(run_attention(c, kc, vc, R, rows_per_seq, c->ingest_blocks == 0));
+  }
   GemmMats o{{w.wo, nullptr, nullptr}, {H, 0, 0}, 1};
   K_TRY(do_gemm(c, c->attn_out, H, o, R, nullptr, 0, &s));
   RowScale ffn = none;
