@@ -294,7 +294,7 @@ __global__ void rope_kv_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__
   v_cache[base + i + half] = from_f<T>(v1);
 }
 
-// One CTA per row; a thread rotates two adjacent pairs (i, i+1) and (i + half, i + half + 1) of
+// One CTA per row (or ROWS of them); a thread rotates two adjacent pairs (i, i+1) and (i + half, i + half + 1) of
 // one head with 8-byte loads.
 template <int NS>
 __device__ __forceinline__ float2 split_sum2(const SplitIn &P, int r, int c, int k) {
@@ -314,52 +314,58 @@ __device__ __forceinline__ void store2(float *p, float a, float b) { *reinterpre
 __device__ __forceinline__ void store2(bf16 *p, float a, float b) {
   *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
-template <typename T, int NS, bool SK>
+// ROWS: consecutive rows of a thread, see several_rows.
+template <typename T, int NS, bool SK, int ROWS>
 __global__ void __launch_bounds__(128)
 rope_kv_vec_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__restrict__ q_out, bf16 *__restrict__ qp_hi,
                    bf16 *__restrict__ qp_lo, T *__restrict__ k_cache, T *__restrict__ v_cache, int rows_per_seq,
-                   int n_heads, int head_dim, int S_max) {
+                   int n_heads, int head_dim, int S_max, int R) {
   pdl_wait();
   pdl_launch_dependents();                // in this order: see rope_kv_write
-  const int r = blockIdx.x;
+  const int r0 = blockIdx.x * ROWS;
   const int half = head_dim >> 1, H = n_heads * head_dim, hq = half >> 1;
-  const int b = plan.cache_of(r / rows_per_seq);
-  const int slot = plan.slot[r];
-  const bool wr = slot >= 0 && slot < S_max;
-  const float rs = sc.of(r);
   // grid.y slices the row's work so that many SMs pull the partial sums
   const int p = blockIdx.y * blockDim.x + threadIdx.x;
   if (p < n_heads * hq) {
     const int h = p / hq, i = (p - h * hq) * 2;
-    const float4 cs = *reinterpret_cast<const float4 *>(&plan.rope[(size_t)r * half + i]);   // c0 s0 c1 s1
     const int c0 = h * head_dim + i, c1 = c0 + half;
     // all partial sums of this thread are requested before the first store (a head lies in one weight
     // tile where tiles are dealt unevenly: there head_dim is 128 and a tile is a multiple of it)
-    const int kq = slots_at<NS, SK>(qkv, r, c0), kk = slots_at<NS, SK>(qkv, r, H + c0), kv = slots_at<NS, SK>(qkv, r, 2 * H + c0);
-    float2 qa = split_sum2<NS>(qkv, r, c0, kq), qb = split_sum2<NS>(qkv, r, c1, kq);
-    float2 ka = split_sum2<NS>(qkv, r, H + c0, kk), kb = split_sum2<NS>(qkv, r, H + c1, kk);
-    float2 va = split_sum2<NS>(qkv, r, 2 * H + c0, kv), vb = split_sum2<NS>(qkv, r, 2 * H + c1, kv);
-    qa.x *= rs; qa.y *= rs; qb.x *= rs; qb.y *= rs;
-    const float2 ra = make_float2(qa.x * cs.x - qb.x * cs.y, qa.y * cs.z - qb.y * cs.w);
-    const float2 rb = make_float2(qb.x * cs.x + qa.x * cs.y, qb.y * cs.z + qa.y * cs.w);
-    store2(q_out + (size_t)r * H + c0, ra.x, ra.y);
-    store2(q_out + (size_t)r * H + c1, rb.x, rb.y);
-    if (qp_hi != nullptr) {      // the same values as a bf16 pair (value + rounding residual)
-      const __nv_bfloat162 ha = __floats2bfloat162_rn(ra.x, ra.y), hb = __floats2bfloat162_rn(rb.x, rb.y);
-      const float2 fa = __bfloat1622float2(ha), fb = __bfloat1622float2(hb);
-      *reinterpret_cast<__nv_bfloat162 *>(qp_hi + (size_t)r * H + c0) = ha;
-      *reinterpret_cast<__nv_bfloat162 *>(qp_hi + (size_t)r * H + c1) = hb;
-      *reinterpret_cast<__nv_bfloat162 *>(qp_lo + (size_t)r * H + c0) = __floats2bfloat162_rn(ra.x - fa.x, ra.y - fa.y);
-      *reinterpret_cast<__nv_bfloat162 *>(qp_lo + (size_t)r * H + c1) = __floats2bfloat162_rn(rb.x - fb.x, rb.y - fb.y);
+    const int kq = slots_at<NS, SK>(qkv, r0, c0), kk = slots_at<NS, SK>(qkv, r0, H + c0), kv = slots_at<NS, SK>(qkv, r0, 2 * H + c0);
+#pragma unroll
+    for (int ri = 0; ri < ROWS; ++ri) {
+      const int r = r0 + ri;
+      if (ROWS > 1 && r >= R) break;
+      const int b = plan.cache_of(r / rows_per_seq);
+      const int slot = plan.slot[r];
+      const bool wr = slot >= 0 && slot < S_max;
+      const float rs = sc.of(r);
+      const float4 cs = *reinterpret_cast<const float4 *>(&plan.rope[(size_t)r * half + i]);   // c0 s0 c1 s1
+      float2 qa = split_sum2<NS>(qkv, r, c0, kq), qb = split_sum2<NS>(qkv, r, c1, kq);
+      float2 ka = split_sum2<NS>(qkv, r, H + c0, kk), kb = split_sum2<NS>(qkv, r, H + c1, kk);
+      float2 va = split_sum2<NS>(qkv, r, 2 * H + c0, kv), vb = split_sum2<NS>(qkv, r, 2 * H + c1, kv);
+      qa.x *= rs; qa.y *= rs; qb.x *= rs; qb.y *= rs;
+      const float2 ra = make_float2(qa.x * cs.x - qb.x * cs.y, qa.y * cs.z - qb.y * cs.w);
+      const float2 rb = make_float2(qb.x * cs.x + qa.x * cs.y, qb.y * cs.z + qa.y * cs.w);
+      store2(q_out + (size_t)r * H + c0, ra.x, ra.y);
+      store2(q_out + (size_t)r * H + c1, rb.x, rb.y);
+      if (qp_hi != nullptr) {      // the same values as a bf16 pair (value + rounding residual)
+        const __nv_bfloat162 ha = __floats2bfloat162_rn(ra.x, ra.y), hb = __floats2bfloat162_rn(rb.x, rb.y);
+        const float2 fa = __bfloat1622float2(ha), fb = __bfloat1622float2(hb);
+        *reinterpret_cast<__nv_bfloat162 *>(qp_hi + (size_t)r * H + c0) = ha;
+        *reinterpret_cast<__nv_bfloat162 *>(qp_hi + (size_t)r * H + c1) = hb;
+        *reinterpret_cast<__nv_bfloat162 *>(qp_lo + (size_t)r * H + c0) = __floats2bfloat162_rn(ra.x - fa.x, ra.y - fa.y);
+        *reinterpret_cast<__nv_bfloat162 *>(qp_lo + (size_t)r * H + c1) = __floats2bfloat162_rn(rb.x - fb.x, rb.y - fb.y);
+      }
+      if (!wr) continue;
+      ka.x *= rs; ka.y *= rs; kb.x *= rs; kb.y *= rs;
+      va.x *= rs; va.y *= rs; vb.x *= rs; vb.y *= rs;
+      const size_t base = (((size_t)b * n_heads + h) * S_max + slot) * head_dim + i;
+      store2(k_cache + base, ka.x * cs.x - kb.x * cs.y, ka.y * cs.z - kb.y * cs.w);
+      store2(k_cache + base + half, kb.x * cs.x + ka.x * cs.y, kb.y * cs.z + ka.y * cs.w);
+      store2(v_cache + base, va.x, va.y);
+      store2(v_cache + base + half, vb.x, vb.y);
     }
-    if (!wr) return;
-    ka.x *= rs; ka.y *= rs; kb.x *= rs; kb.y *= rs;
-    va.x *= rs; va.y *= rs; vb.x *= rs; vb.y *= rs;
-    const size_t base = (((size_t)b * n_heads + h) * S_max + slot) * head_dim + i;
-    store2(k_cache + base, ka.x * cs.x - kb.x * cs.y, ka.y * cs.z - kb.y * cs.w);
-    store2(k_cache + base + half, kb.x * cs.x + ka.x * cs.y, kb.y * cs.z + ka.y * cs.w);
-    store2(v_cache + base, va.x, va.y);
-    store2(v_cache + base + half, vb.x, vb.y);
   }
 }
 
@@ -375,18 +381,25 @@ __global__ void swiglu_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *_
   store_operand(act, act_lo, (size_t)r * F + f, silu_f(rs * gu.at(r, f)) * (rs * gu.at(r, F + f)));
 }
 
-template <typename T, int NS, bool SK>
-__global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int F) {
+template <typename T, int NS, bool SK, int ROWS>
+__global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int R, int F) {
   pdl_launch_dependents();
   pdl_wait();
-  const int r = blockIdx.y;
+  const int r0 = blockIdx.y * ROWS;
   const int f = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (f >= F) return;
-  const float rs = sc.of(r);
-  const float4 a = split_sum4<NS>(gu, r, f, slots_at<NS, SK>(gu, r, f)), b = split_sum4<NS>(gu, r, F + f, slots_at<NS, SK>(gu, r, F + f));
-  store_operand4(act, act_lo, (size_t)r * F + f,
-                 make_float4(silu_f(rs * a.x) * (rs * b.x), silu_f(rs * a.y) * (rs * b.y),
-                             silu_f(rs * a.z) * (rs * b.z), silu_f(rs * a.w) * (rs * b.w)));
+  const int ka = slots_at<NS, SK>(gu, r0, f), kb = slots_at<NS, SK>(gu, r0, F + f);
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    const int r = r0 + i;
+    if (ROWS > 1 && r >= R) break;
+    const float rs = sc.of(r);
+    const float4 a = split_sum4<NS>(gu, r, f, ka), b = split_sum4<NS>(gu, r, F + f, kb);
+    auto silu = [](float v) { return ROWS > 1 ? v / (1.f + expf(-v)) : silu_f(v); };
+    store_operand4(act, act_lo, (size_t)r * F + f,
+                   make_float4(silu(rs * a.x) * (rs * b.x), silu(rs * a.y) * (rs * b.y),
+                               silu(rs * a.z) * (rs * b.z), silu(rs * a.w) * (rs * b.w)));
+  }
 }
 
 // ------------------------------------------------------------------------------- arg-max / top-k
@@ -678,6 +691,14 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
     SPLIT_CASE(12, true, __VA_ARGS__)                                             \
   }
 
+// More than 256 rows with few partial sums each: a thread takes several rows of its columns, so that the number of the
+// partial sums, four integer divisions, is found once for them (token tiles are multiples of 32 rows: consecutive rows share
+// one).  us per launch by rows per thread 1 / 2 / 4 / 8: SwiGLU, 509 rows of the 7B prompt 25.1 / 22.2 / 20.5 / 23.5, about 860 rows of
+// the 13B prompts 57 / 49.5 / 44.5 / 47; rotary step 18.1 / 15.8 / 16.5 / 25.4 and 39 / 34.3 / 33.1 / 34.3.  Up to 256 rows there
+// are too few threads then (128 rows: SwiGLU 5.3 / 5.7 / 8.8; 256 rows 8.6 / 9.0 / 11.5); the residual update, which
+// has up to twelve partial sums in flight per thread, gains nothing (10.6 / 10.5 / 16.5).
+static bool several_rows(const SplitIn &P, int R) { return P.sk_ctas != 0 && P.n <= 3 && R > 256; }
+
 cudaError_t embed_norm(Launch L, int dtype, const int32_t *tok, const void *E, const void *g,
                        float *x, Operand xn, int R, int H, int V, float eps) {
   DISPATCH_T(dtype, return launch_k(embed_norm_kernel<T>, dim3(R), dim3(256), 0, L.st, L.pdl, tok,
@@ -755,9 +776,12 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
     const int work = n_heads * head_dim / 4;
     const int threads = work < 128 ? ((work + 31) / 32) * 32 : 128;
     const int slices = (work + threads - 1) / threads;
-    FOR_SPLIT(dtype, qkv, return launch_k(rope_kv_vec_kernel<T, NS, SK>, dim3(R, slices), dim3(threads), 0, L.st, L.pdl,
+    if (dtype != 0 && several_rows(qkv, R))
+      return launch_k(rope_kv_vec_kernel<bf16, 3, true, 2>, dim3((R + 1) / 2, slices), dim3(threads), 0, L.st, L.pdl, qkv, sc, plan,
+                      q_out, qh, ql, (bf16 *)k_cache, (bf16 *)v_cache, rows_per_seq, n_heads, head_dim, S_max, R);
+    FOR_SPLIT(dtype, qkv, return launch_k(rope_kv_vec_kernel<T, NS, SK, 1>, dim3(R, slices), dim3(threads), 0, L.st, L.pdl,
                                           qkv, sc, plan, q_out, qh, ql, (T *)k_cache, (T *)v_cache, rows_per_seq,
-                                          n_heads, head_dim, S_max);)
+                                          n_heads, head_dim, S_max, R);)
   }
   DISPATCH_T(dtype, return launch_k(rope_kv_kernel<T>, dim3(R, n_heads), dim3(head_dim / 2), 0, L.st,
                                     L.pdl, qkv, sc, plan, q_out, qh, ql, (T *)k_cache, (T *)v_cache,
@@ -766,8 +790,11 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
 
 cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, int R, int F) {
   if (F % 4 == 0 && gu.ld % 4 == 0 && gu.stride % 4 == 0) {
-    FOR_SPLIT(dtype, gu, return launch_k(swiglu_vec_kernel<T, NS, SK>, dim3((F / 4 + 255) / 256, R), dim3(256), 0, L.st,
-                                         L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)
+    if (dtype != 0 && several_rows(gu, R))
+      return launch_k(swiglu_vec_kernel<bf16, 3, true, 4>, dim3((F / 4 + 255) / 256, (R + 3) / 4), dim3(256), 0, L.st, L.pdl, gu, sc,
+                      (bf16 *)act.hi, (bf16 *)act.lo, R, F);
+    FOR_SPLIT(dtype, gu, return launch_k(swiglu_vec_kernel<T, NS, SK, 1>, dim3((F / 4 + 255) / 256, R), dim3(256), 0, L.st,
+                                         L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, R, F);)
   }
   DISPATCH_T(dtype, return launch_k(swiglu_kernel<T>, dim3((F + 255) / 256, R), dim3(256), 0, L.st,
                                     L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)

@@ -75,6 +75,13 @@ def test_7b_shaped_prompts(kind, n, chunk):
     eng.close()
 
 
+@pytest.mark.parametrize("n", [[261], [270], [258, 100]])
+def test_prompts_whose_rows_are_not_whole_groups_of_a_thread(n):
+    """Above 256 rows a thread of the rotary and SwiGLU kernels takes two and four rows: 261 rows (three blocks of 87), 270,
+    and 360 with rows of a second sequence."""
+    test_7b_shaped_prompts("eagle", n, 64)
+
+
 def test_a_prompt_beyond_the_capacity_is_reported():
     cfg = TINY_EAGLE.with_(S_max=100)
     eng, _, _ = make_pair(cfg)
