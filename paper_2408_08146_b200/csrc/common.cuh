@@ -38,14 +38,16 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// CTAs (= partial sums) that share stream-K tile `tile` of sk_kb K-blocks.  Not inlined: the kernels that
-// add partial sums run each instruction once or twice per launch, so what they cost is mostly the fetch
-// of their instructions, and two integer divisions per column group are a large part of them.
-static __device__ __noinline__ int sk_count(unsigned tile, unsigned ctas, unsigned units, unsigned kb) {
+// n / d for 32-bit n, d >= 2, with div_inverse(d) = floor(2^64 / d) + 1: the product is off by less than n / 2^64, below 1 / d.
+static __host__ __device__ __forceinline__ unsigned long long div_inverse(unsigned d) { return ~0ull / d + 1ull; }
+__device__ __forceinline__ unsigned div_by(unsigned n, unsigned long long inv) { return (unsigned)__umul64hi((unsigned long long)n, inv); }
+
+// CTAs (= partial sums) that share stream-K tile `tile` of sk_kb K-blocks, 1 / units given as an inverse: the kernels
+// that add partial sums run each instruction once or twice per launch, and two integer divisions per column group were a
+// large part of them.
+__device__ __forceinline__ int sk_count(unsigned tile, unsigned ctas, unsigned long long units_inv, unsigned kb) {
   const unsigned u0 = tile * kb;
-  const unsigned first = ((u0 + 1u) * ctas - 1u) / units;
-  const unsigned last = ((u0 + kb) * ctas - 1u) / units;
-  return (int)(last - first) + 1;
+  return (int)(div_by((u0 + kb) * ctas - 1u, units_inv) - div_by((u0 + 1u) * ctas - 1u, units_inv)) + 1;
 }
 
 // A matrix given as the sum of partial matrices `stride` floats apart (split-K results).
@@ -64,16 +66,21 @@ struct SplitIn {
   unsigned sk_m0, sk_m1, sk_t0, sk_t1;
   // several token tiles of sk_tt rows dealt in the same launch (0 = one): tile = weight tile * sk_zt + row / sk_tt * sk_wt
   unsigned sk_zt, sk_tt, sk_wt;
+  unsigned long long sk_uinv, sk_tinv;      // div_inverse of sk_units and of sk_tt (set_inverses)
+  void set_inverses() {
+    sk_uinv = sk_units > 1 ? div_inverse(sk_units) : 0ull;
+    sk_tinv = sk_tt > 1 ? div_inverse(sk_tt) : 0ull;
+  }
   // Stream-K tile that column c (of row r) belongs to.
   __device__ __forceinline__ unsigned tile_of(int r, int c) const {
     const unsigned sh = 7u + sk_wide, uc = (unsigned)c;
     unsigned tile = uc >> sh;
     if (sk_m0 != 0 && uc >= sk_m0) tile = uc < sk_m1 ? sk_t0 + ((uc - sk_m0) >> sh) : sk_t1 + ((uc - sk_m1) >> sh);
-    if (sk_tt != 0) tile = tile * sk_zt + (unsigned)r / sk_tt * sk_wt;
+    if (sk_tt != 0) tile = tile * sk_zt + div_by((unsigned)r, sk_tinv) * sk_wt;
     return tile;
   }
   __device__ __forceinline__ int count(int r, int c) const {
-    return sk_ctas == 0 ? n : sk_count(tile_of(r, c), sk_ctas, sk_units, sk_kb);
+    return sk_ctas == 0 ? n : sk_count(tile_of(r, c), sk_ctas, sk_uinv, sk_kb);
   }
   __device__ __forceinline__ float at(int r, int c) const {
     const float *q = p + (size_t)r * ld + c;

@@ -297,12 +297,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       unsigned seg_hi = (unsigned)(tile + 1) * KB;
       if (seg_hi > u_hi) seg_hi = u_hi;
       const int buf = seg % P.nbuf;
-      if (!dry) {
-        ok = mbar_wait(&acc_full[buf], (uint32_t)(seg / P.nbuf) & 1u);
-        if (!ok) break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      int row0, col_off = 0, n_rows = P.n0;
+      int row0, col_off = 0, n_rows = P.n0;                // (where the sums go is found before the wait)
       if (tile >= P.tiles1) { row0 = (tile - P.tiles1) * bm; col_off = P.n0 + P.n1; n_rows = P.n2; }
       else if (tile >= P.tiles0) { row0 = (tile - P.tiles0) * bm; col_off = P.n0; n_rows = P.n1; }
       else row0 = tile * bm;
@@ -311,6 +306,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       int slot = blockIdx.y;
       if (P.sk_ctas > 0)
         slot = (int)blockIdx.x - (int)sk_owner((unsigned)tile * KB, (unsigned)P.sk_ctas, P.sk_units);
+      if (!dry) {
+        ok = mbar_wait(&acc_full[buf], (uint32_t)(seg / P.nbuf) & 1u);
+        if (!ok) break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
       for (int hw = 0; hw < (WIDE ? 2 : 1); ++hw) {      // wide: one accumulator per 128 weight rows
       const int feat = row0 + hw * BM + quarter * 32 + lane;
@@ -1071,6 +1071,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
         si.sk_t0 = (unsigned)q0;
         si.sk_t1 = (unsigned)(q0 + q1);
       }
+      si.set_inverses();
       *out = si;
       const int stage = (chain ? 1 : 2) * PAIR_PART_BYTES + ptt * BK * 2;
       P.stages = (g_smem_optin - 2048) / stage < PAIR_MAX_STAGES ? (g_smem_optin - 2048) / stage : PAIR_MAX_STAGES;
@@ -1190,6 +1191,7 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   if (out) {
     *out = SplitIn{Y, sk ? sk_slots : split, split_stride, ldy, sk ? (unsigned)sk_ctas : 0u, P.sk_units,
                    (unsigned)P.kblocks, (sk && wide) ? 1u : 0u};
+    out->set_inverses();
   }
   // Epilogue warps per 32 accumulator lanes.  256-row tiles keep one accumulator set, so the MMAs
   // of a CTA's next tile wait for the epilogue: sixteen warps (13B-shaped verification of 256 rows:

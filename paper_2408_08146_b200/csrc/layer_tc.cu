@@ -770,7 +770,10 @@ cudaError_t layer_stream(Launch L, const LayerJob &job, unsigned *sync, unsigned
     ph.out_lo = (bf16 *)j.out.lo;
     ph.sumsq = j.sumsq;
     ph.ncols = j.ncols;
-    if (outs) outs[p] = SplitIn{j.Y, slots, j.split_stride, j.ldy, (unsigned)ph.ctas, ph.units, (unsigned)ph.kblocks};
+    if (outs) {
+      outs[p] = SplitIn{j.Y, slots, j.split_stride, j.ldy, (unsigned)ph.ctas, ph.units, (unsigned)ph.kblocks};
+      outs[p].set_inverses();
+    }
     ph.done_target = (use_count[p] + 1u) * (unsigned)grid;     // use_count advances once the launch is accepted
     ph.ready_target = ph.done_target;
     for (int i = 0; i < 3; ++i) {

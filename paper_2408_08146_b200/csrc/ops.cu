@@ -75,7 +75,7 @@ __global__ void row_epilogue_kernel(int mode, float *__restrict__ x, SplitIn P,
 template <int NS, bool SK>
 __device__ __forceinline__ int slots_at(const SplitIn &P, int r, int c) {
   if (!SK) return P.n;
-  return sk_count(P.tile_of(r, c), P.sk_ctas, P.sk_units, P.sk_kb);
+  return sk_count(P.tile_of(r, c), P.sk_ctas, P.sk_uinv, P.sk_kb);
 }
 template <int NS>
 __device__ __forceinline__ float4 split_sum4(const SplitIn &P, int r, int c, int k) {
