@@ -53,7 +53,7 @@ struct TcParams {
   int ldy;
   int R;              // valid tokens
   int bn;             // MMA N = rows of the activation tile in shared memory, multiple of 16, <= 256
-  int tt;             // tokens per tile: bn, or bn / 2 when the activations are a hi/lo pair
+  int tt;             // tokens per tile: bn, or bn / 2 (a multiple of 8) when the activations are a hi/lo pair
   int ztiles;         // token tiles (classic mode; fastest-varying part of blockIdx.x)
   int wtiles;         // CTA pairs in chains: weight tiles
   int tmem_cols;      // power of two >= max(32, bn), per accumulator buffer
@@ -281,7 +281,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
     const int quarter = warp & 3;        // the 32 tensor-memory lanes this warp may read
     // with more than four epilogue warps the warps of a lane quarter share the token columns
     const int n_ch = ((int)(blockDim.x >> 5) - 2) >> 2;
-    const int c_per = (((P.tt >> 4) + n_ch - 1) / n_ch) << 4;
+    const int c_per = ((((P.tt + 15) >> 4) + n_ch - 1) / n_ch) << 4;
     const int c_lo = min(((warp - 2) >> 2) * c_per, P.tt);
     const int c_hi = min(c_lo + c_per, P.tt);
     // A dry pass first: the loop body once with nothing stored and nothing waited for, while the
@@ -316,7 +316,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       const int feat = row0 + hw * BM + quarter * 32 + lane;
       float *Yp = P.Y + (size_t)slot * P.split_stride + col_off + feat;
       const uint32_t lane_base = tmem_acc + (uint32_t)((buf + hw) * P.tmem_cols) + ((uint32_t)(quarter * 32) << 16);
-      // 16 token columns per step, in a rolled loop: the accumulator reads of one warp hide behind the stores
+      // 16 token columns per step (the last eight of a tile may bring eight that are not stored), in a rolled loop: the accumulator reads of one warp hide behind the stores
       // of the others, and the loop's instructions are fetched once.
 #pragma unroll 1
       for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
@@ -967,7 +967,12 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   // weights are passed over once; up to 128 tokens the residual rows are extra accumulator columns.
   const int accp = (pair && R > 128 && !g_tune_no_accp) ? 1 : 0;
   const int tt_max = (pair && !accp) ? 128 : 256;
-  int tt = ((R + 15) / 16) * 16;
+  // (A pair's tile is twice as many MMA columns, so up to 128 rows tokens come in eights: the bytes saved are weight
+  // stages.  Sixteens / eights, six layers, us per pass: 7B one-token step 581 / 575, four sequences 655 / 649, eight
+  // 602 / 594, 13B one token 813 / 796, 40 rows 785 / 778, 72 rows 858 / 854, 100 rows 2184 / 2171.  Not 17 to 24 rows: the
+  // multiplies gain there too, 16.4 -> 16.2 us each, but 20 rows take 745 / 755 in all.)
+  const int unit = pair && R <= 128 && (R <= 16 || R > 24) ? 8 : 16;
+  int tt = (R + unit - 1) / unit * unit;
   if (tt > tt_max) tt = tt_max;
   if (tt > x_rows_alloc) return cudaErrorInvalidValue;
   const int bn = (pair && !accp) ? 2 * tt : tt;
