@@ -71,6 +71,8 @@ constexpr int OSTRIDE = DH + 4;              // floats of a row of the chunk's r
 // the chunk's result goes where the K/V buffers were
 static_assert(64 * OSTRIDE * 4 <= 2 * 4 * SUB && 128 * OSTRIDE * 4 <= 3 * 4 * SUB, "the chunk's result fits");
 
+// Two floats as bf16 value + rounding residual.  (Probabilities too: cutting their value part off instead of rounding it is no
+// faster and leaves a residual twice as large; whole layer of the 7B shape against float64 1.02e-5 instead of 8.4e-6.)
 __device__ __forceinline__ void split_pack(float x, float y, uint32_t &hi, uint32_t &lo) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
   const float2 hf = __bfloat1622float2(h);
@@ -83,14 +85,6 @@ __device__ __forceinline__ float ex2_fast(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-// Probabilities p in [0, 1] as a bf16 pair: hi = p truncated to bf16 (exactly representable, so
-// p - hi is exact), lo = that remainder rounded to bf16.  |p - hi - lo| <= 2^-17 p.
-__device__ __forceinline__ void split_pack_trunc(float x, float y, uint32_t &hi, uint32_t &lo) {
-  const uint32_t xb = __float_as_uint(x) & 0xffff0000u, yb = __float_as_uint(y) & 0xffff0000u;
-  hi = __byte_perm(xb, yb, 0x7632);                 // (y.hi16 << 16) | x.hi16
-  const __nv_bfloat162 l = __floats2bfloat162_rn(x - __uint_as_float(xb), y - __uint_as_float(yb));
-  lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -505,7 +499,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
           const float p0 = ex2_fast(fmaf(__uint_as_float(v[ch * 8 + 2 * e]), sc, -mu));
           const float p1 = ex2_fast(fmaf(__uint_as_float(v[ch * 8 + 2 * e + 1]), sc, -mu));
           l_t += p0 + p1;
-          split_pack_trunc(p0, p1, hi[e], lo[e]);
+          split_pack(p0, p1, hi[e], lo[e]);
         }
         const uint32_t off = (((uint32_t)(ch + (NC / 8) * half)) ^ psw) << 4;
         st_shared_v4(pb + off, hi[0], hi[1], hi[2], hi[3]);
@@ -691,7 +685,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQh, const __grid_const
 
 // Fewer query rows per sequence than this: the mma.sync kernel.  (tcgen05 / mma.sync, 32 heads, eight layers, us per
 // forward: one sequence at context 2000 12 rows 829 / 808, 16 rows 834 / 817, 20 rows 843 / 879; four sequences at
-// 500 8 rows 810 / 835, 15 rows 915 / 966.  Batches would gain from eight rows on, one sequence lose.)
+// 500 8 rows 810 / 835, 15 rows 915 / 966.  Batches of 0.6 to 1 (sequence, head) pairs per SM would gain from three rows on, fifteen
+// rows of four sequences 947 / 902 us a pass, but P V is summed over all of a chunk's tiles in one truncating accumulator here:
+// whole layer against float64 8.4e-6 where mma.sync leaves 8.0e-6.)
 int g_attn_tc_min_rows = 16;
 int g_attn_tc_chunks = 0;      // > 0: this many key chunks whatever the shape (A/B runs)
 int g_attn_tc_dry_pass = 1;
