@@ -1183,7 +1183,12 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   if (g_tune_stages > 0 && g_tune_stages < stages) stages = g_tune_stages;
   if (stages < 2) return cudaErrorInvalidValue;
   P.stages = stages;
-  P.early_w = g_tune_late_w ? 0 : (g_tune_early_stages >= 0 && g_tune_early_stages < stages ? g_tune_early_stages : stages);
+  // Not more than five stages before the dependency wait: the kernel before this one reads its partial sums behind those
+  // requests (residual update at one row 2.9 us with two early stages, 4.4 with five, 4.9 with six).  Six stages, early 3 / 4 / 5 / 6, six
+  // layers of the 7B shape, us per pass: one-token step 577 / 572 / 569 / 573, four sequences 650 / 646 / 640 / 644, chain of
+  // five 1273 / 1266 / 1259 / 1267.
+  const int early = g_tune_early_stages >= 0 ? g_tune_early_stages : 5;
+  P.early_w = g_tune_late_w ? 0 : (early < stages ? early : stages);
   CUtensorMap mw[3], mx, mxlo;
   for (int i = 0; i < 3; ++i) {
     const int j = i < m.n ? i : 0;
