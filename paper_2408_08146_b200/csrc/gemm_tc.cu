@@ -47,6 +47,7 @@ constexpr int THREADS_WIDE = 576;   // most threads a launch uses: producer warp
 constexpr int W_STAGE_BYTES = BM * BK * 2;
 constexpr int E_TIMEOUT = 6;
 constexpr int MAX_STAGES = 12;
+constexpr int EARLY_STAGES = 2, PACE_CYCLES = 1600;      // weights before the dependency wait, see gemm_tc()
 
 struct TcParams {
   float *Y;
@@ -67,6 +68,7 @@ struct TcParams {
   size_t split_stride;
   int stages;
   int early_w;        // how many of the first stages' weight tiles are requested before the dependency wait
+  int pace;           // > 0: the MMA thread requests the stages past early_w, one per so many cycles, until the first stage is complete
   int late_dep;       // 1: the next kernel may start only once everything before this one is complete (one-CTA form)
   int epi_dry;        // 1: the epilogue warps make a dry pass over their loop body (nothing stored) at kernel start
   int *status;
@@ -196,7 +198,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
 #pragma unroll 1
       for (int it = 0; it < pre; ++it) {
         unsigned char *xd = tiles + (size_t)it * stage_bytes + w_stage_bytes;
-        if (it >= P.early_w) {
+        if (it >= P.early_w && P.pace == 0) {
           mbar_expect_tx(&full_bar[it], (uint32_t)stage_bytes);
           load_w(tmW, &full_bar[it], tiles + (size_t)it * stage_bytes, kb, row0);
         }
@@ -231,6 +233,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       // instruction descriptor: D fp32, A and B bf16, both K-major, N = bn, M = 128
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.bn >> 3) << 17) |
                              ((uint32_t)(BM >> 4) << 24);
+      if (P.pace > 0) {
+        // the weight stages past the early ones, spread over the time of the kernel before, until the first stage is complete
+        int tile = (int)(u_lo / KB), kb = (int)(u_lo % KB), row0;
+        for (int it = 0; it < P.early_w && it < pre; ++it)
+          if (++kb == KB) { kb = 0; ++tile; }
+        const CUtensorMap *tmW = tile_map(tile, row0);
+        const long long t0 = clock64();
+#pragma unroll 1
+        for (int it = P.early_w; it < pre; ++it) {
+          while (clock64() - t0 < (long long)(it - P.early_w + 1) * P.pace && !mbar_try(smem_u32(&full_bar[0]), 0)) {}
+          mbar_expect_tx(&full_bar[it], (uint32_t)stage_bytes);
+          load_w(tmW, &full_bar[it], tiles + (size_t)it * stage_bytes, kb, row0);
+          if (++kb == KB) { kb = 0; ++tile; tmW = tile_map(tile, row0); }
+        }
+      }
       bool ok = true;
       int seg = 0;                        // segment = run of units inside one tile
       bool seg_start = true;
@@ -750,6 +767,7 @@ int g_tune_no_pair2 = 0;    // 1 = no CTA-pair kernel; 2 = not for 65 to 128 tok
 int g_tune_pair_min = 0;    // > 0: fewest rows for the CTA-pair kernel
 int g_tune_epi_dry = 1;
 int g_tune_short_sums = 0;  // 1 = the CTA-pair kernel always sums in short chains, from 65 rows up
+int g_tune_pace = PACE_CYCLES;      // 0 = the stages past the early ones come with their activations
 int g_tune_no_wide = 0;      // 1 = 128 weight rows per CTA also for wide token tiles
 int g_tune_traffic_div = 8; // split <= K_in / (div * tokens)
 
@@ -870,6 +888,7 @@ void tc_set_tuning(int key, int value) {
   if (key == 21) g_tune_epi_dry = value;
   if (key == 22) attn_mma_set_chunks(value);
   if (key == 23) g_tune_short_sums = value;
+  if (key == 24) g_tune_pace = value;
   if (key == 2) g_tune_max_split = value;
   if (key == 3) g_tune_no_streamk = value;
   if (key == 6) g_tune_late_w = value;
@@ -1183,12 +1202,15 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   if (g_tune_stages > 0 && g_tune_stages < stages) stages = g_tune_stages;
   if (stages < 2) return cudaErrorInvalidValue;
   P.stages = stages;
-  // Not more than five stages before the dependency wait: the kernel before this one reads its partial sums behind those
-  // requests (residual update at one row 2.9 us with two early stages, 4.4 with five, 4.9 with six).  Six stages, early 3 / 4 / 5 / 6, six
-  // layers of the 7B shape, us per pass: one-token step 577 / 572 / 569 / 573, four sequences 650 / 646 / 640 / 644, chain of
-  // five 1273 / 1266 / 1259 / 1267.
-  const int early = g_tune_early_stages >= 0 ? g_tune_early_stages : 5;
+  // Two stages at once, the rest of the ring one per PACE_CYCLES: the kernel before this one reads its partial sums while they
+  // are on their way, and behind a whole ring of every CTA at once (up to 28 MB) those reads took most of its time - the residual
+  // update at one row 4.9 us, 2.9 with two stages only; paced, the ring is as full when the activations come.  Six layers, us
+  // per pass, whole ring at once / two and one per 800 / 1200 / 1600 / 2000 / 2600 cycles: 7B one-token step 573 / 561 / 554 /
+  // 552 / 554 / 559, four sequences 644 / 628 / 623 / 622 / 626 / 630, chain of five 1266 / 1238 / 1223 / 1222 / 1225 / 1230, 64
+  // nodes 818 / 811 / 811 / 810 / 809 / 811, EAGLE iteration of 60 2016 / 1991 / 1978 / 1971 / 1970 / 1977.
+  const int early = g_tune_early_stages >= 0 ? g_tune_early_stages : EARLY_STAGES;
   P.early_w = g_tune_late_w ? 0 : (early < stages ? early : stages);
+  P.pace = P.early_w > 0 ? g_tune_pace : 0;
   CUtensorMap mw[3], mx, mxlo;
   for (int i = 0; i < 3; ++i) {
     const int j = i < m.n ? i : 0;
