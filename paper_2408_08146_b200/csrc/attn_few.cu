@@ -380,12 +380,16 @@ cudaError_t tree_attention_few(Launch L, int dtype, const float *q, const void *
 }
 
 // Whether a forward of so many rows takes the partial sums itself.  The rotary launch it saves is a time in which the O
-// projection's first weights arrive; where a CTA has many keys to walk they arrive at the attention's expense instead.
-// Six layers of the 7B shape, us per one-token pass, keys of capacity per chunk: one sequence 160 598 -> 583, 528 676
-// -> 653; two 416 630 -> 631, 1056 714 -> 736; four 256 609 -> 591, 448 650 -> 629, 832 (ragged) 659 -> 664; eight 621 -> 604.
+// projection's first weights arrive, and the CTAs come to lie where the multiply's end, not evenly; where they have many keys
+// to walk that costs more.  Six layers, us per one-token pass, rotary launch / sums by keys of capacity per chunk: 7B one
+// sequence (eight chunks) 160 598 / 583, 528 676 / 653; two 416 630 / 631, 560 ragged 605 / 604, 1056 equal 730 / 696 but
+// ragged 648 / 686; four 256 609 / 591, 320 ragged 575 / 563, 448 650 / 629, 576 ragged 595 / 598, 832 equal 687 / 658 but ragged
+// 626 / 649; eight 621 / 604; 13B one 304 784 / 777, 560 811 / 816, 1056 869 / 898; two 608 ragged 794 / 809; three 320 ragged
+// 785 / 775.  The host does not know the lengths.
 bool attn_few_takes_sums(int rows_per_seq, int B, int n_heads, int S_max, int num_sms) {
-  return rows_per_seq >= 1 && rows_per_seq <= ATTN_FEW_ROWS &&
-         S_max <= 640 * few_chunks(true, rows_per_seq, B, n_heads, 1, S_max, num_sms);
+  if (rows_per_seq < 1 || rows_per_seq > ATTN_FEW_ROWS) return false;
+  const int chunks = few_chunks(true, rows_per_seq, B, n_heads, 1, S_max, num_sms);
+  return S_max <= (chunks == MAX_CHUNKS ? 640 : 448) * chunks;
 }
 bool attn_few_rope_supported(const SplitIn &qkv) { return qkv.sk_ctas == 0 && qkv.n <= ROPE_PARTS; }
 
