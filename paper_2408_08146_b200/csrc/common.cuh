@@ -292,6 +292,8 @@ int tc_default_split(int n_tiles, int kblocks, int tokens);
 // split >= 1: classic split-K; split == 0: automatic (stream-K where it applies).  `max_slots`
 // bounds the partial matrices written; *out describes them for the consumer.  short_sums: no sum inside the
 // tensor core is longer than with 64 rows, whatever R.
+struct TcRing { int stages, early, pace; };     // stages of a CTA, weight tiles requested at once, cycles between the others' (0: with the activations)
+TcRing tc_ring(int stage_bytes, int smem_optin, bool wide, bool pdl);
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
                     float *Y, int ldy, int split, size_t split_stride, int *status, int max_slots,
                     SplitIn *out, bool short_sums = false, bool late_dependents = false);

@@ -46,8 +46,8 @@ constexpr int THREADS_WIDE = 576;   // most threads a launch uses: producer warp
                                     // warps (256-row weight tiles); 128-row tiles launch 192 threads
 constexpr int W_STAGE_BYTES = BM * BK * 2;
 constexpr int E_TIMEOUT = 6;
-constexpr int MAX_STAGES = 12;
-constexpr int EARLY_STAGES = 2, PACE_CYCLES = 1600;      // weights before the dependency wait, see gemm_tc()
+constexpr int MAX_STAGES = 8;
+constexpr int EARLY_STAGES = 2, PACE_CYCLES = 1600, ALONE_STAGES = 5;      // see tc_ring()
 
 struct TcParams {
   float *Y;
@@ -758,7 +758,7 @@ int g_tune_stages = 0;      // 0 = as many as fit (at most 8)
 int g_tune_max_split = 0;   // 0 = default rule
 int g_tune_no_streamk = 0;  // 1 = always the per-tile decomposition
 int g_tune_late_w = 0;      // 1 = weights wait for the dependency too
-int g_tune_early_stages = -1; // < 0 = all stages
+int g_tune_early_stages = -1; // < 0: EARLY_STAGES, or the whole ring without programmatic launch
 int g_tune_no_wave_split = 0; // 1 = several token tiles keep the one-wave rule's split factor
 int g_tune_no_accp = 0;      // 1 = pairs of more than 128 tokens as two 128-token tiles with extra columns
 int g_tune_epi = 0;         // 1, 2: that many epilogue warps per lane quarter for 256-row weight tiles (default 4)
@@ -970,6 +970,32 @@ int tc_streamk_ctas(int n_tiles, int kblocks, int tokens, int max_slots, int *sl
   while (g > 1 && slots_of(g) > max_slots) --g;
   *slots_out = slots_of(g);
   return (int)g;
+}
+
+// The ring of the one-CTA form.  As many stages as fit, two CTAs per SM (each with half of the shared memory) where they get
+// two each, so that one CTA's prologue and epilogue overlap the other's streaming.  Behind programmatic launch two weight
+// tiles are requested at once, the rest of the ring one per PACE_CYCLES: the kernel before reads its partial sums while they are
+// on their way, and behind a whole ring of every CTA at once (up to 28 MB) those reads took most of its time - the residual
+// update at one row 4.9 us, 2.9 with two stages only; paced, the ring is as full when the activations come.  Six layers, us
+// per pass, whole ring at once / two and one per 800 / 1200 / 1600 / 2000 / 2600 cycles: 7B one-token step 573 / 561 / 554 /
+// 552 / 554 / 559, four sequences 644 / 628 / 623 / 622 / 626 / 630, chain of five 1266 / 1238 / 1223 / 1222 / 1225 / 1230, 64
+// nodes 818 / 811 / 811 / 810 / 809 / 811, EAGLE iteration of 60 2016 / 1991 / 1978 / 1971 / 1970 / 1977.
+// Without it nothing runs beforehand that could be spared: the whole ring at once, and not six stages, of which all CTAs
+// begin together (us per call, six paced / six at once / five at once: pair of 8 rows, 12288 x 4096 26.0 / 26.0 / 24.7, 4096 x 11008
+// 25.0 / 24.6 / 23.7, 5120 x 13824 32.2 / 32.2 / 31.0; 64 plain rows of 4096 x 4096, three stages, 17.6 paced, 16.9 at once).  Behind
+// programmatic launch five are as fast as six (one-token step 560 / 557, chain 1230 / 1233).
+TcRing tc_ring(int stage_bytes, int smem_optin, bool wide, bool pdl) {
+  TcRing r;
+  r.stages = (smem_optin - 2048) / stage_bytes;
+  if (r.stages > MAX_STAGES) r.stages = MAX_STAGES;
+  const int two_per_sm = (smem_optin / 2 - 2048) / stage_bytes;
+  if (g_tune_stages == 0 && two_per_sm >= 2 && two_per_sm < r.stages && !wide)
+    r.stages = !pdl && two_per_sm > ALONE_STAGES ? ALONE_STAGES : two_per_sm;
+  if (g_tune_stages > 0 && g_tune_stages < r.stages) r.stages = g_tune_stages;
+  const int early = g_tune_early_stages >= 0 ? g_tune_early_stages : (pdl ? EARLY_STAGES : r.stages);
+  r.early = g_tune_late_w ? 0 : (early < r.stages ? early : r.stages);
+  r.pace = r.early > 0 && r.early < r.stages ? g_tune_pace : 0;
+  return r;
 }
 
 cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in, int R,
@@ -1192,25 +1218,12 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   P.epi_dry = g_tune_epi_dry;
   P.late_dep = late_dependents ? 1 : 0;
   const int stage_bytes = (wide ? 2 : 1) * W_STAGE_BYTES + x_bytes;
-  int stages = (g_smem_optin - 2048) / stage_bytes;
-  if (stages > MAX_STAGES) stages = MAX_STAGES;
-  if (stages > 8) stages = 8;
-  // default: two CTAs per SM (each with half of the shared memory), so that one CTA's prologue and
-  // epilogue overlap the other's streaming
-  const int two_per_sm = (g_smem_optin / 2 - 2048) / stage_bytes;
-  if (g_tune_stages == 0 && two_per_sm >= 2 && two_per_sm < stages && !wide) stages = two_per_sm;
-  if (g_tune_stages > 0 && g_tune_stages < stages) stages = g_tune_stages;
+  const TcRing ring = tc_ring(stage_bytes, g_smem_optin, wide, L.pdl);
+  const int stages = ring.stages;
   if (stages < 2) return cudaErrorInvalidValue;
   P.stages = stages;
-  // Two stages at once, the rest of the ring one per PACE_CYCLES: the kernel before this one reads its partial sums while they
-  // are on their way, and behind a whole ring of every CTA at once (up to 28 MB) those reads took most of its time - the residual
-  // update at one row 4.9 us, 2.9 with two stages only; paced, the ring is as full when the activations come.  Six layers, us
-  // per pass, whole ring at once / two and one per 800 / 1200 / 1600 / 2000 / 2600 cycles: 7B one-token step 573 / 561 / 554 /
-  // 552 / 554 / 559, four sequences 644 / 628 / 623 / 622 / 626 / 630, chain of five 1266 / 1238 / 1223 / 1222 / 1225 / 1230, 64
-  // nodes 818 / 811 / 811 / 810 / 809 / 811, EAGLE iteration of 60 2016 / 1991 / 1978 / 1971 / 1970 / 1977.
-  const int early = g_tune_early_stages >= 0 ? g_tune_early_stages : EARLY_STAGES;
-  P.early_w = g_tune_late_w ? 0 : (early < stages ? early : stages);
-  P.pace = P.early_w > 0 ? g_tune_pace : 0;
+  P.early_w = ring.early;
+  P.pace = ring.pace;
   CUtensorMap mw[3], mx, mxlo;
   for (int i = 0; i < 3; ++i) {
     const int j = i < m.n ? i : 0;

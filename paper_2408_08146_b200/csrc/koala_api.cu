@@ -1220,6 +1220,15 @@ int koala_selftest_timeout(koala_ctx *c, int limit_cycles) {
   return KOALA_OK;
 }
 
+int koala_debug_gemm_ring(int stage_bytes, int smem_optin, int wide, int pdl, int *stages, int *early, int *pace) {
+  if (stage_bytes < 1 || !stages || !early || !pace) return KOALA_E_INVALID;
+  const TcRing r = tc_ring(stage_bytes, smem_optin, wide != 0, pdl != 0);
+  *stages = r.stages;
+  *early = r.early;
+  *pace = r.pace;
+  return KOALA_OK;
+}
+
 int koala_debug_deal_blocks(int B, const int32_t *len, int ingest_rows, int fail_at, int *n_blocks, int *n_tokens) {
   if (B < 1 || B > 64 || !len || ingest_rows < 1 || !n_blocks || !n_tokens) return KOALA_E_INVALID;
   IngestLens k;

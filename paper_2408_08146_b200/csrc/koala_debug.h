@@ -18,7 +18,8 @@ extern "C" {
  * bound on the automatic split-K factor (0 = default); key 3 = 1 switches stream-K off (every CTA
  * stays inside one weight tile); key 6 = 1 delays the weight stream until the previous kernel has finished;
  * key 7 = divisor of the split-K partial-sum traffic bound (default 8); key 8 = how many pipeline
- * stages request their weight tile before that wait (< 0 = all, the default); key 9 = fewest query
+ * stages request their weight tile at once, before that wait (< 0, the default: two behind programmatic
+ * launch, else all; the ring's length or more = all in either case); key 9 = fewest query
  * rows per sequence for which the tcgen05 attention kernel is used (default 16); key 10 = 1 keeps
  * the one-wave split-K factor when a launch has several token tiles (more than 128 rows);
  * key 11 = 1 keeps 128 weight rows per CTA also for the widest token tiles (MMA N = 256);
@@ -30,7 +31,8 @@ extern "C" {
  * rows; key 18 = fewest rows for it (default 113); key 20 = 0: no dry pass over its
  * tile loop before the dependency wait; key 21 = 0: no dry pass of the GEMM epilogue warps; key 22 =
  * key chunks of the mma.sync attention kernel (0 = by rule); key 23 = 1: pairs of more than 64 rows always
- * summed in short chains (as in prompt forwards). */
+ * summed in short chains (as in prompt forwards); key 24 = SM cycles between the requests of the stages past those of key 8
+ * (default 1600; 0 = they come with their activations). */
 void koala_set_tuning(int key, int value);
 
 /* Kernels launched by the library in this process so far (all contexts). */
@@ -54,6 +56,11 @@ int koala_debug_check_guards(koala_ctx *ctx, int *n_guards, int *n_damaged);
  * without enqueueing anything: *n_blocks and *n_tokens handed out until the forward with index fail_at
  * (< 0: none) reports KOALA_E_CUDA, which ends the dealing and is returned.  Host memory only. */
 int koala_debug_deal_blocks(int B, const int32_t *len, int ingest_rows, int fail_at, int *n_blocks, int *n_tokens);
+
+/* The ring of a CTA of the one-CTA multiply for stages of stage_bytes on a device with smem_optin bytes of shared memory per
+ * block: *stages, how many of their weight tiles are requested at once (*early) and the cycles between the others' requests
+ * (*pace; 0: they come with the activations).  wide: 256 weight rows per CTA; pdl: programmatic launch.  Host logic only. */
+int koala_debug_gemm_ring(int stage_bytes, int smem_optin, int wide, int pdl, int *stages, int *early, int *pace);
 
 #ifdef __cplusplus
 }
