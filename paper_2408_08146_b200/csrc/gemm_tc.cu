@@ -888,7 +888,7 @@ void tc_set_tuning(int key, int value) {
   if (key == 21) g_tune_epi_dry = value;
   if (key == 22) attn_mma_set_chunks(value);
   if (key == 23) g_tune_short_sums = value;
-  if (key == 24) g_tune_pace = value;
+  if (key == 24) g_tune_pace = value > 0 ? value : 0;      // exactly one thread requests those stages: pace > 0 or == 0
   if (key == 2) g_tune_max_split = value;
   if (key == 3) g_tune_no_streamk = value;
   if (key == 6) g_tune_late_w = value;

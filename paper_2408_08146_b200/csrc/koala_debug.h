@@ -32,7 +32,7 @@ extern "C" {
  * tile loop before the dependency wait; key 21 = 0: no dry pass of the GEMM epilogue warps; key 22 =
  * key chunks of the mma.sync attention kernel (0 = by rule); key 23 = 1: pairs of more than 64 rows always
  * summed in short chains (as in prompt forwards); key 24 = SM cycles between the requests of the stages past those of key 8
- * (default 1600; 0 = they come with their activations). */
+ * (default 1600; 0 or less = they come with their activations). */
 void koala_set_tuning(int key, int value);
 
 /* Kernels launched by the library in this process so far (all contexts). */

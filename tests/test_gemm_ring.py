@@ -29,3 +29,15 @@ def test_two_stages_at_once_and_the_others_paced(stage_bytes):
     stages, early, pace = _ring(stage_bytes)
     assert early == 2 and (pace > 0) == (stages > 2)
     assert 2 * (stages * stage_bytes + 1024) <= SMEM       # two CTAs per SM
+
+
+@pytest.mark.parametrize("value", [-1600, -1, 0])
+def test_no_pace_below_zero(value):
+    """Two threads share the requests of the later stages, one for a pace above zero and one for zero: a negative pace would
+    leave them to nobody, and every multiply would run into its wait limit."""
+    lib = binding.load_library()
+    lib.koala_set_tuning(24, value)
+    try:
+        assert all(_ring(b)[2] == 0 for b in STAGES)
+    finally:
+        lib.koala_set_tuning(24, 1600)
