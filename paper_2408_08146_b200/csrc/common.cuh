@@ -219,6 +219,7 @@ cudaError_t resblock_update(Launch L, int dtype, float *x, SplitIn P, HeadTab ta
 cudaError_t row_update(Launch L, int dtype, float *x, SplitIn P, const void *g, Operand xg, float *sumsq,
                        int R, int H);
 // q_out: rotated queries in fp32; q_pair (bf16 only, may be null): the same as a bf16 pair
+int rope_rows_per_thread(const SplitIn &P, int R, int threads_per_row);
 cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan plan, float *q_out,
                           Operand q_pair, void *k_cache, void *v_cache, int R, int rows_per_seq, int n_heads,
                           int head_dim, int S_max);

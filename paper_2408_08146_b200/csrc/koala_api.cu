@@ -1229,6 +1229,11 @@ int koala_debug_gemm_ring(int stage_bytes, int smem_optin, int wide, int pdl, in
   return KOALA_OK;
 }
 
+int koala_debug_rope_rows(int R, int H, int ctas, int tiles, int kblocks, int n) {
+  const SplitIn s{nullptr, n, 0, 3 * H, (unsigned)ctas, (unsigned)(tiles * kblocks), (unsigned)kblocks};
+  return rope_rows_per_thread(s, R, H / 4);
+}
+
 int koala_debug_deal_blocks(int B, const int32_t *len, int ingest_rows, int fail_at, int *n_blocks, int *n_tokens) {
   if (B < 1 || B > 64 || !len || ingest_rows < 1 || !n_blocks || !n_tokens) return KOALA_E_INVALID;
   IngestLens k;

@@ -62,6 +62,10 @@ int koala_debug_deal_blocks(int B, const int32_t *len, int ingest_rows, int fail
  * (*pace; 0: they come with the activations).  wide: 256 weight rows per CTA; pdl: programmatic launch.  Host logic only. */
 int koala_debug_gemm_ring(int stage_bytes, int smem_optin, int wide, int pdl, int *stages, int *early, int *pace);
 
+/* Rows that a thread of the rotary kernel takes for R rows of a bf16 model of hidden size H whose Q/K/V product left up to n
+ * partial sums per column, its `tiles` tiles of kblocks K blocks dealt to `ctas` CTAs or clusters (0: not dealt).  Host logic only. */
+int koala_debug_rope_rows(int R, int H, int ctas, int tiles, int kblocks, int n);
+
 #ifdef __cplusplus
 }
 #endif

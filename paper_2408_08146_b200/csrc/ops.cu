@@ -7,8 +7,9 @@ namespace koala {
 
 namespace {
 
+__device__ __forceinline__ float silu(float v) { return v / (1.f + expf(-v)); }
 // (not inlined: an exponential and a division, used a dozen times by kernels that run their instructions once)
-__device__ __noinline__ float silu_f(float v) { return v / (1.f + expf(-v)); }
+__device__ __noinline__ float silu_f(float v) { return silu(v); }
 
 // ------------------------------------------------------------------------------- embedding + norm
 template <typename T>
@@ -314,7 +315,7 @@ __device__ __forceinline__ void store2(float *p, float a, float b) { *reinterpre
 __device__ __forceinline__ void store2(bf16 *p, float a, float b) {
   *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
-// ROWS: consecutive rows of a thread, see several_rows.
+// ROWS: consecutive rows of a thread, see rope_rows_per_thread.
 template <typename T, int NS, bool SK, int ROWS>
 __global__ void __launch_bounds__(128)
 rope_kv_vec_kernel(SplitIn qkv, RowScale sc, RowPlan plan, float *__restrict__ q_out, bf16 *__restrict__ qp_hi,
@@ -381,25 +382,21 @@ __global__ void swiglu_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *_
   store_operand(act, act_lo, (size_t)r * F + f, silu_f(rs * gu.at(r, f)) * (rs * gu.at(r, F + f)));
 }
 
-template <typename T, int NS, bool SK, int ROWS>
-__global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int R, int F) {
+// SiLU is inlined: behind the calls of silu_f the second operand's partial sums were not requested before the first's were used
+// (us per launch, calls / inlined: one row of the 7B shape 3.18 / 2.95, 64 rows 5.8 / 5.5, 512 rows 24.4 / 22.7, prompts of 509 tokens
+// 22.5 / 20.9, 860 tokens 35.4 / 33.8, 13B 46.7 / 43.8).
+template <typename T, int NS, bool SK>
+__global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int F) {
   pdl_launch_dependents();
   pdl_wait();
-  const int r0 = blockIdx.y * ROWS;
+  const int r = blockIdx.y;
   const int f = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (f >= F) return;
-  const int ka = slots_at<NS, SK>(gu, r0, f), kb = slots_at<NS, SK>(gu, r0, F + f);
-#pragma unroll
-  for (int i = 0; i < ROWS; ++i) {
-    const int r = r0 + i;
-    if (ROWS > 1 && r >= R) break;
-    const float rs = sc.of(r);
-    const float4 a = split_sum4<NS>(gu, r, f, ka), b = split_sum4<NS>(gu, r, F + f, kb);
-    auto silu = [](float v) { return ROWS > 1 ? v / (1.f + expf(-v)) : silu_f(v); };
-    store_operand4(act, act_lo, (size_t)r * F + f,
-                   make_float4(silu(rs * a.x) * (rs * b.x), silu(rs * a.y) * (rs * b.y),
-                               silu(rs * a.z) * (rs * b.z), silu(rs * a.w) * (rs * b.w)));
-  }
+  const float rs = sc.of(r);
+  const float4 a = split_sum4<NS>(gu, r, f, slots_at<NS, SK>(gu, r, f)), b = split_sum4<NS>(gu, r, F + f, slots_at<NS, SK>(gu, r, F + f));
+  store_operand4(act, act_lo, (size_t)r * F + f,
+                 make_float4(silu(rs * a.x) * (rs * b.x), silu(rs * a.y) * (rs * b.y),
+                             silu(rs * a.z) * (rs * b.z), silu(rs * a.w) * (rs * b.w)));
 }
 
 // ------------------------------------------------------------------------------- arg-max / top-k
@@ -691,13 +688,16 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
     SPLIT_CASE(12, true, __VA_ARGS__)                                             \
   }
 
-// More than 256 rows with few partial sums each: a thread takes several rows of its columns, so that the number of the
-// partial sums, four integer divisions, is found once for them (token tiles are multiples of 32 rows: consecutive rows share
-// one).  us per launch by rows per thread 1 / 2 / 4 / 8: SwiGLU, 509 rows of the 7B prompt 25.1 / 22.2 / 20.5 / 23.5, about 860 rows of
-// the 13B prompts 57 / 49.5 / 44.5 / 47; rotary step 18.1 / 15.8 / 16.5 / 25.4 and 39 / 34.3 / 33.1 / 34.3.  Up to 256 rows there
-// are too few threads then (128 rows: SwiGLU 5.3 / 5.7 / 8.8; 256 rows 8.6 / 9.0 / 11.5); the residual update, which
-// has up to twelve partial sums in flight per thread, gains nothing (10.6 / 10.5 / 16.5).
-static bool several_rows(const SplitIn &P, int R) { return P.sk_ctas != 0 && P.n <= 3 && R > 256; }
+// The rotary kernel takes two consecutive rows per thread where most columns have one or two partial sums (at least five weight
+// tiles per four clusters: prompt forwards; token tiles are multiples of 32 rows, so both rows have the same number) and the half
+// as many CTAs still give an SM 1280 threads; a row's loads follow the other's stores, so with more sums or fewer threads
+// the second trip is exposed.  us per launch, one / two rows: prompts 7B 257 tokens 8.7 / 9.2, 300 9.7 / 9.8, 430 14.1 / 13.8, 509
+// 16.2 / 16.0, 640 21.0 / 18.3, 860 25.6 / 22.5, 13B 300 12.4 / 12.2, 509 20.3 / 18.2, 860 32.0 / 28.6; verifications 7B 260 rows 10.1 /
+// 11.4, 360 12.4 / 12.9, 512 18.6 / 19.4, 13B 300 12.3 / 12.9.
+int rope_rows_per_thread(const SplitIn &P, int R, int threads_per_row) {
+  const bool short_columns = P.sk_ctas != 0 && P.n <= 3 && 4ull * P.sk_units >= 5ull * P.sk_ctas * P.sk_kb;
+  return short_columns && (R + 1LL) / 2 * threads_per_row >= 1280LL * 148 ? 2 : 1;
+}
 
 cudaError_t embed_norm(Launch L, int dtype, const int32_t *tok, const void *E, const void *g,
                        float *x, Operand xn, int R, int H, int V, float eps) {
@@ -776,7 +776,7 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
     const int work = n_heads * head_dim / 4;
     const int threads = work < 128 ? ((work + 31) / 32) * 32 : 128;
     const int slices = (work + threads - 1) / threads;
-    if (dtype != 0 && several_rows(qkv, R))
+    if (dtype != 0 && rope_rows_per_thread(qkv, R, work) == 2)
       return launch_k(rope_kv_vec_kernel<bf16, 3, true, 2>, dim3((R + 1) / 2, slices), dim3(threads), 0, L.st, L.pdl, qkv, sc, plan,
                       q_out, qh, ql, (bf16 *)k_cache, (bf16 *)v_cache, rows_per_seq, n_heads, head_dim, S_max, R);
     FOR_SPLIT(dtype, qkv, return launch_k(rope_kv_vec_kernel<T, NS, SK, 1>, dim3(R, slices), dim3(threads), 0, L.st, L.pdl,
@@ -790,11 +790,8 @@ cudaError_t rope_kv_write(Launch L, int dtype, SplitIn qkv, RowScale sc, RowPlan
 
 cudaError_t swiglu(Launch L, int dtype, SplitIn gu, RowScale sc, Operand act, int R, int F) {
   if (F % 4 == 0 && gu.ld % 4 == 0 && gu.stride % 4 == 0) {
-    if (dtype != 0 && several_rows(gu, R))
-      return launch_k(swiglu_vec_kernel<bf16, 3, true, 4>, dim3((F / 4 + 255) / 256, (R + 3) / 4), dim3(256), 0, L.st, L.pdl, gu, sc,
-                      (bf16 *)act.hi, (bf16 *)act.lo, R, F);
-    FOR_SPLIT(dtype, gu, return launch_k(swiglu_vec_kernel<T, NS, SK, 1>, dim3((F / 4 + 255) / 256, R), dim3(256), 0, L.st,
-                                         L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, R, F);)
+    FOR_SPLIT(dtype, gu, return launch_k(swiglu_vec_kernel<T, NS, SK>, dim3((F / 4 + 255) / 256, R), dim3(256), 0, L.st,
+                                         L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)
   }
   DISPATCH_T(dtype, return launch_k(swiglu_kernel<T>, dim3((F + 255) / 256, R), dim3(256), 0, L.st,
                                     L.pdl, gu, sc, (T *)act.hi, (T *)act.lo, F);)

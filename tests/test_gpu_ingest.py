@@ -75,10 +75,9 @@ def test_7b_shaped_prompts(kind, n, chunk):
     eng.close()
 
 
-@pytest.mark.parametrize("n", [[261], [270], [258, 100]])
+@pytest.mark.parametrize("n", [[261], [270], [258, 100], [429], [381, 102]])
 def test_prompts_whose_rows_are_not_whole_groups_of_a_thread(n):
-    """Above 256 rows a thread of the rotary and SwiGLU kernels takes two and four rows: 261 rows (three blocks of 87), 270,
-    and 360 with rows of a second sequence."""
+    """From about 370 rows on a thread of the rotary kernel takes two: 429 rows, 483 with rows of a second sequence; below it one."""
     test_7b_shaped_prompts("eagle", n, 64)
 
 
