@@ -1013,9 +1013,10 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   const int accp = (pair && R > 128 && !g_tune_no_accp) ? 1 : 0;
   const int tt_max = (pair && !accp) ? 128 : 256;
   // (A pair's tile is twice as many MMA columns, so up to 128 rows tokens come in eights: the bytes saved are weight
-  // stages.  Sixteens / eights, six layers, us per pass: 7B one-token step 581 / 575, four sequences 655 / 649, eight
-  // 602 / 594, 13B one token 813 / 796, 40 rows 785 / 778, 72 rows 858 / 854, 100 rows 2184 / 2171.  Not 17 to 24 rows: the
-  // multiplies gain there too, 16.4 -> 16.2 us each, but 20 rows take 745 / 755 in all.)
+  // stages.  Sixteens / eights, six layers, us per pass: 7B one-token step 565 / 557, four sequences 636 / 627, chain of five 1243 /
+  // 1233, 13B one token 794 / 781; before the stages were paced eight sequences 602 / 594, 40 rows 785 / 778, 72 rows 858 / 854, 100
+  // rows 2184 / 2171.  Not 17 to 24 rows, where five stages come in the place of four: 7B 17 / 20 / 24 rows 713, 715, 718 / 710, 714, 717, but 13B
+  // 958, 959, 963 / 959, 962, 967, and without programmatic launch 893, 899, 901 / 922, 930, 932.)
   const int unit = pair && R <= 128 && (R <= 16 || R > 24) ? 8 : 16;
   int tt = (R + unit - 1) / unit * unit;
   if (tt > tt_max) tt = tt_max;
