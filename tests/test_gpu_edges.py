@@ -155,6 +155,20 @@ def test_scores_that_grow_along_the_context(N, B, n_heads, context, S_max):
     _attention_case(N, B, n_heads, context, S_max, growing=True)
 
 
+@pytest.mark.parametrize("N,context,S_max", [
+    (128, 30, 1024),             # more than 64 rows: three tiles for eight chunks, most of which have none
+    (128, 1500, 2048),
+    (65, 700, 1024),
+    (60, 20, 1024),              # duplicated rows
+    (64, 1900, 2048),
+])
+@pytest.mark.parametrize("growing", [False, True])
+def test_eight_key_chunks(N, context, S_max, growing):
+    """Eight heads leave room for eight chunks per head: merged over the whole cluster, with references that differ from chunk
+    to chunk where the scores grow."""
+    _attention_case(N, 1, 8, context, S_max, growing=growing)
+
+
 def _attention_case(N, B, n_heads, context, S_max, poison=False, growing=False):
     H = n_heads * 128
     cfg = reduced(T7_EAGLE, 1, K=1, N=N, B=B, H=H, n_heads=n_heads, F=2 * H, V=2048, D=min(5, N - 1),
@@ -364,31 +378,53 @@ def test_attention_of_few_rows(N, B, n_heads, context, S_max, kind):
     (2, [63], 32, 256),              # two new rows in different tiles, and so in different chunks
     (2, [127, 62, 5], 16, 512),
     (2, [500, 191], 32, 1024),
-    (1, [900, 64, 130], 32, 1152),
+    (1, [800, 64, 130], 32, 896),
 ])
-def test_few_rows_take_the_sums_of_the_multiply(N, lens, n_heads, S_max):
+@pytest.mark.parametrize("short", [False, True], ids=["all", "last_tree_of_one_node"])
+def test_few_rows_take_the_sums_of_the_multiply(N, lens, n_heads, S_max, short):
     """One or two rows per sequence, where the attention rotates the queries and writes the cache itself: two layers, so
-    that the second layer's context reads lie before its dependency wait; hidden states and the rows written."""
+    that the second layer's context reads lie before its dependency wait; hidden states and the rows written.  A row that no
+    node uses writes nothing."""
+    if short and N == 1:
+        pytest.skip("every row is in use")
     B = len(lens)
     cfg = reduced(T7_EAGLE, 2, K=1, N=N, D=1, topk=1, B=B, H=128 * n_heads, n_heads=n_heads, F=2048, V=2048, S_max=S_max, prompt_len=max(lens))
-    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
+    eng, orc, store = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
     eng.target_k.copy_(random_kv(cfg, "target_k", cfg.L, DEV))
     eng.target_v.copy_(random_kv(cfg, "target_v", cfg.L, DEV))
+    before = (eng.target_k.clone(), eng.target_v.clone())
     for b in range(B):
         for l in range(cfg.L):
             orc.target_k[l][b][...] = kv_to_oracle(eng.target_k, l, b, np.float32)
             orc.target_v[l][b][...] = kv_to_oracle(eng.target_v, l, b, np.float32)
         orc.seq_len[b] = lens[b]
     eng.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    counts = [1 if short and b == B - 1 else N for b in range(B)]
     toks, pars = [[5 + b, 9][:N] for b in range(B)], [[-1, 0][:N]] * B
-    eng.koala_verify(_tree_arrays(eng, toks, pars))
-    orc.verify(list(zip(toks, pars)))
+    tok, par, _, n = _tree_arrays(eng, toks, pars)
+    tree = (tok, par, torch.tensor(counts, dtype=torch.int32, device=DEV), n)
+
+    def launches(e):
+        first = e.launch_count()
+        e.koala_verify(tree)
+        return e.launch_count() - first
+
+    fused = launches(eng)
+    orc.verify([(toks[b][:counts[b]], pars[b][:counts[b]]) for b in range(B)])
     hid = eng.buffers()["verify_hid"]
     for b in range(B):
-        assert_close(hid[b * N:(b + 1) * N].cpu().numpy(), orc.verify_hid[b][:N], cfg.dtype, f"hidden {b}")
+        end = lens[b] + counts[b]
+        assert_close(hid[b * N:b * N + counts[b]].cpu().numpy(), orc.verify_hid[b][:counts[b]], cfg.dtype, f"hidden {b}")
         for l in range(cfg.L):
-            for name, got, want in (("K", eng.target_k, orc.target_k), ("V", eng.target_v, orc.target_v)):
-                assert_close(kv_to_oracle(got, l, b, np.float32)[:lens[b] + N], want[l][b][:lens[b] + N], cfg.dtype, f"{name} {l} {b}")
+            for name, got, want, old in (("K", eng.target_k, orc.target_k, before[0]), ("V", eng.target_v, orc.target_v, before[1])):
+                assert_close(kv_to_oracle(got, l, b, np.float32)[:end], want[l][b][:end], cfg.dtype, f"{name} {l} {b}")
+                assert torch.equal(got[l, b, :, end:], old[l, b, :, end:])
+    assert eng.device_status() == 0
+    eng.close()
+    # the same with more capacity than the sums are taken for: a rotary launch per layer
+    eng = Koala(cfg.with_(S_max=5248), store.tensors)
+    eng.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    assert launches(eng) == fused + cfg.L
     assert eng.device_status() == 0
     eng.close()
 

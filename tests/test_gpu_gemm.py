@@ -47,9 +47,10 @@ def test_cuda_core_gemm(shape):
 
 
 @pytest.mark.parametrize("M", [1, 7, 8, 9, 17, 24, 25, 40, 55, 72, 100, 112])
-@pytest.mark.parametrize("N,K", [(12288, 4096), (200, 192), (1000, 2816), (22016, 512)])
+@pytest.mark.parametrize("N,K", [(12288, 4096), (200, 192), (1000, 2816), (22016, 512), (22016, 4096)])
 def test_token_tiles_of_a_pair_in_eights(M, N, K):
-    """Tiles that are and are not whole sixteens, with ragged weight tiles, split and shared sums."""
+    """Tiles that are and are not whole sixteens, with ragged weight tiles, split sums and (172 tiles of 64 K blocks, dealt to
+    two CTAs per SM) shared ones with two accumulator buffers."""
     xf = normal_tensor(9, f"xe{M}.{N}.{K}", (M, K), 1.0, 0.0, torch.float32, "cuda:0")
     w = normal_tensor(8, f"we{M}.{N}.{K}", (N, K), 0.02, 0.0, torch.bfloat16, "cuda:0")
     hi = xf.to(torch.bfloat16)

@@ -1,6 +1,8 @@
 """How exact the sums inside the tensor core are: it adds by truncation, so the error of a product grows with
 the number of MMAs that one accumulator takes.  Forms are compared with each other on the same inputs and
 with float64."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -8,7 +10,7 @@ import torch
 from paper_2408_08146_b200 import binding, koala_gemm_bf16
 from tests.harness import make_pair
 from workloads import T7_EAGLE, reduced
-from workloads.generate import normal_tensor, uniform_ints
+from workloads.generate import normal_tensor, random_kv, uniform_ints
 
 pytestmark = pytest.mark.gpu
 
@@ -83,5 +85,46 @@ def test_prompt_forwards_are_as_exact_as_their_parts(n):
     eng.target_v.zero_()
     eng.prefill([tok], 64)
     assert differing() <= parts
+    assert eng.device_status() == 0
+    eng.close()
+
+
+def test_tcgen05_attention_is_about_as_exact_as_mma_sync():
+    """One layer over 64 chained rows on a context of 2000, against float64 on the keys and values as stored; the same rows
+    by either kernel (tuning key 9).  P V is added in one truncating accumulator per chunk in the one and in several in the
+    other; a probability is a value rounded to bf16 and a rounded residual in both.  Cutting the value part off instead makes the
+    residual, and its rounding error, up to twice as large: 1.24 times the whole layer's error; rounded it is 1.02 times."""
+    n, ctx, dev = 64, 2000, "cuda:0"
+    cfg = reduced(T7_EAGLE, 1, K=1, N=n, H=1024, n_heads=8, F=2048, V=2048, S_max=2176, prompt_len=ctx, seed=55)
+    eng, _, store = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
+    eng.target_k.copy_(random_kv(cfg, "target_k", 1, dev))
+    eng.target_v.copy_(random_kv(cfg, "target_v", 1, dev))
+    tok = uniform_ints(56, "tokens", n, 0, cfg.V)
+    tree = eng.chain_tree([tok])
+    lib, hid = binding.load_library(), []
+    try:
+        for min_rows in (16, 129):
+            lib.koala_set_tuning(9, min_rows)
+            eng.seq_len.fill_(ctx)
+            eng.koala_verify(tree)
+            hid.append(eng.buffers()["verify_hid"][:n].double())
+    finally:
+        lib.koala_set_tuning(9, 16)
+    w = lambda name: store[name].double()
+    rms = lambda x, gain: x * torch.rsqrt((x * x).mean(-1, keepdim=True) + cfg.rms_eps) * w(gain)
+    x = w("embed")[torch.from_numpy(tok.astype(np.int64)).to(dev)]
+    q = (rms(x, "layers.0.attn_norm") @ w("layers.0.wq").T).view(n, cfg.n_heads, cfg.head_dim)
+    pos = ctx + torch.arange(n, device=dev, dtype=torch.float64)
+    ang = pos[:, None, None] * cfg.rope_base ** (-2.0 * torch.arange(64, device=dev, dtype=torch.float64) / 128)
+    c, s = torch.cos(ang).float().double(), torch.sin(ang).float().double()
+    q = torch.cat([q[..., :64] * c - q[..., 64:] * s, q[..., 64:] * c + q[..., :64] * s], -1)
+    score = torch.einsum("rhd,hkd->hrk", q, eng.target_k[0, 0, :, :ctx + n].double()) / math.sqrt(128)
+    hidden = torch.arange(ctx + n, device=dev)[None] > pos[:, None]
+    p = torch.softmax(score.masked_fill(hidden[None], float("-inf")), -1)
+    x = x + torch.einsum("hrk,hkd->rhd", p, eng.target_v[0, 0, :, :ctx + n].double()).reshape(n, cfg.H) @ w("layers.0.wo").T
+    h = rms(x, "layers.0.ffn_norm")
+    x = x + (torch.nn.functional.silu(h @ w("layers.0.w_gate").T) * (h @ w("layers.0.w_up").T)) @ w("layers.0.w_down").T
+    ref = rms(x, "final_norm")
+    assert _rel(hid[0], ref) <= 1.12 * _rel(hid[1], ref)      # half way between the two
     assert eng.device_status() == 0
     eng.close()
