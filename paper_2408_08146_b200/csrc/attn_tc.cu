@@ -15,7 +15,8 @@
 // MMAs as bf16 pairs (value + rounding residual: two accumulating MMAs), so only the cached K and V
 // carry bf16 rounding.  Q (written as a pair by the rotary-embedding kernel) and the K/V tiles
 // arrive by TMA with the 128-byte swizzle, K/V in a ring of two (up to 64 rows) or three stages.
-// Warps 0..3 own the rows, warp 4 lane 0 issues the copies, warp 5 lane 0 the MMAs (more than 64 rows: warp 6 lane 0 those of S).
+// Warps 0..3 own the rows, warp 4 lane 0 issues the copies, warp 5 lane 0 the MMAs (with more than 64 rows warp 6 lane 0
+// those of S).
 // With several chunks the CTAs of one (head, sequence) form a thread-block cluster: every CTA leaves
 // its unnormalised (O, m, l) in its own shared memory (the K/V ring is free by then); after a cluster
 // barrier every CTA reads its slice of the head dimension from all of them, merges it in chunk order

@@ -333,8 +333,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__
       const int feat = row0 + hw * BM + quarter * 32 + lane;
       float *Yp = P.Y + (size_t)slot * P.split_stride + col_off + feat;
       const uint32_t lane_base = tmem_acc + (uint32_t)((buf + hw) * P.tmem_cols) + ((uint32_t)(quarter * 32) << 16);
-      // 16 token columns per step (the last eight of a tile may bring eight that are not stored), in a rolled loop: the accumulator reads of one warp hide behind the stores
-      // of the others, and the loop's instructions are fetched once.
+      // 16 token columns per step (the last eight of a tile may bring eight that are not stored), in a rolled loop: the
+      // accumulator reads of one warp hide behind the stores of the others, and the loop's instructions are fetched once.
 #pragma unroll 1
       for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
         uint32_t va[16];
@@ -981,9 +981,9 @@ int tc_streamk_ctas(int n_tiles, int kblocks, int tokens, int max_slots, int *sl
 // 552 / 554 / 559, four sequences 644 / 628 / 623 / 622 / 626 / 630, chain of five 1266 / 1238 / 1223 / 1222 / 1225 / 1230, 64
 // nodes 818 / 811 / 811 / 810 / 809 / 811, EAGLE iteration of 60 2016 / 1991 / 1978 / 1971 / 1970 / 1977.
 // Without it nothing runs beforehand that could be spared: the whole ring at once, and not six stages, of which all CTAs
-// begin together (us per call, six paced / six at once / five at once: pair of 8 rows, 12288 x 4096 26.0 / 26.0 / 24.7, 4096 x 11008
-// 25.0 / 24.6 / 23.7, 5120 x 13824 32.2 / 32.2 / 31.0; 64 plain rows of 4096 x 4096, three stages, 17.6 paced, 16.9 at once).  Behind
-// programmatic launch five are as fast as six (one-token step 560 / 557, chain 1230 / 1233).
+// begin together (us per call, six paced / six at once / five at once: pair of 8 rows, 12288 x 4096 26.0 / 26.0 / 24.7,
+// 4096 x 11008 25.0 / 24.6 / 23.7, 5120 x 13824 32.2 / 32.2 / 31.0; 64 plain rows of 4096 x 4096, three stages, 17.6 paced,
+// 16.9 at once).  Behind programmatic launch five are as fast as six (one-token step 560 / 557, chain 1230 / 1233).
 TcRing tc_ring(int stage_bytes, int smem_optin, bool wide, bool pdl) {
   TcRing r;
   r.stages = (smem_optin - 2048) / stage_bytes;
@@ -1013,10 +1013,11 @@ cudaError_t gemm_tc(Launch L, Operand X, int x_rows_alloc, GemmMats m, int K_in,
   const int accp = (pair && R > 128 && !g_tune_no_accp) ? 1 : 0;
   const int tt_max = (pair && !accp) ? 128 : 256;
   // (A pair's tile is twice as many MMA columns, so up to 128 rows tokens come in eights: the bytes saved are weight
-  // stages.  Sixteens / eights, six layers, us per pass: 7B one-token step 565 / 557, four sequences 636 / 627, chain of five 1243 /
-  // 1233, 13B one token 794 / 781; before the stages were paced eight sequences 602 / 594, 40 rows 785 / 778, 72 rows 858 / 854, 100
-  // rows 2184 / 2171.  Not 17 to 24 rows, where five stages come in the place of four: 7B 17 / 20 / 24 rows 713, 715, 718 / 710, 714, 717, but 13B
-  // 958, 959, 963 / 959, 962, 967, and without programmatic launch 893, 899, 901 / 922, 930, 932.)
+  // stages.  Sixteens / eights, six layers, us per pass: 7B one-token step 565 / 557, four sequences 636 / 627, chain of
+  // five 1243 / 1233, 13B one token 794 / 781; before the stages were paced eight sequences 602 / 594, 40 rows 785 / 778, 72
+  // rows 858 / 854, 100 rows 2184 / 2171.  Not 17 to 24 rows, where five stages come in the place of four: 7B 17, 20, 24
+  // rows 713, 715, 718 / 710, 714, 717, but 13B 958, 959, 963 / 959, 962, 967, and without programmatic launch 893, 899, 901 /
+  // 922, 930, 932.)
   const int unit = pair && R <= 128 && (R <= 16 || R > 24) ? 8 : 16;
   int tt = (R + unit - 1) / unit * unit;
   if (tt > tt_max) tt = tt_max;

@@ -362,7 +362,9 @@ int run_layer(koala_ctx *c, const LayerW &w, void *kc, void *vc, int R, int rows
   const RowMap same{0, 0};
   SplitIn s;
   GemmMats qkv{{w.wq, w.wk, w.wv}, {H, H, H}, 3};
-  // with a row or two per sequence the attention may take the multiply's partial sums itself
+  // with a row or two per sequence the attention may take the multiply's partial sums itself (where these turn out to be shared by
+  // the deal, as for the 156 tiles of a 33B shape, the rotary launch takes them after all; that the multiply had held its dependents
+  // back costs nothing there: six layers, one-token step 1204 us with, 1205 without)
   const bool few = c->use_tc && g.dtype == KOALA_BF16 && g.head_dim == 128 && c->ingest_blocks == 0 && !kv_only && tc_supported(qkv, H) &&
                    attn_few_takes_sums(rows_per_seq, g.B, g.n_heads, g.S_max, NUM_SMS);
   K_TRY(do_gemm(c, c->xn, H, qkv, R, nullptr, 0, &s, few));

@@ -382,9 +382,9 @@ __global__ void swiglu_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *_
   store_operand(act, act_lo, (size_t)r * F + f, silu_f(rs * gu.at(r, f)) * (rs * gu.at(r, F + f)));
 }
 
-// SiLU is inlined: behind the calls of silu_f the second operand's partial sums were not requested before the first's were used
-// (us per launch, calls / inlined: one row of the 7B shape 3.18 / 2.95, 64 rows 5.8 / 5.5, 512 rows 24.4 / 22.7, prompts of 509 tokens
-// 22.5 / 20.9, 860 tokens 35.4 / 33.8, 13B 46.7 / 43.8).
+// SiLU is inlined: behind the calls of silu_f the second operand's partial sums were not requested before the first's were
+// used (us per launch, calls / inlined: one row of the 7B shape 3.18 / 2.95, 64 rows 5.8 / 5.5, 512 rows 24.4 / 22.7, prompts
+// of 509 tokens 22.5 / 20.9, 860 tokens 35.4 / 33.8, 13B 46.7 / 43.8).
 template <typename T, int NS, bool SK>
 __global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int F) {
   pdl_launch_dependents();
@@ -688,12 +688,12 @@ topk_logp_cluster_kernel(const float *logits, int32_t *__restrict__ tok, float *
     SPLIT_CASE(12, true, __VA_ARGS__)                                             \
   }
 
-// The rotary kernel takes two consecutive rows per thread where most columns have one or two partial sums (at least five weight
-// tiles per four clusters: prompt forwards; token tiles are multiples of 32 rows, so both rows have the same number) and the half
-// as many CTAs still give an SM 1280 threads; a row's loads follow the other's stores, so with more sums or fewer threads
-// the second trip is exposed.  us per launch, one / two rows: prompts 7B 257 tokens 8.7 / 9.2, 300 9.7 / 9.8, 430 14.1 / 13.8, 509
-// 16.2 / 16.0, 640 21.0 / 18.3, 860 25.6 / 22.5, 13B 300 12.4 / 12.2, 509 20.3 / 18.2, 860 32.0 / 28.6; verifications 7B 260 rows 10.1 /
-// 11.4, 360 12.4 / 12.9, 512 18.6 / 19.4, 13B 300 12.3 / 12.9.
+// The rotary kernel takes two consecutive rows per thread where most columns have one or two partial sums (at least five
+// weight tiles per four clusters: prompt forwards; token tiles are multiples of 32 rows, so both rows have the same number)
+// and half as many CTAs still give an SM 1280 threads; a row's loads follow the other's stores, so with more sums or fewer
+// threads the second trip is exposed.  us per launch, one / two rows: prompts 7B 257 tokens 8.7 / 9.2, 300 9.7 / 9.8, 430 14.1 /
+// 13.8, 509 16.2 / 16.0, 640 21.0 / 18.3, 860 25.6 / 22.5, 13B 300 12.4 / 12.2, 509 20.3 / 18.2, 860 32.0 / 28.6; verifications 7B
+// 260 rows 10.1 / 11.4, 360 12.4 / 12.9, 512 18.6 / 19.4, 13B 300 12.3 / 12.9.
 int rope_rows_per_thread(const SplitIn &P, int R, int threads_per_row) {
   const bool short_columns = P.sk_ctas != 0 && P.n <= 3 && 4ull * P.sk_units >= 5ull * P.sk_ctas * P.sk_kb;
   return short_columns && (R + 1LL) / 2 * threads_per_row >= 1280LL * 148 ? 2 : 1;
