@@ -378,13 +378,47 @@ def test_attention_of_few_rows(N, B, n_heads, context, S_max, kind):
     (2, [63], 32, 256),              # two new rows in different tiles, and so in different chunks
     (2, [127, 62, 5], 16, 512),
     (2, [500, 191], 32, 1024),
-    (1, [800, 64, 130], 32, 896),
+    (1, [900, 64, 130], 32, 1152),
+])
+def test_few_rows_take_the_sums_of_the_multiply(N, lens, n_heads, S_max):
+    """One or two rows per sequence, where the attention rotates the queries and writes the cache itself: two layers, so
+    that the second layer's context reads lie before its dependency wait; hidden states and the rows written."""
+    B = len(lens)
+    cfg = reduced(T7_EAGLE, 2, K=1, N=N, D=1, topk=1, B=B, H=128 * n_heads, n_heads=n_heads, F=2048, V=2048, S_max=S_max, prompt_len=max(lens))
+    eng, orc, _ = make_pair(cfg, oracle_dtype=np.float32, cache_host=False)
+    eng.target_k.copy_(random_kv(cfg, "target_k", cfg.L, DEV))
+    eng.target_v.copy_(random_kv(cfg, "target_v", cfg.L, DEV))
+    for b in range(B):
+        for l in range(cfg.L):
+            orc.target_k[l][b][...] = kv_to_oracle(eng.target_k, l, b, np.float32)
+            orc.target_v[l][b][...] = kv_to_oracle(eng.target_v, l, b, np.float32)
+        orc.seq_len[b] = lens[b]
+    eng.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    toks, pars = [[5 + b, 9][:N] for b in range(B)], [[-1, 0][:N]] * B
+    eng.koala_verify(_tree_arrays(eng, toks, pars))
+    orc.verify(list(zip(toks, pars)))
+    hid = eng.buffers()["verify_hid"]
+    for b in range(B):
+        assert_close(hid[b * N:(b + 1) * N].cpu().numpy(), orc.verify_hid[b][:N], cfg.dtype, f"hidden {b}")
+        for l in range(cfg.L):
+            for name, got, want in (("K", eng.target_k, orc.target_k), ("V", eng.target_v, orc.target_v)):
+                assert_close(kv_to_oracle(got, l, b, np.float32)[:lens[b] + N], want[l][b][:lens[b] + N], cfg.dtype, f"{name} {l} {b}")
+    assert eng.device_status() == 0
+    eng.close()
+
+
+@pytest.mark.parametrize("N,lens,n_heads,S_max", [
+    (1, [63], 32, 256),
+    (1, [1], 8, 128),
+    (2, [63], 32, 256),
+    (2, [127, 62, 5], 16, 512),
+    (2, [500, 191], 32, 1024),
+    (1, [800, 64, 130], 32, 896),    # long and ragged: up to seven tiles per chunk
 ])
 @pytest.mark.parametrize("short", [False, True], ids=["all", "last_tree_of_one_node"])
-def test_few_rows_take_the_sums_of_the_multiply(N, lens, n_heads, S_max, short):
-    """One or two rows per sequence, where the attention rotates the queries and writes the cache itself: two layers, so
-    that the second layer's context reads lie before its dependency wait; hidden states and the rows written.  A row that no
-    node uses writes nothing."""
+def test_rotary_step_inside_the_attention_runs_and_leaves_other_slots_alone(N, lens, n_heads, S_max, short):
+    """The same where the launches say that the fused path ran (a launch less per layer than with more capacity); a row that
+    no node uses writes nothing, nor does any row write past its sequence's end."""
     if short and N == 1:
         pytest.skip("every row is in use")
     B = len(lens)

@@ -75,9 +75,15 @@ def test_7b_shaped_prompts(kind, n, chunk):
     eng.close()
 
 
-@pytest.mark.parametrize("n", [[261], [270], [258, 100], [429], [381, 102]])
+@pytest.mark.parametrize("n", [[261], [270], [258, 100]])
 def test_prompts_whose_rows_are_not_whole_groups_of_a_thread(n):
-    """From about 370 rows on a thread of the rotary kernel takes two: 429 rows, 483 with rows of a second sequence; below it one."""
+    """261 rows (three blocks of 87), 270, and 360 with rows of a second sequence."""
+    test_7b_shaped_prompts("eagle", n, 64)
+
+
+@pytest.mark.parametrize("n", [[429], [381, 102]])
+def test_prompts_whose_last_row_is_alone_in_its_thread(n):
+    """From about 370 rows on a thread of the rotary kernel takes two: 429 rows, 483 with rows of a second sequence."""
     test_7b_shaped_prompts("eagle", n, 64)
 
 
