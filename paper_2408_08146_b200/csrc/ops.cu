@@ -384,7 +384,10 @@ __global__ void swiglu_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *_
 
 // SiLU is inlined: behind the calls of silu_f the second operand's partial sums were not requested before the first's were
 // used (us per launch, calls / inlined: one row of the 7B shape 3.18 / 2.95, 64 rows 5.8 / 5.5, 512 rows 24.4 / 22.7, prompts
-// of 509 tokens 22.5 / 20.9, 860 tokens 35.4 / 33.8, 13B 46.7 / 43.8).
+// of 509 tokens 22.5 / 20.9, 860 tokens 35.4 / 33.8, 13B 46.7 / 43.8).  One row per thread; one / two / four, inlined, at the
+// power cap: prompts 7B 360 tokens 14.4 / 15.4 / 17.6, 509 20.9 / 21.5 / 22.0, 860 34.2 / 34.5 / 33.6, 1020 40.6 / 40.9 / 41.7, 13B
+// 509 26.1 / 26.9 / 25.9, 860 44.1 / 42.6 / 42.2, 1020 52.2 / 51.2 / 49.4, verifications of 512 rows 19.7 / 21.7 / 22.0 and 25.3 / 26.7
+// / 28.3: four gain in the longest 13B prompts only, 0.3 % of a pass at most.
 template <typename T, int NS, bool SK>
 __global__ void __launch_bounds__(256) swiglu_vec_kernel(SplitIn gu, RowScale sc, T *__restrict__ act, T *__restrict__ act_lo, int F) {
   pdl_launch_dependents();
